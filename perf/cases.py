@@ -80,7 +80,15 @@ def listed():
 
 def draw(rng):
     """One more case: a cell on one of the grids it is run on, with a cut-off that the grid holds
-    the products of, an uneven k-mesh, and the options in any combination."""
+    the products of, an uneven k-mesh, and the options in any combination; no more work than the
+    largest listed one (an FP64 flop counted as four)."""
+    while True:
+        c = _draw(rng)
+        if work(c)["flops"] * (4 if c.get("prec") == "fp64" else 1) <= 3.0e11:
+            return c
+
+
+def _draw(rng):
     if rng.random() < 0.15:
         m = round(math.exp(rng.uniform(math.log(40), math.log(3000))))
         return _spectrum_case(m=m, m_total=round(math.exp(rng.uniform(math.log(m), math.log(20000)))),
