@@ -85,7 +85,9 @@ struct Profiler {
 
 ChainBase* make_chain_f64();
 ChainBase* make_chain_f32();
-int footprint_bytes(const ll_system_desc* d, size_t* out, std::string& err);
+// upper bound of the device bytes of a chain whose orbitals are transformed on a grid of `side`
+// points a side (ll_footprint takes the declared side)
+size_t footprint_bytes(const ll_system_desc* d, int side);
 
 #define LL_CK(call)                                                                    \
   do {                                                                                 \
@@ -97,8 +99,10 @@ int footprint_bytes(const ll_system_desc* d, size_t* out, std::string& err);
   } while (0)
 
 // Column/row tables of one sphere family, built on the host from the Miller lists.
+struct Extent { int lo[3], hi[3]; };   // a sphere's smallest and largest Miller index per axis
 struct HostSphere {
   int nks = 0, npw_pad = 0, ncol_max = 0, nrow_max = 0;
+  std::vector<Extent> ext;
   std::vector<int> npw, off, ncol, nrow, colstart;
   std::vector<int4> col, row;
 };
@@ -154,6 +158,7 @@ static inline bool build_sphere(int nks, const int* npw, const int* mil, int n, 
   std::vector<std::vector<int4>> cols(nks), rows(nks);
   std::vector<std::vector<int>> starts(nks);
   std::vector<const char*> kerr(nks, nullptr);
+  h.ext.resize(nks);
   // the tables of one sphere (independent per k: built on several host threads)
   auto one = [&](int k) -> const char* {
     const int* m = mil + 3L * h.off[k];
@@ -167,8 +172,11 @@ static inline bool build_sphere(int nks, const int* npw, const int* mil, int n, 
         if (!less) return "Miller indices of a sphere are not strictly lexicographic";
       }
     }
-    for (int a = 0; a < 3; ++a)
+    for (int a = 0; a < 3; ++a) {
       if (hi[a] - lo[a] >= n) return "a plane-wave sphere does not fit the FFT grid";
+      h.ext[k].lo[a] = lo[a];
+      h.ext[k].hi[a] = hi[a];
+    }
     int i = 0;
     while (i < npw[k]) {
       int j = i;
@@ -252,6 +260,75 @@ static inline void recip(const double a[3][3], double b[3][3]) {
     b[i][1] = f * (u[2] * v[0] - u[0] * v[2]);
     b[i][2] = f * (u[0] * v[1] - u[1] * v[0]);
   }
+}
+
+// The side W <= N of the grid the orbitals are transformed on.  The operator only ever
+// multiplies a potential with an orbital and keeps the product on sphere(k+Q), and the response
+// density is a product of two orbitals, so of V and v' only the components d = G - G' between
+// spheres of one k-point act, and n' has only those.  With every such difference in
+// |d| <= (W - 1)/2 on each axis, V and v' band-limited to that window and sampled on W points
+// give the same products on the spheres as the N points do (the sums G' + d reach 2 max|d| < W,
+// so nothing folds back), and n' on W points holds all of n'.  Only f_xc n' is a product on
+// the declared grid itself: n' is interpolated to it, multiplied, and band-limited back
+// (k_hxcw_*).  The smallest built side that holds the differences is taken: cells whose grid is
+// a size or more above the smallest product grid gain (25 Ry on 32^3: 24^3; 10 Ry on 18^3:
+// 16^3), the others keep W = N.  LL_PRUNE=0 or 1 in the environment: W = N.
+static inline int work_side(const ll_system_desc* d, const Extent* ek, const Extent* eq) {
+  const int n = d->nfft, nsym = d->sym ? d->nsym : 1;
+  const char* pe = getenv("LL_PRUNE");
+  if (pe && (pe[0] == '0' || pe[0] == '1') && pe[1] == 0) return n;
+  int dmax = 0, mmax = 0;
+  for (int k = 0; k < d->nks; ++k) {
+    const Extent &u = ek[k], &x = eq[k];
+    for (int a = 0; a < 3; ++a) {
+      dmax = std::max({dmax, x.hi[a] - x.lo[a], x.hi[a] - u.lo[a], u.hi[a] - x.lo[a]});
+      mmax = std::max({mmax, std::abs(u.lo[a]), std::abs(u.hi[a]), std::abs(x.lo[a]), std::abs(x.hi[a])});
+    }
+  }
+  if (nsym > 1) {
+    // the density averaged over the small group has the rotated differences too: all of
+    // |G| <= max|k+G| + max|k+Q+G| + |Q|, a ball the group's operations keep; they must be
+    // isometries of the lattice (M^T g M = g with g_ij = a_i . a_j)
+    double g[3][3], gmax = 0, r[2] = {0, 0}, q2 = 0;
+    for (int i = 0; i < 3; ++i)
+      for (int j = 0; j < 3; ++j) {
+        g[i][j] = 0;
+        for (int a = 0; a < 3; ++a) g[i][j] += d->lattice[i][a] * d->lattice[j][a];
+        gmax = std::max(gmax, std::abs(g[i][j]));
+      }
+    for (int s = 0; s < nsym; ++s) {
+      const int* m = d->sym + 9 * s;
+      for (int i = 0; i < 3; ++i)
+        for (int j = 0; j < 3; ++j) {
+          double t = 0;
+          for (int k = 0; k < 3; ++k)
+            for (int l = 0; l < 3; ++l) t += m[3 * k + i] * g[k][l] * m[3 * l + j];
+          if (std::abs(t - g[i][j]) > 1e-6 * gmax) return n;
+        }
+    }
+    double b[3][3];
+    recip(d->lattice, b);
+    for (int f = 0; f < 2; ++f) {
+      const int* m = f ? d->miller_kq : d->miller_k;
+      const int* np = f ? d->npw_kq : d->npw_k;
+      for (int k = 0; k < d->nks; ++k)
+        for (int i = 0; i < np[k]; ++i, m += 3) {
+          double t = 0;
+          for (int a = 0; a < 3; ++a) {
+            const double x = d->kcart[3 * k + a] + (f ? d->q_cart[a] : 0.0) + m[0] * b[0][a] + m[1] * b[1][a] + m[2] * b[2][a];
+            t += x * x;
+          }
+          r[f] = std::max(r[f], t);
+        }
+    }
+    for (int a = 0; a < 3; ++a) q2 += d->q_cart[a] * d->q_cart[a];
+    const double rad = std::sqrt(r[0]) + std::sqrt(r[1]) + std::sqrt(q2);
+    for (int a = 0; a < 3; ++a)
+      dmax = std::max(dmax, (int)std::min(1e6, rad * std::sqrt(g[a][a]) / (2.0 * 3.14159265358979323846) + 1e-9));
+  }
+  for (int s : kGridSides)
+    if (s < n && 2 * dmax + 1 <= s && mmax <= s) return s;
+  return n;
 }
 
 // Orbitals per batch of the per-plane kernel: enough axis-1 lines for the 128 threads when
@@ -346,19 +423,6 @@ class Chain : public ChainBase {
     if (!build_sphere(nks_, d->npw_kq, d->miller_kq, n, hq_, err)) return LL_EINVAL;
     for (int k = 0; k < nks_; ++k)
       if (d->npw_kq[k] < nbnd_ + 1) { err = "sphere smaller than the occupied manifold"; return LL_EINVAL; }
-    {   // the largest |m| of the k+Q spheres on any axis picks the pruning bound of the lines:
-        // the tightest built level (tight_prune(N), then N/4) that holds every sphere
-      int pmax = 0;
-      for (int k = 0; k < nks_; ++k)
-        for (int c = 0; c < hq_.ncol[k]; ++c) {
-          const int4 cl = hq_.col[(size_t)k * hq_.ncol_max + c];
-          pmax = std::max({pmax, std::abs(cl.x), std::abs(cl.y), std::abs(cl.z), std::abs(cl.z + cl.w - 1)});
-        }
-      const char* pe = getenv("LL_PRUNE");   // 0: unpruned lines; 1: the N/4 level only
-      const bool off = pe && pe[0] == '0' && pe[1] == 0, wide = pe && pe[0] == '1' && pe[1] == 0;
-      const int tight = tight_prune(n);
-      prune_ = off ? 0 : (!wide && tight > 0 && pmax <= tight) ? tight : (pmax <= n / 4 ? n / 4 : 0);
-    }
     if (!inputs_finite(d, err, false)) return LL_EINVAL;
     if (d->where != LL_WHERE_HOST && d->where != LL_WHERE_DEVICE) { err = "bad where"; return LL_EINVAL; }
     const bool dev_in = d->where == LL_WHERE_DEVICE;
@@ -428,22 +492,45 @@ class Chain : public ChainBase {
                   d->lattice[0][1] * (d->lattice[1][0] * d->lattice[2][2] - d->lattice[1][2] * d->lattice[2][0]) +
                   d->lattice[0][2] * (d->lattice[1][0] * d->lattice[2][1] - d->lattice[1][1] * d->lattice[2][0]));
     for (int a = 0; a < 3; ++a) q_[a] = d->q_cart[a];
+    W_ = work_side(d, hk_.ext.data(), hq_.ext.data());
+    {   // the largest |m| of the k+Q spheres on any axis picks the pruning bound of the lines:
+        // the tightest built level (tight_prune(W), then W/4) that holds every sphere
+      int pmax = 0;
+      for (int k = 0; k < nks_; ++k)
+        for (int c = 0; c < hq_.ncol[k]; ++c) {
+          const int4 cl = hq_.col[(size_t)k * hq_.ncol_max + c];
+          pmax = std::max({pmax, std::abs(cl.x), std::abs(cl.y), std::abs(cl.z), std::abs(cl.z + cl.w - 1)});
+        }
+      const char* pe = getenv("LL_PRUNE");   // 0: unpruned lines; 1: the W/4 level only
+      const bool off = pe && pe[0] == '0' && pe[1] == 0, wide = pe && pe[0] == '1' && pe[1] == 0;
+      const int tight = tight_prune(W_);
+      prune_ = off ? 0 : (!wide && tight > 0 && pmax <= tight) ? tight : (pmax <= W_ / 4 ? W_ / 4 : 0);
+    }
+    const int w = W_;
+    const long w3 = (long)w * w * w;
     const long n3 = (long)n * n * n;
     const int pq = hq_.npw_pad, pk = hk_.npw_pad;
     const long vq = (long)nks_ * nbnd_ * pq;  // one batch vector
     nvec_ = (flavour_ == LL_FLAVOUR_NH) ? 2 : 1;
 
-    // Hartree kernel 4 pi / |Q + G|^2 / N^3 over the box, [m3][m2][m1]
-    std::vector<T> wh(n3);
+    // Hartree kernel 4 pi / |Q + G|^2 / W^3 over the work grid's box, [m3][m2][m1]; Q + G = 0 is
+    // looked for over the whole declared box
+    std::vector<T> wh(w3);
     for (int i3 = 0; i3 < n; ++i3)
       for (int i2 = 0; i2 < n; ++i2)
         for (int i1 = 0; i1 < n; ++i1) {
-          const int m1 = i1 < n / 2 ? i1 : i1 - n, m2 = i2 < n / 2 ? i2 : i2 - n, m3 = i3 < n / 2 ? i3 : i3 - n;
+          const int m[3] = {i1 < n / 2 ? i1 : i1 - n, i2 < n / 2 ? i2 : i2 - n, i3 < n / 2 ? i3 : i3 - n};
           double g[3];
-          for (int a = 0; a < 3; ++a) g[a] = q_[a] + m1 * b[0][a] + m2 * b[1][a] + m3 * b[2][a];
+          for (int a = 0; a < 3; ++a) g[a] = q_[a] + m[0] * b[0][a] + m[1] * b[1][a] + m[2] * b[2][a];
           const double g2 = g[0] * g[0] + g[1] * g[1] + g[2] * g[2];
           if (!(g2 > 1e-20)) { err = "Q + G = 0 on the grid (Q is a reciprocal lattice vector)"; return LL_EINVAL; }
-          wh[((long)i3 * n + i2) * n + i1] = (T)(4.0 * 3.14159265358979323846 / g2 / (double)n3);
+          bool in = true;
+          int i[3];
+          for (int a = 0; a < 3; ++a) {
+            in = in && m[a] >= -(w / 2) && m[a] < (w + 1) / 2;
+            i[a] = m[a] < 0 ? m[a] + w : m[a];
+          }
+          if (in) wh[((long)i[2] * w + i[1]) * w + i[0]] = (T)(4.0 * 3.14159265358979323846 / g2 / (double)w3);
         }
     // kinetic 1/2 |k + Q + G|^2 on sphere(k+Q)
     std::vector<T> kin((size_t)nks_ * pq, T(0));
@@ -567,12 +654,12 @@ class Chain : public ChainBase {
     }
     const long nzp = (long)nks_ * npk_;               // partials per vector and step
     const long nzv = nzp * nvec_;
-    if ((rc = alloc(&whart_, n3)) || (rc = alloc(&kin_, (long)nks_ * pq)) || (rc = alloc(&uk_, (long)nks_ * nbnd_ * pk)) ||
+    if ((rc = alloc(&whart_, w3)) || (rc = alloc(&kin_, (long)nks_ * pq)) || (rc = alloc(&uk_, (long)nks_ * nbnd_ * pk)) ||
         (rc = alloc(&ukq_, vq)) || (rc = alloc(&bkq_, bkq_len)) || (rc = alloc(&eps_, (long)nks_ * nbnd_)) ||
-        (rc = alloc(&dij_, std::max(1, nproj_))) || (rc = alloc(&vloc_, n3)) || (rc = alloc(&rho_, n3)) ||
-        (rc = alloc(&fxc_, n3)) || (rc = ur_alloc((long)nks_ * nbnd_ * n3)) ||
-        (rc = alloc(&cbuf_, (long)norb * n * cb_ncol_)) || (rc = alloc(&nprt_, (long)ngroups_ * n3)) ||
-        (rc = alloc(&nr_, n3)) || (rc = alloc(&ng_, n3)) || (rc = alloc(&vpr_, n3)) ||
+        (rc = alloc(&dij_, std::max(1, nproj_))) || (rc = alloc(&vloc_, w3)) || (rc = alloc(&rho_, n3)) ||
+        (rc = alloc(&fxc_, n3)) || (rc = ur_alloc((long)nks_ * nbnd_ * w3)) ||
+        (rc = alloc(&cbuf_, (long)norb * w * cb_ncol_)) || (rc = alloc(&nprt_, (long)ngroups_ * w3)) ||
+        (rc = alloc(&nr_, w3)) || (rc = alloc(&ng_, w3)) || (rc = alloc(&vpr_, w3)) ||
         (rc = alloc(&y_, vq)) || (rc = alloc(&map_, (long)nks_ * pq)) || (rc = alloc(&part_, std::max(2L * nks_, nzv))) ||
         (rc = alloc(&spart_, nzp)) || (rc = alloc(&vecs_, 3L * nvec_ * vq)) ||
         (rc = alloc(&beta_, cap_ + 2)) || (rc = alloc(&gamma_, cap_ + 2)) || (rc = alloc(&z_, cap_ + 1)) ||
@@ -598,7 +685,7 @@ class Chain : public ChainBase {
                    (rc = alloc(&sp_coef_, nvec_ * (long)nks_ * (nproj_ + nbnd_) * nbnd_))))
       return rc;
     (void)err;
-    LL_CK(cudaMemcpyAsync(whart_, wh.data(), n3 * sizeof(T), cudaMemcpyHostToDevice, st_));
+    LL_CK(cudaMemcpyAsync(whart_, wh.data(), w3 * sizeof(T), cudaMemcpyHostToDevice, st_));
     LL_CK(cudaMemcpyAsync(kin_, kin.data(), kin.size() * sizeof(T), cudaMemcpyHostToDevice, st_));
     {
       int *offk = nullptr, *offq = nullptr;
@@ -610,13 +697,34 @@ class Chain : public ChainBase {
       k_pad_rows<T><<<dim3(nks_, nbnd_), 256, 0, st_>>>(large[0].p, offk, dk_.npw, nbnd_, hk_.npw_pad, ksc, uk_);
       k_pad_rows<T><<<dim3(nks_, nbnd_), 256, 0, st_>>>(large[1].p, offq, dq_.npw, nbnd_, pq, nullptr, ukq_);
       if (nproj_) k_pad_rows<T><<<dim3(nks_, nproj_), 256, 0, st_>>>(large[4].p, offq, dq_.npw, nproj_, pq, nullptr, bkq_);
-      k_grids_in<T><<<256, 256, 0, st_>>>(n, large[2].p, large[3].p, vloc_, rho_);
+      k_grid_in<double><<<256, 256, 0, st_>>>(n, large[3].p, rho_);
+      double *v1 = nullptr, *v2 = nullptr, *rd = nullptr;
+      std::vector<double> rh((size_t)n * w);
+      if (w < n) {   // V_loc band-limited to the work grid, one axis at a time (double)
+        if ((rc = alloc(&v1, (long)n * n * w)) || (rc = alloc(&v2, (long)n * w * w)) || (rc = alloc(&rd, (long)n * w)) ||
+            (rc = alloc(&rup_, (long)n * w)) || (rc = alloc(&t1_, (long)w * n * n)))
+          return rc;
+        resample_table(n, w, rh.data());
+        std::vector<T> rt(rh.begin(), rh.end());
+        LL_CK(cudaMemcpyAsync(rd, rh.data(), rh.size() * sizeof(double), cudaMemcpyHostToDevice, st_));
+        LL_CK(cudaMemcpyAsync(rup_, rt.data(), rt.size() * sizeof(T), cudaMemcpyHostToDevice, st_));
+        LL_CK(cudaStreamSynchronize(st_));   // rt ends here
+        k_resample_axis<<<256, 256, 0, st_>>>((long)n * n, n, 1, w, rd, large[2].p, v1);
+        k_resample_axis<<<256, 256, 0, st_>>>(n, n, w, w, rd, v1, v2);
+        k_resample_axis<<<256, 256, 0, st_>>>(1, n, (long)w * w, w, rd, v2, v1);
+        k_grid_in<T><<<256, 256, 0, st_>>>(w, v1, vloc_);
+      } else {
+        k_grid_in<T><<<256, 256, 0, st_>>>(n, large[2].p, vloc_);
+      }
       LL_CK(cudaGetLastError());
       LL_CK(cudaStreamSynchronize(st_));   // the caller may reuse its arrays once ll_create returns
       release(offk);
       release(offq);
       release(ksc);
       release(stage);
+      release(v1);
+      release(v2);
+      release(rd);
     }
     LL_CK(cudaMemcpyAsync(eps_, d->eps_k, sizeof(double) * nks_ * nbnd_, cudaMemcpyHostToDevice, st_));
     if (nproj_) LL_CK(cudaMemcpyAsync(dij_, d->dij, sizeof(double) * nproj_, cudaMemcpyHostToDevice, st_));
@@ -978,6 +1086,24 @@ class Chain : public ChainBase {
   }
 
  private:
+  // One axis of the band-limited resampling between N and W < N points, [N][W]:
+  // f(j/N) = sum_s R[j][s] f(s/W) for f with |d| <= (W - 1)/2; its transpose times W/N limits a
+  // function of the N points to those components and samples it on the W.
+  static void resample_table(int n, int w, double* r) {
+    const int dm = (w - 1) / 2;
+    for (int j = 0; j < n; ++j)
+      for (int s = 0; s < w; ++s) {
+        // the phase d (j/N - s/W) reduced exactly: an integer over N W
+        const long num = (long)j * w - (long)s * n, den = (long)n * w;
+        double t = 1.0;
+        for (int q = 1; q <= dm; ++q) {
+          const long p = ((num * q) % den + den) % den;
+          t += 2.0 * cos(2.0 * 3.14159265358979323846 * (double)p / (double)den);
+        }
+        r[(size_t)j * w + s] = t / w;
+      }
+  }
+
   // one batch operator application on nvec contiguous vectors (Eqs. 24-28)
   int op(int nvec, const cplx<T>* in, cplx<T>* out, int dens_vec, std::string& err) {
     int rc;
@@ -1064,7 +1190,7 @@ class Chain : public ChainBase {
     return LL_OK;
   }
   int launch_zfwd_proj(int nvec, const cplx<T>* in, cplx<T>* out, std::string& err) {
-    switch (N_) {
+    switch (W_) {
       case 12: return zfwd_proj_n<12>(nvec, in, out, err);
       case 16: return zfwd_proj_n<16>(nvec, in, out, err);
       case 18: return zfwd_proj_n<18>(nvec, in, out, err);
@@ -1204,7 +1330,7 @@ class Chain : public ChainBase {
     return LL_OK;
   }
   int launch_zinv_ph(int j, std::string& err) {
-    switch (N_) {
+    switch (W_) {
       case 12: return zinv_ph_n<12>(j, err);
       case 16: return zinv_ph_n<16>(j, err);
       case 18: return zinv_ph_n<18>(j, err);
@@ -1224,7 +1350,7 @@ class Chain : public ChainBase {
     return cudaGetLastError() == cudaSuccess ? LL_OK : LL_ECUDA;
   }
   int launch_zinv(const SphereDev& s, const cplx<T>* in, int nvec) {
-    switch (N_) {
+    switch (W_) {
       case 12: return zinv_n<12>(s, in, nvec);
       case 16: return zinv_n<16>(s, in, nvec);
       case 18: return zinv_n<18>(s, in, nvec);
@@ -1237,7 +1363,7 @@ class Chain : public ChainBase {
   }
   int groups_for(int norb) const {
     const int target = 4 * nsm_;
-    int g = std::max(1, (target + N_ - 1) / N_);
+    int g = std::max(1, (target + W_ - 1) / W_);
     return std::min(g, norb);
   }
   // Orbital groups of one plane-pass launch (grid N x groups): as many CTAs as fit on the
@@ -1250,7 +1376,7 @@ class Chain : public ChainBase {
         cudaGetLastError();
         occ = 1;
       }
-      cache = std::max(1, (occ * nsm_) / N_);
+      cache = std::max(1, (occ * nsm_) / W_);
     }
     return std::max(1, std::min(std::min(cache, ngroups_), norb));
   }
@@ -1340,7 +1466,7 @@ class Chain : public ChainBase {
     int dev = 0;
     cudaGetDevice(&dev);
     char key[256];
-    snprintf(key, sizeof(key), "%d/%zu/%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%d", dev, sizeof(T), N_, nks_, nbnd_,
+    snprintf(key, sizeof(key), "%d/%zu/%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%d", dev, sizeof(T), N_, W_, nks_, nbnd_,
              hq_.npw_pad, cb_ncol_, hq_.nrow_max, nproj_, (int)split_, xy_pair_, (int)prune_, nsm_);
     {
       std::lock_guard<std::mutex> lock(tune_mutex());
@@ -1368,14 +1494,14 @@ class Chain : public ChainBase {
       return LL_OK;
     };
     float ms = 0.f;
-    const bool can_pair = (N_ == 24 || N_ == 32 || N_ == 36 || N_ == 48) && xy_pair_ < 0;
+    const bool can_pair = (W_ == 24 || W_ == 32 || W_ == 36 || W_ == 48) && xy_pair_ < 0;
     rc = run(approx_ == LL_APPROX_IPA ? -1 : 0, &ms);   // warm-up: lazy module loads, attributes
     const int modes[3] = {XY_PASS1, XY_PASS1_DENS, XY_PASS2};
     for (int mi = 0; mi < 3 && rc == LL_OK; ++mi) {
       const int mode = modes[mi];
       if (mode != XY_PASS1 && approx_ == LL_APPROX_IPA) break;   // no density without K
       const int dens = mode == XY_PASS1 ? -1 : 0;
-      const int bdef = (mode == XY_PASS1) ? 384 / N_ : 256 / N_;
+      const int bdef = (mode == XY_PASS1) ? 384 / W_ : 256 / W_;
       std::vector<XyChoice> cand;
       for (int var = 0; var <= (can_pair ? 1 : 0); ++var) {
         cand.push_back({var, 0});                             // the occupancy-derived batch
@@ -1430,7 +1556,7 @@ class Chain : public ChainBase {
     return xy_nm<N, XY_STORE>(s, norb, o_off, -1, err);
   }
   int launch_xy(const SphereDev& s, int norb, int o_off, int dens_vec, int mode, std::string& err) {
-    switch (N_) {
+    switch (W_) {
       case 12: return xy_n<12>(s, norb, o_off, dens_vec, mode, err);
       case 16: return xy_n<16>(s, norb, o_off, dens_vec, mode, err);
       case 18: return xy_n<18>(s, norb, o_off, dens_vec, mode, err);
@@ -1444,19 +1570,36 @@ class Chain : public ChainBase {
   template <int N>
   int hxc_n(std::string& err) {
     const T scale = (T)(4.0 / (omega_ * nks_));
+    const cplx<T>* np = nprt_;   // the density's groups, or their average over the small group of Q
+    int ng = last_ng_;
+    T sc = scale;
+    const bool wide = W_ < N_ && approx_ == LL_APPROX_TDDFT;   // f_xc n' on the declared grid
     if (nsym_ > 1) {   // the density averaged over the small group of Q, then the same transforms
-      k_dens_sym<T><<<4 * nsm_, 256, 0, st_>>>(nprt_, last_ng_, N, scale, nsym_, sym_, ng_);
-      k_hxc_fwd<T, N><<<N, 256, 0, st_>>>(ng_, 1, T(1), nr_, ng_);
-    } else {
-      k_hxc_fwd<T, N><<<N, 256, 0, st_>>>(nprt_, last_ng_, scale, nr_, ng_);
+      cplx<T>* av = wide ? nr_ : ng_;
+      k_dens_sym<T><<<4 * nsm_, 256, 0, st_>>>(nprt_, last_ng_, N, scale, nsym_, sym_, av);
+      np = av;
+      ng = 1;
+      sc = T(1);
     }
-    k_hxc_z<T, N><<<(N * N + 63) / 64, 64, 0, st_>>>(ng_, whart_);
-    k_hxc_inv<T, N><<<N, 64, 0, st_>>>(ng_, nr_, fxc_, vpr_);
+    if (wide) {
+      int rc;
+      const size_t s1 = hxcw_fwd_smem<T>(N, N_), s2 = hxcw_mid_smem<T>(N, N_), s3 = hxcw_inv_smem<T>(N, N_);
+      if ((rc = set_smem(k_hxcw_fwd<T, N>, s1, err)) || (rc = set_smem(k_hxcw_mid<T, N>, s2, err)) ||
+          (rc = set_smem(k_hxcw_inv<T, N>, s3, err)))
+        return rc;
+      k_hxcw_fwd<T, N><<<dim3(N, 1 + kHxcSlices), 256, s1, st_>>>(np, ng, sc, N_, rup_, ng_, t1_);
+      k_hxcw_mid<T, N><<<hxcw_mid_blocks(N, N_), 128, s2, st_>>>(ng_, whart_, N_, rup_, fxc_, t1_);
+      k_hxcw_inv<T, N><<<dim3(N, kHxcSlices), 256, s3, st_>>>(ng_, N_, rup_, t1_, vpr_);
+    } else {
+      k_hxc_fwd<T, N><<<N, 256, 0, st_>>>(np, ng, sc, nr_, ng_);
+      k_hxc_z<T, N><<<(N * N + 63) / 64, 64, 0, st_>>>(ng_, whart_);
+      k_hxc_inv<T, N><<<N, 64, 0, st_>>>(ng_, nr_, fxc_, vpr_);
+    }
     LL_CK(cudaGetLastError());
     return LL_OK;
   }
   int launch_hxc(std::string& err) {
-    switch (N_) {
+    switch (W_) {
       case 12: return hxc_n<12>(err);
       case 16: return hxc_n<16>(err);
       case 18: return hxc_n<18>(err);
@@ -1513,6 +1656,9 @@ class Chain : public ChainBase {
   // The u_{vk}(r) grids: own (counted in bytes_, freed with the last chain that uses them) or
   // the donor's.
   int ur_alloc(long count) {
+    // (a lender that transforms on another grid side, which depends on the spheres at k+Q, has
+    // grids of another side: this chain then builds its own)
+    if (donor_ && donor_->W_ != W_) donor_ = nullptr;
     if (donor_) {
       ur_share_ = donor_->ur_share_;
       ur_ = donor_->ur_;
@@ -1590,7 +1736,8 @@ class Chain : public ChainBase {
   cplx<T>* Wp() { return vecs_ + 5 * vq(); }
 
   cudaStream_t st_ = nullptr;
-  int N_ = 0, nks_ = 0, nbnd_ = 0, nproj_ = 0, approx_ = 0, flavour_ = 0, cap_ = 0, nvec_ = 1, ngroups_ = 1;
+  int N_ = 0, W_ = 0;       // declared FFT grid side, side of the grid the orbitals are transformed on
+  int nks_ = 0, nbnd_ = 0, nproj_ = 0, approx_ = 0, flavour_ = 0, cap_ = 0, nvec_ = 1, ngroups_ = 1;
   int nsm_ = 152;           // SMs of the device
   int xy_groups_[4] = {0, 0, 0, 0};   // plane-pass groups per mode (one wave), 0 = not yet known
   int cb_ncol_ = 0, steps_ = 0, queued_ = 0, spec_cap_ = 0, last_ng_ = 1;
@@ -1622,6 +1769,8 @@ class Chain : public ChainBase {
   cplx<T> *uk_ = nullptr, *ukq_ = nullptr, *bkq_ = nullptr, *ur_ = nullptr, *cbuf_ = nullptr, *nprt_ = nullptr;
   cplx<T> *nr_ = nullptr, *ng_ = nullptr, *vpr_ = nullptr, *y_ = nullptr, *vecs_ = nullptr;
   cplx<T>* scratch_ = nullptr;
+  T* rup_ = nullptr;             // W_ < N_: resampling table [N_][W_] (resample_table)
+  cplx<T>* t1_ = nullptr;        // W_ < N_: n', then f_xc n', on W_ planes of the declared N_ x N_ grid
   cplx<double> *spart_ = nullptr, *gamma_ = nullptr, *z_ = nullptr, *zpart_ = nullptr, *spec_out_ = nullptr;
   ExtrapTail* tail_ = nullptr;   // continuation constants of the coefficients (spectrum)
   int* jdev_ = nullptr;          // device step counter of the pseudo-Hermitian recursion

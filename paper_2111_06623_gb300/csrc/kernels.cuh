@@ -385,6 +385,209 @@ __global__ void __launch_bounds__(64) k_hxc_inv(const cplx<T>* __restrict__ ng, 
 }
 
 // ---------------------------------------------------------------------------------------
+// The response potential where the orbitals are transformed on a work grid of W < n points a
+// side (the chain's work_side): n' is on the W grid, which holds all its components, the Hartree
+// term stays there, and f_xc n' is formed on the declared n grid.  Both directions between the
+// grids are real n x W matrices per axis (rt [n][W], resample_table): a 24 x 32 matrix is a few
+// dozen FMAs per point, in one pass where a pair of zero-padded FFTs would take two, and the axis-3
+// product up, f_xc, and down again stay in one CTA.  Three launches, as on the declared grid alone.
+//   k_hxcw_fwd  per plane s3: groups summed; slice 0: 2D FFT (Hartree); the other kHxcSlices:
+//               n' interpolated to n x n points of the plane, columns j1 split over the slices
+//               -> t1[s3][j2][j1]
+//   k_hxcw_mid  Hartree lines (axis-3 FFT, kernel, inverse) and, per (j2, j1) column of t1, axis 3
+//               up, times f_xc, axis 3 down, in place
+//   k_hxcw_inv  per plane s3 and slice of s1: inverse 2D FFT of the Hartree part, t1 limited to
+//               W x W points, their sum v'(s3) to vpr.  (Every slice repeats the plane's FFT: its
+//               2 W lines are one warp's work beside the other warps' matrix product.)
+constexpr int kHxcSlices = 4;
+constexpr int kHxcCols = 8;      // t1 columns per CTA of k_hxcw_mid
+static inline __host__ __device__ int hxcw_jslice(int n) { return (n + kHxcSlices - 1) / kHxcSlices; }
+static inline __host__ __device__ int hxcw_sslice(int w) { return (w + kHxcSlices - 1) / kHxcSlices; }
+template <typename T> size_t hxcw_fwd_smem(int w, int n) {
+  return sizeof(cplx<T>) * ((size_t)w * (w + 1) + (size_t)w * hxcw_jslice(n)) + sizeof(T) * (size_t)n * w;
+}
+template <typename T> size_t hxcw_mid_smem(int w, int n) {
+  return sizeof(cplx<T>) * (size_t)kHxcCols * (w + n) + sizeof(T) * (size_t)n * w;
+}
+template <typename T> size_t hxcw_inv_smem(int w, int n) {
+  return sizeof(cplx<T>) * ((size_t)w * (w + 1) + (size_t)n * (n + 1) + (size_t)(n + w) * hxcw_sslice(w)) +
+         sizeof(T) * (size_t)n * w;
+}
+static inline int hxcw_mid_blocks(int w, int n) { return (w * w + 31) / 32 + (n * n + kHxcCols - 1) / kHxcCols; }
+
+template <typename T, int W>
+__global__ void __launch_bounds__(256) k_hxcw_fwd(const cplx<T>* __restrict__ nprt, int ngroups, T scale, int n,
+                                                 const T* __restrict__ rt, cplx<T>* __restrict__ ng,
+                                                 cplx<T>* __restrict__ t1) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cplx<T>* P = reinterpret_cast<cplx<T>*>(smem_raw);        // [W][W + 1]
+  const int js = hxcw_jslice(n);
+  cplx<T>* Q = P + W * (W + 1);                              // [W][js]
+  T* R = reinterpret_cast<T*>(Q + W * js);                   // [n][W]
+  const int iz = blockIdx.x, sl = (int)blockIdx.y - 1;
+  const long plane = (long)W * W;
+  for (int i = threadIdx.x; i < W * W; i += blockDim.x) {
+    const cplx<T>* src = nprt + iz * plane + i;
+    cplx<T> acc = czero<T>();
+#pragma unroll 8
+    for (int gi = 0; gi < ngroups; ++gi) acc = acc + src[(long)gi * W * plane];
+    P[(i / W) * (W + 1) + i % W] = acc * scale;
+  }
+  if (sl >= 0)
+    for (int i = threadIdx.x; i < n * W; i += blockDim.x) R[i] = rt[i];
+  __syncthreads();
+  if (sl < 0) {
+    if (threadIdx.x < W) {  // axis 1, row s2
+      cplx<T>* row = P + threadIdx.x * (W + 1);
+      cplx<T> l[W];
+#pragma unroll
+      for (int p = 0; p < W; ++p) l[p] = row[p];
+      fft_line<T, W, -1>(l);
+#pragma unroll
+      for (int p = 0; p < W; ++p) row[p] = l[p];
+    }
+    __syncthreads();
+    if (threadIdx.x < W) {  // axis 2, column m1
+      const int m1 = threadIdx.x;
+      cplx<T> l[W];
+#pragma unroll
+      for (int p = 0; p < W; ++p) l[p] = P[p * (W + 1) + m1];
+      fft_line<T, W, -1>(l);
+#pragma unroll
+      for (int p = 0; p < W; ++p) ng[iz * plane + p * W + m1] = l[p];
+    }
+    return;
+  }
+  const int j0 = sl * js, nj = min(js, n - j0);
+  for (int i = threadIdx.x; i < W * nj; i += blockDim.x) {   // axis 1
+    const int s2 = i / nj, jl = i - s2 * nj;
+    const T* r = R + (j0 + jl) * W;
+    const cplx<T>* row = P + s2 * (W + 1);
+    cplx<T> acc = czero<T>();
+#pragma unroll
+    for (int s = 0; s < W; ++s) acc = acc + row[s] * r[s];
+    Q[s2 * js + jl] = acc;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n * nj; i += blockDim.x) {   // axis 2
+    const int j2 = i / nj, jl = i - j2 * nj;
+    const T* r = R + j2 * W;
+    cplx<T> acc = czero<T>();
+#pragma unroll
+    for (int s = 0; s < W; ++s) acc = acc + Q[s * js + jl] * r[s];
+    t1[((long)iz * n + j2) * n + j0 + jl] = acc;
+  }
+}
+
+template <typename T, int W>
+__global__ void __launch_bounds__(128) k_hxcw_mid(cplx<T>* __restrict__ ng, const T* __restrict__ whart, int n,
+                                                 const T* __restrict__ rt, const T* __restrict__ fxc,
+                                                 cplx<T>* __restrict__ t1) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int NH = (W * W + 31) / 32;   // CTAs of the Hartree lines
+  const long plane = (long)W * W;
+  if (blockIdx.x < NH) {
+    const int line = blockIdx.x * 32 + threadIdx.x;   // (m2, m1)
+    if (threadIdx.x >= 32 || line >= W * W) return;
+    cplx<T> l[W];
+#pragma unroll
+    for (int p = 0; p < W; ++p) l[p] = ng[p * plane + line];
+    fft_line<T, W, -1>(l);
+#pragma unroll
+    for (int p = 0; p < W; ++p) l[p] = l[p] * whart[p * plane + line];
+    fft_line<T, W, +1>(l);
+#pragma unroll
+    for (int p = 0; p < W; ++p) ng[p * plane + line] = l[p];
+    return;
+  }
+  cplx<T>* X = reinterpret_cast<cplx<T>*>(smem_raw);   // [W][kHxcCols]
+  cplx<T>* Y = X + W * kHxcCols;                        // [n][kHxcCols]
+  T* R = reinterpret_cast<T*>(Y + n * kHxcCols);        // [n][W]
+  const int c0 = (blockIdx.x - NH) * kHxcCols, nn = n * n;
+  const int cl = threadIdx.x % kHxcCols, ln = threadIdx.x / kHxcCols, nl = blockDim.x / kHxcCols;
+  const bool on = c0 + cl < nn;
+  for (int i = threadIdx.x; i < n * W; i += blockDim.x) R[i] = rt[i];
+  for (int s = ln; s < W; s += nl) X[s * kHxcCols + cl] = on ? t1[(long)s * nn + c0 + cl] : czero<T>();
+  __syncthreads();
+  for (int j = ln; j < n; j += nl) {
+    const T* r = R + j * W;
+    cplx<T> acc = czero<T>();
+#pragma unroll
+    for (int s = 0; s < W; ++s) acc = acc + X[s * kHxcCols + cl] * r[s];
+    Y[j * kHxcCols + cl] = acc * (on ? fxc[(long)j * nn + c0 + cl] : T(0));
+  }
+  __syncthreads();
+  const T sc = T(W) / T(n);
+  for (int s = ln; s < W; s += nl) {
+    cplx<T> acc = czero<T>();
+    for (int j = 0; j < n; ++j) acc = acc + Y[j * kHxcCols + cl] * R[j * W + s];
+    if (on) t1[(long)s * nn + c0 + cl] = acc * sc;
+  }
+}
+
+template <typename T, int W>
+__global__ void __launch_bounds__(256) k_hxcw_inv(const cplx<T>* __restrict__ ng, int n, const T* __restrict__ rt,
+                                                 const cplx<T>* __restrict__ t1, cplx<T>* __restrict__ vpr) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int ss = hxcw_sslice(W), s0 = blockIdx.y * ss, ns = min(ss, W - s0);
+  cplx<T>* F = reinterpret_cast<cplx<T>*>(smem_raw);       // [W][W + 1] the Hartree part
+  cplx<T>* X = F + W * (W + 1);                             // [n][n + 1] f_xc n'
+  cplx<T>* Q = X + n * (n + 1);                             // [n][ss]
+  cplx<T>* O = Q + n * ss;                                  // [W][ss]
+  T* R = reinterpret_cast<T*>(O + W * ss);                  // [n][W]
+  const int iz = blockIdx.x;
+  const long plane = (long)W * W;
+  for (int i = threadIdx.x; i < W * W; i += blockDim.x) F[(i / W) * (W + 1) + i % W] = ng[iz * plane + i];
+  for (int i = threadIdx.x; i < n * n; i += blockDim.x) X[(i / n) * (n + 1) + i % n] = t1[(long)iz * n * n + i];
+  for (int i = threadIdx.x; i < n * W; i += blockDim.x) R[i] = rt[i];
+  __syncthreads();
+  constexpr int NF = (W + 31) / 32 * 32;   // threads of the FFT lines, the rest: the matrix product
+  const T sc = T(W) / T(n);
+  if (threadIdx.x < NF) {
+    if (threadIdx.x < W) {  // axis 2 inverse, column m1
+      const int m1 = threadIdx.x;
+      cplx<T> l[W];
+#pragma unroll
+      for (int p = 0; p < W; ++p) l[p] = F[p * (W + 1) + m1];
+      fft_line<T, W, +1>(l);
+#pragma unroll
+      for (int p = 0; p < W; ++p) F[p * (W + 1) + m1] = l[p];
+    }
+  } else {
+    for (int i = threadIdx.x - NF; i < n * ns; i += blockDim.x - NF) {   // axis 1
+      const int j2 = i / ns, sl = i - j2 * ns;
+      cplx<T> acc = czero<T>();
+      for (int j = 0; j < n; ++j) acc = acc + X[j2 * (n + 1) + j] * R[j * W + s0 + sl];
+      Q[j2 * ss + sl] = acc * sc;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < NF) {
+    if (threadIdx.x < W) {  // axis 1 inverse, row s2
+      cplx<T>* row = F + threadIdx.x * (W + 1);
+      cplx<T> l[W];
+#pragma unroll
+      for (int p = 0; p < W; ++p) l[p] = row[p];
+      fft_line<T, W, +1>(l);
+#pragma unroll
+      for (int p = 0; p < W; ++p) row[p] = l[p];
+    }
+  } else {
+    for (int i = threadIdx.x - NF; i < W * ns; i += blockDim.x - NF) {   // axis 2
+      const int s2 = i / ns, sl = i - s2 * ns;
+      cplx<T> acc = czero<T>();
+      for (int j = 0; j < n; ++j) acc = acc + Q[j * ss + sl] * R[j * W + s2];
+      O[s2 * ss + sl] = acc * sc;
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < W * ns; i += blockDim.x) {
+    const int s2 = i / ns, sl = i - s2 * ns;
+    vpr[iz * plane + s2 * W + s0 + sl] = F[s2 * (W + 1) + s0 + sl] + O[s2 * ss + sl];
+  }
+}
+
+// ---------------------------------------------------------------------------------------
 // Reductions.  Every sum below runs in a fixed order (per-thread strided partial sums, lanes,
 // then warps), so results are bitwise reproducible.
 __device__ __forceinline__ double warp_sum(double v) {
@@ -1015,16 +1218,26 @@ __global__ void k_pad_rows(const double* __restrict__ src, const int* __restrict
     d[g] = g < n ? mk((T)(f * s[2 * g]), (T)(f * s[2 * g + 1])) : czero<T>();
 }
 
-// Grids [j1][j2][j3] -> [j3][j2][j1]: V in T, the density in double.
+// A grid [j1][j2][j3] -> [j3][j2][j1] in T.
 template <typename T>
-__global__ void k_grids_in(int n, const double* __restrict__ vloc, const double* __restrict__ rho, T* __restrict__ vl,
-                           double* __restrict__ rh) {
+__global__ void k_grid_in(int n, const double* __restrict__ src, T* __restrict__ dst) {
   const long n3 = (long)n * n * n;
-  for (long dst = (long)blockIdx.x * blockDim.x + threadIdx.x; dst < n3; dst += (long)gridDim.x * blockDim.x) {
-    const long j1 = dst % n, j2 = (dst / n) % n, j3 = dst / ((long)n * n);
-    const long src = (j1 * n + j2) * n + j3;
-    vl[dst] = (T)vloc[src];
-    rh[dst] = rho[src];
+  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += (long)gridDim.x * blockDim.x) {
+    const long j1 = i % n, j2 = (i / n) % n, j3 = i / ((long)n * n);
+    dst[i] = (T)src[(j1 * n + j2) * n + j3];
+  }
+}
+
+// One axis of a grid band-limited and sampled on w of its n points: in [na][n][nb] ->
+// out [na][w][nb] = (w/n) sum_j r[j][s] in[.][j][.] (r: the resampling table [n][w]).
+static __global__ void k_resample_axis(long na, int n, long nb, int w, const double* __restrict__ r,
+                                       const double* __restrict__ in, double* __restrict__ out) {
+  const double sc = (double)w / (double)n;
+  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < na * w * nb; i += (long)gridDim.x * blockDim.x) {
+    const long b = i % nb, s = (i / nb) % w, a = i / (nb * w);
+    double t = 0.0;
+    for (int j = 0; j < n; ++j) t += r[(long)j * w + s] * in[(a * n + j) * nb + b];
+    out[i] = t * sc;
   }
 }
 

@@ -80,6 +80,46 @@ int fma_peak(double* tflops, cudaStream_t st) {
 }  // namespace
 
 
+namespace ll {
+size_t footprint_bytes(const ll_system_desc* d, int side) {
+  const size_t elem = (d->precision == LL_PREC_FP64) ? 16 : 8;
+  int mk = 1, mq = 1;
+  for (int k = 0; k < d->nks; ++k) {
+    mk = d->npw_k[k] > mk ? d->npw_k[k] : mk;
+    mq = d->npw_kq[k] > mq ? d->npw_kq[k] : mq;
+  }
+  const size_t pk = (mk + 3) / 4 * 4, pq = (mq + 3) / 4 * 4;
+  const size_t n = d->nfft, w = side, n3 = n * n * n, w3 = w * w * w;
+  const size_t nvec = (d->flavour == LL_FLAVOUR_NH) ? 2 : 1;
+  const size_t vq = (size_t)d->nks * d->nbnd * pq;
+  const size_t orb = (size_t)d->nks * d->nbnd;
+  // columns per sphere are at most the sphere size; bounded by pq for the estimate
+  const size_t cb = nvec * orb * w * pq;
+  // density slot planes: 4 per SM of the current device (152 where none can be queried)
+  int nsm = 152;
+  {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+      nsm = std::max(nsm, n);
+    cudaGetLastError();
+  }
+  const size_t ngroups = (4 * (size_t)nsm + w - 1) / w;
+  // vectors: 3 nvec Lanczos vectors, nvec partial copies, y, U_{k+Q}, and the 2-vector scratch
+  // of the plane-pass tuner and ll_apply
+  size_t b = elem * (vq * (3 * nvec + nvec + 2 + 2) + orb * pk + orb * w3 + cb + ngroups * w3 + 3 * w3 +
+                     (size_t)d->nks * d->nproj * pq);
+  // Lanczos partials: up to max(bands, plane-wave chunks) per k and step (band groups or the
+  // split path), and the split path's chunk partials and coefficient blocks
+  const size_t npk = (size_t)std::max(d->nbnd, (int)((pq + 511) / 512));
+  const size_t pairs = (size_t)(d->nproj + d->nbnd) * d->nbnd;
+  b += (elem / 2) * (2 * n3 + (size_t)d->nks * pq) + 8 * n3 +
+       40 * (size_t)(d->max_steps + 2) * (d->nks * npk + 2) + 48 * nvec * (size_t)d->nks * npk * pairs;
+  if (w < n) b += elem * (w * n * n + n * w);   // between the grids: n' on W planes, the table
+  if (d->occ_k) b += 32 * (size_t)d->nks * d->nbnd * d->nbnd;   // the metal's projector tables
+  return b;
+}
+}  // namespace ll
+
 extern "C" {
 
 const char* ll_last_error(void) { return g_err.c_str(); }
@@ -465,40 +505,7 @@ int ll_bytes(ll_handle* h, size_t* bytes) {
 int ll_footprint(const ll_system_desc* d, size_t* bytes) {
   if (!d || !bytes || !d->npw_k || !d->npw_kq || d->nks < 1 || d->nbnd < 1 || d->nfft < 1)
     return fail(LL_EINVAL, "bad footprint arguments");
-  const size_t elem = (d->precision == LL_PREC_FP64) ? 16 : 8;
-  int mk = 1, mq = 1;
-  for (int k = 0; k < d->nks; ++k) {
-    mk = d->npw_k[k] > mk ? d->npw_k[k] : mk;
-    mq = d->npw_kq[k] > mq ? d->npw_kq[k] : mq;
-  }
-  const size_t pk = (mk + 3) / 4 * 4, pq = (mq + 3) / 4 * 4;
-  const size_t n3 = (size_t)d->nfft * d->nfft * d->nfft;
-  const size_t nvec = (d->flavour == LL_FLAVOUR_NH) ? 2 : 1;
-  const size_t vq = (size_t)d->nks * d->nbnd * pq;
-  const size_t orb = (size_t)d->nks * d->nbnd;
-  // columns per sphere are at most the sphere size; bounded by pq for the estimate
-  const size_t cb = nvec * orb * d->nfft * pq;
-  // density slot planes: 4 per SM of the current device (152 where none can be queried)
-  int nsm = 152;
-  {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
-      nsm = std::max(nsm, n);
-    cudaGetLastError();
-  }
-  const size_t ngroups = (4 * (size_t)nsm + d->nfft - 1) / d->nfft;
-  // vectors: 3 nvec Lanczos vectors, nvec partial copies, y, U_{k+Q}, and the 2-vector scratch
-  // of the plane-pass tuner and ll_apply
-  size_t b = elem * (vq * (3 * nvec + nvec + 2 + 2) + orb * pk + orb * n3 + cb + ngroups * n3 + 3 * n3 +
-                     (size_t)d->nks * d->nproj * pq);
-  // Lanczos partials: up to max(bands, plane-wave chunks) per k and step (band groups or the
-  // split path), and the split path's chunk partials and coefficient blocks
-  const size_t npk = (size_t)std::max(d->nbnd, (int)((pq + 511) / 512));
-  const size_t pairs = (size_t)(d->nproj + d->nbnd) * d->nbnd;
-  b += (elem / 2) * (2 * n3 + (size_t)d->nks * pq) + 8 * n3 +
-       40 * (size_t)(d->max_steps + 2) * (d->nks * npk + 2) + 48 * nvec * (size_t)d->nks * npk * pairs;
-  if (d->occ_k) b += 32 * (size_t)d->nks * d->nbnd * d->nbnd;   // the metal's projector tables
-  *bytes = b;
+  *bytes = ll::footprint_bytes(d, d->nfft);
   return LL_OK;
 }
 
