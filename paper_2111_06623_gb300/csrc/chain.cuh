@@ -86,8 +86,9 @@ struct Profiler {
 ChainBase* make_chain_f64();
 ChainBase* make_chain_f32();
 // upper bound of the device bytes of a chain whose orbitals are transformed on a grid of `side`
-// points a side (ll_footprint takes the declared side)
-size_t footprint_bytes(const ll_system_desc* d, int side);
+// points a side, with at most `cols` columns per sphere (ll_footprint, which reads no Miller
+// index, takes the declared side and one column per plane wave)
+size_t footprint_bytes(const ll_system_desc* d, int side, int cols);
 
 #define LL_CK(call)                                                                    \
   do {                                                                                 \

@@ -81,7 +81,7 @@ int fma_peak(double* tflops, cudaStream_t st) {
 
 
 namespace ll {
-size_t footprint_bytes(const ll_system_desc* d, int side) {
+size_t footprint_bytes(const ll_system_desc* d, int side, int cols) {
   const size_t elem = (d->precision == LL_PREC_FP64) ? 16 : 8;
   int mk = 1, mq = 1;
   for (int k = 0; k < d->nks; ++k) {
@@ -93,8 +93,7 @@ size_t footprint_bytes(const ll_system_desc* d, int side) {
   const size_t nvec = (d->flavour == LL_FLAVOUR_NH) ? 2 : 1;
   const size_t vq = (size_t)d->nks * d->nbnd * pq;
   const size_t orb = (size_t)d->nks * d->nbnd;
-  // columns per sphere are at most the sphere size; bounded by pq for the estimate
-  const size_t cb = nvec * orb * w * pq;
+  const size_t cb = nvec * orb * w * (size_t)(cols + 1);   // rows of an even length
   // density slot planes: 4 per SM of the current device (152 where none can be queried)
   int nsm = 152;
   {
@@ -505,7 +504,9 @@ int ll_bytes(ll_handle* h, size_t* bytes) {
 int ll_footprint(const ll_system_desc* d, size_t* bytes) {
   if (!d || !bytes || !d->npw_k || !d->npw_kq || d->nks < 1 || d->nbnd < 1 || d->nfft < 1)
     return fail(LL_EINVAL, "bad footprint arguments");
-  *bytes = ll::footprint_bytes(d, d->nfft);
+  int mq = 1;
+  for (int k = 0; k < d->nks; ++k) mq = std::max(mq, d->npw_kq[k]);
+  *bytes = ll::footprint_bytes(d, d->nfft, (mq + 3) / 4 * 4 - 1);
   return LL_OK;
 }
 

@@ -428,20 +428,25 @@ int ll_submit(ll_server* s, const ll_job_desc* jd, uint64_t* job_id) {
   j->eta = jd->eta_ev;
   {   // admitted by the bytes of the grid the chain will transform on (at most ll_footprint's)
     std::vector<ll::Extent> e[2];
+    int cols = 1;
     for (int f = 0; f < 2; ++f) {
       const int* m = f ? j->desc.miller_kq : j->desc.miller_k;
       for (int k = 0; k < j->desc.nks; ++k) {
         const int np = (f ? j->desc.npw_kq : j->desc.npw_k)[k];
         ll::Extent x{{m[0], m[1], m[2]}, {m[0], m[1], m[2]}};
-        for (int i = 0; i < np; ++i, m += 3)
+        int nc = 1;
+        for (int i = 0; i < np; ++i, m += 3) {
+          nc += i > 0 && (m[0] != m[-3] || m[1] != m[-2]);
           for (int a = 0; a < 3; ++a) {
             x.lo[a] = std::min(x.lo[a], m[a]);
             x.hi[a] = std::max(x.hi[a], m[a]);
           }
+        }
+        cols = std::max(cols, nc);
         e[f].push_back(x);
       }
     }
-    fp = std::min(fp, ll::footprint_bytes(&j->desc, ll::work_side(&j->desc, e[0].data(), e[1].data())) +
+    fp = std::min(fp, ll::footprint_bytes(&j->desc, ll::work_side(&j->desc, e[0].data(), e[1].data()), cols) +
                           LL_SPECTRUM_BYTES(jd->n_omega));
   }
   j->footprint = fp;
