@@ -1019,7 +1019,7 @@ class Chain : public ChainBase {
       if (!tail_ && (rc = alloc(&tail_, 1))) return rc;
       k_extrap_tail<<<1, 256, 0, st_>>>(m, kind, beta_, gamma_, tail_);
     }
-    k_spectrum<<<(nw + 127) / 128, 128, 0, st_>>>(m, m_total, m_total > m ? tail_ : nullptr, beta_, gamma_, z_, nw,
+    k_spectrum<<<(nw + 31) / 32, 32, 0, st_>>>(m, m_total, m_total > m ? tail_ : nullptr, beta_, gamma_, z_, nw,
                                                   spec_w_, eta_ev / ha, 4.0 / omega_,
                                                   4.0 * 3.14159265358979323846 / q2, spec_out_, spec_out_ + nw,
                                                   spec_out_ + 2L * nw);

@@ -1280,7 +1280,7 @@ __global__ void __launch_bounds__(128) k_dot_re(int nks, int nbnd, int npw_pad, 
 // = u_1 where A^T u = z, eliminated from the bottom row up (the continued fraction):
 //   d_M = w, r_M = z_M;  d_j = w - beta_{j+1} gamma_{j+1} / d_{j+1},
 //   r_j = z_j + beta_{j+1} r_{j+1} / d_{j+1};  u_1 = r_1 / d_1.
-// chi = pref b_1 u_1, eps^-1 = 1 + v_Q chi, eps = 1/eps^-1.  One thread per frequency.
+// chi = pref b_1 u_1, eps^-1 = 1 + v_Q chi, eps = 1/eps^-1.
 __device__ __forceinline__ cplx<double> cdiv(cplx<double> a, cplx<double> b) {
   const double d = b.x * b.x + b.y * b.y;
   return mk((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
@@ -1329,27 +1329,103 @@ static __global__ void __launch_bounds__(256) k_extrap_tail(int m, int kind, con
   }
 }
 
-// m_total > m continues the chain with `tail` (T grows to m_total x m_total; z stays m long).
-static __global__ void k_spectrum(int m, int m_total, const ExtrapTail* __restrict__ tail,
-                                  const double* __restrict__ beta, const cplx<double>* __restrict__ gamma,
-                                  const cplx<double>* __restrict__ z, int nw, const double* __restrict__ w_ha,
-                                  double eta, double pref, double vq, cplx<double>* __restrict__ chi,
-                                  cplx<double>* __restrict__ epsi, cplx<double>* __restrict__ eps) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nw) return;
-  if (m_total < m || !tail) m_total = m;
-  const cplx<double> w = mk(w_ha[i], eta);
-  cplx<double> d = w, r = (m_total > m) ? mk(0.0, 0.0) : z[m - 1];
-  for (int j = m_total - 2; j >= 0; --j) {
-    const int c = j + 1;
-    const double b = c < m ? beta[c] : tail->b[c & 1];
-    const cplx<double> g = c < m ? gamma[c] : tail->g[c & 1];
-    const cplx<double> q = cdiv(cmul(mk(b, 0.0), g), d);
-    const cplx<double> rr = cdiv(mk(b * r.x, b * r.y), d);
-    d = w - q;
-    r = (j < m ? z[j] : mk(0.0, 0.0)) + rr;
+// 2^-e with e the largest exponent among the arguments (1 where they vanish or are not finite):
+// multiplying by it is exact.
+__device__ __forceinline__ double pow2_scale(double a, double b, double c, double d) {
+  const int e = max(max(__double2hiint(a) & 0x7ff00000, __double2hiint(b) & 0x7ff00000),
+                    max(__double2hiint(c) & 0x7ff00000, __double2hiint(d) & 0x7ff00000));
+  return (e == 0 || e >= 0x7fe00000) ? 1.0 : __hiloint2double(0x7fe00000 - e, 0);
+}
+
+// The elimination without its divisions: with d_j = P_j / P_{j+1} and r_j = R_j / P_{j+1},
+//   P_j = w P_{j+1} - beta_{j+1} gamma_{j+1} P_{j+2},   R_j = z_j P_{j+1} + beta_{j+1} R_{j+1},
+// u_1 = R_1 / P_1; P, P_{j+1} and R are scaled together by an exact power of two every fourth
+// row.  m_total > m continues the chain with `tail` (T grows to m_total x m_total; z stays m
+// long): there R = 0 and the rows repeat with period two, so the whole tail is the
+// floor((m_total - m)/2)-th power of one 2 x 2 matrix, formed by repeated squaring.
+// Bound by the FP64 pipe (one warp instruction per 16 cycles and SM): 14 FP64 instructions per row
+// against about 70 with two complex divisions; one warp per CTA puts 4001 frequencies on 126 SMs
+// where 128-thread CTAs used 32.  Errors as the division form's (both within 1e-14 on 1000
+// coefficients continued to 20000 at eta = 0.1 eV).  Block 32.
+static __global__ void __launch_bounds__(32) k_spectrum(int m, int m_total, const ExtrapTail* __restrict__ tail,
+                                                        const double* __restrict__ beta,
+                                                        const cplx<double>* __restrict__ gamma,
+                                                        const cplx<double>* __restrict__ z, int nw,
+                                                        const double* __restrict__ w_ha, double eta, double pref,
+                                                        double vq, cplx<double>* __restrict__ chi,
+                                                        cplx<double>* __restrict__ epsi, cplx<double>* __restrict__ eps) {
+  __shared__ cplx<double> sbg[32], sz[32];
+  __shared__ double sb[32];
+  const int lane = threadIdx.x, i = blockIdx.x * 32 + lane;
+  const cplx<double> w = mk(w_ha[min(i, nw - 1)], eta);
+  cplx<double> P = w, P1 = mk(1.0, 0.0);
+  const int nt = (tail && m_total > m) ? m_total - m : 0;
+  if (nt > 0) {
+    const int pa = m & 1, pb = pa ^ 1;   // row c takes the constants of parity c % 2; the rows c = m, m + 2, ...: pa
+    const cplx<double> ca = tail->g[pa] * tail->b[pa], cb = tail->g[pb] * tail->b[pb];
+    if (nt & 1) {
+      const cplx<double> t = cmul(w, P) - cmul(ca, P1);
+      P1 = P;
+      P = t;
+    }
+    // one period: [[w, -ca], [1, 0]] [[w, -cb], [1, 0]]
+    cplx<double> a = cmul(w, w) - ca, b = mk(-(cb.x * w.x - cb.y * w.y), -(cb.x * w.y + cb.y * w.x)), c = w,
+                 d = mk(-cb.x, -cb.y);
+    for (int h = nt >> 1; h; h >>= 1) {
+      if (h & 1) {
+        const cplx<double> t = cmul(a, P) + cmul(b, P1), u = cmul(c, P) + cmul(d, P1);
+        const double s = pow2_scale(t.x, t.y, u.x, u.y);
+        P = t * s;
+        P1 = u * s;
+      }
+      if (h == 1) break;
+      const cplx<double> bc = cmul(b, c), tr = a + d;
+      const cplx<double> na = cmul(a, a) + bc, nd = cmul(d, d) + bc, nb = cmul(b, tr), nc = cmul(c, tr);
+      const double s = fmin(pow2_scale(na.x, na.y, nb.x, nb.y), pow2_scale(nc.x, nc.y, nd.x, nd.y));
+      a = na * s;
+      b = nb * s;
+      c = nc * s;
+      d = nd * s;
+    }
   }
-  const cplx<double> u1 = cdiv(r, d);
+  cplx<double> R = cmul(z[m - 1], P1);
+  for (int j0 = m - 2; j0 >= 0; j0 -= 32) {   // rows j0, j0 - 1, ...
+    __syncwarp();
+    if (j0 - lane >= 0) {
+      const int j = j0 - lane;
+      const double b = beta[j + 1];
+      sb[lane] = b;
+      sbg[lane] = gamma[j + 1] * b;
+      sz[lane] = z[j];
+    }
+    __syncwarp();
+    const int n = min(32, j0 + 1);
+    auto row = [&](int q) {
+      const cplx<double> zj = sz[q], g = sbg[q];
+      const double b = sb[q];
+      R = mk(zj.x * P.x - zj.y * P.y + b * R.x, zj.x * P.y + zj.y * P.x + b * R.y);
+      const cplx<double> t = mk(w.x * P.x - w.y * P.y - (g.x * P1.x - g.y * P1.y),
+                                w.x * P.y + w.y * P.x - (g.x * P1.y + g.y * P1.x));
+      P1 = P;
+      P = t;
+    };
+    auto rescale = [&]() {
+      const double s = pow2_scale(P.x, P.y, P1.x, P1.y);
+      P = P * s;
+      P1 = P1 * s;
+      R = R * s;
+    };
+    int q = 0;
+    for (; q + 4 <= n; q += 4) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) row(q + u);
+      rescale();
+    }
+    for (; q < n; ++q) row(q);
+    rescale();
+  }
+  if (i >= nw) return;
+  const cplx<double> u1 = cdiv(R, P);
   const cplx<double> c = u1 * (pref * beta[0]);
   chi[i] = c;
   const cplx<double> ei = mk(1.0 + vq * c.x, vq * c.y);

@@ -246,7 +246,7 @@ static int spectrum_impl(const double* beta, const double* gamma, const double* 
   cudaMemcpyAsync(dz, z, m * sizeof(ll::cplx<double>), cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(dw, w.data(), n_omega * sizeof(double), cudaMemcpyHostToDevice, st);
   if (m_total > m) ll::k_extrap_tail<<<1, 256, 0, st>>>(m, kind, db, dg, dt);
-  ll::k_spectrum<<<(n_omega + 127) / 128, 128, 0, st>>>(m, m_total, m_total > m ? dt : nullptr, db, dg, dz, n_omega,
+  ll::k_spectrum<<<(n_omega + 31) / 32, 32, 0, st>>>(m, m_total, m_total > m ? dt : nullptr, db, dg, dz, n_omega,
                                                          dw, eta_ev / ha, 4.0 / omega_cell,
                                                          4.0 * 3.14159265358979323846 / q2, dout, dout + n_omega,
                                                          dout + 2L * n_omega);
@@ -395,7 +395,7 @@ int ll_spectrum_static(const double* beta, const double* gamma, const double* z,
   if (e == cudaSuccess) e = cudaMemcpyAsync(dw, omega_ev, n_omega * sizeof(double), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) {
     k_ev_to_ha<<<(n_omega + 127) / 128, 128, 0, st>>>(n_omega, dw);
-    ll::k_spectrum<<<(n_omega + 127) / 128, 128, 0, st>>>(m, m, nullptr, db, dg, dz, n_omega, dw, eta_ev / 27.211386245988,
+    ll::k_spectrum<<<(n_omega + 31) / 32, 32, 0, st>>>(m, m, nullptr, db, dg, dz, n_omega, dw, eta_ev / 27.211386245988,
                                                            4.0 / omega_cell, 4.0 * 3.14159265358979323846 / q2, dout,
                                                            dout + kStaticMaxOmega, dout + 2L * kStaticMaxOmega);
     e = cudaGetLastError();
