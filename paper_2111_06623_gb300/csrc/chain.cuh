@@ -627,8 +627,9 @@ class Chain : public ChainBase {
       // k-point when they fit: the Lanczos partials are then one per k)
       auto fused = [&](int b) {
         bpc_ = b;
-        return 2 * (size_t)b * pq * sizeof(cplx<T>) + (size_t)std::max(nproj_, nbnd_) * b * sizeof(cplx<double>) +
-               red_bytes(256) + 32 * 32 * sizeof(cplx<T>) + 4096;
+        return 2 * (size_t)b * pq * sizeof(cplx<T>) +
+               (size_t)(nproj_ + nbnd_) * b * (sizeof(cplx<double>) + sizeof(cplx<T>)) +
+               red_doubles(256) * sizeof(double) + 32 * 32 * sizeof(cplx<T>) + 4096;
       };
       int best = 0;
       for (int b = nbnd_; b >= 1 && !best; --b)
@@ -680,9 +681,9 @@ class Chain : public ChainBase {
       const char* xp = getenv("LL_XY_PAIR");   // 1: lane pairs for every even N, 0: never (k_xy)
       xy_pair_ = (xp && xp[1] == 0 && (xp[0] == '0' || xp[0] == '1')) ? xp[0] - '0' : -1;
     }
+    if ((rc = alloc(&ub_, (long)nks_ * nbnd_ * std::max(1, nproj_)))) return rc;
     // chunk partials: U^H x per vector (two per vector on the non-Hermitian update), B^H x
     if (split_ && ((rc = alloc(&sp_s_, 2 * nzv * nbnd_ * nbnd_)) || (rc = alloc(&sp_c_, nzv * std::max(1, nproj_ * nbnd_))) ||
-                   (rc = alloc(&ub_, (long)nks_ * nbnd_ * std::max(1, nproj_))) ||
                    (rc = alloc(&sp_coef_, nvec_ * (long)nks_ * (nproj_ + nbnd_) * nbnd_))))
       return rc;
     (void)err;
@@ -738,12 +739,16 @@ class Chain : public ChainBase {
     LL_CK(cudaMemsetAsync(zpart_, 0, (long)(cap_ + 1) * nzp * sizeof(cplx<double>), st_));
     k_fxc<T><<<256, 256, 0, st_>>>(n3, rho_, fxc_, approx_ == LL_APPROX_TDDFT ? 1 : 0);
     LL_CK(cudaGetLastError());
-    if (split_ && nproj_ > 0) {  // U^H B per k (the KB part of P_c on the split path)
+    if (nproj_ > 0) {  // U^H B per k (the KB part of P_c)
+      const int nc = (pq + kChunk - 1) / kChunk;
+      cplx<double>* pt = sp_c_;   // chunk partials
+      if (!split_ && (rc = alloc(&pt, (long)nks_ * nc * nbnd_ * nproj_))) return rc;
       const size_t sm = (size_t)(nbnd_ + nproj_) * kTileP * sizeof(cplx<T>);
       if ((rc = set_smem(k_sp_ub<T>, sm, err))) return rc;
-      k_sp_ub<T><<<dim3(nks_, nchunk_), 256, sm, st_>>>(nbnd_, pq, dq_.npw, nchunk_, nproj_, ukq_, bkq_, sp_c_);
-      k_sp_reduce<<<nks_, 256, 0, st_>>>(nchunk_, nbnd_ * nproj_, sp_c_, ub_);
+      k_sp_ub<T><<<dim3(nks_, nc), 256, sm, st_>>>(nbnd_, pq, dq_.npw, nc, nproj_, ukq_, bkq_, pt);
+      k_sp_reduce<<<nks_, 256, 0, st_>>>(nc, nbnd_ * nproj_, pt, ub_);
       LL_CK(cudaGetLastError());
+      if (!split_) release(pt);
     }
 
     // index map sphere(k+Q) -> sphere(k) (on the device, from the Miller lists)
@@ -833,7 +838,7 @@ class Chain : public ChainBase {
     int rc;
     const int pq = hq_.npw_pad;
     const size_t smem_nh = 2 * (size_t)bpc_ * pq * sizeof(cplx<T>) + (size_t)nbnd_ * bpc_ * sizeof(cplx<double>) +
-                           16 * 4 * sizeof(double);
+                           red_doubles(128) * sizeof(double);
     Coef co{beta_, gamma_, zpart_, err_};
     if (flavour_ == LL_FLAVOUR_PH && n > 0) {
       k_step_set<<<1, 1, 0, st_>>>(jdev_, queued_ + 1);
@@ -1138,7 +1143,7 @@ class Chain : public ChainBase {
       prof_.count(LL_PROF_ZINV, 3);
       return img_;
     }
-    k_metal_image<T><<<dim3(nks_, nvec), 128, 0, st_>>>(nks_, nbnd_, hq_.npw_pad, dq_.npw, ukq_, in, img_, zp_, md_);
+    k_metal_image<T><<<dim3(nks_, nvec), 256, 0, st_>>>(nks_, nbnd_, hq_.npw_pad, dq_.npw, ukq_, in, img_, zp_, md_);
     prof_.count(LL_PROF_ZINV);
     return img_;
   }
@@ -1168,16 +1173,12 @@ class Chain : public ChainBase {
     return LL_OK;
   }
 
-  // reduction scratch of the per-k dot routines: max(16, 2*ni*nj) doubles per warp
-  size_t red_bytes(int threads) const {
-    const int pairs = std::max(std::max(nproj_, nbnd_) * std::max(bpc_, 1), 8);
-    return (size_t)(threads / 32) * 2 * pairs * sizeof(double);
-  }
   template <int N>
   int zfwd_proj_n(int nvec, const cplx<T>* in, cplx<T>* out, std::string& err) {
     if (split_) return zfwd_split_n<N>(nvec, in, out, err);
     const size_t smem = 2 * (size_t)bpc_ * hq_.npw_pad * sizeof(cplx<T>) +
-                        (size_t)std::max(nproj_, nbnd_) * bpc_ * sizeof(cplx<double>) + red_bytes(256);
+                        (size_t)(nproj_ + nbnd_) * bpc_ * (sizeof(cplx<double>) + sizeof(cplx<T>)) +
+                        red_doubles(256) * sizeof(double);
     int rc;
     auto kern = k_zfwd_proj<T, N>;
     if constexpr (tight_prune(N) > 0)
@@ -1186,7 +1187,7 @@ class Chain : public ChainBase {
     if ((rc = set_smem(kern, smem, err))) return rc;
     kern<<<dim3(nks_, nvec, ngrp_), 256, smem, st_>>>(dq_, nbnd_, bpc_, cbuf_, cb_ncol_,
                                                                     metal_ ? img_ : in, kin_, eps_, ukq_, bkq_,
-                                                                    dij_, nproj_, out, part_, md_, zp_);
+                                                                    dij_, ub_, nproj_, out, part_, md_, zp_);
     LL_CK(cudaGetLastError());
     return LL_OK;
   }
@@ -1319,7 +1320,7 @@ class Chain : public ChainBase {
   int zinv_ph_n(int j, std::string& err) {
     if (split_) return zinv_split_n<N>(j, err);
     const size_t smem = (size_t)bpc_ * hq_.npw_pad * sizeof(cplx<T>) + (size_t)nbnd_ * bpc_ * sizeof(cplx<double>) +
-                        red_bytes(256);
+                        red_doubles(256) * sizeof(double);
     int rc;
     Coef co{beta_, gamma_, zpart_, err_};
     // the per-(k, band group) update, then the axis-3 inverse FFTs, one thread per column line

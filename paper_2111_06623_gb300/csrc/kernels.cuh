@@ -603,117 +603,146 @@ __device__ __forceinline__ T warp_sum_t(T v) {
   return v;
 }
 
-// All-pairs dots out[i*nj + j] = mult[i] * sum_g conj(A[i*lda + g]) B[j*ldb + g] over g < npw,
-// eight pairs at a time: per-thread partial sums in T, warp sums in T, warps summed in
-// double.  `red`: 16 doubles per warp.  Called by the whole block; ends synchronised.
-template <typename T>
-__device__ void block_dots(const cplx<T>* A, long lda, const cplx<T>* B, long ldb, int npw, int ni, int nj,
-                           const double* mult, cplx<double>* out, double* red) {
-  const int np = ni * nj;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int c0 = 0; c0 < np; c0 += 8) {
-    T acc[16];
+// Warp sums of NV values per lane at once (NV a power of two <= 32): at every step a lane keeps
+// half of its values and gives its partner the other half, so 32 values take 31 exchanges
+// instead of 5 each.  Returns the total of value number lane / (32 / NV).
+template <typename T, int NV>
+__device__ __forceinline__ T warp_sums(T (&v)[NV]) {
+  const int lane = threadIdx.x & 31;
+  int o = 16;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) acc[q] = T(0);
-    for (int g = threadIdx.x; g < npw; g += blockDim.x) {
+  for (int n = NV / 2; n > 0; n /= 2, o /= 2) {
+    const bool up = lane & o;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int pr = c0 + q;
-        if (pr < np) {
-          const int i = pr / nj, j = pr - i * nj;
-          const cplx<T> t = cjmul(A[i * lda + g], B[j * ldb + g]);
-          acc[2 * q] += t.x;
-          acc[2 * q + 1] += t.y;
-        }
-      }
+    for (int i = 0; i < n; ++i) {
+      const T give = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
     }
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const T v = warp_sum_t(acc[q]);
-      if (lane == 0) red[warp * 16 + q] = (double)v;
-    }
-    __syncthreads();
-    if (threadIdx.x < 8 && c0 + (int)threadIdx.x < np) {
-      const int pr = c0 + threadIdx.x;
-      double re = 0.0, im = 0.0;
-      for (int w = 0; w < nw; ++w) {
-        re += red[w * 16 + 2 * threadIdx.x];
-        im += red[w * 16 + 2 * threadIdx.x + 1];
-      }
-      const double m = mult ? mult[pr / nj] : 1.0;
-      out[pr] = mk(re * m, im * m);
-    }
-    __syncthreads();
   }
+  T t = v[0];
+#pragma unroll
+  for (; o > 0; o /= 2) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
 }
 
-// The same for compile-time NI x NJ (the common small shapes) in one pass: every thread keeps
-// all NI*NJ complex partial sums in registers.  `red`: 2*NI*NJ doubles per warp.
-template <typename T, int NI, int NJ>
-__device__ void block_dots_fixed(const cplx<T>* A, long lda, const cplx<T>* B, long ldb, int npw,
-                                 const double* mult, cplx<double>* out, double* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  T acc[NI][NJ][2];
+// Dot blocks of the per-k kernels: out[i*nj + j] = mult[i] sum_{g < npw} conj(A_i[g]) B_j[g] for
+// all ni x nj pairs, in tiles of 4 x NJ pairs whose sums a thread keeps in registers (4 + NJ
+// loads per 4 NJ complex products); warp sums in T by halving exchange (warp_sums), warps summed
+// in double.  `red`: kRedPairs complex doubles per warp; the tiles fill it before the block
+// synchronises.  Bound by latency and by the reductions, not by the products: at 570 plane waves
+// a thread of 256 holds 2 of them per tile, 128 FMAs beside the 31 exchanges (160 with a warp
+// reduction per value; in FP64, where an add takes 16 cycles of the SM's pipe, the reductions
+// were most of the block).  Called by the whole block; ends synchronised.
+constexpr int kRedPairs = 64;
+__host__ __device__ constexpr size_t red_doubles(int threads) { return (size_t)(threads / 32) * 2 * kRedPairs; }
+
+template <typename T, int NJ>
+__device__ __forceinline__ void dots_tile(const cplx<T>* __restrict__ A, long lda, const cplx<T>* B, long ldb, int npw,
+                                          int ni, int nj, double* red) {
+  T acc[8 * NJ];   // [i][j][re, im]
 #pragma unroll
-  for (int i = 0; i < NI; ++i)
+  for (int q = 0; q < 8 * NJ; ++q) acc[q] = T(0);
+  const cplx<T>*pa[4], *pb[NJ];   // rows past the block's edge repeat its last one
 #pragma unroll
-    for (int j = 0; j < NJ; ++j) acc[i][j][0] = acc[i][j][1] = T(0);
+  for (int i = 0; i < 4; ++i) pa[i] = A + (long)min(i, ni - 1) * lda;
+#pragma unroll
+  for (int j = 0; j < NJ; ++j) pb[j] = B + (long)min(j, nj - 1) * ldb;
   for (int g = threadIdx.x; g < npw; g += blockDim.x) {
-    cplx<T> a[NI], b[NJ];
+    cplx<T> x[4], y[NJ];
 #pragma unroll
-    for (int i = 0; i < NI; ++i) a[i] = A[i * lda + g];
+    for (int i = 0; i < 4; ++i) x[i] = pa[i][g];
 #pragma unroll
-    for (int j = 0; j < NJ; ++j) b[j] = B[j * ldb + g];
+    for (int j = 0; j < NJ; ++j) y[j] = pb[j][g];
 #pragma unroll
-    for (int i = 0; i < NI; ++i)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int j = 0; j < NJ; ++j) {
-        acc[i][j][0] += a[i].x * b[j].x + a[i].y * b[j].y;
-        acc[i][j][1] += a[i].x * b[j].y - a[i].y * b[j].x;
+        acc[(i * NJ + j) * 2] += x[i].x * y[j].x + x[i].y * y[j].y;
+        acc[(i * NJ + j) * 2 + 1] += x[i].x * y[j].y - x[i].y * y[j].x;
       }
   }
-#pragma unroll
-  for (int i = 0; i < NI; ++i)
-#pragma unroll
-    for (int j = 0; j < NJ; ++j)
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const T v = warp_sum_t(acc[i][j][c]);
-        if (lane == 0) red[warp * (2 * NI * NJ) + (i * NJ + j) * 2 + c] = (double)v;
-      }
-  __syncthreads();
-  if (threadIdx.x < NI * NJ) {
-    double re = 0.0, im = 0.0;
-    for (int w = 0; w < nw; ++w) {
-      re += red[w * (2 * NI * NJ) + 2 * threadIdx.x];
-      im += red[w * (2 * NI * NJ) + 2 * threadIdx.x + 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int NV = 8 * NJ;
+  const T t = warp_sums<T, NV>(acc);
+  if (lane % (32 / NV) == 0) red[(long)warp * 2 * kRedPairs + lane / (32 / NV)] = (double)t;
+}
+
+template <typename T, int NJ>
+__device__ __forceinline__ void block_dots_nj(const cplx<T>* A, long lda, const cplx<T>* B, long ldb, int npw, int ni,
+                                              int nj, const double* mult, cplx<double>* out, double* red) {
+  constexpr int TP = 4 * NJ, TB = kRedPairs / TP;   // pairs per tile, tiles per batch
+  const int tj = (nj + NJ - 1) / NJ, nt = ((ni + 3) / 4) * tj, nw = blockDim.x >> 5;
+  for (int t0 = 0; t0 < nt; t0 += TB) {
+    const int n = min(TB, nt - t0);
+    for (int t = 0; t < n; ++t) {
+      const int i0 = (t0 + t) / tj * 4, j0 = (t0 + t) % tj * NJ;
+      dots_tile<T, NJ>(A + i0 * lda, lda, B + j0 * ldb, ldb, npw, ni - i0, nj - j0, red + t * 2 * TP);
     }
-    const double m = mult ? mult[threadIdx.x / NJ] : 1.0;
-    out[threadIdx.x] = mk(re * m, im * m);
+    __syncthreads();
+    for (int p = threadIdx.x; p < n * TP; p += blockDim.x) {
+      const int t = t0 + p / TP, i = t / tj * 4 + (p % TP) / NJ, j = t % tj * NJ + p % NJ;
+      if (i < ni && j < nj) {
+        double re = 0.0, im = 0.0;
+        for (int w = 0; w < nw; ++w) {
+          re += red[w * 2 * kRedPairs + 2 * p];
+          im += red[w * 2 * kRedPairs + 2 * p + 1];
+        }
+        const double m = mult ? mult[i] : 1.0;
+        out[i * nj + j] = mk(re * m, im * m);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+template <typename T>
+__device__ __forceinline__ void block_dots(const cplx<T>* A, long lda, const cplx<T>* B, long ldb, int npw, int ni,
+                                           int nj, const double* mult, cplx<double>* out, double* red) {
+  if (nj == 1) block_dots_nj<T, 1>(A, lda, B, ldb, npw, ni, nj, mult, out, red);
+  else block_dots_nj<T, 4>(A, lda, B, ldb, npw, ni, nj, mult, out, red);
+}
+
+// The sum over the block of conj(a[g]) b[g], g < n (one pair): `red` as above, out[0].
+template <typename T>
+__device__ __forceinline__ void block_dot1(const cplx<T>* a, const cplx<T>* b, int n, cplx<double>* out, double* red) {
+  T acc[2] = {T(0), T(0)};
+  for (int g = threadIdx.x; g < n; g += blockDim.x) {
+    const cplx<T> x = a[g], y = b[g];
+    acc[0] += x.x * y.x + x.y * y.y;
+    acc[1] += x.x * y.y - x.y * y.x;
+  }
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const T t = warp_sums<T, 2>(acc);
+  if (lane % 16 == 0) red[(threadIdx.x >> 5) * 2 + lane / 16] = (double)t;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double re = 0.0, im = 0.0;
+    for (int w = 0; w < nw; ++w) re += red[2 * w], im += red[2 * w + 1];
+    out[0] = mk(re, im);
   }
   __syncthreads();
 }
 
-// Fixed-shape dots when (ni, nj) is one of the compiled shapes, else the chunked form.
-// `red` must hold max(16, 2*ni*nj) doubles per warp.
-template <typename T>
-__device__ __forceinline__ void small_dots(const cplx<T>* A, long lda, const cplx<T>* B, long ldb, int npw, int ni,
-                                           int nj, const double* mult, cplx<double>* out, double* red) {
-  if (ni == 4 && nj == 4) block_dots_fixed<T, 4, 4>(A, lda, B, ldb, npw, mult, out, red);
-  else if (ni == 8 && nj == 4) block_dots_fixed<T, 8, 4>(A, lda, B, ldb, npw, mult, out, red);
-  else if (ni == 2 && nj == 4) block_dots_fixed<T, 2, 4>(A, lda, B, ldb, npw, mult, out, red);
-  else if (ni == 1 && nj == 1) block_dots_fixed<T, 1, 1>(A, lda, B, ldb, npw, mult, out, red);
-  else block_dots<T>(A, lda, B, ldb, npw, ni, nj, mult, out, red);
-}
-
-// The P_c dot block S = U^H x (nbnd x nv): the 4 x 4 shape in registers, others chunked.
-// (A separate dispatcher from small_dots keeps the 8 x 4 KB shape's registers out of the
-// kernels that only project.)
-template <typename T>
-__device__ __forceinline__ void proj_dots(const cplx<T>* A, long lda, const cplx<T>* B, long ldb, int npw, int ni,
-                                          int nj, cplx<double>* out, double* red) {
-  if (ni == 4 && nj == 4) block_dots_fixed<T, 4, 4>(A, lda, B, ldb, npw, nullptr, out, red);
-  else block_dots<T>(A, lda, B, ldb, npw, ni, nj, nullptr, out, red);
+// acc[v] += sign sum_r M[r][g] C[r*ldc + v], v < 4, over nr rows of M (row stride ldm; C in shared
+// memory): every value of M is loaded once for four bands.
+template <typename T, int SIGN>
+__device__ __forceinline__ void rows_times(cplx<T> (&acc)[4], const cplx<T>* __restrict__ M, long ldm, int nr,
+                                           const cplx<T>* C, int ldc, int nv) {
+#pragma unroll 4
+  for (int r = 0; r < nr; ++r) {
+    const cplx<T> m = M[r * ldm];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const cplx<T> c = C[r * ldc + min(v, nv - 1)];
+      if (SIGN > 0) {
+        acc[v].x += m.x * c.x - m.y * c.y;
+        acc[v].y += m.x * c.y + m.y * c.x;
+      } else {
+        acc[v].x -= m.x * c.x - m.y * c.y;
+        acc[v].y -= m.x * c.y + m.y * c.x;
+      }
+    }
+  }
 }
 
 // x[v][g] -= sum_w U[w][g] S[w][v] for nv orbitals x of one k against its nbnd occupied
@@ -725,11 +754,16 @@ __device__ __forceinline__ void subtract_projection(cplx<T>* x, const cplx<T>* u
   __shared__ cplx<T> St[32 * 32];
   for (int i = threadIdx.x; i < nbnd * nv; i += blockDim.x) St[i] = mk((T)S[i].x, (T)S[i].y);
   __syncthreads();
-  for (int i = threadIdx.x; i < nv * npw_pad; i += blockDim.x) {
-    const int v = i / npw_pad, gi = i - v * npw_pad;
-    cplx<T> t = x[i];
-    for (int w = 0; w < nbnd; ++w) t = t - cmul(uk[(long)w * npw_pad + gi], St[w * nv + v]);
-    x[i] = t;
+  const int nb4 = (nv + 3) / 4;
+  for (int i = threadIdx.x; i < nb4 * npw_pad; i += blockDim.x) {
+    const int v0 = i / npw_pad * 4, gi = i % npw_pad, n = min(4, nv - v0);
+    cplx<T> acc[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) acc[v] = v < n ? x[(long)(v0 + v) * npw_pad + gi] : czero<T>();
+    rows_times<T, -1>(acc, uk + gi, npw_pad, nbnd, St + v0, nv, n);
+#pragma unroll
+    for (int v = 0; v < 4; ++v)
+      if (v < n) x[(long)(v0 + v) * npw_pad + gi] = acc[v];
   }
   __syncthreads();
 }
@@ -772,6 +806,19 @@ __device__ __forceinline__ double block_sum(double v) {
   return t;
 }
 
+// The same with the lanes summed in T, the warps in double.
+template <typename T>
+__device__ __forceinline__ double block_sum_t(T v) {
+  __shared__ double wsum[32];
+  v = warp_sum_t(v);
+  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = (double)v;
+  __syncthreads();
+  double t = 0.0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += wsum[w];
+  __syncthreads();
+  return t;
+}
+
 // x <- P_c x for every orbital of k (in place); with coef ([nks][nbnd][nbnd], m-major), the
 // component along u_m of band v is removed with weight coef[k][m][v] instead of 1.  The bands
 // of k are independent: grid (nks, nvec, nsplit) with nsplit dividing nbnd, each CTA taking
@@ -781,7 +828,7 @@ __global__ void __launch_bounds__(128) k_project(int nks, int nbnd, int npw_pad,
                                                  const cplx<T>* __restrict__ ukq, cplx<T>* __restrict__ x,
                                                  const double* __restrict__ coef) {
   __shared__ cplx<double> cf[32 * 32];
-  __shared__ double red[4 * 16];
+  __shared__ double red[red_doubles(128)];
   const int k = blockIdx.x, vec = blockIdx.y;
   const int nv = nbnd / gridDim.z, v0 = blockIdx.z * nv;
   const long base = (((long)vec * nks + k) * nbnd + v0) * npw_pad;
@@ -799,14 +846,14 @@ __global__ void __launch_bounds__(128) k_project(int nks, int nbnd, int npw_pad,
 }
 
 // A metal's image of a batch vector z for the FFT pipeline: img = Q z = z - U (qh Z) and
-// zp = [c > 0] Z, Z = U^H z (double), per (vector, k).  grid (nks, nvec), block 128.
+// zp = [c > 0] Z, Z = U^H z (double), per (vector, k).  grid (nks, nvec), block 256.
 template <typename T>
-__global__ void __launch_bounds__(128) k_metal_image(int nks, int nbnd, int npw_pad, const int* __restrict__ npw,
+__global__ void __launch_bounds__(256) k_metal_image(int nks, int nbnd, int npw_pad, const int* __restrict__ npw,
                                                      const cplx<T>* __restrict__ ukq, const cplx<T>* __restrict__ z,
                                                      cplx<T>* __restrict__ img, cplx<double>* __restrict__ zp,
                                                      MetalDev md) {
   __shared__ cplx<double> cf[32 * 32];
-  __shared__ double red[4 * 16];
+  __shared__ double red[red_doubles(256)];
   const int k = blockIdx.x, vec = blockIdx.y;
   const long base = ((long)vec * nks + k) * nbnd * npw_pad;
   const cplx<T>* uk = ukq + (long)k * nbnd * npw_pad;
@@ -860,7 +907,7 @@ __device__ __forceinline__ double block_mean(const double* p, int n, int stride 
 // k_zinv.  grid (nks, ngrp), block 256.  smem: r [bpc][npw_pad], S [nbnd*bpc] (double
 // complex), reduction scratch.
 template <typename T>
-__global__ void __launch_bounds__(256) k_ph_update(const int* __restrict__ jdev, SphereDev s, int nbnd, int bpc,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_ph_update(const int* __restrict__ jdev, SphereDev s, int nbnd, int bpc,
                                                    const double* __restrict__ part, cplx<T>* __restrict__ R,
                                                    const cplx<T>* __restrict__ X, cplx<T>* __restrict__ Vp,
                                                    const cplx<T>* __restrict__ y, const cplx<T>* __restrict__ ukq,
@@ -887,7 +934,7 @@ __global__ void __launch_bounds__(256) k_ph_update(const int* __restrict__ jdev,
   const int np = s.npw[k];
   const long zi = (long)(j - 1) * nks * ngrp + (long)k * ngrp + grp;
   if (r_upper) {  // z_j partial = (y, r_j)/beta_j over the group's bands
-    block_dots_fixed<T, 1, 1>(y + base, 0, R + base, 0, bpc * npw_pad, nullptr, cf, red);
+    block_dot1<T>(y + base, R + base, bpc * npw_pad, cf, red);
     if (threadIdx.x == 0) co.zpart[zi] = mk(cf[0].x / b, cf[0].y / b);
   } else if (threadIdx.x == 0) {
     co.zpart[zi] = mk(0.0, 0.0);
@@ -900,7 +947,7 @@ __global__ void __launch_bounds__(256) k_ph_update(const int* __restrict__ jdev,
   }
   __syncthreads();
   const cplx<T>* uk = ukq + (long)k * nbnd * npw_pad;
-  proj_dots<T>(uk, npw_pad, rs, npw_pad, np, nbnd, bpc, cf, red);
+  block_dots<T>(uk, npw_pad, rs, npw_pad, np, nbnd, bpc, nullptr, cf, red);
   if (keep) {  // a metal: only the states with c_mv = 0 are removed
     for (int i = threadIdx.x; i < nbnd * bpc; i += blockDim.x) {
       const int m = i / bpc;
@@ -935,17 +982,24 @@ static __device__ __noinline__ double metal_operator_coefs(const MetalDev md, in
 
 // Last stage of the operator fused with the per-k projections, for one group of bpc bands of
 // one k-point (the kinetic, KB and P_c terms act band by band): forward FFT of the group's
-// columns along axis 3 and gather of the sphere (1/N^3), + (1/2|k+Q+G|^2 - eps_vk) x, + KB
+// columns along axis 3 and gather of the sphere (1/W^3), + (1/2|k+Q+G|^2 - eps_vk) x, + KB
 // sum_p beta_p D_p <beta_p|x>, then P_c, the output X and the group's partial Re(x^H X)
 // (a metal: x is the image Q z, zp holds Z = U^H z per vector; the output is the operator
 // on z through the MetalDev tables, and the partial Re(z^H X)).
+// P_c of the KB term goes through the overlaps ub = U^H B of the set-up, S = U^H t + ub c, so
+// both dot blocks are formed on the same data and KB, P_c, the output and the norm partial
+// are one pass over the plane waves, four bands of a plane wave per thread (rows_times).
 // grid (nks, nvec, ngrp), block 256.  smem: x, t [bpc][npw_pad]; coefficients; scratch.
+// Measured (GB300, FP32, us per launch, before -> after the shared dot blocks and the one pass):
+// eight-atom cell (16 bands, 1632 plane waves, 64 k) 313 -> 124, KB workload (4 bands, 570, 512 k)
+// 77 -> 61.
 template <typename T, int N, int PR = 0>
 __global__ void __launch_bounds__(256, 2) k_zfwd_proj(SphereDev s, int nbnd, int bpc, const cplx<T>* __restrict__ cbuf,
                                                    int cb_ncol, const cplx<T>* __restrict__ xin,
                                                    const T* __restrict__ kin, const double* __restrict__ eps,
                                                    const cplx<T>* __restrict__ ukq, const cplx<T>* __restrict__ bkq,
-                                                   const double* __restrict__ dij, int nproj,
+                                                   const double* __restrict__ dij,
+                                                   const cplx<double>* __restrict__ ub, int nproj,
                                                    cplx<T>* __restrict__ xout, double* __restrict__ part,
                                                    MetalDev md, const cplx<double>* __restrict__ zp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -954,8 +1008,9 @@ __global__ void __launch_bounds__(256, 2) k_zfwd_proj(SphereDev s, int nbnd, int
   const int v0 = grp * bpc;
   cplx<T>* xs = reinterpret_cast<cplx<T>*>(smem_raw);
   cplx<T>* ts = xs + bpc * npw_pad;
-  cplx<double>* cf = reinterpret_cast<cplx<double>*>(ts + bpc * npw_pad);   // [max(nproj, nbnd) * bpc]
-  double* red = reinterpret_cast<double*>(cf + (nproj > nbnd ? nproj : nbnd) * bpc);
+  cplx<double>* cf = reinterpret_cast<cplx<double>*>(ts + bpc * npw_pad);   // [nproj + nbnd][bpc]: c, then S
+  double* red = reinterpret_cast<double*>(cf + (nproj + nbnd) * bpc);
+  cplx<T>* ct = reinterpret_cast<cplx<T>*>(red + red_doubles(256));         // the coefficients in T
   __shared__ T epsk[32];
   const long o0 = ((long)vec * nks + k) * nbnd + v0;      // first orbital of the group
   const long base = o0 * npw_pad;
@@ -991,26 +1046,42 @@ __global__ void __launch_bounds__(256, 2) k_zfwd_proj(SphereDev s, int nbnd, int
     }
   }
   __syncthreads();
+  cplx<double>* sf = cf + nproj * bpc;
+  if (nproj > 0) block_dots<T>(bk, npw_pad, xs, npw_pad, np, nproj, bpc, dij, cf, red);   // D_p <beta_p|x_v>
+  block_dots<T>(uk, npw_pad, ts, npw_pad, np, nbnd, bpc, nullptr, sf, red);
   if (nproj > 0) {
-    small_dots<T>(bk, npw_pad, xs, npw_pad, np, nproj, bpc, dij, cf, red);   // D_p <beta_p|x_v>
-    cplx<T>* ct = reinterpret_cast<cplx<T>*>(red);    // the coefficients in T (red is free now)
-    for (int i = threadIdx.x; i < nproj * bpc; i += blockDim.x) ct[i] = mk((T)cf[i].x, (T)cf[i].y);
-    __syncthreads();
-    for (int i = threadIdx.x; i < bpc * npw_pad; i += blockDim.x) {
-      const int v = i / npw_pad, gi = i - v * npw_pad;
-      cplx<T> acc = ts[i];
-      for (int p = 0; p < nproj; ++p) acc = acc + cmul(bk[(long)p * npw_pad + gi], ct[p * bpc + v]);
-      ts[i] = acc;
+    const cplx<double>* ubk = ub + (long)k * nbnd * nproj;
+    for (int i = threadIdx.x; i < nbnd * bpc; i += blockDim.x) {   // + U^H B c
+      const int w = i / bpc, v = i - w * bpc;
+      cplx<double> a = sf[i];
+      for (int p = 0; p < nproj; ++p) a = a + cmul(ubk[w * nproj + p], cf[p * bpc + v]);
+      sf[i] = a;
     }
     __syncthreads();
   }
-  small_dots<T>(uk, npw_pad, ts, npw_pad, np, nbnd, bpc, nullptr, cf, red);
   const double corr =
-      md.sp ? metal_operator_coefs(md, k, v0, nbnd, bpc, zp + (long)vec * nks * nbnd * nbnd, cf) : 0.0;
-  subtract_projection<T>(ts, uk, cf, nbnd, bpc, npw_pad);
-  for (int i = threadIdx.x; i < bpc * npw_pad; i += blockDim.x) xout[base + i] = ts[i];
-  small_dots<T>(xs, 0, ts, 0, bpc * npw_pad, 1, 1, nullptr, cf, red);
-  if (threadIdx.x == 0) part[((long)vec * nks + k) * ngrp + grp] = cf[0].x + corr;
+      md.sp ? metal_operator_coefs(md, k, v0, nbnd, bpc, zp + (long)vec * nks * nbnd * nbnd, sf) : 0.0;
+  for (int i = threadIdx.x; i < (nproj + nbnd) * bpc; i += blockDim.x) ct[i] = mk((T)cf[i].x, (T)cf[i].y);
+  __syncthreads();
+  const int nb4 = (bpc + 3) / 4;
+  T nr = T(0);
+  for (int i = threadIdx.x; i < nb4 * npw_pad; i += blockDim.x) {
+    const int b0 = i / npw_pad * 4, gi = i % npw_pad, n = min(4, bpc - b0);
+    cplx<T> acc[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) acc[v] = v < n ? ts[(b0 + v) * npw_pad + gi] : czero<T>();
+    rows_times<T, +1>(acc, bk + gi, npw_pad, nproj, ct + b0, bpc, n);
+    rows_times<T, -1>(acc, uk + gi, npw_pad, nbnd, ct + nproj * bpc + b0, bpc, n);
+#pragma unroll
+    for (int v = 0; v < 4; ++v)
+      if (v < n) {
+        const cplx<T> x = xs[(b0 + v) * npw_pad + gi];
+        nr += x.x * acc[v].x + x.y * acc[v].y;
+        xout[base + (long)(b0 + v) * npw_pad + gi] = acc[v];
+      }
+  }
+  const double t = block_sum_t(nr);
+  if (threadIdx.x == 0) part[((long)vec * nks + k) * ngrp + grp] = t + corr;
 }
 
 // Non-Hermitian step j after the two operator applications XV = L v_j, XW = L^dag w_j, for
@@ -1039,7 +1110,7 @@ __global__ void __launch_bounds__(128) k_nh_update(int j, int upper, int nks, in
   const cplx<double> gj = co.gamma[j - 1];
   const cplx<T> g = mk((T)gj.x, (T)gj.y), bc = mk((T)bj, (T)0);
   if (upper) {  // z_j partial = (y, v_j) over the group's bands
-    block_dots<T>(y + base, 0, Vc + base, 0, bpc * npw_pad, 1, 1, nullptr, cf, red);
+    block_dot1<T>(y + base, Vc + base, bpc * npw_pad, cf, red);
     if (threadIdx.x == 0) co.zpart[zi] = cf[0];
   } else if (threadIdx.x == 0) {
     co.zpart[zi] = mk(0.0, 0.0);
@@ -1067,7 +1138,7 @@ __global__ void __launch_bounds__(128) k_nh_update(int j, int upper, int nks, in
     XV[base + i] = vs[i];
     XW[base + i] = ws[i];
   }
-  block_dots<T>(ws, 0, vs, 0, bpc * npw_pad, 1, 1, nullptr, cf, red);
+  block_dot1<T>(ws, vs, bpc * npw_pad, cf, red);
   if (threadIdx.x == 0) spart[(long)k * ngrp + grp] = cf[0];
 }
 
