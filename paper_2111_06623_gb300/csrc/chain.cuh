@@ -627,9 +627,11 @@ class Chain : public ChainBase {
       // k-point when they fit: the Lanczos partials are then one per k)
       auto fused = [&](int b) {
         bpc_ = b;
-        return 2 * (size_t)b * pq * sizeof(cplx<T>) +
-               (size_t)(nproj_ + nbnd_) * b * (sizeof(cplx<double>) + sizeof(cplx<T>)) +
-               red_doubles(256) * sizeof(double) + 32 * 32 * sizeof(cplx<T>) + 4096;
+        const size_t op = (size_t)(nproj_ + nbnd_) * b * (sizeof(cplx<double>) + sizeof(cplx<T>)) +
+                          32 * 32 * sizeof(cplx<T>);
+        const size_t nh = (size_t)nbnd_ * 2 * b * sizeof(cplx<double>) + 2 * 32 * 32 * sizeof(cplx<T>);
+        return 2 * (size_t)b * pq * sizeof(cplx<T>) + (flavour_ == LL_FLAVOUR_NH ? std::max(op, nh) : op) +
+               red_doubles(256) * sizeof(double) + 4096;
       };
       int best = 0;
       for (int b = nbnd_; b >= 1 && !best; --b)
@@ -665,7 +667,7 @@ class Chain : public ChainBase {
         (rc = alloc(&y_, vq)) || (rc = alloc(&map_, (long)nks_ * pq)) || (rc = alloc(&part_, std::max(2L * nks_, nzv))) ||
         (rc = alloc(&spart_, nzp)) || (rc = alloc(&vecs_, 3L * nvec_ * vq)) ||
         (rc = alloc(&beta_, cap_ + 2)) || (rc = alloc(&gamma_, cap_ + 2)) || (rc = alloc(&z_, cap_ + 1)) ||
-        (rc = alloc(&zpart_, (long)(cap_ + 1) * nzp)) || (rc = alloc(&err_, 2)) || (rc = alloc(&jdev_, 1)))
+        (rc = alloc(&zpart_, (long)(cap_ + 1) * nzp)) || (rc = alloc(&err_, 2)) || (rc = alloc(&jdev_, 1)) || (rc = alloc(&scal_, 4)))
       return rc;
     if (metal_) {
       const long sz = (long)nks_ * nbnd_ * nbnd_;
@@ -837,11 +839,11 @@ class Chain : public ChainBase {
     if (stopped_) { err = "the chain stopped at a breakdown"; return LL_EBREAKDOWN; }
     int rc;
     const int pq = hq_.npw_pad;
-    const size_t smem_nh = 2 * (size_t)bpc_ * pq * sizeof(cplx<T>) + (size_t)nbnd_ * bpc_ * sizeof(cplx<double>) +
-                           red_doubles(128) * sizeof(double);
+    const size_t smem_nh = 2 * (size_t)bpc_ * pq * sizeof(cplx<T>) + (size_t)nbnd_ * 2 * bpc_ * sizeof(cplx<double>) +
+                           red_doubles(256) * sizeof(double);
     Coef co{beta_, gamma_, zpart_, err_};
     if (flavour_ == LL_FLAVOUR_PH && n > 0) {
-      k_step_set<<<1, 1, 0, st_>>>(jdev_, queued_ + 1);
+      k_step_set<<<1, 1, 0, st_>>>(jdev_, queued_);
       LL_CK(cudaGetLastError());
       prof_.count(LL_PROF_UPDATE);
     }
@@ -880,19 +882,20 @@ class Chain : public ChainBase {
           prof_.count(LL_PROF_UPDATE, 1);
         } else {
           if ((rc = set_smem(k_nh_update<T>, smem_nh, err))) return rc;
-          k_nh_update<T><<<dim3(nks_, ngrp_), 128, smem_nh, st_>>>(j, upper, nks_, nbnd_, bpc_, pq, dq_.npw, XV(),
+          k_nh_update<T><<<dim3(nks_, ngrp_), 256, smem_nh, st_>>>(j, upper, nks_, nbnd_, bpc_, pq, dq_.npw, XV(),
                                                                    XW(), VpNH(), Wp(),
                                                       Vc(), y_, ukq_, co, spart_, md_.keep);
         }
-        k_nh_normalize<T><<<nks_, 128, 0, st_>>>(j, nks_, nbnd_, pq, npk_, spart_, XV(), XW(), Vc(), VpNH(), Wc(),
-                                                 Wp(), co, tol_);
-        prof_.count(LL_PROF_UPDATE, 2);
+        k_nh_scalars<<<1, 256, 0, st_>>>(j, nks_ * npk_, nks_, spart_, co, tol_, scal_);
+        k_nh_normalize<T><<<4 * nsm_, 256, 0, st_>>>(vq(), XV(), XW(), scal_);
+        nh_rot_ = (nh_rot_ + 2) % 3;   // v_hat, w_hat become v_j, w_j; those v_{j-1}, w_{j-1}
+        prof_.count(LL_PROF_UPDATE, 3);
         prof_.span(LL_PROF_UPDATE, u0, prof_.mark(st_));
       }
       LL_CK(cudaGetLastError());
     }
     if (n > 0) {
-      k_reduce_z<<<(n + 127) / 128, 128, 0, st_>>>(zpart_, nks_ * npk_, nks_, queued_, queued_ + n, z_);
+      k_reduce_z<<<n, 128, 0, st_>>>(zpart_, nks_ * npk_, nks_, queued_, z_);
       LL_CK(cudaGetLastError());
       prof_.count(LL_PROF_UPDATE);
     }
@@ -901,16 +904,17 @@ class Chain : public ChainBase {
   }
 
   // One pseudo-Hermitian step (the step index comes from the device counter jdev_, which the
-  // step advances at its end): update of the Lanczos vectors and the axis-3 inverse FFT of
+  // step advances first): beta_j, update of the Lanczos vectors and the axis-3 inverse FFT of
   // r_{j+1}, then the rest of the operator (D + K when j is odd: r_{j+1} is then upper).
   int ph_step(int j, std::string& err) {
     int rc;
     const int u0 = prof_.mark(st_);
+    const Coef co{beta_, gamma_, zpart_, err_};
+    k_ph_beta<<<1, 256, 0, st_>>>(jdev_, part_, nks_ * npk_, nks_, co, tol_, scal_);
     if ((rc = launch_zinv_ph(j, err))) return rc;
     prof_.span(LL_PROF_ZINV, u0, prof_.mark(st_));
     const int dens = (j % 2 == 1 && approx_ != LL_APPROX_IPA) ? 0 : -1;
     if ((rc = op_rest(1, R(), X(), dens, err))) return rc;
-    k_step_next<<<1, 1, 0, st_>>>(jdev_);
     prof_.count(LL_PROF_ZINV, split_ ? 4 : 2);
     prof_.count(LL_PROF_UPDATE);
     LL_CK(cudaGetLastError());
@@ -1295,8 +1299,8 @@ class Chain : public ChainBase {
     int rc;
     if ((rc = set_smem(k_sp_start<T>, sm, err))) return rc;
     Coef co{beta_, gamma_, zpart_, err_};
-    k_sp_start<T><<<dim3(nks_, nchunk_), 256, sm, st_>>>(jdev_, nks_, nbnd_, pq, dq_.npw, nchunk_, part_, R(), X(), Vp(),
-                                                         y_, ukq_, co, tol_, sp_s_, tc_u_ ? 0 : 1);
+    k_sp_start<T><<<dim3(nks_, nchunk_), 256, sm, st_>>>(jdev_, nks_, nbnd_, pq, dq_.npw, nchunk_, scal_, R(), X(), Vp(),
+                                                         y_, ukq_, co, sp_s_, tc_u_ ? 0 : 1);
     if (tc_u_ && (rc = tc_dots<TC_U>(1, tc_nb_u_, nullptr, R(), nullptr, nullptr, sp_s_, err))) return rc;
     // P_c with the chunk-reduced coefficients, tiled (U read once per chunk for all bands),
     // then the axis-3 inverse FFTs over many CTAs per k
@@ -1325,8 +1329,8 @@ class Chain : public ChainBase {
     Coef co{beta_, gamma_, zpart_, err_};
     // the per-(k, band group) update, then the axis-3 inverse FFTs, one thread per column line
     if ((rc = set_smem(k_ph_update<T>, smem, err))) return rc;
-    k_ph_update<T><<<dim3(nks_, ngrp_), 256, smem, st_>>>(jdev_, dq_, nbnd_, bpc_, part_, R(), X(), Vp(), y_, ukq_, co,
-                                                          tol_, md_.keep);
+    k_ph_update<T><<<dim3(nks_, ngrp_), 256, smem, st_>>>(jdev_, dq_, nbnd_, bpc_, scal_, R(), X(), Vp(), y_, ukq_, co,
+                                                          md_.keep);
     k_zinv<T, N><<<dim3(nks_, 1, zsplit()), 128, 0, st_>>>(dq_, metal_image(R(), 1), nbnd_, cbuf_, cb_ncol_);
     LL_CK(cudaGetLastError());
     return LL_OK;
@@ -1725,17 +1729,20 @@ class Chain : public ChainBase {
     return LL_OK;
   }
 
-  // batch vectors: PH uses [R | X | v_{j-1}], NH uses [v_j w_j | XV XW | v_{j-1} w_{j-1}]
+  // batch vectors: PH uses [R | X | v_{j-1}], NH three pairs [v w] that take turns as the current
+  // vectors, the operator's outputs (then v_hat, w_hat) and the previous vectors
   long vq() const { return (long)nks_ * nbnd_ * hq_.npw_pad; }
   cplx<T>* R() { return vecs_; }
   cplx<T>* X() { return vecs_ + vq(); }
   cplx<T>* Vp() { return vecs_ + 2 * vq(); }
-  cplx<T>* Vc() { return vecs_; }
-  cplx<T>* Wc() { return vecs_ + vq(); }
-  cplx<T>* XV() { return vecs_ + 2 * vq(); }
-  cplx<T>* XW() { return vecs_ + 3 * vq(); }
-  cplx<T>* VpNH() { return vecs_ + 4 * vq(); }
-  cplx<T>* Wp() { return vecs_ + 5 * vq(); }
+  cplx<T>* nh_pair(int i) { return vecs_ + 2 * vq() * ((nh_rot_ + i) % 3); }
+  cplx<T>* Vc() { return nh_pair(0); }
+  cplx<T>* Wc() { return nh_pair(0) + vq(); }
+  cplx<T>* VpNH() { return nh_pair(1); }
+  cplx<T>* Wp() { return nh_pair(1) + vq(); }
+  cplx<T>* XV() { return nh_pair(2); }
+  cplx<T>* XW() { return nh_pair(2) + vq(); }
+  int nh_rot_ = 0;
 
   cudaStream_t st_ = nullptr;
   int N_ = 0, W_ = 0;       // declared FFT grid side, side of the grid the orbitals are transformed on
@@ -1775,6 +1782,7 @@ class Chain : public ChainBase {
   cplx<T>* t1_ = nullptr;        // W_ < N_: n', then f_xc n', on W_ planes of the declared N_ x N_ grid
   cplx<double> *spart_ = nullptr, *gamma_ = nullptr, *z_ = nullptr, *zpart_ = nullptr, *spec_out_ = nullptr;
   ExtrapTail* tail_ = nullptr;   // continuation constants of the coefficients (spectrum)
+  double* scal_ = nullptr;       // the step's scalars for the update kernels (k_ph_beta, k_nh_scalars)
   int* jdev_ = nullptr;          // device step counter of the pseudo-Hermitian recursion
   bool use_graphs_ = true;       // replay captured steps (LL_GRAPHS=0 in the environment: eager)
   bool eager_done_[2] = {false, false};

@@ -748,10 +748,11 @@ __device__ __forceinline__ void rows_times(cplx<T> (&acc)[4], const cplx<T>* __r
 // x[v][g] -= sum_w U[w][g] S[w][v] for nv orbitals x of one k against its nbnd occupied
 // states U (S = U^H x, nbnd x nv).  The coefficients are rounded to T once: conversions from
 // double run on the slow FP64 pipe.
-template <typename T>
+// nv <= NB nbnd: NB blocks of bands (v_hat and w_hat of the non-Hermitian update: 2).
+template <typename T, int NB = 1>
 __device__ __forceinline__ void subtract_projection(cplx<T>* x, const cplx<T>* uk, const cplx<double>* S, int nbnd,
                                                     int nv, int npw_pad) {
-  __shared__ cplx<T> St[32 * 32];
+  __shared__ cplx<T> St[NB * 32 * 32];
   for (int i = threadIdx.x; i < nbnd * nv; i += blockDim.x) St[i] = mk((T)S[i].x, (T)S[i].y);
   __syncthreads();
   const int nb4 = (nv + 3) / 4;
@@ -898,20 +899,47 @@ __device__ __forceinline__ double block_mean(const double* p, int n, int stride 
   return t / n;
 }
 
-// Pseudo-Hermitian step j (read from the device step counter, so that a captured step can be
-// replayed) for one band group of one k-point (P_c, the norm and z act band by
-// band, so groups of bpc bands are independent): beta_j from the ngrp partials per k of
-// Re(r_j^H X_j) (every block re-reduces them in the same order), the group's z_j partial,
-// r_{j+1} = P_c(X_j/beta_j - beta_j v_{j-1}) formed in shared memory and written to R (a
-// metal: keep = MetalDev::keep, the projection P'_v), v_j = r_j/beta_j.  The sphere columns of r_{j+1} are then inverse-FFT'd along axis 3 by
-// k_zinv.  grid (nks, ngrp), block 256.  smem: r [bpc][npw_pad], S [nbnd*bpc] (double
-// complex), reduction scratch.
+// Start of pseudo-Hermitian step j: the device step counter is advanced to j (so that a captured
+// step can be replayed), and beta_j from the n partials of Re(r_j^H X_j) in a fixed order;
+// scal = {beta_j, 1/beta_j} for the update kernels.  One block.  (Every CTA of the update
+// reduced the partials and divided by itself before: on the KB workload 512 CTAs x 256 threads of
+// FP64 adds and divisions, 2 FP64 lanes per SM and cycle.)
+static __global__ void __launch_bounds__(256) k_ph_beta(int* __restrict__ jdev, const double* __restrict__ part, int n,
+                                                       int nks, Coef co, double tol, double* __restrict__ scal) {
+  __shared__ double wsum[8];
+  double s = 0.0;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n; i += 256) s += part[i];
+  s = warp_sum(s);
+  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const int j = *jdev + 1;
+    double t = 0.0, b = 1.0;
+    for (int w = 0; w < 8; ++w) t += wsum[w];
+    const double b2 = t / nks;
+    if (!(b2 > tol)) flag_error(co.err, b2 <= 0.0 ? DEV_NOTPD : DEV_BREAKDOWN, j);
+    else b = sqrt(b2);
+    co.beta[j - 1] = b;
+    co.gamma[j - 1] = mk(b, 0.0);
+    scal[0] = b;
+    scal[1] = 1.0 / b;
+    *jdev = j;
+  }
+}
+
+// Pseudo-Hermitian step j (device step counter) for one band group of one k-point (P_c, the norm
+// and z act band by band, so groups of bpc bands are independent): with beta_j from k_ph_beta,
+// the group's z_j partial, r_{j+1} = P_c(X_j/beta_j - beta_j v_{j-1}) formed in shared memory and
+// written to R (a metal: keep = MetalDev::keep, the projection P'_v), v_j = r_j/beta_j.  The
+// sphere columns of r_{j+1} are then inverse-FFT'd along axis 3 by k_zinv.  grid (nks, ngrp),
+// block 256.  smem: r [bpc][npw_pad], S [nbnd*bpc] (double complex), reduction scratch.
 template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_ph_update(const int* __restrict__ jdev, SphereDev s, int nbnd, int bpc,
-                                                   const double* __restrict__ part, cplx<T>* __restrict__ R,
+                                                   const double* __restrict__ scal, cplx<T>* __restrict__ R,
                                                    const cplx<T>* __restrict__ X, cplx<T>* __restrict__ Vp,
                                                    const cplx<T>* __restrict__ y, const cplx<T>* __restrict__ ukq,
-                                                   Coef co, double tol, const double* __restrict__ keep) {
+                                                   Coef co, const double* __restrict__ keep) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int j = *jdev, r_upper = (j % 2 == 0) ? 1 : 0;   // step index from the device counter
   const int npw_pad = s.npw_pad, nks = s.nks;
@@ -919,27 +947,16 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_ph_update(const
   cplx<T>* rs = reinterpret_cast<cplx<T>*>(smem_raw);
   cplx<double>* cf = reinterpret_cast<cplx<double>*>(rs + bpc * npw_pad);
   double* red = reinterpret_cast<double*>(cf + nbnd * bpc);
-  __shared__ double sbeta;
-  const double b2 = block_mean(part, nks * ngrp) * ngrp;
-  if (threadIdx.x == 0) {
-    double b = 1.0;
-    if (!(b2 > tol)) flag_error(co.err, b2 <= 0.0 ? DEV_NOTPD : DEV_BREAKDOWN, j);
-    else b = sqrt(b2);
-    sbeta = b;
-    if (k == 0 && grp == 0) { co.beta[j - 1] = b; co.gamma[j - 1] = mk(b, 0.0); }
-  }
-  __syncthreads();
-  const double b = sbeta;
   const long base = ((long)k * nbnd + grp * bpc) * npw_pad;
   const int np = s.npw[k];
   const long zi = (long)(j - 1) * nks * ngrp + (long)k * ngrp + grp;
   if (r_upper) {  // z_j partial = (y, r_j)/beta_j over the group's bands
     block_dot1<T>(y + base, R + base, bpc * npw_pad, cf, red);
-    if (threadIdx.x == 0) co.zpart[zi] = mk(cf[0].x / b, cf[0].y / b);
+    if (threadIdx.x == 0) co.zpart[zi] = mk(cf[0].x * scal[1], cf[0].y * scal[1]);
   } else if (threadIdx.x == 0) {
     co.zpart[zi] = mk(0.0, 0.0);
   }
-  const T ib = (T)(1.0 / b), bb = (T)b;
+  const T ib = (T)scal[1], bb = (T)scal[0];
   for (int i = threadIdx.x; i < bpc * npw_pad; i += blockDim.x) {
     const cplx<T> r = R[base + i];
     rs[i] = X[base + i] * ib - Vp[base + i] * bb;
@@ -1088,9 +1105,9 @@ __global__ void __launch_bounds__(256, 2) k_zfwd_proj(SphereDev s, int nbnd, int
 // one group of bpc bands of one k-point: v_hat = P_c(XV - gamma_j v_{j-1}), w_hat =
 // P_c(XW - conj(beta_j) w_{j-1}) (stored in XV, XW), the group's partials of s = (w_hat,
 // v_hat) and of z_j = (y, v_j) (a metal: keep = MetalDev::keep, the projection P'_v).
-// grid (nks, ngrp), block 128.
+// grid (nks, ngrp), block 256.
 template <typename T>
-__global__ void __launch_bounds__(128) k_nh_update(int j, int upper, int nks, int nbnd, int bpc, int npw_pad,
+__global__ void __launch_bounds__(256) k_nh_update(int j, int upper, int nks, int nbnd, int bpc, int npw_pad,
                                                    const int* __restrict__ npw, cplx<T>* __restrict__ XV,
                                                    cplx<T>* __restrict__ XW, const cplx<T>* __restrict__ Vp,
                                                    const cplx<T>* __restrict__ Wp, const cplx<T>* __restrict__ Vc,
@@ -1100,8 +1117,8 @@ __global__ void __launch_bounds__(128) k_nh_update(int j, int upper, int nks, in
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cplx<T>* vs = reinterpret_cast<cplx<T>*>(smem_raw);          // [bpc][npw_pad]
   cplx<T>* ws = vs + bpc * npw_pad;
-  cplx<double>* cf = reinterpret_cast<cplx<double>*>(ws + bpc * npw_pad);   // [nbnd * bpc]
-  double* red = reinterpret_cast<double*>(cf + nbnd * bpc);
+  cplx<double>* cf = reinterpret_cast<cplx<double>*>(ws + bpc * npw_pad);   // [nbnd * 2 bpc]
+  double* red = reinterpret_cast<double*>(cf + nbnd * 2 * bpc);
   const int k = blockIdx.x, grp = blockIdx.y, ngrp = gridDim.y;
   const long base = ((long)k * nbnd + grp * bpc) * npw_pad;
   const long zi = (long)(j - 1) * nks * ngrp + (long)k * ngrp + grp;
@@ -1121,19 +1138,17 @@ __global__ void __launch_bounds__(128) k_nh_update(int j, int upper, int nks, in
   }
   __syncthreads();
   const cplx<T>* uk = ukq + (long)k * nbnd * npw_pad;
-  for (int h = 0; h < 2; ++h) {
-    cplx<T>* xs = h ? ws : vs;
-    block_dots<T>(uk, npw_pad, xs, npw_pad, np, nbnd, bpc, nullptr, cf, red);
-    if (keep) {  // a metal: P'_v, only the states with c_mv = 0 removed
-      for (int i = threadIdx.x; i < nbnd * bpc; i += blockDim.x) {
-        const int m = i / bpc;
-        const double c = keep[metal_idx(k, m, grp * bpc + i - m * bpc, nbnd)];
-        cf[i] = mk(cf[i].x * c, cf[i].y * c);
-      }
-      __syncthreads();
+  // v_hat and w_hat are 2 bpc consecutive rows: one dot block and one pass of P_c for both
+  block_dots<T>(uk, npw_pad, vs, npw_pad, np, nbnd, 2 * bpc, nullptr, cf, red);
+  if (keep) {  // a metal: P'_v, only the states with c_mv = 0 removed
+    for (int i = threadIdx.x; i < nbnd * 2 * bpc; i += blockDim.x) {
+      const int m = i / (2 * bpc), v = (i - m * 2 * bpc) % bpc;
+      const double c = keep[metal_idx(k, m, grp * bpc + v, nbnd)];
+      cf[i] = mk(cf[i].x * c, cf[i].y * c);
     }
-    subtract_projection<T>(xs, uk, cf, nbnd, bpc, npw_pad);
+    __syncthreads();
   }
+  subtract_projection<T, 2>(vs, uk, cf, nbnd, 2 * bpc, npw_pad);
   for (int i = threadIdx.x; i < bpc * npw_pad; i += blockDim.x) {
     XV[base + i] = vs[i];
     XW[base + i] = ws[i];
@@ -1142,59 +1157,73 @@ __global__ void __launch_bounds__(128) k_nh_update(int j, int upper, int nks, in
   if (threadIdx.x == 0) spart[(long)k * ngrp + grp] = cf[0];
 }
 
-// Non-Hermitian normalisation at the end of step j: beta_{j+1} = sqrt|s|, gamma_{j+1} =
-// s/beta_{j+1}; v_{j-1} <- v_j, v_j <- v_hat/beta; w_{j-1} <- w_j, w_j <- w_hat/conj(gamma).
-template <typename T>
-__global__ void __launch_bounds__(128) k_nh_normalize(int j, int nks, int nbnd, int npw_pad, int nchunk,
-                                                      const cplx<double>* __restrict__ spart,
-                                                      const cplx<T>* __restrict__ XV, const cplx<T>* __restrict__ XW,
-                                                      cplx<T>* __restrict__ Vc, cplx<T>* __restrict__ Vp,
-                                                      cplx<T>* __restrict__ Wc, cplx<T>* __restrict__ Wp, Coef co,
-                                                      double tol) {
-  __shared__ cplx<double> sc[2];
-  const int k = blockIdx.x;
-  // spart: nks nchunk partials (one per k, or per (k, chunk) on the split path)
-  const double sr = block_mean(reinterpret_cast<const double*>(spart), nks * nchunk, 2, 0) * nchunk;
-  const double si = block_mean(reinterpret_cast<const double*>(spart), nks * nchunk, 2, 1) * nchunk;
+// Non-Hermitian scalars at the end of step j from the n partials of s = (w_hat, v_hat) (fixed
+// order): beta_{j+1} = sqrt|s|, gamma_{j+1} = s/beta_{j+1}; scal = {1/beta, Re, Im of
+// 1/conj(gamma)}.  One block.
+static __global__ void __launch_bounds__(256) k_nh_scalars(int j, int n, int nks, const cplx<double>* __restrict__ spart,
+                                                           Coef co, double tol, double* __restrict__ scal) {
+  __shared__ double wr[8], wi[8];
+  double sr = 0.0, si = 0.0;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n; i += 256) {
+    sr += spart[i].x;
+    si += spart[i].y;
+  }
+  sr = warp_sum(sr);
+  si = warp_sum(si);
+  if ((threadIdx.x & 31) == 0) { wr[threadIdx.x >> 5] = sr; wi[threadIdx.x >> 5] = si; }
+  __syncthreads();
   if (threadIdx.x == 0) {
+    sr = si = 0.0;
+    for (int w = 0; w < 8; ++w) sr += wr[w], si += wi[w];
+    sr /= nks;
+    si /= nks;
     const double a = sqrt(sr * sr + si * si);
     double b = sqrt(a);
     cplx<double> gm = mk(sr / b, si / b);
     if (!(a > tol)) { flag_error(co.err, DEV_BREAKDOWN, j + 1); b = 1.0; gm = mk(1.0, 0.0); }
-    sc[0] = mk(b, 0.0);
-    sc[1] = gm;
-    if (k == 0) { co.beta[j] = b; co.gamma[j] = gm; }
-  }
-  __syncthreads();
-  const double b = sc[0].x;
-  const cplx<double> gm = sc[1];
-  // 1/conj(gamma) = gamma/|gamma|^2
-  const double gg = gm.x * gm.x + gm.y * gm.y;
-  const cplx<T> igc = mk((T)(gm.x / gg), (T)(gm.y / gg));
-  const T ib = (T)(1.0 / b);
-  const long base = (long)k * nbnd * npw_pad;
-  for (int i = threadIdx.x; i < nbnd * npw_pad; i += blockDim.x) {
-    Vp[base + i] = Vc[base + i];
-    Vc[base + i] = XV[base + i] * ib;
-    Wp[base + i] = Wc[base + i];
-    Wc[base + i] = cmul(XW[base + i], igc);
+    co.beta[j] = b;
+    co.gamma[j] = gm;
+    const double gg = gm.x * gm.x + gm.y * gm.y;   // 1/conj(gamma) = gamma/|gamma|^2
+    scal[0] = 1.0 / b;
+    scal[1] = gm.x / gg;
+    scal[2] = gm.y / gg;
   }
 }
 
-// z_j = (1/nks) sum_k zpart[j][k] for j in [j0, j1)
-// Device step counter of the pseudo-Hermitian recursion: set before a run of steps, advanced
-// at the end of every step (one thread).
-static __global__ void k_step_set(int* jdev, int j) { *jdev = j; }
-static __global__ void k_step_next(int* jdev) { *jdev += 1; }
+// Non-Hermitian normalisation in place, v_hat/beta and w_hat/conj(gamma) (one vector's n values
+// after the other): they are v_{j+1}, w_{j+1}, and the chain's three pairs of vectors take turns
+// (v_j stays where it is and is v_{j-1} of the next step).  Bound by memory: 4 n values moved
+// (8 n when v_j was copied).
+template <typename T>
+__global__ void __launch_bounds__(256) k_nh_normalize(long n, cplx<T>* __restrict__ XV, cplx<T>* __restrict__ XW,
+                                                      const double* __restrict__ scal) {
+  const T ib = (T)scal[0];
+  const cplx<T> igc = mk((T)scal[1], (T)scal[2]);
+  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
+    XV[i] = XV[i] * ib;
+    XW[i] = cmul(XW[i], igc);
+  }
+}
 
-// (nzp partials per step: one per k, or one per (k, chunk) on the split path)
-static __global__ void k_reduce_z(const cplx<double>* __restrict__ zpart, int nzp, int nks, int j0, int j1,
-                                  cplx<double>* __restrict__ z) {
-  const int j = j0 + blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= j1) return;
+// The device step counter of the pseudo-Hermitian recursion before a run of steps (k_ph_beta
+// advances it).
+static __global__ void k_step_set(int* jdev, int j) { *jdev = j; }
+
+// z_j = (1/nks) sum zpart[j][0..nzp) for j in [j0, j0 + gridDim.x): nzp partials per step, one per
+// (k, band group) or (k, chunk) on the split path, one block per step, fixed order.  (One thread
+// per step took 68 us for the KB workload's 512 partials.)
+static __global__ void __launch_bounds__(128) k_reduce_z(const cplx<double>* __restrict__ zpart, int nzp, int nks, int j0,
+                                                        cplx<double>* __restrict__ z) {
+  __shared__ double wr[4], wi[4];
+  const int j = j0 + blockIdx.x;
   double zr = 0, zi = 0;
-  for (int k = 0; k < nzp; ++k) { zr += zpart[(long)j * nzp + k].x; zi += zpart[(long)j * nzp + k].y; }
-  z[j] = mk(zr / nks, zi / nks);
+  for (int k = threadIdx.x; k < nzp; k += 128) { zr += zpart[(long)j * nzp + k].x; zi += zpart[(long)j * nzp + k].y; }
+  zr = warp_sum(zr);
+  zi = warp_sum(zi);
+  if ((threadIdx.x & 31) == 0) { wr[threadIdx.x >> 5] = zr; wi[threadIdx.x >> 5] = zi; }
+  __syncthreads();
+  if (threadIdx.x == 0) z[j] = mk((wr[0] + wr[1] + wr[2] + wr[3]) / nks, (wi[0] + wi[1] + wi[2] + wi[3]) / nks);
 }
 
 // ---------------------------------------------------------------------------------------

@@ -25,20 +25,6 @@ constexpr int kTile = 32;      // plane waves per shared-memory tile of the dot 
 constexpr int kTileP = kTile + 1;  // padded row of a tile (conflict-free column reads)
 constexpr int kMaxPairs = 2048;  // ni * nj of one dot block (nproj <= 64, nbnd <= 32)
 
-// sum_i p[i], i < n, by the whole block in a fixed order; every thread gets the result.
-__device__ __forceinline__ double block_sum(const double* p, int n) {
-  __shared__ double wsum[32];
-  double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s += p[i];
-  s = warp_sum(s);
-  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = s;
-  __syncthreads();
-  double t = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += wsum[w];
-  __syncthreads();
-  return t;
-}
-
 // out[i*nj + j] = sum_{g0 <= g < g1} conj(A[i*lda + g]) B[j*ldb + g] for all ni x nj pairs.
 // Each thread owns up to kMaxPairs/blockDim pairs; the plane waves stream through shared
 // memory in tiles of kTile, each tile summed in T and added to a double accumulator.
@@ -87,34 +73,23 @@ __device__ void chunk_dots(const cplx<T>* A, long lda, const cplx<T>* B, long ld
   __syncthreads();
 }
 
-// Step j, first part: beta_j = sqrt((1/nks) sum of the norm partials), the z_j partial of
+// Step j, first part, with beta_j from k_ph_beta: the z_j partial of
 // the chunk, r_{j+1} = X_j/beta_j - beta_j v_{j-1} into R, v_j = r_j/beta_j into Vp, and the
 // chunk's partial U^H r_{j+1}.  grid (nks, nchunk), block 256.
 template <typename T>
 __global__ void __launch_bounds__(256) k_sp_start(const int* __restrict__ jdev, int nks, int nbnd, int npw_pad,
                                                   const int* __restrict__ npw, int nchunk,
-                                                  const double* __restrict__ part, cplx<T>* __restrict__ R,
+                                                  const double* __restrict__ scal, cplx<T>* __restrict__ R,
                                                   const cplx<T>* __restrict__ X, cplx<T>* __restrict__ Vp,
                                                   const cplx<T>* __restrict__ y, const cplx<T>* __restrict__ ukq,
-                                                  Coef co, double tol, cplx<double>* __restrict__ spart,
+                                                  Coef co, cplx<double>* __restrict__ spart,
                                                   int dots) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int j = *jdev, r_upper = (j % 2 == 0) ? 1 : 0;   // step index from the device counter
   cplx<T>* tile = reinterpret_cast<cplx<T>*>(smem_raw);
-  __shared__ double sbeta;
   __shared__ double zred[2][8];
   const int k = blockIdx.x, c = blockIdx.y;
   const int g0 = c * kChunk, g1 = min(npw_pad, g0 + kChunk);
-  const double b2 = block_sum(part, nks * nchunk) / nks;
-  if (threadIdx.x == 0) {
-    double b = 1.0;
-    if (!(b2 > tol)) flag_error(co.err, b2 <= 0.0 ? DEV_NOTPD : DEV_BREAKDOWN, j);
-    else b = sqrt(b2);
-    sbeta = b;
-    if (k == 0 && c == 0) { co.beta[j - 1] = b; co.gamma[j - 1] = mk(b, 0.0); }
-  }
-  __syncthreads();
-  const double b = sbeta;
   const long base = (long)k * nbnd * npw_pad;
   const int zi = (j - 1) * nks * nchunk + k * nchunk + c;
   if (r_upper) {  // z_j partial = (y, r_j)/beta_j over the chunk
@@ -132,13 +107,13 @@ __global__ void __launch_bounds__(256) k_sp_start(const int* __restrict__ jdev, 
     if (threadIdx.x == 0) {
       double sr = 0.0, si = 0.0;
       for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { sr += zred[0][w]; si += zred[1][w]; }
-      co.zpart[zi] = mk(sr / b, si / b);
+      co.zpart[zi] = mk(sr * scal[1], si * scal[1]);
     }
   } else if (threadIdx.x == 0) {
     co.zpart[zi] = mk(0.0, 0.0);
   }
   __syncthreads();
-  const T ib = (T)(1.0 / b), bb = (T)b;
+  const T ib = (T)scal[1], bb = (T)scal[0];
   for (int e = threadIdx.x; e < nbnd * (g1 - g0); e += blockDim.x) {
     const int v = e / (g1 - g0), g = g0 + e - v * (g1 - g0);
     const long i = base + (long)v * npw_pad + g;
