@@ -278,7 +278,7 @@ def _sc16(stream, steps: int = 2000):
 
 def source_digest() -> str:
     """sha256 of the code that sets the plane pass's DRAM traffic per launch: common.cuh,
-    fft.cuh, the k_xy section of kernels.cuh and its batch sizes and launch in chain.cuh."""
+    fft.cuh, plane.cuh and its launch in chain.cuh."""
     import hashlib
     csrc = os.path.join(ROOT, "paper_2111_06623_gb300", "csrc")
 
@@ -290,12 +290,8 @@ def source_digest() -> str:
         i = text.index(start)
         return text[i:text.index(end, i)]
 
-    k = read("kernels.cuh")
-    c = read("chain.cuh")
-    parts = [read("common.cuh"), read("fft.cuh"),
-             between(k, "// Per-plane pass of one operator application.", "// Response potential of one density"),
-             between(c, "template <int N, int MODE> struct BO", "};"),
-             between(c, "  int xy_nm(", "  // mode 0: operator pass 1")]
+    parts = [read("common.cuh"), read("fft.cuh"), read("plane.cuh"),
+             between(read("chain.cuh"), "  int xy_nm(", "  int xy_launch(")]
     return hashlib.sha256("\0".join(parts).encode()).hexdigest()[:16]
 
 
@@ -691,7 +687,7 @@ def main():
     roofline = None
     if dom == "xy1":
         ach = flops / (ms_cls[dom] / n_dom / 1e3) / 1e12
-        roofline = {"bound": "alu", "kernel": "k_xy (pass 1: per-plane 2D FFTs, V x, density)", "achieved": ach,
+        roofline = {"bound": "alu", "kernel": "k_plane (pass 1: per-plane 2D FFTs, V x, density)", "achieved": ach,
                     "peak": peak, "unit": "TFLOP/s", "frac": ach / peak, "traffic": profiled_traffic("work_grid_traffic_bytes_per_launch"),
                     "traffic_unit": "bytes per launch (mean of the D+K and D launches)",
                     "peak_source": "FP32 FMA: 152 SMs x 128 lanes x 2 flops x max SM clock (derived)"}

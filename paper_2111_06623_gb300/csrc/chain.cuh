@@ -20,7 +20,7 @@
 #include "ll.h"
 #include "split.cuh"
 #include "tcproj.cuh"
-#include "xypair.cuh"
+#include "plane.cuh"
 
 #include <type_traits>
 
@@ -380,6 +380,11 @@ static inline uint64_t ground_state_hash(const ll_system_desc* d) {
   return h;
 }
 
+// The bounds |m| <= PR the plane pass is built for at side W: W/4 (spheres whose products just
+// fit the grid), two ninths more at W = 48 (the sixteen-atom cell's |m| <= 13), and W/2 - 1, the
+// largest with unique signed indices.
+constexpr int plane_level(int w, int l) { return l == 0 ? w / 4 : l == 1 && w == 48 ? 14 : w / 2 - 1; }
+
 template <typename T>
 class Chain : public ChainBase {
  public:
@@ -494,18 +499,15 @@ class Chain : public ChainBase {
                   d->lattice[0][2] * (d->lattice[1][0] * d->lattice[2][1] - d->lattice[1][1] * d->lattice[2][0]));
     for (int a = 0; a < 3; ++a) q_[a] = d->q_cart[a];
     W_ = work_side(d, hk_.ext.data(), hq_.ext.data());
-    {   // the largest |m| of the k+Q spheres on any axis picks the pruning bound of the lines:
-        // the tightest built level (tight_prune(W), then W/4) that holds every sphere
+    {   // the largest |m| of the k+Q spheres on any axis picks the bound the lines are built with:
+        // the smallest of plane_level's that holds every sphere, 0 (k_xy) where none does
       int pmax = 0;
-      for (int k = 0; k < nks_; ++k)
-        for (int c = 0; c < hq_.ncol[k]; ++c) {
-          const int4 cl = hq_.col[(size_t)k * hq_.ncol_max + c];
-          pmax = std::max({pmax, std::abs(cl.x), std::abs(cl.y), std::abs(cl.z), std::abs(cl.z + cl.w - 1)});
-        }
-      const char* pe = getenv("LL_PRUNE");   // 0: unpruned lines; 1: the W/4 level only
-      const bool off = pe && pe[0] == '0' && pe[1] == 0, wide = pe && pe[0] == '1' && pe[1] == 0;
-      const int tight = tight_prune(W_);
-      prune_ = off ? 0 : (!wide && tight > 0 && pmax <= tight) ? tight : (pmax <= W_ / 4 ? W_ / 4 : 0);
+      for (const Extent& e : hq_.ext)
+        for (int a = 0; a < 3; ++a) pmax = std::max({pmax, std::abs(e.lo[a]), std::abs(e.hi[a])});
+      const char* pe = getenv("LL_PRUNE");   // 0: lines not pruned (the largest bound); 1: W = N
+      prune_ = 0;
+      for (int l = (pe && pe[0] == '0' && pe[1] == 0) ? 2 : 0; l < 3 && !prune_; ++l)
+        if (pmax <= plane_level(W_, l)) prune_ = plane_level(W_, l);
     }
     const int w = W_;
     const long w3 = (long)w * w * w;
@@ -680,8 +682,6 @@ class Chain : public ChainBase {
     {
       const char* g = getenv("LL_GRAPHS");
       use_graphs_ = use_graphs_ && !(g && g[0] == '0' && g[1] == 0);
-      const char* xp = getenv("LL_XY_PAIR");   // 1: lane pairs for every even N, 0: never (k_xy)
-      xy_pair_ = (xp && xp[1] == 0 && (xp[0] == '0' || xp[0] == '1')) ? xp[0] - '0' : -1;
     }
     if ((rc = alloc(&ub_, (long)nks_ * nbnd_ * std::max(1, nproj_)))) return rc;
     // chunk partials: U^H x per vector (two per vector on the non-Hermitian update), B^H x
@@ -783,9 +783,6 @@ class Chain : public ChainBase {
       LL_CK(cudaGetLastError());
     }
 
-
-    // the plane pass's kernel variant and batch per mode, timed on this system (cached per shape)
-    if ((rc = tune_plane_pass(err))) return rc;
 
     // start of the recursion
     if (flavour_ == LL_FLAVOUR_PH) {
@@ -1185,8 +1182,6 @@ class Chain : public ChainBase {
                         red_doubles(256) * sizeof(double);
     int rc;
     auto kern = k_zfwd_proj<T, N>;
-    if constexpr (tight_prune(N) > 0)
-      if (prune_ == tight_prune(N)) kern = k_zfwd_proj<T, N, tight_prune(N)>;
     if (prune_ == N / 4) kern = k_zfwd_proj<T, N, N / 4>;
     if ((rc = set_smem(kern, smem, err))) return rc;
     kern<<<dim3(nks_, nvec, ngrp_), 256, smem, st_>>>(dq_, nbnd_, bpc_, cbuf_, cb_ncol_,
@@ -1372,10 +1367,11 @@ class Chain : public ChainBase {
     int g = std::max(1, (target + W_ - 1) / W_);
     return std::min(g, norb);
   }
-  // Orbital groups of one plane-pass launch (grid N x groups): as many CTAs as fit on the
-  // GPU at once for this mode's occupancy, so that the launch is a single wave.
+  // Orbital groups of one plane-pass launch (grid W x groups): as many CTAs as fit on the GPU at
+  // once for this kernel's occupancy, so that the launch is a single wave (the density pass: at
+  // most the groups its partials are allocated for).
   template <typename K>
-  int groups_for_kernel(K kernel, size_t smem, int norb, int& cache, int threads = 128) {
+  int groups_for_kernel(K kernel, size_t smem, int norb, int& cache, int threads, bool dens) {
     if (cache == 0) {
       int occ = 0;
       if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem) != cudaSuccess || occ < 1) {
@@ -1384,30 +1380,9 @@ class Chain : public ChainBase {
       }
       cache = std::max(1, (occ * nsm_) / W_);
     }
-    return std::max(1, std::min(std::min(cache, ngroups_), norb));
+    return std::max(1, std::min(dens ? std::min(cache, ngroups_) : cache, norb));
   }
-  template <int N, int MODE>
-  int xy_nm(const SphereDev& s, int norb, int o_off, int dens_vec, std::string& err) {
-    const XyChoice c = xy_choice_[MODE];
-    if constexpr (N == 24 || N == 32 || N == 36 || N == 48) {
-      // every line transform split over a lane pair (xypair.cuh): half the registers per thread.
-      // Untuned default: N = 48 only (measured on GB300: faster at N = 48, 16-atom cell pass 2
-      // 0.67 -> 0.55 ms per step; slower at N = 32, KB workload pass 1 0.26 -> 0.29 ms)
-      const bool pair = xy_pair_ >= 0 ? xy_pair_ == 1 : (c.var >= 0 ? c.var == 1 : N == 48);
-      if (pair) return xy_launch<N, MODE>(k_xyp<T, N, MODE>, 4 * N, 2, c.bo, s, norb, o_off, dens_vec, err);
-    }
-    if constexpr (MODE != XY_STORE) {   // lines pruned to the spheres' extent
-      if constexpr (tight_prune(N) > 0)
-        if (prune_ == tight_prune(N))
-          return xy_launch<N, MODE>(k_xy<T, N, MODE, tight_prune(N)>, 128, 128 / N, c.bo, s, norb, o_off, dens_vec, err);
-      if (prune_ == N / 4) return xy_launch<N, MODE>(k_xy<T, N, MODE, N / 4>, 128, 128 / N, c.bo, s, norb, o_off, dens_vec, err);
-    }
-    return xy_launch<N, MODE>(k_xy<T, N, MODE>, 128, 128 / N, c.bo, s, norb, o_off, dens_vec, err);
-  }
-  template <int N, int MODE, typename K>
-  int xy_launch(K kernel, int threads, int slots, int bo, const SphereDev& s, int norb, int o_off, int dens_vec,
-                std::string& err) {
-    int B = bo > 0 ? bo : BO<N, MODE>::v;
+  XYArgs xy_args(const SphereDev& s, int norb, int o_off, int dens_vec) const {
     XYArgs a;
     a.s = s;
     a.nbnd = nbnd_;
@@ -1420,7 +1395,37 @@ class Chain : public ChainBase {
     a.f_nbnd = FastDiv((unsigned)nbnd_);
     a.f_nks = FastDiv((unsigned)s.nks);
     a.f_pervec = FastDiv((unsigned)(s.nks * nbnd_));
-    const int NP = N + 1;
+    return a;
+  }
+  template <int N, int MODE>
+  int xy_nm(const SphereDev& s, int norb, int o_off, int dens_vec, std::string& err) {
+    if constexpr (MODE != XY_STORE) {
+      if (prune_ == plane_level(N, 0)) return plane_launch<N, MODE, plane_level(N, 0)>(s, norb, o_off, dens_vec, err);
+      if constexpr (plane_level(N, 1) != plane_level(N, 2))
+        if (prune_ == plane_level(N, 1)) return plane_launch<N, MODE, plane_level(N, 1)>(s, norb, o_off, dens_vec, err);
+      if (prune_ == plane_level(N, 2)) return plane_launch<N, MODE, plane_level(N, 2)>(s, norb, o_off, dens_vec, err);
+    }
+    return xy_launch<N, MODE>(s, norb, o_off, dens_vec, err);
+  }
+  template <int N, int MODE, int PR>
+  int plane_launch(const SphereDev& s, int norb, int o_off, int dens_vec, std::string& err) {
+    constexpr int threads = PlaneCfg<T, N, MODE>::TH;
+    XYArgs a = xy_args(s, norb, o_off, dens_vec);
+    a.bo = PlaneCfg<T, N, MODE>::SL;
+    const size_t smem = plane_smem<T, N, MODE>(cb_ncol_, s.nrow_max);
+    int rc;
+    if ((rc = set_smem(k_plane<T, N, MODE, PR>, smem, err))) return rc;
+    const int ng = groups_for_kernel(k_plane<T, N, MODE, PR>, smem, norb, xy_groups_[MODE], threads, MODE == XY_PASS1_DENS);
+    a.per_group = (norb + ng - 1) / ng;
+    k_plane<T, N, MODE, PR><<<dim3(N, ng), threads, smem, st_>>>(a, cbuf_, vloc_, vpr_, ur_, nprt_, err_);
+    if (MODE == XY_PASS1_DENS) last_ng_ = ng;
+    LL_CK(cudaGetLastError());
+    return LL_OK;
+  }
+  template <int N, int MODE>
+  int xy_launch(const SphereDev& s, int norb, int o_off, int dens_vec, std::string& err) {
+    XYArgs a = xy_args(s, norb, o_off, dens_vec);
+    const int NP = N + 1, slots = 128 / N;
     auto smem_for = [&](int b) {
       size_t m = (size_t)b * cb_ncol_ + (size_t)b * s.nrow_max * NP;
       if (MODE == XY_PASS2) m += (size_t)N * N;
@@ -1429,130 +1434,21 @@ class Chain : public ChainBase {
       if (MODE == XY_PASS1 || MODE == XY_PASS1_DENS) m += (size_t)N * N * sizeof(T);
       return m;
     };
-    // fewer orbitals per batch where the default batch's tiles exceed shared memory (FP64 at
-    // N = 48 on the 16-atom cell), or would keep the SM below the CTA count its registers
-    // allow (N = 48: 116 KB for 8 orbitals left one 4-warp CTA per SM)
-    if (xy_occ_reg_[MODE] == 0) {
-      int occ = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, 0) != cudaSuccess || occ < 1) {
-        cudaGetLastError();
-        occ = 1;
-      }
-      xy_occ_reg_[MODE] = std::min(occ, 8);
-    }
-    const size_t per_sm = 227 * 1024 - 2048 * (size_t)xy_occ_reg_[MODE];
-    if (bo > 0) {   // a tuned batch: only the shared-memory limit applies
-      while (B > 1 && smem_for(B) > 200 * 1024) --B;
-    } else {
-      while (B > 1 && (smem_for(B) > 200 * 1024 || smem_for(B) * xy_occ_reg_[MODE] > per_sm)) --B;
-    }
+    // fewer orbitals per batch where the default batch's tiles exceed shared memory, or would keep
+    // the SM below four CTAs
+    int B = BO<N, MODE>::v;
+    while (B > 1 && (smem_for(B) > 200 * 1024 || smem_for(B) * 4 > 227 * 1024 - 4 * 2048)) --B;
     const size_t smem = smem_for(B);
     a.bo = B;
     int rc;
-    if ((rc = set_smem(kernel, smem, err))) return rc;
-    const int ng = groups_for_kernel(kernel, smem, norb, xy_groups_[MODE], threads);
+    if ((rc = set_smem(k_xy<T, N, MODE>, smem, err))) return rc;
+    const int ng = groups_for_kernel(k_xy<T, N, MODE>, smem, norb, xy_groups_[MODE], 128, MODE == XY_PASS1_DENS);
     a.per_group = (norb + ng - 1) / ng;
-    kernel<<<dim3(N, ng), threads, smem, st_>>>(a, cbuf_, vloc_, vpr_, ur_, nprt_, ur_);
+    k_xy<T, N, MODE><<<dim3(N, ng), 128, smem, st_>>>(a, cbuf_, vloc_, vpr_, ur_, nprt_, ur_);
     if (MODE == XY_PASS1_DENS) last_ng_ = ng;
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) { err = std::string("k_xy: ") + cudaGetErrorString(e); return LL_ECUDA; }
+    LL_CK(cudaGetLastError());
     return LL_OK;
   }
-  // ---- autotuner of the plane pass ----------------------------------------------------
-  // For each mode of the operator's plane pass (pass 1, pass 1 with the density, pass 2) the
-  // kernel variant (one thread or a lane pair per line transform) and the orbital batch are
-  // chosen by timing whole operator applications on a scratch copy of the starting vector
-  // (CUDA events on the chain's stream; one mode at a time, the others at their current
-  // choice).  The choice is kept per system shape and device for the whole process, so every
-  // chain of one shape in a process uses the same launches (their results agree bit for bit
-  // whatever else runs); LL_TUNE=0 keeps the untuned defaults.
-  int tune_plane_pass(std::string& err) {
-    const char* te = getenv("LL_TUNE");
-    if (te && te[0] == '0' && te[1] == 0) return LL_OK;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    char key[256];
-    snprintf(key, sizeof(key), "%d/%zu/%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%d", dev, sizeof(T), N_, W_, nks_, nbnd_,
-             hq_.npw_pad, cb_ncol_, hq_.nrow_max, nproj_, (int)split_, xy_pair_, (int)prune_, nsm_);
-    {
-      std::lock_guard<std::mutex> lock(tune_mutex());
-      auto it = tune_cache().find(key);
-      if (it != tune_cache().end()) {
-        for (int m = 0; m < 3; ++m) xy_choice_[m] = {it->second[2 * m], it->second[2 * m + 1]};
-        for (int m = 0; m < 3; ++m) xy_occ_reg_[m] = xy_groups_[m] = 0;
-        return LL_OK;
-      }
-    }
-    const long vq = (long)nks_ * nbnd_ * hq_.npw_pad;
-    int rc;
-    if (!scratch_ && (rc = alloc(&scratch_, 2 * vq))) return rc;
-    cudaEvent_t ea, eb;
-    LL_CK(cudaEventCreate(&ea));
-    LL_CK(cudaEventCreate(&eb));
-    auto run = [&](int dens, float* ms) -> int {
-      LL_CK(cudaMemcpyAsync(scratch_, y_, vq * sizeof(cplx<T>), cudaMemcpyDeviceToDevice, st_));
-      LL_CK(cudaEventRecord(ea, st_));
-      int r = op(1, scratch_, scratch_ + vq, dens, err);
-      if (r) return r;
-      LL_CK(cudaEventRecord(eb, st_));
-      LL_CK(cudaEventSynchronize(eb));
-      LL_CK(cudaEventElapsedTime(ms, ea, eb));
-      return LL_OK;
-    };
-    float ms = 0.f;
-    const bool can_pair = (W_ == 24 || W_ == 32 || W_ == 36 || W_ == 48) && xy_pair_ < 0;
-    rc = run(approx_ == LL_APPROX_IPA ? -1 : 0, &ms);   // warm-up: lazy module loads, attributes
-    const int modes[3] = {XY_PASS1, XY_PASS1_DENS, XY_PASS2};
-    for (int mi = 0; mi < 3 && rc == LL_OK; ++mi) {
-      const int mode = modes[mi];
-      if (mode != XY_PASS1 && approx_ == LL_APPROX_IPA) break;   // no density without K
-      const int dens = mode == XY_PASS1 ? -1 : 0;
-      const int bdef = (mode == XY_PASS1) ? 384 / W_ : 256 / W_;
-      std::vector<XyChoice> cand;
-      for (int var = 0; var <= (can_pair ? 1 : 0); ++var) {
-        cand.push_back({var, 0});                             // the occupancy-derived batch
-        for (int b : {bdef, std::max(1, bdef / 2)}) cand.push_back({var, b});
-      }
-      // every candidate timed twice, the rounds interleaved; the fastest of its two times counts
-      std::vector<float> tmin(cand.size(), 1e30f);
-      for (int rep = 0; rep < 2 && rc == LL_OK; ++rep)
-        for (size_t ci = 0; ci < cand.size(); ++ci) {
-          xy_choice_[mode] = cand[ci];
-          xy_occ_reg_[mode] = xy_groups_[mode] = 0;
-          if ((rc = run(dens, &ms)) != LL_OK) break;
-          tmin[ci] = std::min(tmin[ci], ms);
-        }
-      XyChoice pick = cand[0];
-      float best = 1e30f;
-      for (size_t ci = 0; ci < cand.size(); ++ci)
-        if (tmin[ci] < best) { best = tmin[ci]; pick = cand[ci]; }
-      xy_choice_[mode] = pick;
-      xy_occ_reg_[mode] = xy_groups_[mode] = 0;
-    }
-    cudaEventDestroy(ea);
-    cudaEventDestroy(eb);
-    if (rc != LL_OK) return rc;
-    std::lock_guard<std::mutex> lock(tune_mutex());
-    auto it = tune_cache().find(key);
-    if (it != tune_cache().end()) {   // another chain of this shape tuned meanwhile: use its choice
-      for (int m = 0; m < 3; ++m) xy_choice_[m] = {it->second[2 * m], it->second[2 * m + 1]};
-      for (int m = 0; m < 3; ++m) xy_occ_reg_[m] = xy_groups_[m] = 0;
-    } else {
-      std::array<int, 6> v;
-      for (int m = 0; m < 3; ++m) v[2 * m] = xy_choice_[m].var, v[2 * m + 1] = xy_choice_[m].bo;
-      tune_cache()[key] = v;
-    }
-    return LL_OK;
-  }
-  static std::mutex& tune_mutex() {
-    static std::mutex m;
-    return m;
-  }
-  static std::map<std::string, std::array<int, 6>>& tune_cache() {
-    static std::map<std::string, std::array<int, 6>> c;
-    return c;
-  }
-
   // mode 0: operator pass 1 (with the density when dens_vec >= 0); 1: pass 2; 2: store x(r)
   template <int N>
   int xy_n(const SphereDev& s, int norb, int o_off, int dens_vec, int mode, std::string& err) {
@@ -1788,11 +1684,7 @@ class Chain : public ChainBase {
   bool eager_done_[2] = {false, false};
   cudaGraphExec_t graph_[2] = {nullptr, nullptr};   // one captured step per parity of j
   bool split_ = false;      // per-k work split over chunks of plane waves (split.cuh)
-  int xy_occ_reg_[4] = {0, 0, 0, 0};   // CTAs per SM the plane pass's registers allow, per mode
-  int xy_pair_ = -1;                   // LL_XY_PAIR: 1 lane pairs for every even N, 0 never, -1 not forced
-  int prune_ = 0;                      // line transforms pruned to |m| <= prune_ (0: unpruned)
-  struct XyChoice { int var; int bo; };    // plane-pass kernel (0 k_xy, 1 k_xyp) and orbital batch
-  XyChoice xy_choice_[4] = {{-1, 0}, {-1, 0}, {-1, 0}, {-1, 0}};   // per mode; -1 / 0: the untuned default
+  int prune_ = 0;                      // bound |m| <= prune_ of the plane pass's lines (0: k_xy)
   bool tc_op_ = false, tc_u_ = false, tc_u2_ = false;   // split-path dot blocks on the tensor cores
   bool tc_ap_ = false;                                    // split-path projections applied on the tensor cores
   int tc_nb_op_ = 32, tc_nb_u_ = 32, tc_nb_ap_ = 32;      // N of those MMAs (Bop rows, padded to 32)

@@ -57,42 +57,80 @@ __device__ __forceinline__ cplx<T> twiddle(int e) {
   return w;
 }
 
+// Arithmetic with explicit rounding: what the compiler may contract is written out, so a
+// transform's result does not depend on what surrounds it (a pruned instantiation rounds as the
+// dense one).
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+template <typename T> __device__ __forceinline__ cplx<T> cadd(cplx<T> a, cplx<T> b) { return mk(add_rn(a.x, b.x), add_rn(a.y, b.y)); }
+template <typename T> __device__ __forceinline__ cplx<T> csub(cplx<T> a, cplx<T> b) { return mk(add_rn(a.x, -b.x), add_rn(a.y, -b.y)); }
+template <typename T> __device__ __forceinline__ cplx<T> cmul_rn(cplx<T> a, cplx<T> w) {
+  return mk(fma_rn(a.x, w.x, mul_rn(-a.y, w.y)), fma_rn(a.x, w.y, mul_rn(a.y, w.x)));
+}
+// a + w b and a - w b in six FMAs (a complex product and two additions: eight operations)
+template <typename T> __device__ __forceinline__ void butterfly(cplx<T> a, cplx<T> b, cplx<T> w, cplx<T>& s, cplx<T>& d) {
+  s = mk(fma_rn(w.x, b.x, fma_rn(-w.y, b.y, a.x)), fma_rn(w.x, b.y, fma_rn(w.y, b.x, a.y)));
+  d = mk(fma_rn(T(2), a.x, -s.x), fma_rn(T(2), a.y, -s.y));
+}
+
 // R-point DFT in place with exponent sign SIGN.
 template <typename T, int R, int SIGN> struct Dft;
 
+// w1 multiplies input 1 and w1^2 input 2 (and w1^3 input 3) where TW (a twiddled pass).
 template <typename T, int SIGN> struct Dft<T, 2, SIGN> {
-  static __device__ __forceinline__ void run(cplx<T>* v) {
-    cplx<T> a = v[0], b = v[1];
-    v[0] = a + b;
-    v[1] = a - b;
+  template <bool TW>
+  static __device__ __forceinline__ void run(cplx<T>* v, cplx<T> w1, cplx<T>) {
+    const cplx<T> a = v[0], b = v[1];
+    if (TW) {
+      butterfly(a, b, w1, v[0], v[1]);
+    } else {
+      v[0] = cadd(a, b);
+      v[1] = csub(a, b);
+    }
   }
 };
 
 template <typename T, int SIGN> struct Dft<T, 3, SIGN> {
-  static __device__ __forceinline__ void run(cplx<T>* v) {
+  template <bool TW>
+  static __device__ __forceinline__ void run(cplx<T>* v, cplx<T> w1, cplx<T> w2) {
     // W_3 = -1/2 + SIGN i sqrt(3)/2
     const T c = T(-0.5);
     const T s = T(SIGN) * T(0.86602540378443864676372317075294);
-    cplx<T> a = v[0], b = v[1], d = v[2];
-    cplx<T> sum = b + d, dif = b - d;
-    v[0] = a + sum;
-    cplx<T> m = mk(a.x + c * sum.x, a.y + c * sum.y);
+    cplx<T> a = v[0], sum, dif;
+    if (TW) butterfly(cmul_rn(v[1], w1), v[2], w2, sum, dif);
+    else sum = cadd(v[1], v[2]), dif = csub(v[1], v[2]);
+    v[0] = cadd(a, sum);
+    cplx<T> m = mk(fma_rn(c, sum.x, a.x), fma_rn(c, sum.y, a.y));
     // i s dif = (-s dif.y, s dif.x)
-    v[1] = mk(m.x - s * dif.y, m.y + s * dif.x);
-    v[2] = mk(m.x + s * dif.y, m.y - s * dif.x);
+    v[1] = mk(fma_rn(-s, dif.y, m.x), fma_rn(s, dif.x, m.y));
+    v[2] = mk(fma_rn(s, dif.y, m.x), fma_rn(-s, dif.x, m.y));
   }
 };
 
 template <typename T, int SIGN> struct Dft<T, 4, SIGN> {
-  static __device__ __forceinline__ void run(cplx<T>* v) {
-    cplx<T> a0 = v[0] + v[2], a1 = v[0] - v[2];
-    cplx<T> b0 = v[1] + v[3], b1 = v[1] - v[3];
-    // SIGN i b1
-    cplx<T> jb1 = (SIGN > 0) ? mk(-b1.y, b1.x) : mk(b1.y, -b1.x);
-    v[0] = a0 + b0;
-    v[2] = a0 - b0;
-    v[1] = a1 + jb1;
-    v[3] = a1 - jb1;
+  template <bool TW>
+  static __device__ __forceinline__ void run(cplx<T>* v, cplx<T> w1, cplx<T> w2) {
+    cplx<T> a0, a1, b0, b1;
+    if (TW) {   // w1 v1 +- w3 v3 = w1 (v1 +- w2 v3): the factor w1 goes into the last butterflies
+      butterfly(v[0], v[2], w2, a0, a1);
+      butterfly(v[1], v[3], w2, b0, b1);
+      butterfly(a0, b0, w1, v[0], v[2]);
+      const cplx<T> jw = (SIGN > 0) ? mk(-w1.y, w1.x) : mk(w1.y, -w1.x);   // SIGN i w1
+      butterfly(a1, b1, jw, v[1], v[3]);
+    } else {
+      a0 = cadd(v[0], v[2]), a1 = csub(v[0], v[2]);
+      b0 = cadd(v[1], v[3]), b1 = csub(v[1], v[3]);
+      // SIGN i b1
+      const cplx<T> jb1 = (SIGN > 0) ? mk(-b1.y, b1.x) : mk(b1.y, -b1.x);
+      v[0] = cadd(a0, b0);
+      v[2] = csub(a0, b0);
+      v[1] = cadd(a1, jb1);
+      v[3] = csub(a1, jb1);
+    }
   }
 };
 
@@ -103,12 +141,10 @@ __device__ __forceinline__ void stockham_pass(const cplx<T>* in, cplx<T>* out) {
   for (int j = 0; j < N / R; ++j) {
     cplx<T> v[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      v[r] = in[j + r * (N / R)];
-      const int e = ((j % Ns) * r * (N / (Ns * R))) % N;
-      if (e != 0) v[r] = cmul(v[r], twiddle<T, N, SIGN>(e));
-    }
-    Dft<T, R, SIGN>::run(v);
+    for (int r = 0; r < R; ++r) v[r] = in[j + r * (N / R)];
+    const int e = (j % Ns) * (N / (Ns * R));   // twiddle exponent of input 1
+    if (e != 0) Dft<T, R, SIGN>::template run<true>(v, twiddle<T, N, SIGN>(e), twiddle<T, N, SIGN>(2 * e));
+    else Dft<T, R, SIGN>::template run<false>(v, v[0], v[0]);
     const int d = (j / Ns) * Ns * R + (j % Ns);
 #pragma unroll
     for (int r = 0; r < R; ++r) out[d + r * Ns] = v[r];
@@ -140,11 +176,10 @@ __device__ __forceinline__ void fft_line(cplx<T> (&a)[N]) {
   }
 }
 
-// Input pruning.  A point p of a line whose sphere keeps only |m| <= PR (p <= PR or p >= N - PR)
-// is zero on input; the first pass knows these zeros at compile time (a value with a constant
-// flag) and skips every add whose operand is such a zero.  The arithmetic on the other values
-// is the dense pass's, operation for operation, so the result equals fft_line's (up to the
-// sign of exact zeros).
+// Input pruning.  A line whose points i are zero unless i <= LO or i >= N - HI: the first pass
+// knows these zeros at compile time (a value with a constant flag) and skips every add whose
+// operand is such a zero.  The arithmetic on the other values is the dense pass's, operation for
+// operation, so the result equals fft_line's (up to the sign of exact zeros).
 template <typename T>
 struct ZC {
   cplx<T> v;
@@ -154,13 +189,13 @@ template <typename T>
 __device__ __forceinline__ ZC<T> zadd(ZC<T> a, ZC<T> b) {
   if (a.z) return b;
   if (b.z) return a;
-  return {a.v + b.v, false};
+  return {cadd(a.v, b.v), false};
 }
 template <typename T>
 __device__ __forceinline__ ZC<T> zsub(ZC<T> a, ZC<T> b) {
   if (b.z) return a;
   if (a.z) return {mk(-b.v.x, -b.v.y), false};
-  return {a.v - b.v, false};
+  return {csub(a.v, b.v), false};
 }
 
 template <typename T, int R, int SIGN> struct ZDft;
@@ -186,15 +221,14 @@ template <typename T, int SIGN> struct ZDft<T, 3, SIGN> {   // all zero, or the 
   static __device__ __forceinline__ void run(ZC<T>* v) {
     if (v[0].z && v[1].z && v[2].z) return;
     cplx<T> d[3] = {v[0].z ? czero<T>() : v[0].v, v[1].z ? czero<T>() : v[1].v, v[2].z ? czero<T>() : v[2].v};
-    Dft<T, 3, SIGN>::run(d);
+    Dft<T, 3, SIGN>::template run<false>(d, d[0], d[0]);
     for (int r = 0; r < 3; ++r) v[r] = {d[r], false};
   }
 };
 
-// fft_line<T, N, SIGN> of a line that is zero outside |m| <= PR (PR = 0: fft_line itself).
-template <typename T, int N, int SIGN, int PR>
+template <typename T, int N, int SIGN, int LO, int HI>
 __device__ __forceinline__ void fft_line_in(cplx<T> (&a)[N]) {
-  if constexpr (PR == 0) {
+  if constexpr (LO + HI + 1 >= N) {
     fft_line<T, N, SIGN>(a);
   } else {
     constexpr int R0 = Plan<N>::r[0], R1 = Plan<N>::r[1], R2 = Plan<N>::r[2];
@@ -205,7 +239,7 @@ __device__ __forceinline__ void fft_line_in(cplx<T> (&a)[N]) {
 #pragma unroll
       for (int r = 0; r < R0; ++r) {
         const int i = j + r * (N / R0);
-        const bool kept = i <= PR || i >= N - PR;
+        const bool kept = i <= LO || i >= N - HI;
         v[r] = {kept ? a[i] : czero<T>(), !kept};
       }
       ZDft<T, R0, SIGN>::run(v);
@@ -233,33 +267,47 @@ __device__ __forceinline__ cplx<T> shfl_pair(cplx<T> v, unsigned mask) {
   return mk(__shfl_xor_sync(mask, v.x, 1), __shfl_xor_sync(mask, v.y, 1));
 }
 
-template <typename T, int H, int SIGN>
+template <typename T, int H, int SIGN, int LO = H, int HI = H>   // points a[m] zero unless m <= LO or m >= H - HI
 __device__ __forceinline__ void fft_pair_dit(cplx<T> (&a)[H], int h, unsigned mask) {
-  fft_line<T, H, SIGN>(a);               // Y_h[k] = sum_m x[2m + h] W_H^(mk)
+  fft_line_in<T, H, SIGN, LO, HI>(a);    // Y_h[k] = sum_m x[2m + h] W_H^(mk)
   if (h) {
 #pragma unroll
-    for (int k = 1; k < H; ++k) a[k] = cmul(a[k], twiddle<T, 2 * H, SIGN>(k));   // W_2H^k Y_1[k]
+    for (int k = 1; k < H; ++k) a[k] = cmul_rn(a[k], twiddle<T, 2 * H, SIGN>(k));   // W_2H^k Y_1[k]
   }
+  const T s = h ? T(-1) : T(1);
 #pragma unroll
   for (int k = 0; k < H; ++k) {
     const cplx<T> o = shfl_pair(a[k], mask);
-    a[k] = h ? o - a[k] : a[k] + o;        // X[k] = Y0 + W Y1,  X[k + H] = Y0 - W Y1
+    a[k] = mk(fma_rn(s, a[k].x, o.x), fma_rn(s, a[k].y, o.y));   // X[k] = Y0 + W Y1,  X[k + H] = Y0 - W Y1
   }
 }
 
 template <typename T, int H, int SIGN>
 __device__ __forceinline__ void fft_pair_dif(cplx<T> (&a)[H], int h, unsigned mask) {
+  const T s = h ? T(-1) : T(1);
 #pragma unroll
-  for (int j = 0; j < H; ++j) {
+  for (int j = 0; j < H; ++j) {            // x[j] + x[j + H], or x[j] - x[j + H]
     const cplx<T> o = shfl_pair(a[j], mask);
-    if (h) {
-      a[j] = o - a[j];                     // x[j] - x[j + H]
-      if (j) a[j] = cmul(a[j], twiddle<T, 2 * H, SIGN>(j));
-    } else {
-      a[j] = a[j] + o;                     // x[j] + x[j + H]
-    }
+    a[j] = mk(fma_rn(s, a[j].x, o.x), fma_rn(s, a[j].y, o.y));
+  }
+  if (h) {
+#pragma unroll
+    for (int j = 1; j < H; ++j) a[j] = cmul_rn(a[j], twiddle<T, 2 * H, SIGN>(j));
   }
   fft_line<T, H, SIGN>(a);               // even (h = 0) or odd (h = 1) outputs
+}
+
+// A line of W points on P lanes (P = 1: one thread; P = 2: a lane pair, h its lane):
+// inverse from points that are zero outside i <= LO, i >= W/P - HI, and forward.
+template <typename T, int W, int P, int LO, int HI>
+__device__ __forceinline__ void line_inv(cplx<T> (&a)[W / P], int h, unsigned mask) {
+  if constexpr (P == 1) fft_line_in<T, W, +1, LO, HI>(a);
+  else fft_pair_dit<T, W / 2, +1, LO, HI>(a, h, mask);
+}
+template <typename T, int W, int P>
+__device__ __forceinline__ void line_fwd(cplx<T> (&a)[W / P], int h, unsigned mask) {
+  if constexpr (P == 1) fft_line<T, W, -1>(a);
+  else fft_pair_dif<T, W / 2, -1>(a, h, mask);
 }
 
 }  // namespace ll

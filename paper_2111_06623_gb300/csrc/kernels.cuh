@@ -68,7 +68,10 @@ __device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
 }
 
 // ---------------------------------------------------------------------------------------
-// Per-plane pass of one operator application.  grid (N planes, groups), block 128.
+// Per-plane pass of one operator application, for any Miller indices that fit the grid (the
+// orbital grids at set-up, and spheres beyond |m| < N/2, a Q far outside the first zone; every
+// other application takes k_plane, plane.cuh, with the same modes).  grid (N planes, groups),
+// block 128.
 // The sphere's columns are ordered by (m2, m1) and grouped in rows of equal m2 (consecutive
 // m1).  For every orbital of the group (BO at a time), at plane j3 = blockIdx.x:
 //   rows     1D FFT along axis 1 (m1 <-> j1) of every sphere row, between the column buffer
@@ -104,11 +107,7 @@ struct XYArgs {
   FastDiv f_pervec;            // orbital -> vector: o / (nks nbnd)
 };
 
-// The pruning bounds built besides N/4: 3N/16 at N = 32 (the spheres of a 25 Ry cutoff on the
-// two-atom cell reach |m| = 6), none elsewhere.
-__host__ __device__ constexpr int tight_prune(int n) { return n == 32 ? 3 * n / 16 : 0; }
-
-// Output pruning of the forward line transforms: with PR > 0 every sphere of the system has
+// Output pruning of the forward column transforms: with PR > 0 every sphere of the system has
 // |m| <= PR on all three axes, so only the points p <= PR and p >= N - PR of a forward line
 // are kept; with the stores of the other points gone at compile time, the compiler drops
 // the butterflies that only feed them.  PR = 0: every point.
@@ -117,7 +116,7 @@ __device__ __forceinline__ constexpr bool line_kept(int p) {
   return PR == 0 || p <= PR || p >= N - PR;
 }
 
-template <typename T, int N, int MODE, int PR = 0>
+template <typename T, int N, int MODE>
 __global__ void __launch_bounds__(128, N > 36 ? 2 : (MODE == XY_PASS1_DENS ? 3 : 4)) k_xy(XYArgs a, cplx<T>* __restrict__ cbuf, const T* __restrict__ vloc,
                                                const cplx<T>* __restrict__ vpr, const cplx<T>* __restrict__ ur,
                                                cplx<T>* __restrict__ nprt, cplx<T>* __restrict__ grid_out) {
@@ -187,7 +186,7 @@ __global__ void __launch_bounds__(128, N > 36 ? 2 : (MODE == XY_PASS1_DENS ? 3 :
           const int j = wrapn<N>(p - rw.z);
           l[p] = (j < rw.w && LL_INB(rw.y >= 0 && rw.y + j < a.cb_ncol)) ? cs[j] : czero<T>();
         }
-        fft_line_in<T, N, +1, (MODE == XY_STORE ? 0 : PR)>(l);
+        fft_line<T, N, +1>(l);
         cplx<T>* ys = Ys + (b * s.nrow_max + r) * NP;
 #pragma unroll
         for (int p = 0; p < N; ++p) ys[p] = l[p];
@@ -212,7 +211,7 @@ __global__ void __launch_bounds__(128, N > 36 ? 2 : (MODE == XY_PASS1_DENS ? 3 :
           const int r = wrapn<N>(p - m2min);
           l[p] = (r < nr && LL_INB(r < s.nrow_max)) ? Ys[(b * s.nrow_max + r) * NP + j1] : czero<T>();
         }
-        fft_line_in<T, N, +1, (MODE == XY_STORE ? 0 : PR)>(l);
+        fft_line<T, N, +1>(l);
         if (MODE == XY_STORE) {
           cplx<T>* dst = grid_out + (long)o * N * plane + iz * plane + j1;
 #pragma unroll
@@ -233,7 +232,7 @@ __global__ void __launch_bounds__(128, N > 36 ? 2 : (MODE == XY_PASS1_DENS ? 3 :
 #pragma unroll
       for (int p = 0; p < N; ++p) {
         const int r = wrapn<N>(p - m2min);
-        if (line_kept<N, PR>(p) && r < nr && LL_INB(r < s.nrow_max)) Ys[(b * s.nrow_max + r) * NP + j1] = l[p];
+        if (r < nr && LL_INB(r < s.nrow_max)) Ys[(b * s.nrow_max + r) * NP + j1] = l[p];
       }
     }
     __syncthreads();
@@ -253,7 +252,7 @@ __global__ void __launch_bounds__(128, N > 36 ? 2 : (MODE == XY_PASS1_DENS ? 3 :
 #pragma unroll
       for (int p = 0; p < N; ++p) {
         const int j = wrapn<N>(p - rw.z);
-        if (line_kept<N, PR>(p) && j < rw.w && LL_INB(rw.y >= 0 && rw.y + j < a.cb_ncol)) cs[j] = l[p];
+        if (j < rw.w && LL_INB(rw.y >= 0 && rw.y + j < a.cb_ncol)) cs[j] = l[p];
       }
     }
     __syncthreads();
