@@ -633,7 +633,7 @@ class Chain : public ChainBase {
                           32 * 32 * sizeof(cplx<T>);
         const size_t nh = (size_t)nbnd_ * 2 * b * sizeof(cplx<double>) + 2 * 32 * 32 * sizeof(cplx<T>);
         return 2 * (size_t)b * pq * sizeof(cplx<T>) + (flavour_ == LL_FLAVOUR_NH ? std::max(op, nh) : op) +
-               red_doubles(256) * sizeof(double) + 4096;
+               red_elems(512) * sizeof(T) + 4096;
       };
       int best = 0;
       for (int b = nbnd_; b >= 1 && !best; --b)
@@ -837,7 +837,7 @@ class Chain : public ChainBase {
     int rc;
     const int pq = hq_.npw_pad;
     const size_t smem_nh = 2 * (size_t)bpc_ * pq * sizeof(cplx<T>) + (size_t)nbnd_ * 2 * bpc_ * sizeof(cplx<double>) +
-                           red_doubles(256) * sizeof(double);
+                           red_elems(proj_threads(hq_.npw_pad)) * sizeof(T);
     Coef co{beta_, gamma_, zpart_, err_};
     if (flavour_ == LL_FLAVOUR_PH && n > 0) {
       k_step_set<<<1, 1, 0, st_>>>(jdev_, queued_);
@@ -879,7 +879,7 @@ class Chain : public ChainBase {
           prof_.count(LL_PROF_UPDATE, 1);
         } else {
           if ((rc = set_smem(k_nh_update<T>, smem_nh, err))) return rc;
-          k_nh_update<T><<<dim3(nks_, ngrp_), 256, smem_nh, st_>>>(j, upper, nks_, nbnd_, bpc_, pq, dq_.npw, XV(),
+          k_nh_update<T><<<dim3(nks_, ngrp_), proj_threads(hq_.npw_pad), smem_nh, st_>>>(j, upper, nks_, nbnd_, bpc_, pq, dq_.npw, XV(),
                                                                    XW(), VpNH(), Wp(),
                                                       Vc(), y_, ukq_, co, spart_, md_.keep);
         }
@@ -926,7 +926,7 @@ class Chain : public ChainBase {
       prof_.count(LL_PROF_HXC, 3);
       prof_.count(LL_PROF_XY2);
     }
-    prof_.count(LL_PROF_ZFWD, split_ ? 4 + (metal_ ? 1 : 0) : 1);
+    prof_.count(LL_PROF_ZFWD, split_ ? 4 + (metal_ ? 1 : 0) : 2);
   }
   int capture_step(int j, std::string& err) {
     cudaGraph_t g = nullptr;
@@ -1169,24 +1169,33 @@ class Chain : public ChainBase {
       prof_.span(LL_PROF_XY2, e3, e2);
     }
     if ((rc = launch_zfwd_proj(nvec, in, out, err))) return rc;
-    prof_.count(LL_PROF_ZFWD, split_ ? 4 + (metal_ ? 1 : 0) : 1);
+    prof_.count(LL_PROF_ZFWD, split_ ? 4 + (metal_ ? 1 : 0) : 2);
     prof_.span(LL_PROF_ZFWD, e2, prof_.mark(st_));
     return LL_OK;
   }
 
   template <int N>
+  int zfwd_n(int nvec, const cplx<T>* in, cplx<T>* out) {   // columns -> t = kinetic + gathered, in `out`
+    const dim3 grid(nks_, nvec, (nbnd_ * hq_.ncol_max + kLines - 1) / kLines);
+    if (prune_ == plane_level(N, 0))
+      k_zfwd<T, N, plane_level(N, 0)><<<grid, kLines, 0, st_>>>(dq_, nbnd_, cbuf_, cb_ncol_, in, kin_, eps_, out);
+    else if (prune_ > 0 && prune_ == plane_level(N, 1))
+      k_zfwd<T, N, plane_level(N, 1)><<<grid, kLines, 0, st_>>>(dq_, nbnd_, cbuf_, cb_ncol_, in, kin_, eps_, out);
+    else
+      k_zfwd<T, N><<<grid, kLines, 0, st_>>>(dq_, nbnd_, cbuf_, cb_ncol_, in, kin_, eps_, out);
+    return cudaGetLastError() == cudaSuccess ? LL_OK : LL_ECUDA;
+  }
+  template <int N>
   int zfwd_proj_n(int nvec, const cplx<T>* in, cplx<T>* out, std::string& err) {
-    if (split_) return zfwd_split_n<N>(nvec, in, out, err);
-    const size_t smem = 2 * (size_t)bpc_ * hq_.npw_pad * sizeof(cplx<T>) +
-                        (size_t)(nproj_ + nbnd_) * bpc_ * (sizeof(cplx<double>) + sizeof(cplx<T>)) +
-                        red_doubles(256) * sizeof(double);
     int rc;
-    auto kern = k_zfwd_proj<T, N>;
-    if (prune_ == N / 4) kern = k_zfwd_proj<T, N, N / 4>;
-    if ((rc = set_smem(kern, smem, err))) return rc;
-    kern<<<dim3(nks_, nvec, ngrp_), 256, smem, st_>>>(dq_, nbnd_, bpc_, cbuf_, cb_ncol_,
-                                                                    metal_ ? img_ : in, kin_, eps_, ukq_, bkq_,
-                                                                    dij_, ub_, nproj_, out, part_, md_, zp_);
+    const cplx<T>* x = metal_ ? img_ : in;   // a metal: the kinetic, KB and norm terms act on the image Q z
+    if ((rc = zfwd_n<N>(nvec, x, out))) { err = "zfwd launch"; return rc; }
+    if (split_) return proj_split(nvec, x, out, err);
+    const size_t smem = (size_t)(nproj_ + nbnd_) * bpc_ * (sizeof(cplx<double>) + sizeof(cplx<T>)) +
+                        red_elems(proj_threads(hq_.npw_pad)) * sizeof(T);
+    if ((rc = set_smem(k_op_proj<T>, smem, err))) return rc;
+    k_op_proj<T><<<dim3(nks_, nvec, ngrp_), proj_threads(hq_.npw_pad), smem, st_>>>(
+        dq_, nbnd_, bpc_, x, ukq_, bkq_, dij_, ub_, nproj_, out, part_, md_, zp_);
     LL_CK(cudaGetLastError());
     return LL_OK;
   }
@@ -1256,12 +1265,8 @@ class Chain : public ChainBase {
   }
 
   // split per-k path (split.cuh): several CTAs per k-point, chunk partials reduced in order
-  template <int N>
-  int zfwd_split_n(int nvec, const cplx<T>* in, cplx<T>* out, std::string& err) {
+  int proj_split(int nvec, const cplx<T>* in, cplx<T>* out, std::string& err) {
     const int pq = hq_.npw_pad;
-    if (metal_) in = img_;   // a metal: the kinetic, KB and norm terms act on the image Q z
-    const int lines = (nbnd_ * hq_.ncol_max + kLines - 1) / kLines;
-    k_sp_zfwd<T, N><<<dim3(nks_, nvec, lines), kLines, 0, st_>>>(dq_, nbnd_, cbuf_, cb_ncol_, in, kin_, eps_, out);
     const size_t sm_d = (size_t)(std::max(nproj_, nbnd_) + nbnd_) * kTileP * sizeof(cplx<T>);
     const size_t sm_a = (size_t)(nproj_ + nbnd_) * (nbnd_ + kSub) * sizeof(cplx<T>);
     int rc;
@@ -1311,24 +1316,23 @@ class Chain : public ChainBase {
     }
     const cplx<T>* rin = metal_image(R(), 1);
     if (!rin) { err = "metal image launch"; return LL_ECUDA; }
-    k_zinv<T, N><<<dim3(nks_, 1, zsplit()), 128, 0, st_>>>(dq_, rin, nbnd_, cbuf_, cb_ncol_);
-    LL_CK(cudaGetLastError());
-    return LL_OK;
+    return zinv_n<N>(dq_, rin, 1);
   }
   template <int N>
   int zinv_ph_n(int j, std::string& err) {
     if (split_) return zinv_split_n<N>(j, err);
     const size_t smem = (size_t)bpc_ * hq_.npw_pad * sizeof(cplx<T>) + (size_t)nbnd_ * bpc_ * sizeof(cplx<double>) +
-                        red_doubles(256) * sizeof(double);
+                        red_elems(proj_threads(hq_.npw_pad)) * sizeof(T);
     int rc;
     Coef co{beta_, gamma_, zpart_, err_};
     // the per-(k, band group) update, then the axis-3 inverse FFTs, one thread per column line
     if ((rc = set_smem(k_ph_update<T>, smem, err))) return rc;
-    k_ph_update<T><<<dim3(nks_, ngrp_), 256, smem, st_>>>(jdev_, dq_, nbnd_, bpc_, scal_, R(), X(), Vp(), y_, ukq_, co,
+    k_ph_update<T><<<dim3(nks_, ngrp_), proj_threads(hq_.npw_pad), smem, st_>>>(jdev_, dq_, nbnd_, bpc_, scal_, R(), X(), Vp(), y_, ukq_, co,
                                                           md_.keep);
-    k_zinv<T, N><<<dim3(nks_, 1, zsplit()), 128, 0, st_>>>(dq_, metal_image(R(), 1), nbnd_, cbuf_, cb_ncol_);
     LL_CK(cudaGetLastError());
-    return LL_OK;
+    const cplx<T>* rin = metal_image(R(), 1);
+    if (!rin) { err = "metal image launch"; return LL_ECUDA; }
+    return zinv_n<N>(dq_, rin, 1);
   }
   int launch_zinv_ph(int j, std::string& err) {
     switch (W_) {
@@ -1347,7 +1351,14 @@ class Chain : public ChainBase {
   int zsplit() const { return std::max(1, (nbnd_ * std::max(hk_.ncol_max, hq_.ncol_max) + 127) / 128); }
   template <int N>
   int zinv_n(const SphereDev& s, const cplx<T>* in, int nvec) {
-    k_zinv<T, N><<<dim3(nks_, nvec, zsplit()), 128, 0, st_>>>(s, in, nbnd_, cbuf_, cb_ncol_);
+    // pruned where the spheres are the k+Q ones the bound holds for (not sphere(k) at set-up)
+    const dim3 grid(nks_, nvec, zsplit());
+    if (s.col == dq_.col && prune_ == plane_level(N, 0))
+      k_zinv<T, N, plane_level(N, 0)><<<grid, 128, 0, st_>>>(s, in, nbnd_, cbuf_, cb_ncol_);
+    else if (s.col == dq_.col && prune_ > 0 && prune_ == plane_level(N, 1))
+      k_zinv<T, N, plane_level(N, 1)><<<grid, 128, 0, st_>>>(s, in, nbnd_, cbuf_, cb_ncol_);
+    else
+      k_zinv<T, N><<<grid, 128, 0, st_>>>(s, in, nbnd_, cbuf_, cb_ncol_);
     return cudaGetLastError() == cudaSuccess ? LL_OK : LL_ECUDA;
   }
   int launch_zinv(const SphereDev& s, const cplx<T>* in, int nvec) {

@@ -31,11 +31,20 @@ struct SphereDev {
 template <int N>
 __device__ __forceinline__ int wrapn(int m) { return (int)((unsigned)(m + N) % (unsigned)N); }
 
+// Pruned lines: with PR > 0 every sphere of the system has |m| <= PR on all three axes, so only the
+// points p <= PR and p >= N - PR of a line are kept; with the stores of the other points gone at
+// compile time, the compiler drops the butterflies that only feed them.  PR = 0: every point.
+template <int N, int PR>
+__device__ __forceinline__ constexpr bool line_kept(int p) {
+  return PR == 0 || p <= PR || p >= N - PR;
+}
+
 // ---------------------------------------------------------------------------------------
 // Sphere -> columns: scatter each column's points and inverse-FFT along axis 3.
 // grid (nks, nvec, split), block 128; item = (v, column), the k block's items spread over
-// the split CTAs.
-template <typename T, int N>
+// the split CTAs.  PR > 0: every point of the spheres has |m| <= PR (PR < N/2), so a point's
+// offset is a compile-time constant and the zeros outside are known (PR = 0: any indices).
+template <typename T, int N, int PR = 0>
 __global__ void __launch_bounds__(128) k_zinv(SphereDev s, const cplx<T>* __restrict__ x, int nbnd,
                                               cplx<T>* __restrict__ cbuf, int cb_ncol) {
   const int k = blockIdx.x, vec = blockIdx.y;
@@ -49,10 +58,14 @@ __global__ void __launch_bounds__(128) k_zinv(SphereDev s, const cplx<T>* __rest
     cplx<T> a[N];
 #pragma unroll
     for (int p = 0; p < N; ++p) {
-      const int i = wrapn<N>(p - cl.z);
-      a[p] = (i < cl.w && LL_INB(st >= 0 && st + i < s.npw_pad)) ? src[i] : czero<T>();
+      a[p] = czero<T>();
+      if (line_kept<N, PR>(p)) {
+        const int i = PR > 0 ? (p <= PR ? p : p - N) - cl.z : wrapn<N>(p - cl.z);
+        if ((unsigned)i < (unsigned)cl.w && LL_INB(st >= 0 && st + i < s.npw_pad)) a[p] = src[i];
+      }
     }
-    fft_line<T, N, +1>(a);
+    if constexpr (PR > 0) fft_line_in<T, N, +1, PR, PR>(a);
+    else fft_line<T, N, +1>(a);
     if (!LL_INB(c < cb_ncol)) continue;
     cplx<T>* dst = cbuf + o * (long)N * cb_ncol + c;
 #pragma unroll
@@ -106,15 +119,6 @@ struct XYArgs {
   FastDiv f_nbnd, f_nks;       // orbital -> k: (o / nbnd) mod nks
   FastDiv f_pervec;            // orbital -> vector: o / (nks nbnd)
 };
-
-// Output pruning of the forward column transforms: with PR > 0 every sphere of the system has
-// |m| <= PR on all three axes, so only the points p <= PR and p >= N - PR of a forward line
-// are kept; with the stores of the other points gone at compile time, the compiler drops
-// the butterflies that only feed them.  PR = 0: every point.
-template <int N, int PR>
-__device__ __forceinline__ constexpr bool line_kept(int p) {
-  return PR == 0 || p <= PR || p >= N - PR;
-}
 
 template <typename T, int N, int MODE>
 __global__ void __launch_bounds__(128, N > 36 ? 2 : (MODE == XY_PASS1_DENS ? 3 : 4)) k_xy(XYArgs a, cplx<T>* __restrict__ cbuf, const T* __restrict__ vloc,
@@ -602,6 +606,25 @@ __device__ __forceinline__ T warp_sum_t(T v) {
   return v;
 }
 
+// A sum of T values held to at least twice T's precision without the FP64 pipe (2 lanes per SM
+// and cycle): FP32 adds with the rounding error of each kept (Knuth's two-sum, seven FP32
+// operations against a conversion and an add of 16 cycles each); plain for double.
+template <typename T> struct DSum;
+template <> struct DSum<double> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <> struct DSum<float> {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float v) {
+    const float s = __fadd_rn(hi, v), b = __fadd_rn(s, -hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -b)), __fadd_rn(v, -b)));
+    hi = s;
+  }
+  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
 // Warp sums of NV values per lane at once (NV a power of two <= 32): at every step a lane keeps
 // half of its values and gives its partner the other half, so 32 values take 31 exchanges
 // instead of 5 each.  Returns the total of value number lane / (32 / NV).
@@ -624,20 +647,19 @@ __device__ __forceinline__ T warp_sums(T (&v)[NV]) {
   return t;
 }
 
-// Dot blocks of the per-k kernels: out[i*nj + j] = mult[i] sum_{g < npw} conj(A_i[g]) B_j[g] for
-// all ni x nj pairs, in tiles of 4 x NJ pairs whose sums a thread keeps in registers (4 + NJ
-// loads per 4 NJ complex products); warp sums in T by halving exchange (warp_sums), warps summed
-// in double.  `red`: kRedPairs complex doubles per warp; the tiles fill it before the block
+// Dot blocks of the per-k kernels, in tiles of 4 x NJ pairs whose sums a thread keeps in registers
+// (4 + NJ loads per 4 NJ complex products); warp sums in T by halving exchange (warp_sums), warps
+// summed with DSum.  `red`: kRedPairs complex T per warp; the tiles fill it before the block
 // synchronises.  Bound by latency and by the reductions, not by the products: at 570 plane waves
 // a thread of 256 holds 2 of them per tile, 128 FMAs beside the 31 exchanges (160 with a warp
 // reduction per value; in FP64, where an add takes 16 cycles of the SM's pipe, the reductions
-// were most of the block).  Called by the whole block; ends synchronised.
-constexpr int kRedPairs = 64;
-__host__ __device__ constexpr size_t red_doubles(int threads) { return (size_t)(threads / 32) * 2 * kRedPairs; }
+// were most of the block).
+constexpr int kRedPairs = 128;
+__host__ __device__ constexpr size_t red_elems(int threads) { return (size_t)(threads / 32) * 2 * kRedPairs; }
 
 template <typename T, int NJ>
 __device__ __forceinline__ void dots_tile(const cplx<T>* __restrict__ A, long lda, const cplx<T>* B, long ldb, int npw,
-                                          int ni, int nj, double* red) {
+                                          int ni, int nj, T* red) {
   T acc[8 * NJ];   // [i][j][re, im]
 #pragma unroll
   for (int q = 0; q < 8 * NJ; ++q) acc[q] = T(0);
@@ -661,33 +683,44 @@ __device__ __forceinline__ void dots_tile(const cplx<T>* __restrict__ A, long ld
       }
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp * 32 >= npw) return;   // a warp without plane waves
   constexpr int NV = 8 * NJ;
   const T t = warp_sums<T, NV>(acc);
-  if (lane % (32 / NV) == 0) red[(long)warp * 2 * kRedPairs + lane / (32 / NV)] = (double)t;
+  if (lane % (32 / NV) == 0) red[(long)warp * 2 * kRedPairs + lane / (32 / NV)] = t;
 }
 
+// Two dot blocks at once (n1 = 0: one): out[i*nj + j] = mult[i] sum_{g < npw} conj(A0_i[g]) B0_j[g]
+// for i < n0 (mult null: 1), then conj(A1_i) B1_j for i < n1 in the n1 rows after them; every row
+// stride ld.  Called by the whole block; ends synchronised.
 template <typename T, int NJ>
-__device__ __forceinline__ void block_dots_nj(const cplx<T>* A, long lda, const cplx<T>* B, long ldb, int npw, int ni,
-                                              int nj, const double* mult, cplx<double>* out, double* red) {
+__device__ __forceinline__ void block_dots_nj(const cplx<T>* A0, const cplx<T>* B0, int n0, const double* mult,
+                                              const cplx<T>* A1, const cplx<T>* B1, int n1, long ld, int npw, int nj,
+                                              cplx<double>* out, T* red) {
   constexpr int TP = 4 * NJ, TB = kRedPairs / TP;   // pairs per tile, tiles per batch
-  const int tj = (nj + NJ - 1) / NJ, nt = ((ni + 3) / 4) * tj, nw = blockDim.x >> 5;
-  for (int t0 = 0; t0 < nt; t0 += TB) {
-    const int n = min(TB, nt - t0);
-    for (int t = 0; t < n; ++t) {
-      const int i0 = (t0 + t) / tj * 4, j0 = (t0 + t) % tj * NJ;
-      dots_tile<T, NJ>(A + i0 * lda, lda, B + j0 * ldb, ldb, npw, ni - i0, nj - j0, red + t * 2 * TP);
+  const int tj = (nj + NJ - 1) / NJ, t0n = ((n0 + 3) / 4) * tj, nt = t0n + ((n1 + 3) / 4) * tj;
+  const int nw = min((int)blockDim.x, npw + 31) >> 5;   // warps with plane waves
+  for (int b0 = 0; b0 < nt; b0 += TB) {
+    const int n = min(TB, nt - b0);
+    for (int q = 0; q < n; ++q) {
+      const bool first = b0 + q < t0n;
+      const int t = first ? b0 + q : b0 + q - t0n, i0 = t / tj * 4, j0 = t % tj * NJ;
+      dots_tile<T, NJ>((first ? A0 : A1) + i0 * ld, ld, (first ? B0 : B1) + j0 * ld, ld, npw, (first ? n0 : n1) - i0,
+                       nj - j0, red + q * 2 * TP);
     }
     __syncthreads();
     for (int p = threadIdx.x; p < n * TP; p += blockDim.x) {
-      const int t = t0 + p / TP, i = t / tj * 4 + (p % TP) / NJ, j = t % tj * NJ + p % NJ;
-      if (i < ni && j < nj) {
-        double re = 0.0, im = 0.0;
+      const int q = b0 + p / TP;
+      const bool first = q < t0n;
+      const int t = first ? q : q - t0n, i = t / tj * 4 + (p % TP) / NJ, j = t % tj * NJ + p % NJ;
+      if (i < (first ? n0 : n1) && j < nj) {
+        DSum<T> re, im;
+#pragma unroll 4
         for (int w = 0; w < nw; ++w) {
-          re += red[w * 2 * kRedPairs + 2 * p];
-          im += red[w * 2 * kRedPairs + 2 * p + 1];
+          re.add(red[w * 2 * kRedPairs + 2 * p]);
+          im.add(red[w * 2 * kRedPairs + 2 * p + 1]);
         }
-        const double m = mult ? mult[i] : 1.0;
-        out[i * nj + j] = mk(re * m, im * m);
+        const double a = re.value(), b = im.value();
+        out[((first ? 0 : n0) + i) * nj + j] = first && mult ? mk(a * mult[i], b * mult[i]) : mk(a, b);
       }
     }
     __syncthreads();
@@ -695,29 +728,31 @@ __device__ __forceinline__ void block_dots_nj(const cplx<T>* A, long lda, const 
 }
 
 template <typename T>
-__device__ __forceinline__ void block_dots(const cplx<T>* A, long lda, const cplx<T>* B, long ldb, int npw, int ni,
-                                           int nj, const double* mult, cplx<double>* out, double* red) {
-  if (nj == 1) block_dots_nj<T, 1>(A, lda, B, ldb, npw, ni, nj, mult, out, red);
-  else block_dots_nj<T, 4>(A, lda, B, ldb, npw, ni, nj, mult, out, red);
+__device__ __forceinline__ void block_dots2(const cplx<T>* A0, const cplx<T>* B0, int n0, const double* mult,
+                                            const cplx<T>* A1, const cplx<T>* B1, int n1, long ld, int npw, int nj,
+                                            cplx<double>* out, T* red) {
+  if (nj == 1) block_dots_nj<T, 1>(A0, B0, n0, mult, A1, B1, n1, ld, npw, nj, out, red);
+  else block_dots_nj<T, 4>(A0, B0, n0, mult, A1, B1, n1, ld, npw, nj, out, red);
+}
+template <typename T>
+__device__ __forceinline__ void block_dots(const cplx<T>* A, const cplx<T>* B, long ld, int npw, int ni, int nj,
+                                           cplx<double>* out, T* red) {
+  block_dots2<T>(A, B, ni, nullptr, A, B, 0, ld, npw, nj, out, red);
 }
 
-// The sum over the block of conj(a[g]) b[g], g < n (one pair): `red` as above, out[0].
+// The sums over the block of every thread's (re, im), lanes in T, warps with DSum, to thread 0 as
+// out[0].  `red`: two T per warp.  Called by the whole block; ends synchronised.
 template <typename T>
-__device__ __forceinline__ void block_dot1(const cplx<T>* a, const cplx<T>* b, int n, cplx<double>* out, double* red) {
-  T acc[2] = {T(0), T(0)};
-  for (int g = threadIdx.x; g < n; g += blockDim.x) {
-    const cplx<T> x = a[g], y = b[g];
-    acc[0] += x.x * y.x + x.y * y.y;
-    acc[1] += x.x * y.y - x.y * y.x;
-  }
-  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const T t = warp_sums<T, 2>(acc);
-  if (lane % 16 == 0) red[(threadIdx.x >> 5) * 2 + lane / 16] = (double)t;
+__device__ __forceinline__ void block_sum2(T re, T im, cplx<double>* out, T* red) {
+  T v[2] = {re, im};
+  const int lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
+  const T t = warp_sums<T, 2>(v);
+  if (lane % 16 == 0) red[(threadIdx.x >> 5) * 2 + lane / 16] = t;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double re = 0.0, im = 0.0;
-    for (int w = 0; w < nw; ++w) re += red[2 * w], im += red[2 * w + 1];
-    out[0] = mk(re, im);
+    DSum<T> a, b;
+    for (int w = 0; w < nw; ++w) a.add(red[2 * w]), b.add(red[2 * w + 1]);
+    out[0] = mk(a.value(), b.value());
   }
   __syncthreads();
 }
@@ -749,7 +784,7 @@ __device__ __forceinline__ void rows_times(cplx<T> (&acc)[4], const cplx<T>* __r
 // double run on the slow FP64 pipe.
 // nv <= NB nbnd: NB blocks of bands (v_hat and w_hat of the non-Hermitian update: 2).
 template <typename T, int NB = 1>
-__device__ __forceinline__ void subtract_projection(cplx<T>* x, const cplx<T>* uk, const cplx<double>* S, int nbnd,
+__device__ __forceinline__ void subtract_projection(cplx<T>* x, const cplx<T>* __restrict__ uk, const cplx<double>* S, int nbnd,
                                                     int nv, int npw_pad) {
   __shared__ cplx<T> St[NB * 32 * 32];
   for (int i = threadIdx.x; i < nbnd * nv; i += blockDim.x) St[i] = mk((T)S[i].x, (T)S[i].y);
@@ -806,19 +841,6 @@ __device__ __forceinline__ double block_sum(double v) {
   return t;
 }
 
-// The same with the lanes summed in T, the warps in double.
-template <typename T>
-__device__ __forceinline__ double block_sum_t(T v) {
-  __shared__ double wsum[32];
-  v = warp_sum_t(v);
-  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = (double)v;
-  __syncthreads();
-  double t = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += wsum[w];
-  __syncthreads();
-  return t;
-}
-
 // x <- P_c x for every orbital of k (in place); with coef ([nks][nbnd][nbnd], m-major), the
 // component along u_m of band v is removed with weight coef[k][m][v] instead of 1.  The bands
 // of k are independent: grid (nks, nvec, nsplit) with nsplit dividing nbnd, each CTA taking
@@ -828,12 +850,12 @@ __global__ void __launch_bounds__(128) k_project(int nks, int nbnd, int npw_pad,
                                                  const cplx<T>* __restrict__ ukq, cplx<T>* __restrict__ x,
                                                  const double* __restrict__ coef) {
   __shared__ cplx<double> cf[32 * 32];
-  __shared__ double red[red_doubles(128)];
+  __shared__ T red[red_elems(128)];
   const int k = blockIdx.x, vec = blockIdx.y;
   const int nv = nbnd / gridDim.z, v0 = blockIdx.z * nv;
   const long base = (((long)vec * nks + k) * nbnd + v0) * npw_pad;
   const cplx<T>* uk = ukq + (long)k * nbnd * npw_pad;
-  block_dots<T>(uk, npw_pad, x + base, npw_pad, npw[k], nbnd, nv, nullptr, cf, red);
+  block_dots<T>(uk, x + base, npw_pad, npw[k], nbnd, nv, cf, red);
   if (coef) {
     for (int i = threadIdx.x; i < nbnd * nv; i += blockDim.x) {
       const int m = i / nv;
@@ -853,11 +875,11 @@ __global__ void __launch_bounds__(256) k_metal_image(int nks, int nbnd, int npw_
                                                      cplx<T>* __restrict__ img, cplx<double>* __restrict__ zp,
                                                      MetalDev md) {
   __shared__ cplx<double> cf[32 * 32];
-  __shared__ double red[red_doubles(256)];
+  __shared__ T red[red_elems(256)];
   const int k = blockIdx.x, vec = blockIdx.y;
   const long base = ((long)vec * nks + k) * nbnd * npw_pad;
   const cplx<T>* uk = ukq + (long)k * nbnd * npw_pad;
-  block_dots<T>(uk, npw_pad, z + base, npw_pad, npw[k], nbnd, nbnd, nullptr, cf, red);
+  block_dots<T>(uk, z + base, npw_pad, npw[k], nbnd, nbnd, cf, red);
   for (int i = threadIdx.x; i < nbnd * nbnd; i += blockDim.x) {
     const long ci = (long)k * nbnd * nbnd + i;
     const cplx<double> v = cf[i];
@@ -932,9 +954,9 @@ static __global__ void __launch_bounds__(256) k_ph_beta(int* __restrict__ jdev, 
 // the group's z_j partial, r_{j+1} = P_c(X_j/beta_j - beta_j v_{j-1}) formed in shared memory and
 // written to R (a metal: keep = MetalDev::keep, the projection P'_v), v_j = r_j/beta_j.  The
 // sphere columns of r_{j+1} are then inverse-FFT'd along axis 3 by k_zinv.  grid (nks, ngrp),
-// block 256.  smem: r [bpc][npw_pad], S [nbnd*bpc] (double complex), reduction scratch.
+// block proj_threads.  smem: r [bpc][npw_pad], S [nbnd*bpc] (double complex), reduction scratch.
 template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_ph_update(const int* __restrict__ jdev, SphereDev s, int nbnd, int bpc,
+__global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_ph_update(const int* __restrict__ jdev, SphereDev s, int nbnd, int bpc,
                                                    const double* __restrict__ scal, cplx<T>* __restrict__ R,
                                                    const cplx<T>* __restrict__ X, cplx<T>* __restrict__ Vp,
                                                    const cplx<T>* __restrict__ y, const cplx<T>* __restrict__ ukq,
@@ -945,25 +967,28 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_ph_update(const
   const int k = blockIdx.x, grp = blockIdx.y, ngrp = gridDim.y;
   cplx<T>* rs = reinterpret_cast<cplx<T>*>(smem_raw);
   cplx<double>* cf = reinterpret_cast<cplx<double>*>(rs + bpc * npw_pad);
-  double* red = reinterpret_cast<double*>(cf + nbnd * bpc);
+  T* red = reinterpret_cast<T*>(cf + nbnd * bpc);
   const long base = ((long)k * nbnd + grp * bpc) * npw_pad;
   const int np = s.npw[k];
   const long zi = (long)(j - 1) * nks * ngrp + (long)k * ngrp + grp;
-  if (r_upper) {  // z_j partial = (y, r_j)/beta_j over the group's bands
-    block_dot1<T>(y + base, R + base, bpc * npw_pad, cf, red);
-    if (threadIdx.x == 0) co.zpart[zi] = mk(cf[0].x * scal[1], cf[0].y * scal[1]);
-  } else if (threadIdx.x == 0) {
-    co.zpart[zi] = mk(0.0, 0.0);
-  }
   const T ib = (T)scal[1], bb = (T)scal[0];
+  T zr = T(0), zim = T(0);   // z_j partial = (y, r_j)/beta_j over the group's bands (r_j upper)
+#pragma unroll 4
   for (int i = threadIdx.x; i < bpc * npw_pad; i += blockDim.x) {
-    const cplx<T> r = R[base + i];
-    rs[i] = X[base + i] * ib - Vp[base + i] * bb;
+    const cplx<T> r = R[base + i], x = X[base + i], v = Vp[base + i];
+    if (r_upper) {
+      const cplx<T> yv = y[base + i];
+      zr += yv.x * r.x + yv.y * r.y;
+      zim += yv.x * r.y - yv.y * r.x;
+    }
+    rs[i] = x * ib - v * bb;
     Vp[base + i] = r * ib;
   }
-  __syncthreads();
+  if (r_upper) block_sum2<T>(zr, zim, cf, red);
+  else __syncthreads();
+  if (threadIdx.x == 0) co.zpart[zi] = r_upper ? mk(cf[0].x * scal[1], cf[0].y * scal[1]) : mk(0.0, 0.0);
   const cplx<T>* uk = ukq + (long)k * nbnd * npw_pad;
-  block_dots<T>(uk, npw_pad, rs, npw_pad, np, nbnd, bpc, nullptr, cf, red);
+  block_dots<T>(uk, rs, npw_pad, np, nbnd, bpc, cf, red);
   if (keep) {  // a metal: only the states with c_mv = 0 are removed
     for (int i = threadIdx.x; i < nbnd * bpc; i += blockDim.x) {
       const int m = i / bpc;
@@ -996,75 +1021,82 @@ static __device__ __noinline__ double metal_operator_coefs(const MetalDev md, in
   return block_sum(corr);
 }
 
-// Last stage of the operator fused with the per-k projections, for one group of bpc bands of
-// one k-point (the kinetic, KB and P_c terms act band by band): forward FFT of the group's
-// columns along axis 3 and gather of the sphere (1/W^3), + (1/2|k+Q+G|^2 - eps_vk) x, + KB
-// sum_p beta_p D_p <beta_p|x>, then P_c, the output X and the group's partial Re(x^H X)
-// (a metal: x is the image Q z, zp holds Z = U^H z per vector; the output is the operator
-// on z through the MetalDev tables, and the partial Re(z^H X)).
+// Columns -> sphere: forward FFT of the columns along axis 3, gather (1/N^3) and the kinetic term,
+// t = (1/2|k+Q+G|^2 - eps_vk) x + gathered, written to xout.  One thread per column line;
+// grid (nks, nvec, lines), block kLines.  PR as for k_zinv.
+constexpr int kLines = 128;
+template <typename T, int N, int PR = 0>
+__global__ void __launch_bounds__(kLines) k_zfwd(SphereDev s, int nbnd, const cplx<T>* __restrict__ cbuf, int cb_ncol,
+                                                 const cplx<T>* __restrict__ xin, const T* __restrict__ kin,
+                                                 const double* __restrict__ eps, cplx<T>* __restrict__ xout) {
+  const int k = blockIdx.x, vec = blockIdx.y, nks = s.nks, npw_pad = s.npw_pad;
+  const int nc = s.ncol[k];
+  const int it = blockIdx.z * kLines + threadIdx.x;
+  if (it >= nbnd * nc) return;
+  const int v = it / nc, c = it - v * nc;
+  const long o = ((long)vec * nks + k) * nbnd + v;
+  const int4 cl = s.col[k * s.ncol_max + c];
+  if (!LL_INB(c < cb_ncol)) return;
+  const cplx<T>* src = cbuf + o * (long)N * cb_ncol + c;
+  cplx<T> a[N];
+#pragma unroll
+  for (int p = 0; p < N; ++p) a[p] = src[(long)p * cb_ncol];
+  const T ev = (T)eps[k * nbnd + v];
+  const int st = s.colstart[k * s.ncol_max + c];
+  const cplx<T>* x = xin + o * npw_pad + st;
+  const T* kn = kin + (long)k * npw_pad + st;
+  cplx<T>* t = xout + o * npw_pad + st;
+  fft_line<T, N, -1>(a);
+  const T scale = T(1) / T(N * N * N);
+#pragma unroll
+  for (int p = 0; p < N; ++p)
+    if (line_kept<N, PR>(p)) {
+      const int i = PR > 0 ? (p <= PR ? p : p - N) - cl.z : wrapn<N>(p - cl.z);
+      if ((unsigned)i < (unsigned)cl.w && LL_INB(st >= 0 && st + i < npw_pad)) t[i] = x[i] * (kn[i] - ev) + a[p] * scale;
+    }
+}
+
+// Threads of the per-k projection kernels: 512 where a band has more plane waves than two rounds
+// of 256 hold three times over (their loops then have few, long rounds of loads in flight: the
+// eight-atom cell has 1.7 CTAs per SM), else 256 (four CTAs per SM: the KB workload's 512
+// k-points are one wave).
+static inline int proj_threads(int npw_pad) { return npw_pad > 768 ? 512 : 256; }
+
+// Last stage of the operator, for one group of bpc bands of one k-point (the KB and P_c terms act
+// band by band): from t (k_zfwd's output, in xout), + KB sum_p beta_p D_p <beta_p|x>, then P_c,
+// the output X (in place) and the group's partial Re(x^H X) (a metal: x is the image Q z, zp
+// holds Z = U^H z per vector; the output is the operator on z through the MetalDev tables, and the
+// partial Re(z^H X)).
 // P_c of the KB term goes through the overlaps ub = U^H B of the set-up, S = U^H t + ub c, so
 // both dot blocks are formed on the same data and KB, P_c, the output and the norm partial
 // are one pass over the plane waves, four bands of a plane wave per thread (rows_times).
-// grid (nks, nvec, ngrp), block 256.  smem: x, t [bpc][npw_pad]; coefficients; scratch.
-// Measured (GB300, FP32, us per launch, before -> after the shared dot blocks and the one pass):
-// eight-atom cell (16 bands, 1632 plane waves, 64 k) 313 -> 124, KB workload (4 bands, 570, 512 k)
-// 77 -> 61.
-template <typename T, int N, int PR = 0>
-__global__ void __launch_bounds__(256, 2) k_zfwd_proj(SphereDev s, int nbnd, int bpc, const cplx<T>* __restrict__ cbuf,
-                                                   int cb_ncol, const cplx<T>* __restrict__ xin,
-                                                   const T* __restrict__ kin, const double* __restrict__ eps,
-                                                   const cplx<T>* __restrict__ ukq, const cplx<T>* __restrict__ bkq,
-                                                   const double* __restrict__ dij,
+// grid (nks, nvec, ngrp), block proj_threads.  smem: coefficients, scratch.
+// A kernel of its own: with the column transforms in front it needed 123 registers, two CTAs per
+// SM and 1.7 waves on the KB workload's 512 k-points, and shared memory for x and t.  Measured
+// (GB300, FP32, us per launch; the one kernel -> k_zfwd + this one): eight-atom cell (16 bands,
+// 1632 plane waves) 128 -> 27 + 79, KB workload (4 bands, 570) 61 -> 18 + 41, two-atom 10 Ry cell
+// (147) 15 -> 6 + 11.
+template <typename T>
+__global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_op_proj(SphereDev s, int nbnd, int bpc,
+                                                   const cplx<T>* __restrict__ xin, const cplx<T>* __restrict__ ukq,
+                                                   const cplx<T>* __restrict__ bkq, const double* __restrict__ dij,
                                                    const cplx<double>* __restrict__ ub, int nproj,
-                                                   cplx<T>* __restrict__ xout, double* __restrict__ part,
-                                                   MetalDev md, const cplx<double>* __restrict__ zp) {
+                                                   cplx<T>* xout, double* __restrict__ part, MetalDev md,
+                                                   const cplx<double>* __restrict__ zp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int npw_pad = s.npw_pad, nks = s.nks;
   const int k = blockIdx.x, vec = blockIdx.y, grp = blockIdx.z, ngrp = gridDim.z;
   const int v0 = grp * bpc;
-  cplx<T>* xs = reinterpret_cast<cplx<T>*>(smem_raw);
-  cplx<T>* ts = xs + bpc * npw_pad;
-  cplx<double>* cf = reinterpret_cast<cplx<double>*>(ts + bpc * npw_pad);   // [nproj + nbnd][bpc]: c, then S
-  double* red = reinterpret_cast<double*>(cf + (nproj + nbnd) * bpc);
-  cplx<T>* ct = reinterpret_cast<cplx<T>*>(red + red_doubles(256));         // the coefficients in T
-  __shared__ T epsk[32];
-  const long o0 = ((long)vec * nks + k) * nbnd + v0;      // first orbital of the group
-  const long base = o0 * npw_pad;
+  cplx<double>* cf = reinterpret_cast<cplx<double>*>(smem_raw);   // [nproj + nbnd][bpc]: c, then S
+  cplx<T>* ct = reinterpret_cast<cplx<T>*>(cf + (nproj + nbnd) * bpc);      // the coefficients in T
+  T* red = reinterpret_cast<T*>(ct + (nproj + nbnd) * bpc);
+  const long base = (((long)vec * nks + k) * nbnd + v0) * npw_pad;          // first orbital of the group
   const int np = s.npw[k];
   const cplx<T>* bk = bkq + (long)k * nproj * npw_pad;
   const cplx<T>* uk = ukq + (long)k * nbnd * npw_pad;
-  if (threadIdx.x < bpc) epsk[threadIdx.x] = (T)eps[k * nbnd + v0 + threadIdx.x];
-  __syncthreads();
-  for (int i = threadIdx.x; i < bpc * npw_pad; i += blockDim.x) {
-    const int v = i / npw_pad, gi = i - v * npw_pad;
-    const cplx<T> xv = xin[base + i];
-    xs[i] = xv;
-    ts[i] = xv * (kin[(long)k * npw_pad + gi] - epsk[v]);
-  }
-  __syncthreads();
-  const int nc = s.ncol[k];
-  const T scale = T(1) / T(N * N * N);
-  for (int it = threadIdx.x; it < bpc * nc; it += blockDim.x) {
-    const int v = it / nc, c = it - v * nc;
-    const int4 cl = s.col[k * s.ncol_max + c];
-    if (!LL_INB(c < cb_ncol)) continue;
-    const cplx<T>* src = cbuf + (o0 + v) * (long)N * cb_ncol + c;
-    cplx<T> a[N];
-#pragma unroll
-    for (int p = 0; p < N; ++p) a[p] = src[(long)p * cb_ncol];
-    fft_line<T, N, -1>(a);
-    const int st = s.colstart[k * s.ncol_max + c];
-    cplx<T>* dst = ts + v * npw_pad + st;
-#pragma unroll
-    for (int p = 0; p < N; ++p) {
-      const int i = wrapn<N>(p - cl.z);
-      if (line_kept<N, PR>(p) && i < cl.w && LL_INB(st >= 0 && st + i < npw_pad)) dst[i] = dst[i] + a[p] * scale;
-    }
-  }
-  __syncthreads();
+  cplx<T>* ts = xout + base;   // a thread meets the same plane waves of t in both passes (L1)
   cplx<double>* sf = cf + nproj * bpc;
-  if (nproj > 0) block_dots<T>(bk, npw_pad, xs, npw_pad, np, nproj, bpc, dij, cf, red);   // D_p <beta_p|x_v>
-  block_dots<T>(uk, npw_pad, ts, npw_pad, np, nbnd, bpc, nullptr, sf, red);
+  block_dots2<T>(bk, xin + base, nproj, dij, uk, ts, nbnd, npw_pad, np, bpc, cf, red);   // D_p <beta_p|x_v>, U^H t
   if (nproj > 0) {
     const cplx<double>* ubk = ub + (long)k * nbnd * nproj;
     for (int i = threadIdx.x; i < nbnd * bpc; i += blockDim.x) {   // + U^H B c
@@ -1091,22 +1123,23 @@ __global__ void __launch_bounds__(256, 2) k_zfwd_proj(SphereDev s, int nbnd, int
 #pragma unroll
     for (int v = 0; v < 4; ++v)
       if (v < n) {
-        const cplx<T> x = xs[(b0 + v) * npw_pad + gi];
+        const long o = base + (long)(b0 + v) * npw_pad + gi;
+        const cplx<T> x = xin[o];
         nr += x.x * acc[v].x + x.y * acc[v].y;
-        xout[base + (long)(b0 + v) * npw_pad + gi] = acc[v];
+        xout[o] = acc[v];
       }
   }
-  const double t = block_sum_t(nr);
-  if (threadIdx.x == 0) part[((long)vec * nks + k) * ngrp + grp] = t + corr;
+  block_sum2<T>(nr, T(0), cf, red);
+  if (threadIdx.x == 0) part[((long)vec * nks + k) * ngrp + grp] = cf[0].x + corr;
 }
 
 // Non-Hermitian step j after the two operator applications XV = L v_j, XW = L^dag w_j, for
 // one group of bpc bands of one k-point: v_hat = P_c(XV - gamma_j v_{j-1}), w_hat =
 // P_c(XW - conj(beta_j) w_{j-1}) (stored in XV, XW), the group's partials of s = (w_hat,
 // v_hat) and of z_j = (y, v_j) (a metal: keep = MetalDev::keep, the projection P'_v).
-// grid (nks, ngrp), block 256.
+// grid (nks, ngrp), block proj_threads.
 template <typename T>
-__global__ void __launch_bounds__(256) k_nh_update(int j, int upper, int nks, int nbnd, int bpc, int npw_pad,
+__global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_nh_update(int j, int upper, int nks, int nbnd, int bpc, int npw_pad,
                                                    const int* __restrict__ npw, cplx<T>* __restrict__ XV,
                                                    cplx<T>* __restrict__ XW, const cplx<T>* __restrict__ Vp,
                                                    const cplx<T>* __restrict__ Wp, const cplx<T>* __restrict__ Vc,
@@ -1117,7 +1150,7 @@ __global__ void __launch_bounds__(256) k_nh_update(int j, int upper, int nks, in
   cplx<T>* vs = reinterpret_cast<cplx<T>*>(smem_raw);          // [bpc][npw_pad]
   cplx<T>* ws = vs + bpc * npw_pad;
   cplx<double>* cf = reinterpret_cast<cplx<double>*>(ws + bpc * npw_pad);   // [nbnd * 2 bpc]
-  double* red = reinterpret_cast<double*>(cf + nbnd * 2 * bpc);
+  T* red = reinterpret_cast<T*>(cf + nbnd * 2 * bpc);
   const int k = blockIdx.x, grp = blockIdx.y, ngrp = gridDim.y;
   const long base = ((long)k * nbnd + grp * bpc) * npw_pad;
   const long zi = (long)(j - 1) * nks * ngrp + (long)k * ngrp + grp;
@@ -1125,20 +1158,23 @@ __global__ void __launch_bounds__(256) k_nh_update(int j, int upper, int nks, in
   const double bj = co.beta[j - 1];
   const cplx<double> gj = co.gamma[j - 1];
   const cplx<T> g = mk((T)gj.x, (T)gj.y), bc = mk((T)bj, (T)0);
-  if (upper) {  // z_j partial = (y, v_j) over the group's bands
-    block_dot1<T>(y + base, Vc + base, bpc * npw_pad, cf, red);
-    if (threadIdx.x == 0) co.zpart[zi] = cf[0];
-  } else if (threadIdx.x == 0) {
-    co.zpart[zi] = mk(0.0, 0.0);
-  }
+  T zr = T(0), zim = T(0);   // z_j partial = (y, v_j) over the group's bands
+#pragma unroll 2
   for (int i = threadIdx.x; i < bpc * npw_pad; i += blockDim.x) {
+    if (upper) {
+      const cplx<T> yv = y[base + i], v = Vc[base + i];
+      zr += yv.x * v.x + yv.y * v.y;
+      zim += yv.x * v.y - yv.y * v.x;
+    }
     vs[i] = XV[base + i] - cmul(g, Vp[base + i]);
     ws[i] = XW[base + i] - cmul(bc, Wp[base + i]);
   }
-  __syncthreads();
+  if (upper) block_sum2<T>(zr, zim, cf, red);
+  else __syncthreads();
+  if (threadIdx.x == 0) co.zpart[zi] = upper ? cf[0] : mk(0.0, 0.0);
   const cplx<T>* uk = ukq + (long)k * nbnd * npw_pad;
   // v_hat and w_hat are 2 bpc consecutive rows: one dot block and one pass of P_c for both
-  block_dots<T>(uk, npw_pad, vs, npw_pad, np, nbnd, 2 * bpc, nullptr, cf, red);
+  block_dots<T>(uk, vs, npw_pad, np, nbnd, 2 * bpc, cf, red);
   if (keep) {  // a metal: P'_v, only the states with c_mv = 0 removed
     for (int i = threadIdx.x; i < nbnd * 2 * bpc; i += blockDim.x) {
       const int m = i / (2 * bpc), v = (i - m * 2 * bpc) % bpc;
@@ -1148,11 +1184,15 @@ __global__ void __launch_bounds__(256) k_nh_update(int j, int upper, int nks, in
     __syncthreads();
   }
   subtract_projection<T, 2>(vs, uk, cf, nbnd, 2 * bpc, npw_pad);
+  T sr = T(0), si = T(0);
   for (int i = threadIdx.x; i < bpc * npw_pad; i += blockDim.x) {
-    XV[base + i] = vs[i];
-    XW[base + i] = ws[i];
+    const cplx<T> v = vs[i], w = ws[i];
+    XV[base + i] = v;
+    XW[base + i] = w;
+    sr += w.x * v.x + w.y * v.y;
+    si += w.x * v.y - w.y * v.x;
   }
-  block_dot1<T>(ws, vs, bpc * npw_pad, cf, red);
+  block_sum2<T>(sr, si, cf, red);
   if (threadIdx.x == 0) spart[(long)k * ngrp + grp] = cf[0];
 }
 

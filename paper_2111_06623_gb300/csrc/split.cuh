@@ -1,6 +1,6 @@
 // Per-k work of the pseudo-Hermitian step split over several CTAs per k-point (sm_103a).
 //
-// The fused per-k kernels (k_ph_update, k_zfwd_proj) hold a whole k block of two vectors,
+// The fused per-k kernels (k_ph_update, k_op_proj) hold a whole k block of two vectors,
 // 2 nbnd npw complex values, in one CTA's shared memory.  Systems whose k blocks do not fit
 // (the eight-atom cell: 16 bands x 1632 plane waves, 420 KB in FP32) take this path: every
 // k block is cut into chunks of kChunk plane waves (for the projections) or of kLines column
@@ -11,7 +11,7 @@
 // One pseudo-Hermitian step here: k_sp_start (beta_j, z_j partial, r_{j+1} before P_c,
 // partial U^H r) -> k_sp_coef, k_sp_apply (P_c) -> k_zinv (axis-3 inverse FFT over several
 // CTAs per k) -> planes and response
-// potential as in the fused path -> k_sp_zfwd (axis-3 forward FFT, gather, kinetic - eps)
+// potential as in the fused path -> k_zfwd (axis-3 forward FFT, gather, kinetic - eps)
 // -> k_sp_dots (partial B^H x, U^H t) -> k_sp_coef (coefficients) -> k_sp_apply (KB, P_c,
 // output, norm partial).
 #pragma once
@@ -20,7 +20,6 @@
 namespace ll {
 
 constexpr int kChunk = 512;    // plane waves per projection chunk
-constexpr int kLines = 256;    // column lines per axis-3 CTA
 constexpr int kTile = 32;      // plane waves per shared-memory tile of the dot blocks
 constexpr int kTileP = kTile + 1;  // padded row of a tile (conflict-free column reads)
 constexpr int kMaxPairs = 2048;  // ni * nj of one dot block (nproj <= 64, nbnd <= 32)
@@ -125,39 +124,6 @@ __global__ void __launch_bounds__(256) k_sp_start(const int* __restrict__ jdev, 
   __syncthreads();
   chunk_dots<T>(ukq + base, npw_pad, R + base, npw_pad, g0, max(g0, min(g1, npw[k])), nbnd, nbnd, tile,
                 spart + ((long)k * nchunk + c) * nbnd * nbnd);
-}
-
-// Operator, last stage, first part: forward FFT of the columns along axis 3, gather of the
-// sphere (1/N^3) plus (1/2|k+Q+G|^2 - eps_vk) x into t = out.  grid (nks, nvec, lines).
-template <typename T, int N>
-__global__ void __launch_bounds__(kLines) k_sp_zfwd(SphereDev s, int nbnd, const cplx<T>* __restrict__ cbuf,
-                                                    int cb_ncol, const cplx<T>* __restrict__ xin,
-                                                    const T* __restrict__ kin, const double* __restrict__ eps,
-                                                    cplx<T>* __restrict__ xout) {
-  const int k = blockIdx.x, vec = blockIdx.y, nks = s.nks, npw_pad = s.npw_pad;
-  const int nc = s.ncol[k];
-  const int it = blockIdx.z * kLines + threadIdx.x;
-  if (it >= nbnd * nc) return;
-  const int v = it / nc, c = it - v * nc;
-  const long o = ((long)vec * nks + k) * nbnd + v;
-  const int4 cl = s.col[k * s.ncol_max + c];
-  if (!LL_INB(c < cb_ncol)) return;
-  const cplx<T>* src = cbuf + o * (long)N * cb_ncol + c;
-  cplx<T> a[N];
-#pragma unroll
-  for (int p = 0; p < N; ++p) a[p] = src[(long)p * cb_ncol];
-  fft_line<T, N, -1>(a);
-  const T scale = T(1) / T(N * N * N);
-  const T ev = (T)eps[k * nbnd + v];
-  const int st = s.colstart[k * s.ncol_max + c];
-  const cplx<T>* x = xin + o * npw_pad + st;
-  const T* kn = kin + (long)k * npw_pad + st;
-  cplx<T>* t = xout + o * npw_pad + st;
-#pragma unroll
-  for (int p = 0; p < N; ++p) {
-    const int i = wrapn<N>(p - cl.z);
-    if (i < cl.w && LL_INB(st >= 0 && st + i < npw_pad)) t[i] = x[i] * (kn[i] - ev) + a[p] * scale;
-  }
 }
 
 // Partial dot blocks of one chunk: C = B^H x (nproj x nbnd, when nproj > 0) and
