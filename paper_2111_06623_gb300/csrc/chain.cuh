@@ -674,7 +674,7 @@ class Chain : public ChainBase {
     if (metal_) {
       const long sz = (long)nks_ * nbnd_ * nbnd_;
       if ((rc = alloc(&mc_, 4 * sz)) || (rc = alloc(&img_, nvec_ * vq)) || (rc = alloc(&zp_, nvec_ * sz)) ||
-          (rc = alloc(&mcorr_, (long)nvec_ * nks_)))
+          (rc = alloc(&mcorr_, (long)nvec_ * nks_ * kCoefSlices)))
         return rc;
       LL_CK(cudaMemcpyAsync(mc_, mtab_.data(), 4 * sz * sizeof(double), cudaMemcpyHostToDevice, st_));
       md_ = MetalDev{mc_, mc_ + sz, mc_ + 2 * sz, mc_ + 3 * sz};
@@ -1137,7 +1137,7 @@ class Chain : public ChainBase {
       if (set_smem(k_sp_dots<T>, sm_d, e) || set_smem(k_sp_apply<T>, sm_a, e)) return nullptr;
       k_sp_dots<T><<<dim3(nks_, nvec, nchunk_), 256, sm_d, st_>>>(nks_, nbnd_, pq, dq_.npw, nchunk_, 0, in, in, ukq_,
                                                                   bkq_, sp_c_, sp_s_);
-      k_sp_coef<T><<<nks_ * nvec, 256, 0, st_>>>(nks_, nbnd_, nchunk_, 0, dij_, ub_, sp_c_, sp_s_, sp_coef_, 3, md_,
+      k_sp_coef<T><<<dim3(nks_ * nvec, kCoefSlices), 256, 0, st_>>>(nks_, nbnd_, nchunk_, 0, dij_, ub_, sp_c_, sp_s_, sp_coef_, 3, md_,
                                                  zp_, nullptr);
       k_sp_apply<T><<<dim3(nks_, nvec, nchunk_), 256, sm_a, st_>>>(nks_, nbnd_, pq, dq_.npw, nchunk_, 0, nullptr,
                                                                    img_, ukq_, bkq_, sp_coef_, nullptr);
@@ -1255,7 +1255,7 @@ class Chain : public ChainBase {
       const size_t sm = tc_apply_smem(a.nb, a.nks_k);
       int rc;
       if ((rc = set_smem(k_tc_apply, sm, err))) return rc;
-      k_tc_apply<<<dim3(nks_, nvec, nchunk_), kTcThreads, sm, st_>>>(a);
+      k_tc_apply<<<dim3(nks_, nvec, nchunk_), kTaThreads, sm, st_>>>(a);
       LL_CK(cudaGetLastError());
       return LL_OK;
     } else {
@@ -1270,7 +1270,7 @@ class Chain : public ChainBase {
     const size_t sm_d = (size_t)(std::max(nproj_, nbnd_) + nbnd_) * kTileP * sizeof(cplx<T>);
     const size_t sm_a = (size_t)(nproj_ + nbnd_) * (nbnd_ + kSub) * sizeof(cplx<T>);
     int rc;
-    const size_t sm_c = (size_t)nproj_ * nbnd_ * sizeof(cplx<double>);
+    const size_t sm_c = (size_t)nproj_ * coef_slice(nbnd_) * sizeof(cplx<double>);
     if ((rc = set_smem(k_sp_dots<T>, sm_d, err)) || (rc = set_smem(k_sp_coef<T>, sm_c, err)) ||
         (rc = set_smem(k_sp_apply<T>, sm_a, err)))
       return rc;
@@ -1280,7 +1280,7 @@ class Chain : public ChainBase {
       k_sp_dots<T><<<dim3(nks_, nvec, nchunk_), 256, sm_d, st_>>>(nks_, nbnd_, pq, dq_.npw, nchunk_, nproj_, in, out,
                                                                   ukq_, bkq_, sp_c_, sp_s_);
     }
-    k_sp_coef<T><<<nks_ * nvec, 256, sm_c, st_>>>(nks_, nbnd_, nchunk_, nproj_, dij_, ub_, sp_c_, sp_s_, sp_coef_,
+    k_sp_coef<T><<<dim3(nks_ * nvec, kCoefSlices), 256, sm_c, st_>>>(nks_, nbnd_, nchunk_, nproj_, dij_, ub_, sp_c_, sp_s_, sp_coef_,
                                                   metal_ ? 1 : 0, md_, zp_, mcorr_);
     if (tc_ap_) {
       if ((rc = tc_apply(nvec, nproj_, in, out, part_, err))) return rc;
@@ -1306,7 +1306,7 @@ class Chain : public ChainBase {
     // then the axis-3 inverse FFTs over many CTAs per k
     const size_t sm_a = (size_t)nbnd_ * (nbnd_ + kSub) * sizeof(cplx<T>);
     if ((rc = set_smem(k_sp_apply<T>, sm_a, err))) return rc;
-    k_sp_coef<T><<<nks_, 256, 0, st_>>>(nks_, nbnd_, nchunk_, 0, dij_, ub_, sp_c_, sp_s_, sp_coef_, metal_ ? 2 : 0,
+    k_sp_coef<T><<<dim3(nks_, kCoefSlices), 256, 0, st_>>>(nks_, nbnd_, nchunk_, 0, dij_, ub_, sp_c_, sp_s_, sp_coef_, metal_ ? 2 : 0,
                                         md_);
     if (tc_ap_) {
       if ((rc = tc_apply(1, 0, nullptr, R(), nullptr, err))) return rc;

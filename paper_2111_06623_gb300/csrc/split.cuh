@@ -90,35 +90,34 @@ __global__ void __launch_bounds__(256) k_sp_start(const int* __restrict__ jdev, 
   const int k = blockIdx.x, c = blockIdx.y;
   const int g0 = c * kChunk, g1 = min(npw_pad, g0 + kChunk);
   const long base = (long)k * nbnd * npw_pad;
-  const int zi = (j - 1) * nks * nchunk + k * nchunk + c;
-  if (r_upper) {  // z_j partial = (y, r_j)/beta_j over the chunk
-    double zr = 0.0, zim = 0.0;
-    for (int e = threadIdx.x; e < nbnd * (g1 - g0); e += blockDim.x) {
-      const int v = e / (g1 - g0), g = g0 + e - v * (g1 - g0);
-      const cplx<T> a = y[base + (long)v * npw_pad + g], r = R[base + (long)v * npw_pad + g];
-      zr += (double)(a.x * r.x + a.y * r.y);
-      zim += (double)(a.x * r.y - a.y * r.x);
+  const long zi = (long)(j - 1) * nks * nchunk + k * nchunk + c;
+  const T ib = (T)scal[1], bb = (T)scal[0];
+  const int n = g1 - g0;
+  DSum<T> zr, zim;   // z_j partial = (y, r_j)/beta_j over the chunk (r_j upper)
+#pragma unroll 4
+  for (int e = threadIdx.x; e < nbnd * n; e += blockDim.x) {
+    const int v = e / n, g = g0 + e - v * n;
+    const long i = base + (long)v * npw_pad + g;
+    const cplx<T> r = R[i], x = X[i], w = Vp[i];
+    if (r_upper) {
+      const cplx<T> a = y[i];
+      zr.add(a.x * r.x + a.y * r.y);
+      zim.add(a.x * r.y - a.y * r.x);
     }
-    zr = warp_sum(zr);
-    zim = warp_sum(zim);
-    if ((threadIdx.x & 31) == 0) { zred[0][threadIdx.x >> 5] = zr; zred[1][threadIdx.x >> 5] = zim; }
+    R[i] = x * ib - w * bb;
+    Vp[i] = r * ib;
+  }
+  if (r_upper) {
+    const double sr = warp_sum(zr.value()), si = warp_sum(zim.value());
+    if ((threadIdx.x & 31) == 0) { zred[0][threadIdx.x >> 5] = sr; zred[1][threadIdx.x >> 5] = si; }
     __syncthreads();
     if (threadIdx.x == 0) {
-      double sr = 0.0, si = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { sr += zred[0][w]; si += zred[1][w]; }
-      co.zpart[zi] = mk(sr * scal[1], si * scal[1]);
+      double tr = 0.0, ti = 0.0;
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { tr += zred[0][w]; ti += zred[1][w]; }
+      co.zpart[zi] = mk(tr * scal[1], ti * scal[1]);
     }
   } else if (threadIdx.x == 0) {
     co.zpart[zi] = mk(0.0, 0.0);
-  }
-  __syncthreads();
-  const T ib = (T)scal[1], bb = (T)scal[0];
-  for (int e = threadIdx.x; e < nbnd * (g1 - g0); e += blockDim.x) {
-    const int v = e / (g1 - g0), g = g0 + e - v * (g1 - g0);
-    const long i = base + (long)v * npw_pad + g;
-    const cplx<T> r = R[i];
-    R[i] = X[i] * ib - Vp[i] * bb;
-    Vp[i] = r * ib;
   }
   if (!dots) return;   // the partial U^H r_{j+1} comes from the tensor-core kernel
   __syncthreads();
@@ -154,7 +153,11 @@ __global__ void __launch_bounds__(256) k_sp_dots(int nks, int nbnd, int npw_pad,
 // Z with Z = zp[kv] from the image, and mcorr[kv] = sum qh Re(conj(Z) (S - C)), the term that
 // makes the norm partial of the image Re(z, X); kind 2 (the update) keep S; kind 3 (the image
 // Q z, S = U^H z) qh S, with zp[kv] = S on the kept states.  kind 0: S itself.
-// grid nks * nvec, block 256.
+// The bands are split over kCoefSlices CTAs per (vector, k) (one took 80 us on the sixteen-atom
+// cell: U^H B c is 524k FP64 FMAs per k on one SM's two FP64 lanes).
+// grid (nks * nvec, kCoefSlices), block 256.
+constexpr int kCoefSlices = 4;
+static inline __host__ __device__ int coef_slice(int nbnd) { return (nbnd + kCoefSlices - 1) / kCoefSlices; }
 template <typename T>
 __global__ void __launch_bounds__(256) k_sp_coef(int nks, int nbnd, int nchunk, int nproj,
                                                  const double* __restrict__ dij, const cplx<double>* __restrict__ ub,
@@ -164,31 +167,36 @@ __global__ void __launch_bounds__(256) k_sp_coef(int nks, int nbnd, int nchunk, 
                                                  cplx<double>* __restrict__ zp = nullptr,
                                                  double* __restrict__ mcorr = nullptr) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cplx<double>* cd = reinterpret_cast<cplx<double>*>(smem_raw);   // [nproj * nbnd]
   const long kv = blockIdx.x;
-  const int k = (int)(kv % nks);
+  const int k = (int)(kv % nks), vs = coef_slice(nbnd), v0 = blockIdx.y * vs, nv = min(vs, nbnd - v0);
+  cplx<double>* cd = reinterpret_cast<cplx<double>*>(smem_raw);   // [nproj][nv]
   cplx<T>* out = coef + kv * (long)(nproj + nbnd) * nbnd;
-  for (int p = threadIdx.x; p < nproj * nbnd; p += blockDim.x) {
+  for (int i = threadIdx.x; i < nproj * nv; i += blockDim.x) {
+    const int q = i / nv, p = q * nbnd + v0 + i - q * nv;
     double re = 0.0, im = 0.0;
+#pragma unroll 4
     for (int cc = 0; cc < nchunk; ++cc) {
-      re += cpart[(kv * nchunk + cc) * nproj * nbnd + p].x;
-      im += cpart[(kv * nchunk + cc) * nproj * nbnd + p].y;
+      const cplx<double> a = cpart[(kv * nchunk + cc) * nproj * nbnd + p];
+      re += a.x;
+      im += a.y;
     }
-    const double m = dij[p / nbnd];
-    cd[p] = mk(re * m, im * m);
+    const double m = dij[q];
+    cd[i] = mk(re * m, im * m);
     out[p] = mk((T)(re * m), (T)(im * m));
   }
   __syncthreads();
   double corr = 0.0;
-  for (int p = threadIdx.x; p < nbnd * nbnd; p += blockDim.x) {
+  for (int i = threadIdx.x; i < nbnd * nv; i += blockDim.x) {
+    const int w = i / nv, v = v0 + i - w * nv, p = w * nbnd + v;
     double re = 0.0, im = 0.0;
+#pragma unroll 4
     for (int cc = 0; cc < nchunk; ++cc) {
-      re += spart[(kv * nchunk + cc) * nbnd * nbnd + p].x;
-      im += spart[(kv * nchunk + cc) * nbnd * nbnd + p].y;
+      const cplx<double> a = spart[(kv * nchunk + cc) * nbnd * nbnd + p];
+      re += a.x;
+      im += a.y;
     }
-    const int w = p / nbnd, v = p - w * nbnd;
     for (int q = 0; q < nproj; ++q) {
-      const cplx<double> a = ub[((long)k * nbnd + w) * nproj + q], d = cd[q * nbnd + v];
+      const cplx<double> a = ub[((long)k * nbnd + w) * nproj + q], d = cd[q * nv + v - v0];
       re += a.x * d.x - a.y * d.y;
       im += a.x * d.y + a.y * d.x;
     }
@@ -214,14 +222,18 @@ __global__ void __launch_bounds__(256) k_sp_coef(int nks, int nbnd, int nchunk, 
   }
   if (kind == 1) {
     corr = block_sum(corr);
-    if (threadIdx.x == 0) mcorr[kv] = corr;
+    if (threadIdx.x == 0) mcorr[kv * kCoefSlices + blockIdx.y] = corr;
   }
 }
 
 // A metal's term of the norm partial (k_sp_coef, kind 1) added to the first chunk's partial of
 // each (vector, k).  grid 1, block 256.
 static __global__ void k_sp_addcorr(int nkv, int nchunk, const double* __restrict__ mcorr, double* __restrict__ part) {
-  for (int kv = threadIdx.x; kv < nkv; kv += blockDim.x) part[(long)kv * nchunk] += mcorr[kv];
+  for (int kv = threadIdx.x; kv < nkv; kv += blockDim.x) {
+    double t = 0.0;
+    for (int q = 0; q < kCoefSlices; ++q) t += mcorr[kv * kCoefSlices + q];
+    part[(long)kv * nchunk] += t;
+  }
 }
 
 // Operator, last stage, applied: t <- t + B c - U S (= P_c (t + B c)) on one chunk of plane
@@ -254,7 +266,7 @@ __global__ void __launch_bounds__(256) k_sp_apply(int nks, int nbnd, int npw_pad
   const cplx<T>* uk = ukq + (long)k * nbnd * npw_pad;
   const cplx<T>* bk = bkq + (long)k * nproj * npw_pad;
   const int gl = threadIdx.x % kSub, vb = threadIdx.x / kSub;
-  double nr = 0.0;
+  DSum<T> nra;
   for (int s0 = g0; s0 < g1; s0 += kSub) {
     __syncthreads();
     for (int e = threadIdx.x; e < nrow * kSub; e += blockDim.x) {
@@ -275,7 +287,7 @@ __global__ void __launch_bounds__(256) k_sp_apply(int nks, int nbnd, int npw_pad
           for (int w = 0; w < nbnd; ++w) acc = acc - cmul(Bt[(nproj + w) * kSub + gl], Ct[(nproj + w) * nbnd + v]);
           if (part) {
             const cplx<T> x = xin[i];
-            nr += (double)(x.x * acc.x + x.y * acc.y);
+            nra.add(x.x * acc.x + x.y * acc.y);
           }
         }
         t[i] = acc;
@@ -283,7 +295,7 @@ __global__ void __launch_bounds__(256) k_sp_apply(int nks, int nbnd, int npw_pad
     }
   }
   if (!part) return;   // the projection of the update step: no norm
-  nr = warp_sum(nr);
+  const double nr = warp_sum(nra.value());
   if ((threadIdx.x & 31) == 0) wred[threadIdx.x >> 5] = nr;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -338,35 +350,33 @@ __global__ void __launch_bounds__(256) k_sp_nh_start(int j, int upper, int nks, 
   const int g0 = c * kChunk, g1 = min(npw_pad, g0 + kChunk), n = g1 - g0;
   const long base = (long)k * nbnd * npw_pad;
   const int zi = (j - 1) * nks * nchunk + k * nchunk + c;
-  if (upper) {  // z_j partial = (y, v_j) over the chunk
-    double zr = 0.0, zim = 0.0;
-    for (int e = threadIdx.x; e < nbnd * n; e += blockDim.x) {
-      const int v = e / n;
-      const long i = base + (long)v * npw_pad + g0 + e - v * n;
-      const cplx<T> a = y[i], r = Vc[i];
-      zr += (double)(a.x * r.x + a.y * r.y);
-      zim += (double)(a.x * r.y - a.y * r.x);
-    }
-    zr = warp_sum(zr);
-    zim = warp_sum(zim);
-    if ((threadIdx.x & 31) == 0) { zred[0][threadIdx.x >> 5] = zr; zred[1][threadIdx.x >> 5] = zim; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double sr = 0.0, si = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { sr += zred[0][w]; si += zred[1][w]; }
-      co.zpart[zi] = mk(sr, si);
-    }
-  } else if (threadIdx.x == 0) {
-    co.zpart[zi] = mk(0.0, 0.0);
-  }
   const double bj = co.beta[j - 1];
   const cplx<double> gj = co.gamma[j - 1];
   const cplx<T> g = mk((T)gj.x, (T)gj.y), bc = mk((T)bj, (T)0);
+  DSum<T> zr, zim;   // z_j partial = (y, v_j) over the chunk
+#pragma unroll 2
   for (int e = threadIdx.x; e < nbnd * n; e += blockDim.x) {
     const int v = e / n;
     const long i = base + (long)v * npw_pad + g0 + e - v * n;
+    if (upper) {
+      const cplx<T> a = y[i], r = Vc[i];
+      zr.add(a.x * r.x + a.y * r.y);
+      zim.add(a.x * r.y - a.y * r.x);
+    }
     XV[i] = XV[i] - cmul(g, Vp[i]);
     XW[i] = XW[i] - cmul(bc, Wp[i]);
+  }
+  if (upper) {
+    const double sr = warp_sum(zr.value()), si = warp_sum(zim.value());
+    if ((threadIdx.x & 31) == 0) { zred[0][threadIdx.x >> 5] = sr; zred[1][threadIdx.x >> 5] = si; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double tr = 0.0, ti = 0.0;
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { tr += zred[0][w]; ti += zred[1][w]; }
+      co.zpart[zi] = mk(tr, ti);
+    }
+  } else if (threadIdx.x == 0) {
+    co.zpart[zi] = mk(0.0, 0.0);
   }
   if (!dots) return;   // the partials U^H v_hat, U^H w_hat come from the tensor-core kernel
   __syncthreads();
@@ -405,7 +415,7 @@ __global__ void __launch_bounds__(256) k_sp_nh_proj(int nks, int nbnd, int npw_p
   const int np = npw[k];
   const long base = (long)k * nbnd * npw_pad;
   const cplx<T>* uk = ukq + base;
-  double sr = 0.0, si = 0.0;
+  DSum<T> sra, sia;
   for (int e = threadIdx.x; e < nbnd * n; e += blockDim.x) {
     const int v = e / n, g = g0 + e - v * n;
     const long i = base + (long)v * npw_pad + g;
@@ -418,12 +428,11 @@ __global__ void __launch_bounds__(256) k_sp_nh_proj(int nks, int nbnd, int npw_p
     XV[i] = a;
     XW[i] = b;
     if (g < np) {
-      sr += (double)(b.x * a.x + b.y * a.y);
-      si += (double)(b.x * a.y - b.y * a.x);
+      sra.add(b.x * a.x + b.y * a.y);
+      sia.add(b.x * a.y - b.y * a.x);
     }
   }
-  sr = warp_sum(sr);
-  si = warp_sum(si);
+  const double sr = warp_sum(sra.value()), si = warp_sum(sia.value());
   if ((threadIdx.x & 31) == 0) { sred[0][threadIdx.x >> 5] = sr; sred[1][threadIdx.x >> 5] = si; }
   __syncthreads();
   if (threadIdx.x == 0) {

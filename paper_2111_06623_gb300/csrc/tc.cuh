@@ -129,4 +129,23 @@ __device__ __forceinline__ void bf16_split3(float a, __nv_bfloat16& hi, __nv_bfl
   lo = __float2bfloat16_rn(r2);
 }
 
+// The same for two values at once, each part packed (a in the low half): one conversion per
+// part, and a part's float value is its bits moved to the top half of a word.
+__device__ __forceinline__ uint32_t bf16_pack(float a, float b) {
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+  return r;
+}
+__device__ __forceinline__ void bf16_split3x2(float a, float b, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+  hi = bf16_pack(a, b);
+  a -= __uint_as_float(hi << 16);
+  b -= __uint_as_float(hi & 0xffff0000u);
+  mid = bf16_pack(a, b);
+  a -= __uint_as_float(mid << 16);
+  b -= __uint_as_float(mid & 0xffff0000u);
+  lo = bf16_pack(a, b);
+}
+// (a, b) -> (b, -a) of a packed pair: the parts of (im, -re) from those of (re, im)
+__device__ __forceinline__ uint32_t bf16_swapneg(uint32_t v) { return __byte_perm(v, v, 0x1032) ^ 0x80000000u; }
+
 }  // namespace ll

@@ -112,23 +112,10 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-__device__ __forceinline__ uint2 pack_bf16x4(__nv_bfloat16 a, __nv_bfloat16 b, __nv_bfloat16 c, __nv_bfloat16 d) {
-  uint2 r;
-  r.x = (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
-  r.y = (uint32_t)__bfloat16_as_ushort(c) | ((uint32_t)__bfloat16_as_ushort(d) << 16);
-  return r;
-}
-
 // Split four FP32 values into the three BF16 levels, packed four to eight bytes.
 __device__ __forceinline__ void split4(float4 v, uint2& hi, uint2& mid, uint2& lo) {
-  __nv_bfloat16 h[4], m[4], l[4];
-  bf16_split3(v.x, h[0], m[0], l[0]);
-  bf16_split3(v.y, h[1], m[1], l[1]);
-  bf16_split3(v.z, h[2], m[2], l[2]);
-  bf16_split3(v.w, h[3], m[3], l[3]);
-  hi = pack_bf16x4(h[0], h[1], h[2], h[3]);
-  mid = pack_bf16x4(m[0], m[1], m[2], m[3]);
-  lo = pack_bf16x4(l[0], l[1], l[2], l[3]);
+  bf16_split3x2(v.x, v.y, hi.x, mid.x, lo.x);
+  bf16_split3x2(v.z, v.w, hi.y, mid.y, lo.y);
 }
 
 // Piece i of this thread in a stage: source row and 16-byte piece f of the row.  A warp's 32
@@ -226,7 +213,9 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_dots(TcDotsArgs a) {
             *reinterpret_cast<uint2*>(base + 2 * lev_bytes + o) = l;
           }
           if (das >= 0 || dbs >= 0) {   // swap: (im, -re) per complex value
-            split4(make_float4(v.y, -v.x, v.w, -v.z), h, m, l);
+            h = make_uint2(bf16_swapneg(h.x), bf16_swapneg(h.y));
+            m = make_uint2(bf16_swapneg(m.x), bf16_swapneg(m.y));
+            l = make_uint2(bf16_swapneg(l.x), bf16_swapneg(l.y));
             const uint32_t o = das >= 0 ? tc_off(das, kin) : kTcATile + tc_off(dbs, kin);
             *reinterpret_cast<uint2*>(base + o) = h;
             *reinterpret_cast<uint2*>(base + lev_bytes + o) = m;
@@ -331,7 +320,7 @@ constexpr int kTaKs = 2;         // K steps per stage: 2 x 8 rows q of W
 constexpr int kTaRows = 8 * kTaKs;
 constexpr int kTaRing = 5;       // FP32 stages of W in flight (cp.async ring)
 constexpr int kTaRawRow = 128 * 8 + 64;   // bytes of one W row of a raw stage (padded)
-constexpr int kTaBands = 16;     // bands per epilogue group (a multiple of 8)
+constexpr int kTaThreads = 512;
 
 struct TcApplyArgs {
   int nks, nbnd, npw_pad, nchunk, nproj, nb, nks_k;  // nb = N (2 nbnd padded to 32); nks_k = K steps of K'
@@ -347,17 +336,20 @@ struct TcApplyArgs {
 };
 
 __host__ __device__ inline size_t tc_apply_smem(int nb, int nks_k) {
-  return (size_t)3 * nks_k * 32 * nb + (size_t)3 * kTaKs * kTcATile + (size_t)kTaRing * kTaRows * kTaRawRow;
+  return (size_t)3 * nks_k * 32 * nb + (size_t)2 * 3 * kTaKs * kTcATile + (size_t)kTaRing * kTaRows * kTaRawRow;
 }
 
-// grid (nks, nvec, nchunk), block kTcThreads, dynamic shared memory tc_apply_smem(nb, nks_k).
+// grid (nks, nvec, nchunk), block kTaThreads, dynamic shared memory tc_apply_smem(nb, nks_k).
 // The rows of W of stage (tile, st) stream into a ring of FP32 stages (cp.async, kTaRing - 1
-// stages ahead, across tiles), are split into the BF16 A tile and multiplied.
-static __global__ void __launch_bounds__(kTcThreads, 1) k_tc_apply(TcApplyArgs a) {
+// stages ahead, across tiles), are split into one of two BF16 A tiles and multiplied while the
+// next stage is split into the other.  One CTA per SM (coefficients 72 KB, tiles 48 KB, ring
+// 85 KB on the sixteen-atom cell), so it has 16 warps; the split, not HBM or the tensor pipe, is
+// what it spends its issue slots on.  Sixteen-atom cell, per launch (operator / update): PLACE_TA.
+static __global__ void __launch_bounds__(kTaThreads, 1) k_tc_apply(TcApplyArgs a) {
   extern __shared__ __align__(1024) unsigned char tsm[];
-  __shared__ __align__(8) uint64_t bar;
+  __shared__ __align__(8) uint64_t bar[2];
   __shared__ uint32_t tslot;
-  __shared__ double wred[kTcThreads / 32];
+  __shared__ double wred[kTaThreads / 32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int k = blockIdx.x, vec = blockIdx.y, c = blockIdx.z;
   const long kv = (long)vec * a.nks + k;
@@ -367,22 +359,23 @@ static __global__ void __launch_bounds__(kTcThreads, 1) k_tc_apply(TcApplyArgs a
   const int g0 = c * kChunk, g1 = min(a.npw_pad, g0 + kChunk);
   const size_t bop_lev = (size_t)nks_k * 32 * nb;           // one level of the coefficient operand
   unsigned char* bop = tsm;
-  unsigned char* ast = tsm + 3 * bop_lev;                    // A stage: [level][kTaKs][128 rows x 32 B]
   const size_t ast_lev = (size_t)kTaKs * kTcATile;
-  unsigned char* ring = ast + 3 * ast_lev;                   // [kTaRing][kTaRows][kTaRawRow]
+  unsigned char* ast2 = tsm + 3 * bop_lev;                   // two A stages: [level][kTaKs][128 rows x 32 B]
+  unsigned char* ring = ast2 + 2 * 3 * ast_lev;                   // [kTaRing][kTaRows][kTaRawRow]
   const int nstage = (nq + kTaRows - 1) / kTaRows;          // stages per tile
   const int ntile = (g1 - g0 + 127) / 128;
   const int nseq = ntile * nstage;                           // (tile, stage) in order
 
   if (warp == 0) tc_alloc(&tslot, 128);
   if (tid == 0) {
-    mbar_init(&bar, 1);
+    mbar_init(&bar[0], 1);
+    mbar_init(&bar[1], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // the coefficient operand, all three levels, zero outside the 2 nbnd x 2 nq block
   {
     const float2* cf = a.coef + kv * (long)nq * nbnd;
-    for (int e = tid; e < nb * nks_k * 16; e += kTcThreads) {
+    for (int e = tid; e < nb * nks_k * 16; e += kTaThreads) {
       const int n = e / (nks_k * 16), kk = e - n * (nks_k * 16);
       const int q = kk >> 1, v = n >> 1;
       float val = 0.f;
@@ -411,8 +404,8 @@ static __global__ void __launch_bounds__(kTcThreads, 1) k_tc_apply(TcApplyArgs a
     const int gt = g0 + (sq / nstage) * 128, st = sq % nstage;
     unsigned char* slot = ring + (size_t)(sq % kTaRing) * kTaRows * kTaRawRow;
 #pragma unroll
-    for (int i = 0; i < kTaRows * 64 / kTcThreads; ++i) {
-      const int e = tid + i * kTcThreads;
+    for (int i = 0; i < kTaRows * 64 / kTaThreads; ++i) {
+      const int e = tid + i * kTaThreads;
       const int ql = e >> 6, gp = e & 63;
       const int q = st * kTaRows + ql, g = gt + 2 * gp;
       const int bytes = (q < nq && g < npw) ? (g + 1 < npw ? 16 : 8) : 0;
@@ -423,33 +416,39 @@ static __global__ void __launch_bounds__(kTcThreads, 1) k_tc_apply(TcApplyArgs a
   };
   // convert mapping: lane = (g % 8, q % 4), conflict-free 4-byte BF16 stores
   auto convert = [&](int sq) {
+    unsigned char* ast = ast2 + (sq & 1) * 3 * ast_lev;
     const unsigned char* slot = ring + (size_t)(sq % kTaRing) * kTaRows * kTaRawRow;
 #pragma unroll
-    for (int i = 0; i < kTaRows * 128 / kTcThreads; ++i) {
-      const int e = tid + i * kTcThreads;
+    for (int i = 0; i < kTaRows * 128 / kTaThreads; ++i) {
+      const int e = tid + i * kTaThreads;
       const int item = e >> 5, ln = e & 31;
       const int gl = (item & 15) * 8 + (ln & 7);         // plane wave in the tile
       const int ql = (item >> 4) * 4 + (ln >> 3);         // row q in the stage
       const float2 v = *reinterpret_cast<const float2*>(slot + ql * kTaRawRow + gl * 8);
-      __nv_bfloat16 hr, mr, lr, hi, mi, li;
-      bf16_split3(v.x, hr, mr, lr);
-      bf16_split3(v.y, hi, mi, li);
+      uint32_t vh, vm, vl;
+      bf16_split3x2(v.x, v.y, vh, vm, vl);
       const int kk = 2 * ql;
       const uint32_t o = (uint32_t)((kk >> 4) * kTcATile) + tc_off(gl, kk & 15);
-      *reinterpret_cast<uint32_t*>(ast + o) = (uint32_t)__bfloat16_as_ushort(hr) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-      *reinterpret_cast<uint32_t*>(ast + ast_lev + o) =
-          (uint32_t)__bfloat16_as_ushort(mr) | ((uint32_t)__bfloat16_as_ushort(mi) << 16);
-      *reinterpret_cast<uint32_t*>(ast + 2 * ast_lev + o) =
-          (uint32_t)__bfloat16_as_ushort(lr) | ((uint32_t)__bfloat16_as_ushort(li) << 16);
+      *reinterpret_cast<uint32_t*>(ast + o) = vh;
+      *reinterpret_cast<uint32_t*>(ast + ast_lev + o) = vm;
+      *reinterpret_cast<uint32_t*>(ast + 2 * ast_lev + o) = vl;
     }
   };
 
   bool ok = true;
-  uint32_t phase = 0;
-  bool pending = false;          // MMAs committed and not yet waited for
-  double nr = 0.0;
+  uint32_t waits = 0;            // phases of bar[] waited for, by buffer (bit 0, bit 1: parity)
+  int done = 0;                  // stages whose MMAs are known to be complete
+  // every MMA of stages < n complete (stage q commits to bar[q & 1])
+  auto wait_stages = [&](int n) {
+    for (; done < n; ++done) {
+      const int f = done & 1;
+      if (!mbar_wait(&bar[f], (waits >> f) & 1)) ok = false;
+      waits ^= 1u << f;
+    }
+    tc_fence_after();
+  };
+  DSum<float> nr;
   const int row = (warp & 3) * 32 + lane;
-  const int half = nb / 2, cbeg = (warp >> 2) * half;
   for (int i = 0; i < kTaRing - 1; ++i) {
     issue(i);
     cp_async_commit();
@@ -459,19 +458,14 @@ static __global__ void __launch_bounds__(kTcThreads, 1) k_tc_apply(TcApplyArgs a
     issue(sq + kTaRing - 1);
     cp_async_commit();
     cp_async_wait<kTaRing - 1>();       // this thread's pieces of stage sq have landed
-    if (pending) {                      // the tensor core has finished with the A tile
-      if (!mbar_wait(&bar, phase)) ok = false;
-      phase ^= 1;
-      pending = false;
-      tc_fence_after();
-    }
+    if (sq >= 2) wait_stages(sq - 1);   // the tensor core has finished with this A tile (stage sq - 2)
     __syncthreads();                    // every thread's pieces of stage sq are in the ring
     convert(sq);
     fence_async_smem();
     __syncthreads();
     if (tid == 0) {
       tc_fence_after();
-      const uint32_t sa0 = smem_u32(ast), sb0 = smem_u32(bop);
+      const uint32_t sa0 = smem_u32(ast2 + (sq & 1) * 3 * ast_lev), sb0 = smem_u32(bop);
       const int pa[6] = {0, 0, 1, 0, 2, 1}, pb[6] = {0, 1, 0, 2, 0, 1};
 #pragma unroll
       for (int ks = 0; ks < kTaKs; ++ks) {
@@ -484,55 +478,46 @@ static __global__ void __launch_bounds__(kTcThreads, 1) k_tc_apply(TcApplyArgs a
           tc_mma(taddr, tc_desc(sa), tc_desc(sb), idesc, (st > 0 || ks > 0 || p > 0) ? 1 : 0);
         }
       }
-      tc_commit(&bar);
+      tc_commit(&bar[sq & 1]);
     }
-    pending = true;
     if (st + 1 < nstage) continue;
-    // epilogue: thread = plane wave gt + row, the bands of its column half, in groups of
-    // kTaBands.  The group's t and x values are loaded before the wait for the tile's last
-    // MMAs (the first group) or before its tensor-memory loads, so that their latency overlaps.
+    // epilogue: thread = plane wave gt + row, blocks of 16 columns (eight bands) by warp group.  The
+    // block's t and x values are loaded before the wait for the tile's last MMAs.
     const int gt = g0 + tile * 128;
     const int g = gt + row;
     const bool live = g < npw;
-    for (int vb = 0; vb < half / 2; vb += kTaBands) {
-      const int v0 = (cbeg >> 1) + vb;
-      float2 tv[kTaBands], xv[kTaBands];
+    for (int cbk = warp >> 2; cbk < nb / 16; cbk += kTaThreads / 128) {
+      const int v0 = 8 * cbk;
+      float2 tv[8], xv[8];
 #pragma unroll
-      for (int j = 0; j < kTaBands; ++j) {
+      for (int j = 0; j < 8; ++j) {
         tv[j] = xv[j] = make_float2(0.f, 0.f);
         const int v = v0 + j;
-        if (live && vb + j < half / 2 && v < nbnd) {
+        if (live && v < nbnd) {
           const long idx = (kv * nbnd + v) * pad + g;
           tv[j] = a.t[idx];
           if (a.x) xv[j] = a.x[idx];
         }
       }
-      if (vb == 0) {   // the tile's accumulator is complete once its last MMAs are
-        if (!mbar_wait(&bar, phase)) ok = false;
-        phase ^= 1;
-        pending = false;
-        tc_fence_after();
-      }
+      wait_stages(sq + 1);   // the tile's accumulator is complete once its last MMAs are
+      float d[16];
+      tc_ld16(taddr + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(16 * cbk), d);
+      if (ok && g < g1) {
 #pragma unroll
-      for (int h = 0; h < kTaBands / 8; ++h) {
-        const int c0 = cbeg + 2 * vb + 16 * h;
-        if (c0 >= cbeg + half) break;
-        float d[16];
-        tc_ld16(taddr + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0, d);
-        if (!ok || g >= g1) continue;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int j = 8 * h + i, v = v0 + j;
+        for (int j = 0; j < 8; ++j) {
+          const int v = v0 + j;
           if (v >= nbnd) continue;
           float2 r = make_float2(0.f, 0.f);
           if (live) {
-            r = make_float2(tv[j].x + d[2 * i], tv[j].y + d[2 * i + 1]);
-            nr += (double)(xv[j].x * r.x + xv[j].y * r.y);
+            r = make_float2(tv[j].x + d[2 * j], tv[j].y + d[2 * j + 1]);
+            nr.add(xv[j].x * r.x + xv[j].y * r.y);
           }
           a.t[(kv * nbnd + v) * pad + g] = r;
         }
       }
+      __syncwarp();
     }
+    wait_stages(sq + 1);
     tc_fence_before();
     __syncthreads();   // every thread has read the accumulator before the next tile's MMAs
     tc_fence_after();
@@ -540,12 +525,12 @@ static __global__ void __launch_bounds__(kTcThreads, 1) k_tc_apply(TcApplyArgs a
   cp_async_wait<0>();
   if (!ok && lane == 0) flag_error(a.err, DEV_TIMEOUT, a.jdev ? *a.jdev : 0);
   if (a.part) {
-    nr = warp_sum(nr);
-    if (lane == 0) wred[warp] = nr;
+    const double ws = warp_sum(nr.value());
+    if (lane == 0) wred[warp] = ws;
     __syncthreads();
     if (tid == 0) {
       double s = 0.0;
-      for (int w = 0; w < kTcThreads / 32; ++w) s += wred[w];
+      for (int w = 0; w < kTaThreads / 32; ++w) s += wred[w];
       a.part[kv * a.nchunk + c] = s;
     }
   }
