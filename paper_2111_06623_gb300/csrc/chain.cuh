@@ -1255,7 +1255,9 @@ class Chain : public ChainBase {
       const size_t sm = tc_apply_smem(a.nb, a.nks_k);
       int rc;
       if ((rc = set_smem(k_tc_apply, sm, err))) return rc;
-      k_tc_apply<<<dim3(nks_, nvec, nchunk_), kTaThreads, sm, st_>>>(a);
+      a.tiles = tc_apply_tiles(nks_ * nvec, a.npw_pad, nsm_);
+      const int ng = ((a.npw_pad + 127) / 128 + a.tiles - 1) / a.tiles;
+      k_tc_apply<<<dim3(nks_, nvec, ng), kTaThreads, sm, st_>>>(a);
       LL_CK(cudaGetLastError());
       return LL_OK;
     } else {

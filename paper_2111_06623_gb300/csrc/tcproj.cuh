@@ -26,6 +26,8 @@
 // BF16 tiles; one elected thread issues the MMAs and commits them to an mbarrier that the CTA
 // waits on (bounded) before it overwrites the tiles.
 #pragma once
+#include <algorithm>
+
 #include "split.cuh"
 #include "tc.cuh"
 
@@ -163,67 +165,63 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_dots(TcDotsArgs a) {
   const uint32_t taddr = tslot;
   const uint32_t idesc = tc_idesc_bf16(128, nb);
 
-  // the FP32 pieces of stage st into ring slot st % kTcRaw (zero beyond the chunk's sphere)
-  auto issue = [&](int st) {
-    const int gs = g0 + st * kTcPw;
-    unsigned char* slot = raw + (size_t)(st % kTcRaw) * raw_slot;
+  // this thread's pieces (the same of every stage): source address at the chunk's start, offset in
+  // a ring slot, and the offsets in a BF16 level where its values and their swap go (-1: nowhere)
+  const float4* psrc[kTcMaxF4];
+  int pg[kTcMaxF4], pslot[kTcMaxF4], pdst[kTcMaxF4], pswp[kTcMaxF4];
 #pragma unroll
-    for (int i = 0; i < kTcMaxF4; ++i) {
-      const int e = tid + i * kTcThreads;
-      if (e < npiece) {
-        int row, f;
-        tc_piece(e, row, f);
-        if (row < nsrc) {
-          const int g = gs + 2 * f;
-          int da, das, db, dbs;
-          const float4* src = tc_src<MODE>(a, k, kv, row, da, das, db, dbs);
-          const int bytes = g < g1 ? (g + 1 < g1 ? 16 : 8) : 0;
-          cp_async16(slot + row * kTcRawRow + f * 16, src + (bytes ? (g >> 1) : 0), bytes);
-        }
+  for (int i = 0; i < kTcMaxF4; ++i) {
+    const int e = tid + i * kTcThreads;
+    pg[i] = pslot[i] = pdst[i] = pswp[i] = -1;
+    psrc[i] = nullptr;
+    if (e < npiece) {
+      int row, f;
+      tc_piece(e, row, f);
+      if (row < nsrc) {
+        int da, das, db, dbs;
+        psrc[i] = tc_src<MODE>(a, k, kv, row, da, das, db, dbs) + (g0 + 2 * f) / 2;
+        pg[i] = g0 + 2 * f;
+        pslot[i] = row * kTcRawRow + f * 16;
+        const int ks = (int)((f >> 2) * step_bytes), kin = (f & 3) * 4;
+        // a source row has one place of its own (A or Bop) and at most one for its swap
+        pdst[i] = ks + (int)(da >= 0 ? tc_off(da, kin) : kTcATile + tc_off(db, kin));
+        if (das >= 0 || dbs >= 0) pswp[i] = ks + (int)(das >= 0 ? tc_off(das, kin) : kTcATile + tc_off(dbs, kin));
       }
     }
+  }
+  // the FP32 pieces of stage st into ring slot st % kTcRaw (zero beyond the chunk's sphere)
+  auto issue = [&](int st) {
+    unsigned char* slot = raw + (size_t)(st % kTcRaw) * raw_slot;
+#pragma unroll
+    for (int i = 0; i < kTcMaxF4; ++i)
+      if (pslot[i] >= 0) {
+        const int g = pg[i] + st * kTcPw;
+        const int bytes = g < g1 ? (g + 1 < g1 ? 16 : 8) : 0;
+        cp_async16(slot + pslot[i], bytes ? psrc[i] + st * (kTcPw / 2) : a.ukq, bytes);
+      }
   };
   // ring slot st % kTcRaw -> the three BF16 levels of A and Bop (and the swapped copies)
   auto convert = [&](int st) {
     const unsigned char* slot = raw + (size_t)(st % kTcRaw) * raw_slot;
 #pragma unroll
-    for (int i = 0; i < kTcMaxF4; ++i) {
-      const int e = tid + i * kTcThreads;
-      if (e < npiece) {
-        int row, f;
-        tc_piece(e, row, f);
-        if (row < nsrc) {
-          int da, das, db, dbs;
-          tc_src<MODE>(a, k, kv, row, da, das, db, dbs);
-          const int ks = f >> 2, kin = (f & 3) * 4;
-          const float4 v = *reinterpret_cast<const float4*>(slot + row * kTcRawRow + f * 16);
-          uint2 h, m, l;
-          split4(v, h, m, l);
-          unsigned char* base = tile + ks * step_bytes;
-          if (da >= 0) {
-            const uint32_t o = tc_off(da, kin);
-            *reinterpret_cast<uint2*>(base + o) = h;
-            *reinterpret_cast<uint2*>(base + lev_bytes + o) = m;
-            *reinterpret_cast<uint2*>(base + 2 * lev_bytes + o) = l;
-          }
-          if (db >= 0) {
-            const uint32_t o = kTcATile + tc_off(db, kin);
-            *reinterpret_cast<uint2*>(base + o) = h;
-            *reinterpret_cast<uint2*>(base + lev_bytes + o) = m;
-            *reinterpret_cast<uint2*>(base + 2 * lev_bytes + o) = l;
-          }
-          if (das >= 0 || dbs >= 0) {   // swap: (im, -re) per complex value
-            h = make_uint2(bf16_swapneg(h.x), bf16_swapneg(h.y));
-            m = make_uint2(bf16_swapneg(m.x), bf16_swapneg(m.y));
-            l = make_uint2(bf16_swapneg(l.x), bf16_swapneg(l.y));
-            const uint32_t o = das >= 0 ? tc_off(das, kin) : kTcATile + tc_off(dbs, kin);
-            *reinterpret_cast<uint2*>(base + o) = h;
-            *reinterpret_cast<uint2*>(base + lev_bytes + o) = m;
-            *reinterpret_cast<uint2*>(base + 2 * lev_bytes + o) = l;
-          }
+    for (int i = 0; i < kTcMaxF4; ++i)
+      if (pslot[i] >= 0) {
+        uint2 h, m, l;
+        split4(*reinterpret_cast<const float4*>(slot + pslot[i]), h, m, l);
+        unsigned char* d = tile + pdst[i];
+        *reinterpret_cast<uint2*>(d) = h;
+        *reinterpret_cast<uint2*>(d + lev_bytes) = m;
+        *reinterpret_cast<uint2*>(d + 2 * lev_bytes) = l;
+        if (pswp[i] >= 0) {   // swap: (im, -re) per complex value
+          h = make_uint2(bf16_swapneg(h.x), bf16_swapneg(h.y));
+          m = make_uint2(bf16_swapneg(m.x), bf16_swapneg(m.y));
+          l = make_uint2(bf16_swapneg(l.x), bf16_swapneg(l.y));
+          d = tile + pswp[i];
+          *reinterpret_cast<uint2*>(d) = h;
+          *reinterpret_cast<uint2*>(d + lev_bytes) = m;
+          *reinterpret_cast<uint2*>(d + 2 * lev_bytes) = l;
         }
       }
-    }
   };
 
   bool ok = true;
@@ -324,6 +322,7 @@ constexpr int kTaThreads = 512;
 
 struct TcApplyArgs {
   int nks, nbnd, npw_pad, nchunk, nproj, nb, nks_k;  // nb = N (2 nbnd padded to 32); nks_k = K steps of K'
+  int tiles;             // tiles of 128 plane waves per CTA
   const int* npw;
   const float2* x;       // operator input (norm partial), or null
   float2* t;             // vector updated in place
@@ -339,7 +338,22 @@ __host__ __device__ inline size_t tc_apply_smem(int nb, int nks_k) {
   return (size_t)3 * nks_k * 32 * nb + (size_t)2 * 3 * kTaKs * kTcATile + (size_t)kTaRing * kTaRows * kTaRawRow;
 }
 
-// grid (nks, nvec, nchunk), block kTaThreads, dynamic shared memory tc_apply_smem(nb, nks_k).
+// Tiles of 128 plane waves per CTA, at least a chunk's four (the partials then have a place): one
+// CTA runs per SM, so the launch takes waves x (tiles + the set-up of the coefficient operand,
+// about one tile's time); the least of that (sixteen-atom cell, 64 k of 47 tiles on 152 SMs: 7
+// tiles, 3 waves, where a chunk each made 5.05).
+static inline int tc_apply_tiles(int nkv, int npw_pad, int nsm) {
+  const int t = (npw_pad + 127) / 128;
+  int best = 4;
+  long cost = -1;
+  for (int n = 4; n <= 16; ++n) {
+    const long waves = ((long)nkv * ((t + n - 1) / n) + nsm - 1) / nsm, c = waves * (std::min(n, t) + 1);
+    if (cost < 0 || c < cost) cost = c, best = n;
+  }
+  return best;
+}
+
+// grid (nks, nvec, tile groups), block kTaThreads, dynamic shared memory tc_apply_smem(nb, nks_k).
 // The rows of W of stage (tile, st) stream into a ring of FP32 stages (cp.async, kTaRing - 1
 // stages ahead, across tiles), are split into one of two BF16 A tiles and multiplied while the
 // next stage is split into the other.  One CTA per SM (coefficients 72 KB, tiles 48 KB, ring
@@ -356,7 +370,7 @@ static __global__ void __launch_bounds__(kTaThreads, 1) k_tc_apply(TcApplyArgs a
   const int nb = a.nb, nbnd = a.nbnd, np = a.nproj, nq = np + nbnd, nks_k = a.nks_k;
   const long pad = a.npw_pad;
   const int npw = a.npw[k];
-  const int g0 = c * kChunk, g1 = min(a.npw_pad, g0 + kChunk);
+  const int g0 = c * a.tiles * 128, g1 = min(a.npw_pad, g0 + a.tiles * 128);
   const size_t bop_lev = (size_t)nks_k * 32 * nb;           // one level of the coefficient operand
   unsigned char* bop = tsm;
   const size_t ast_lev = (size_t)kTaKs * kTcATile;
@@ -532,6 +546,8 @@ static __global__ void __launch_bounds__(kTaThreads, 1) k_tc_apply(TcApplyArgs a
       double s = 0.0;
       for (int w = 0; w < kTaThreads / 32; ++w) s += wred[w];
       a.part[kv * a.nchunk + c] = s;
+      if (c == 0)   // the partials of the chunked path that this grid has no CTA for
+        for (int q = gridDim.z; q < a.nchunk; ++q) a.part[kv * a.nchunk + q] = 0.0;
     }
   }
   tc_fence_before();
