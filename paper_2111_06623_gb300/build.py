@@ -20,6 +20,9 @@ UNITS = ("ll_api", "ll_f64", "ll_f32", "ll_server")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include")]
 
+# the FP64 unit's integer transforms take minutes on one thread; the others' code is better unsplit
+UNIT_FLAGS = {"ll_f64": ["-split-compile=0"]}
+
 
 def _nvcc() -> str:
     for cand in (shutil.which("nvcc"), "/usr/local/cuda/bin/nvcc"):
@@ -36,7 +39,7 @@ def source_hash(extra_flags: list[str] | None = None) -> str:
         h.update(os.path.basename(p).encode() + b"\0")
         with open(p, "rb") as fh:
             h.update(fh.read())
-    h.update("\0".join(ARCH + FLAGS + list(extra_flags or []) + [platform.machine()]).encode())
+    h.update("\0".join(ARCH + FLAGS + sum(UNIT_FLAGS.values(), []) + list(extra_flags or []) + [platform.machine()]).encode())
     r = subprocess.run([_nvcc(), "--version"], capture_output=True, text=True)
     h.update(r.stdout.encode())
     return h.hexdigest()
@@ -61,7 +64,7 @@ def build_library(force: bool = False, extra_flags: list[str] | None = None, che
 
     def compile_one(u):
         obj = os.path.join(build_dir, u + ".o")
-        cmd = [nvcc, *ARCH, *flags, "-c", os.path.join(SRC, u + ".cu"), "-o", obj]
+        cmd = [nvcc, *ARCH, *flags, *UNIT_FLAGS.get(u, []), "-c", os.path.join(SRC, u + ".cu"), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed for {u}:\n{r.stderr[-4000:]}")

@@ -20,7 +20,7 @@
 #include "ll.h"
 #include "split.cuh"
 #include "tcproj.cuh"
-#include "plane.cuh"
+#include "plane64.cuh"
 
 #include <type_traits>
 
@@ -1427,10 +1427,11 @@ class Chain : public ChainBase {
     a.bo = PlaneCfg<T, N, MODE>::SL;
     const size_t smem = plane_smem<T, N, MODE>(cb_ncol_, s.nrow_max);
     int rc;
-    if ((rc = set_smem(k_plane<T, N, MODE, PR>, smem, err))) return rc;
-    const int ng = groups_for_kernel(k_plane<T, N, MODE, PR>, smem, norb, xy_groups_[MODE], threads, MODE == XY_PASS1_DENS);
+    auto* kernel = plane_kernel<T, N, MODE, PR>();
+    if ((rc = set_smem(kernel, smem, err))) return rc;
+    const int ng = groups_for_kernel(kernel, smem, norb, xy_groups_[MODE], threads, MODE == XY_PASS1_DENS);
     a.per_group = (norb + ng - 1) / ng;
-    k_plane<T, N, MODE, PR><<<dim3(N, ng), threads, smem, st_>>>(a, cbuf_, vloc_, vpr_, ur_, nprt_, err_);
+    kernel<<<dim3(N, ng), threads, smem, st_>>>(a, cbuf_, vloc_, vpr_, ur_, nprt_, err_);
     if (MODE == XY_PASS1_DENS) last_ng_ = ng;
     LL_CK(cudaGetLastError());
     return LL_OK;

@@ -10,6 +10,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "fixed.cuh"
 
 namespace ll {
 
@@ -17,19 +18,32 @@ namespace ll {
 // them with tw_tables_upload() on every device it uses.
 static __constant__ double2 c_tw64[kTwTotal];
 static __constant__ float2 c_tw32[kTwTotal];
+static __constant__ int c_twfx[6 * kTwTotal];
 
+// A line of type T and its twiddles: W(e), type (the real pair; in fixed point fixed.cuh's limbs).
 template <typename T> struct TwTab;
 template <> struct TwTab<double> {
+  using type = cplx<double>;
   static __device__ __forceinline__ cplx<double> get(int i) { double2 w = c_tw64[i]; return mk(w.x, w.y); }
 };
 template <> struct TwTab<float> {
+  using type = cplx<float>;
   static __device__ __forceinline__ cplx<float> get(int i) { float2 w = c_tw32[i]; return mk(w.x, w.y); }
+};
+
+template <> struct TwTab<fx64> {
+  using type = FxTw;
+  static __device__ __forceinline__ FxTw get(int i) {
+    const int* w = c_twfx + 6 * i;
+    return FxTw{w[0], w[1], w[2], w[3], w[4], w[5]};
+  }
 };
 
 // exp(-2 pi i e / N) from the host libm in double (and rounded to float), for every side.
 static inline cudaError_t tw_tables_upload(cudaStream_t stream) {
   double2 h64[kTwTotal];
   float2 h32[kTwTotal];
+  int hfx[6 * kTwTotal];
   int off = 0;
   for (int n : kGridSides) {
     for (int e = 0; e < n; ++e) {
@@ -40,6 +54,7 @@ static inline cudaError_t tw_tables_upload(cudaStream_t stream) {
       if (4 * e == 3 * n) { c = 0.0; s = 1.0; }
       h64[off + e] = make_double2(c, s);
       h32[off + e] = make_float2((float)c, (float)s);
+      fx_twiddle_limbs(e, n, hfx + 6 * (off + e));
     }
     off += n;
   }
@@ -47,14 +62,20 @@ static inline cudaError_t tw_tables_upload(cudaStream_t stream) {
   if (err != cudaSuccess) return err;
   err = cudaMemcpyToSymbolAsync(c_tw32, h32, sizeof(h32), 0, cudaMemcpyHostToDevice, stream);
   if (err != cudaSuccess) return err;
+  err = cudaMemcpyToSymbolAsync(c_twfx, hfx, sizeof(hfx), 0, cudaMemcpyHostToDevice, stream);
+  if (err != cudaSuccess) return err;
   return cudaStreamSynchronize(stream);
 }
 
+template <typename T> __device__ __forceinline__ cplx<T> conj_tw(cplx<T> w) { return mk(w.x, -w.y); }
 template <typename T, int N, int SIGN>
-__device__ __forceinline__ cplx<T> twiddle(int e) {
-  cplx<T> w = TwTab<T>::get(TwOff<N>::v + e);
-  if (SIGN > 0) w.y = -w.y;
-  return w;
+__device__ __forceinline__ typename TwTab<T>::type twiddle(int e) {
+  const typename TwTab<T>::type w = TwTab<T>::get(TwOff<N>::v + e);
+  return SIGN > 0 ? conj_tw(w) : w;
+}
+// SIGN i w
+template <int SIGN, typename T> __device__ __forceinline__ cplx<T> turn_tw(cplx<T> w) {
+  return (SIGN > 0) ? mk(-w.y, w.x) : mk(w.y, -w.x);
 }
 
 // Arithmetic with explicit rounding: what the compiler may contract is written out, so a
@@ -77,13 +98,30 @@ template <typename T> __device__ __forceinline__ void butterfly(cplx<T> a, cplx<
   d = mk(fma_rn(T(2), a.x, -s.x), fma_rn(T(2), a.y, -s.y));
 }
 
+// o + a, or o - a where h
+template <typename T> __device__ __forceinline__ cplx<T> addsub(int h, cplx<T> a, cplx<T> o) {
+  const T s = h ? T(-1) : T(1);
+  return mk(fma_rn(s, a.x, o.x), fma_rn(s, a.y, o.y));
+}
+// the rest of a three-point DFT from a and sum, dif = b +- c
+template <int SIGN, typename T> __device__ __forceinline__ void third(cplx<T> a, cplx<T> sum, cplx<T> dif, cplx<T>* v) {
+  // W_3 = -1/2 + SIGN i sqrt(3)/2
+  const T c = T(-0.5);
+  const T s = T(SIGN) * T(0.86602540378443864676372317075294);
+  const cplx<T> m = mk(fma_rn(c, sum.x, a.x), fma_rn(c, sum.y, a.y));
+  // i s dif = (-s dif.y, s dif.x)
+  v[1] = mk(fma_rn(-s, dif.y, m.x), fma_rn(s, dif.x, m.y));
+  v[2] = mk(fma_rn(s, dif.y, m.x), fma_rn(-s, dif.x, m.y));
+}
+
 // R-point DFT in place with exponent sign SIGN.
 template <typename T, int R, int SIGN> struct Dft;
 
 // w1 multiplies input 1 and w1^2 input 2 (and w1^3 input 3) where TW (a twiddled pass).
 template <typename T, int SIGN> struct Dft<T, 2, SIGN> {
+  using Tw = typename TwTab<T>::type;
   template <bool TW>
-  static __device__ __forceinline__ void run(cplx<T>* v, cplx<T> w1, cplx<T>) {
+  static __device__ __forceinline__ void run(cplx<T>* v, Tw w1, Tw) {
     const cplx<T> a = v[0], b = v[1];
     if (TW) {
       butterfly(a, b, w1, v[0], v[1]);
@@ -95,32 +133,28 @@ template <typename T, int SIGN> struct Dft<T, 2, SIGN> {
 };
 
 template <typename T, int SIGN> struct Dft<T, 3, SIGN> {
+  using Tw = typename TwTab<T>::type;
   template <bool TW>
-  static __device__ __forceinline__ void run(cplx<T>* v, cplx<T> w1, cplx<T> w2) {
-    // W_3 = -1/2 + SIGN i sqrt(3)/2
-    const T c = T(-0.5);
-    const T s = T(SIGN) * T(0.86602540378443864676372317075294);
-    cplx<T> a = v[0], sum, dif;
+  static __device__ __forceinline__ void run(cplx<T>* v, Tw w1, Tw w2) {
+    const cplx<T> a = v[0];
+    cplx<T> sum, dif;
     if (TW) butterfly(cmul_rn(v[1], w1), v[2], w2, sum, dif);
     else sum = cadd(v[1], v[2]), dif = csub(v[1], v[2]);
     v[0] = cadd(a, sum);
-    cplx<T> m = mk(fma_rn(c, sum.x, a.x), fma_rn(c, sum.y, a.y));
-    // i s dif = (-s dif.y, s dif.x)
-    v[1] = mk(fma_rn(-s, dif.y, m.x), fma_rn(s, dif.x, m.y));
-    v[2] = mk(fma_rn(s, dif.y, m.x), fma_rn(-s, dif.x, m.y));
+    third<SIGN>(a, sum, dif, v);
   }
 };
 
 template <typename T, int SIGN> struct Dft<T, 4, SIGN> {
+  using Tw = typename TwTab<T>::type;
   template <bool TW>
-  static __device__ __forceinline__ void run(cplx<T>* v, cplx<T> w1, cplx<T> w2) {
+  static __device__ __forceinline__ void run(cplx<T>* v, Tw w1, Tw w2) {
     cplx<T> a0, a1, b0, b1;
     if (TW) {   // w1 v1 +- w3 v3 = w1 (v1 +- w2 v3): the factor w1 goes into the last butterflies
       butterfly(v[0], v[2], w2, a0, a1);
       butterfly(v[1], v[3], w2, b0, b1);
       butterfly(a0, b0, w1, v[0], v[2]);
-      const cplx<T> jw = (SIGN > 0) ? mk(-w1.y, w1.x) : mk(w1.y, -w1.x);   // SIGN i w1
-      butterfly(a1, b1, jw, v[1], v[3]);
+      butterfly(a1, b1, turn_tw<SIGN>(w1), v[1], v[3]);
     } else {
       a0 = cadd(v[0], v[2]), a1 = csub(v[0], v[2]);
       b0 = cadd(v[1], v[3]), b1 = csub(v[1], v[3]);
@@ -144,7 +178,7 @@ __device__ __forceinline__ void stockham_pass(const cplx<T>* in, cplx<T>* out) {
     for (int r = 0; r < R; ++r) v[r] = in[j + r * (N / R)];
     const int e = (j % Ns) * (N / (Ns * R));   // twiddle exponent of input 1
     if (e != 0) Dft<T, R, SIGN>::template run<true>(v, twiddle<T, N, SIGN>(e), twiddle<T, N, SIGN>(2 * e));
-    else Dft<T, R, SIGN>::template run<false>(v, v[0], v[0]);
+    else Dft<T, R, SIGN>::template run<false>(v, {}, {});
     const int d = (j / Ns) * Ns * R + (j % Ns);
 #pragma unroll
     for (int r = 0; r < R; ++r) out[d + r * Ns] = v[r];
@@ -221,7 +255,7 @@ template <typename T, int SIGN> struct ZDft<T, 3, SIGN> {   // all zero, or the 
   static __device__ __forceinline__ void run(ZC<T>* v) {
     if (v[0].z && v[1].z && v[2].z) return;
     cplx<T> d[3] = {v[0].z ? czero<T>() : v[0].v, v[1].z ? czero<T>() : v[1].v, v[2].z ? czero<T>() : v[2].v};
-    Dft<T, 3, SIGN>::template run<false>(d, d[0], d[0]);
+    Dft<T, 3, SIGN>::template run<false>(d, {}, {});
     for (int r = 0; r < 3; ++r) v[r] = {d[r], false};
   }
 };
@@ -274,22 +308,14 @@ __device__ __forceinline__ void fft_pair_dit(cplx<T> (&a)[H], int h, unsigned ma
 #pragma unroll
     for (int k = 1; k < H; ++k) a[k] = cmul_rn(a[k], twiddle<T, 2 * H, SIGN>(k));   // W_2H^k Y_1[k]
   }
-  const T s = h ? T(-1) : T(1);
 #pragma unroll
-  for (int k = 0; k < H; ++k) {
-    const cplx<T> o = shfl_pair(a[k], mask);
-    a[k] = mk(fma_rn(s, a[k].x, o.x), fma_rn(s, a[k].y, o.y));   // X[k] = Y0 + W Y1,  X[k + H] = Y0 - W Y1
-  }
+  for (int k = 0; k < H; ++k) a[k] = addsub(h, a[k], shfl_pair(a[k], mask));   // X[k] = Y0 + W Y1,  X[k + H] = Y0 - W Y1
 }
 
 template <typename T, int H, int SIGN>
 __device__ __forceinline__ void fft_pair_dif(cplx<T> (&a)[H], int h, unsigned mask) {
-  const T s = h ? T(-1) : T(1);
 #pragma unroll
-  for (int j = 0; j < H; ++j) {            // x[j] + x[j + H], or x[j] - x[j + H]
-    const cplx<T> o = shfl_pair(a[j], mask);
-    a[j] = mk(fma_rn(s, a[j].x, o.x), fma_rn(s, a[j].y, o.y));
-  }
+  for (int j = 0; j < H; ++j) a[j] = addsub(h, a[j], shfl_pair(a[j], mask));   // x[j] + x[j + H], or x[j] - x[j + H]
   if (h) {
 #pragma unroll
     for (int j = 1; j < H; ++j) a[j] = cmul_rn(a[j], twiddle<T, 2 * H, SIGN>(j));

@@ -51,15 +51,18 @@ __device__ __forceinline__ void mbar_expect(uint64_t* bar, uint32_t bytes) {
 // ---- launch shape ------------------------------------------------------------------------
 // P lanes per line and SL line slots for a side, type and mode.  A lane holds W/P points; two
 // lanes where one would not keep a line in registers beside its temporaries (W >= 36 in FP32,
-// W >= 32 in FP64) or beside the density's column (W = 32).
+// W >= 24 in FP64) or beside the density's column (W = 32).
 template <typename T, int W, int MODE> struct PlaneCfg {
   static constexpr bool f64 = sizeof(T) == 8;
-  static constexpr int P = (W >= 36 || (W >= 32 && (f64 || MODE == XY_PASS1_DENS))) ? 2 : 1;
+  static constexpr int P = (W >= 36 || (W >= 24 && f64) || (W >= 32 && MODE == XY_PASS1_DENS)) ? 2 : 1;
   static constexpr int SL = W == 48 ? (f64 ? 1 : 2) : W == 36 ? 2 : W == 32 ? (P == 2 ? 2 : 4) : W == 24 ? (f64 ? 4 : 8) : 8;
   static constexpr int H = W / P, TH = SL * W * P;
-  static constexpr bool acc_reg = MODE == XY_PASS1_DENS && !f64;   // density column in registers, else in shared memory
-  static constexpr int regs = (2 * H * (f64 ? 2 : 1) + (acc_reg ? 2 * H : 0) + 52 + 7) / 8 * 8;
-  static constexpr int min_ctas = 65536 / ((TH + 31) / 32 * 32 * regs) < 1 ? 1 : 65536 / ((TH + 31) / 32 * 32 * regs);
+  static constexpr bool acc_reg = MODE == XY_PASS1_DENS && !f64;   // density column in registers (FP64: in shared memory)
+  // CTAs per SM that the registers allow, a scheduler's quarter of them (512 per thread of a warp) shared by whole warps
+  static constexpr int regs = (f64 ? 4 * H + 96 : 2 * H + (acc_reg ? 2 * H : 0) + 52) + 7;
+  static constexpr int warps = (TH + 31) / 32;
+  static constexpr int ctas = f64 ? 4 * (512 / (regs / 8 * 8)) / warps : 65536 / (warps * 32 * (regs / 8 * 8));
+  static constexpr int min_ctas = ctas < 1 ? 1 : ctas;
 };
 
 // Dynamic shared memory: Cs [2][SL][cb_ncol], Us [SL][W][W] (modes with u), Ys [SL][nrow][W + 1],
@@ -92,7 +95,7 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
   cplx<T>* Us = Cs + 2 * SL * cb;
   cplx<T>* Ys = Us + (HAS_U ? SL * WW : 0);
   cplx<T>* Pb = Ys + SL * s.nrow_max * NP;
-  cplx<T>* Pl = Pb + (MODE == XY_PASS1_DENS ? (C::acc_reg ? 1 : SL) * WW : 0);
+  cplx<T>* Pl = Pb + (MODE == XY_PASS1_DENS ? WW : 0);
   T* Pv = reinterpret_cast<T*>(Pl);
   const int t = threadIdx.x;
   if (t == 0) {
@@ -107,8 +110,6 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
   } else {
     for (int i = t; i < WW; i += TH) Pv[i] = vloc[(long)iz * WW + i];
   }
-  if (MODE == XY_PASS1_DENS && !C::acc_reg)
-    for (int i = t; i < SL * WW; i += TH) Pb[i] = czero<T>();
   __syncthreads();
 
   const int o_begin = a.o_off + g * a.per_group;
@@ -162,9 +163,9 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
     }
   };
   if (nbat > 0) tables(o_begin);
-  cplx<T> acc[C::acc_reg ? H : 1];
+  cplx<T> acc[MODE == XY_PASS1_DENS ? H : 1];
 #pragma unroll
-  for (int i = 0; i < (C::acc_reg ? H : 1); ++i) acc[i] = czero<T>();
+  for (int i = 0; i < (MODE == XY_PASS1_DENS ? H : 1); ++i) acc[i] = czero<T>();
   // signed index of point i of this lane: m(i) = (p <= PR ? p : p - W) at h = 0, + h
   auto m_of = [](int i) constexpr { return P == 1 ? (i <= LO ? i : i - W) : (i <= LO ? 2 * i : 2 * i - W); };
   auto kept = [](int i) constexpr { return i <= LO || i >= H - HI; };
@@ -216,23 +217,11 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
         }
         line_inv<T, W, P, LO, HI>(l, h, pmask);
         if (MODE == XY_PASS1_DENS && dens_orb(ob + ls)) {
-          if constexpr (C::acc_reg) {
 #pragma unroll
-            for (int i = 0; i < H; ++i) {
-              const cplx<T> x = u[i * W];
-              acc[i].x = fma_rn(x.y, l[i].y, fma_rn(x.x, l[i].x, acc[i].x));
-              acc[i].y = fma_rn(-x.y, l[i].x, fma_rn(x.x, l[i].y, acc[i].y));
-            }
-          } else {
-            cplx<T>* pb = Pb + ls * WW + H * h * W + j1;
-#pragma unroll
-            for (int i = 0; i < H; ++i) {
-              const cplx<T> x = u[i * W];
-              cplx<T> q = pb[i * W];
-              q.x = fma_rn(x.y, l[i].y, fma_rn(x.x, l[i].x, q.x));
-              q.y = fma_rn(-x.y, l[i].x, fma_rn(x.x, l[i].y, q.y));
-              pb[i * W] = q;
-            }
+          for (int i = 0; i < H; ++i) {
+            const cplx<T> x = u[i * W];
+            acc[i].x = fma_rn(x.y, l[i].y, fma_rn(x.x, l[i].x, acc[i].x));
+            acc[i].y = fma_rn(-x.y, l[i].x, fma_rn(x.x, l[i].y, acc[i].y));
           }
         }
 #pragma unroll
@@ -282,24 +271,17 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
   if (bad && t == 0 && err) flag_error(err, DEV_TIMEOUT, 1);
   if (MODE == XY_PASS1_DENS) {   // the slots summed in order
     __syncthreads();
-    if constexpr (C::acc_reg) {
-      for (int q = 0; q < SL; ++q) {
-        if (ls == q) {
+    for (int q = 0; q < SL; ++q) {
+      if (ls == q) {
 #pragma unroll
-          for (int i = 0; i < H; ++i) {
-            cplx<T>* p = Pb + (H * h + i) * W + j1;
-            *p = q == 0 ? acc[i] : *p + acc[i];
-          }
+        for (int i = 0; i < H; ++i) {
+          cplx<T>* p = Pb + (H * h + i) * W + j1;
+          *p = q == 0 ? acc[i] : *p + acc[i];
         }
-        __syncthreads();
       }
+      __syncthreads();
     }
-    for (int i = t; i < WW; i += TH) {
-      cplx<T> v = Pb[i];
-      if (!C::acc_reg)
-        for (int q = 1; q < SL; ++q) v = v + Pb[q * WW + i];
-      nprt[((long)g * W + iz) * WW + i] = v;
-    }
+    for (int i = t; i < WW; i += TH) nprt[((long)g * W + iz) * WW + i] = Pb[i];
   }
   if (t < SL) bulk_wait();   // the stores leave shared memory before the CTA does
 }
