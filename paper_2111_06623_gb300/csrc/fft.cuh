@@ -336,4 +336,31 @@ __device__ __forceinline__ void line_fwd(cplx<T> (&a)[W / P], int h, unsigned ma
   else fft_pair_dif<T, W / 2, -1>(a, h, mask);
 }
 
+// ---- FP64 lines in fixed point (fixed.cuh) ------------------------------------------------------
+__device__ __forceinline__ long long fx_raw(double a) { return __double_as_longlong(a); }
+__device__ __forceinline__ cplx<fx64> fx_raw(cplx<double> a) { return mk(fx64(fx_raw(a.x)), fx64(fx_raw(a.y))); }
+__device__ __forceinline__ cplx<double> fx_value(cplx<fx64> a, int e) {
+  return mk(__longlong_as_double(fx_bits(a.x.v, e)), __longlong_as_double(fx_bits(a.y.v, e)));
+}
+
+// One whole line per thread, doubles in and out: the transform itself (FP32), or through fixed point
+// (FP64).  Points are zero outside i <= LO, i >= N - HI.
+template <typename T, int N, int SIGN, int LO = N, int HI = N>
+__device__ __forceinline__ void line_transform(cplx<T> (&a)[N]) {
+  if constexpr (sizeof(T) == 8) {
+    constexpr int G = fx_growth(N);
+    cplx<fx64> l[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) l[i] = fx_raw(a[i]);
+    const int E = fx_line_exp<1>(l, 0u);
+    fx_line_from<8 - G>(l, E);
+    fft_line_in<fx64, N, SIGN, LO, HI>(l);
+    const int e = fx_exp(E, 8 - G);
+#pragma unroll
+    for (int i = 0; i < N; ++i) a[i] = fx_value(l[i], e);
+  } else {
+    fft_line_in<T, N, SIGN, LO, HI>(a);
+  }
+}
+
 }  // namespace ll

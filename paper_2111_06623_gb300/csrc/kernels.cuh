@@ -64,8 +64,8 @@ __global__ void __launch_bounds__(128) k_zinv(SphereDev s, const cplx<T>* __rest
         if ((unsigned)i < (unsigned)cl.w && LL_INB(st >= 0 && st + i < s.npw_pad)) a[p] = src[i];
       }
     }
-    if constexpr (PR > 0) fft_line_in<T, N, +1, PR, PR>(a);
-    else fft_line<T, N, +1>(a);
+    if constexpr (PR > 0) line_transform<T, N, +1, PR, PR>(a);
+    else line_transform<T, N, +1>(a);
     if (!LL_INB(c < cb_ncol)) continue;
     cplx<T>* dst = cbuf + o * (long)N * cb_ncol + c;
 #pragma unroll
@@ -1046,7 +1046,7 @@ __global__ void __launch_bounds__(kLines) k_zfwd(SphereDev s, int nbnd, const cp
   const cplx<T>* x = xin + o * npw_pad + st;
   const T* kn = kin + (long)k * npw_pad + st;
   cplx<T>* t = xout + o * npw_pad + st;
-  fft_line<T, N, -1>(a);
+  line_transform<T, N, -1>(a);
   const T scale = T(1) / T(N * N * N);
 #pragma unroll
   for (int p = 0; p < N; ++p)

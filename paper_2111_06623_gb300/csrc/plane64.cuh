@@ -21,10 +21,57 @@
 
 namespace ll {
 
-__device__ __forceinline__ long long fx_raw(double a) { return __double_as_longlong(a); }
-__device__ __forceinline__ cplx<fx64> fx_raw(cplx<double> a) { return mk(fx64(fx_raw(a.x)), fx64(fx_raw(a.y))); }
-__device__ __forceinline__ cplx<double> fx_value(cplx<fx64> a, int e) {
-  return mk(__longlong_as_double(fx_bits(a.x.v, e)), __longlong_as_double(fx_bits(a.y.v, e)));
+// A line of 2H points on a lane pair (h: the lane).  In grid order lane h holds the points
+// Q h + (0 .. Q-1) and those H further on (Q = H/2), so that each lane computes Q of the H twiddled
+// butterflies and exchanges Q values with its partner (fft_pair_dit's lanes hold a half each: lane
+// 1 multiplies all H values while lane 0 waits, and all H are exchanged).  In sphere order lane h
+// holds the points 2 i + h.  The twiddle of butterfly Q h + k is W^k, turned by +-i at h = 1.
+template <int SIGN>
+__device__ __forceinline__ cplx<fx64> fx_turn(cplx<fx64> a, int h) {   // h: times SIGN i
+  if (SIGN > 0) return mk(h ? -a.y : a.x, h ? a.x : a.y);
+  return mk(h ? a.y : a.x, h ? -a.x : a.y);
+}
+template <int SIGN> __device__ __forceinline__ FxTw fx_turn(FxTw w, int h) {
+  const FxTw r = turn_tw<SIGN>(w);
+  return FxTw{h ? r.xh : w.xh, h ? r.xl : w.xl, h ? r.yh : w.yh, h ? r.yl : w.yl, h ? r.nh : w.nh, h ? r.nl : w.nl};
+}
+__device__ __forceinline__ cplx<fx64> fx_sel(int h, cplx<fx64> a, cplx<fx64> b) {   // h ? a : b
+  return mk(h ? a.x : b.x, h ? a.y : b.y);
+}
+template <int W, int P, int LO, int HI>
+__device__ __forceinline__ void fx_line_inv(cplx<fx64> (&l)[W / P], int h, unsigned mask) {
+  if constexpr (P == 1) {
+    fft_line_in<fx64, W, +1, LO, HI>(l);
+  } else {
+    constexpr int H = W / 2, Q = H / 2;
+    static_assert(H % 2 == 0, "half lines of an even length");
+    fft_line_in<fx64, H, +1, LO, HI>(l);   // Y_h
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+      const cplx<fx64> r = shfl_pair(fx_sel(h, l[k], l[k + Q]), mask);
+      const cplx<fx64> y0 = fx_sel(h, r, l[k]), y1 = fx_sel(h, l[k + Q], r);
+      const cplx<fx64> p = k == 0 ? fx_turn<+1>(y1, h) : cmul_rn(y1, fx_turn<+1>(twiddle<fx64, W, +1>(k), h));
+      l[k] = cadd(y0, p);
+      l[k + Q] = csub(y0, p);
+    }
+  }
+}
+template <int W, int P>
+__device__ __forceinline__ void fx_line_fwd(cplx<fx64> (&l)[W / P], int h, unsigned mask) {
+  if constexpr (P == 1) {
+    fft_line<fx64, W, -1>(l);
+  } else {
+    constexpr int H = W / 2, Q = H / 2;
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+      const cplx<fx64> a = cadd(l[k], l[k + Q]), b = csub(l[k], l[k + Q]);
+      const cplx<fx64> d = k == 0 ? fx_turn<-1>(b, h) : cmul_rn(b, fx_turn<-1>(twiddle<fx64, W, -1>(k), h));
+      const cplx<fx64> r = shfl_pair(fx_sel(h, a, d), mask);
+      l[k] = fx_sel(h, r, a);
+      l[k + Q] = fx_sel(h, d, r);
+    }
+    fft_line<fx64, H, -1>(l);              // even (h = 0) or odd (h = 1) outputs
+  }
 }
 
 template <int W, int MODE, int PR>
@@ -134,6 +181,9 @@ __global__ void __launch_bounds__(PlaneCfg<double, W, MODE>::TH, PlaneCfg<double
     }
   };
   if (nbat > 0) tables(o_begin);
+  // grid point i of this lane: hb + pos(i)
+  auto pos = [](int i) constexpr { return P == 1 || i < H / 2 ? i : i + H / 2; };
+  const int hb = P == 1 ? 0 : H / 2 * h;
   bool bad = false;
 
   for (int it = 0; it < nbat; ++it) {
@@ -180,45 +230,46 @@ __global__ void __launch_bounds__(PlaneCfg<double, W, MODE>::TH, PlaneCfg<double
           }
           e += G;
         } else if (ph == 1) {                       // v'(r) u(r)
-          const cplx<T>* u = Us + ls * WW + H * h * W + j1;
+          const cplx<T>* u = Us + ls * WW + hb * W + j1;
 #pragma unroll
-          for (int i = 0; i < H; ++i) l[i] = fx_raw(u[i * W]);
+          for (int i = 0; i < H; ++i) l[i] = fx_raw(u[pos(i) * W]);
           e = fx_line_exp<P>(l, pmask);
           fx_line_from<8>(l, e);
           e = fx_exp(e, 8) + ev;
-          const int4* pl = reinterpret_cast<const int4*>(Pv) + H * h * W + j1;
+          const int4* pl = reinterpret_cast<const int4*>(Pv) + hb * W + j1;
 #pragma unroll
           for (int i = 0; i < H; ++i) {
-            const int4 w = pl[i * W];
+            const int4 w = pl[pos(i) * W];
             l[i] = cmul_rn(l[i], FxTw{w.x, w.y, w.z, w.w, -w.z, -w.w});
           }
         } else {                                    // the lines brought to one exponent
-          const int* el = s_el + rb * W + H * h;
+          const int* el = s_el + rb * W + hb;
           e = -(1 << 30);
 #pragma unroll
-          for (int i = 0; i < H; ++i) e = max(e, el[i]);
+          for (int i = 0; i < H; ++i) e = max(e, el[pos(i)]);
           if (P == 2) e = max(e, __shfl_xor_sync(pmask, e, 1));
 #pragma unroll
-          for (int i = 0; i < H; ++i) l[i] = fx_down(ysr[H * h + i], min(e - el[i] + G, 63));
+          for (int i = 0; i < H; ++i) l[i] = fx_down(ysr[hb + pos(i)], min(e - el[pos(i)] + G, 63));
           e += G;
         }
-        if (MODE != XY_PASS2 && ph < 2) line_inv<fx64, W, P, LO, HI>(l, h, pmask);
+        if (MODE != XY_PASS2 && ph < 2) fx_line_inv<W, P, LO, HI>(l, h, pmask);
         if (ph == 1 && MODE != XY_PASS2) {
           if (MODE == XY_PASS1_DENS && dens_orb(ob + ls)) {
-            cplx<T>* pb = Pb + ls * WW + H * h * W + j1;
-            const cplx<T>* u = Us + ls * WW + H * h * W + j1;
+            cplx<T>* pb = Pb + ls * WW + hb * W + j1;
+            const cplx<T>* u = Us + ls * WW + hb * W + j1;
 #pragma unroll
             for (int i = 0; i < H; ++i) {
-              const cplx<T> x = u[i * W], r = fx_value(l[i], e);
-              cplx<T> q = pb[i * W];
+              const cplx<T> x = u[pos(i) * W], r = fx_value(l[i], e);
+              cplx<T> q = pb[pos(i) * W];
               q.x = fma_rn(x.y, r.y, fma_rn(x.x, r.x, q.x));
               q.y = fma_rn(-x.y, r.x, fma_rn(x.x, r.y, q.y));
-              pb[i * W] = q;
+              pb[pos(i) * W] = q;
             }
           }
+          const int2* pv = Pv + hb * W + j1;
 #pragma unroll
           for (int i = 0; i < H; ++i) {
-            const int2 w = Pv[(H * h + i) * W + j1];
+            const int2 w = pv[pos(i) * W];
             l[i] = mk(fx_mul(l[i].x, w.x, w.y), fx_mul(l[i].y, w.x, w.y));
           }
           e += ev;
@@ -234,10 +285,10 @@ __global__ void __launch_bounds__(PlaneCfg<double, W, MODE>::TH, PlaneCfg<double
           }
           if (h == 0) (ph == 0 ? s_er : s_el)[pr] = e;
         }
-        if (ph > 0) line_fwd<fx64, W, P>(l, h, pmask);
+        if (ph > 0) fx_line_fwd<W, P>(l, h, pmask);
         if (ph == 0) {
 #pragma unroll
-          for (int i = 0; i < H; ++i) ysr[H * h + i] = l[i];
+          for (int i = 0; i < H; ++i) ysr[hb + pos(i)] = l[i];
         } else if (ph == 1) {
 #pragma unroll
           for (int i = 0; i < H; ++i)
