@@ -98,11 +98,6 @@ template <typename T> __device__ __forceinline__ void butterfly(cplx<T> a, cplx<
   d = mk(fma_rn(T(2), a.x, -s.x), fma_rn(T(2), a.y, -s.y));
 }
 
-// o + a, or o - a where h
-template <typename T> __device__ __forceinline__ cplx<T> addsub(int h, cplx<T> a, cplx<T> o) {
-  const T s = h ? T(-1) : T(1);
-  return mk(fma_rn(s, a.x, o.x), fma_rn(s, a.y, o.y));
-}
 // the rest of a three-point DFT from a and sum, dif = b +- c
 template <int SIGN, typename T> __device__ __forceinline__ void third(cplx<T> a, cplx<T> sum, cplx<T> dif, cplx<T>* v) {
   // W_3 = -1/2 + SIGN i sqrt(3)/2
@@ -308,14 +303,22 @@ __device__ __forceinline__ void fft_pair_dit(cplx<T> (&a)[H], int h, unsigned ma
 #pragma unroll
     for (int k = 1; k < H; ++k) a[k] = cmul_rn(a[k], twiddle<T, 2 * H, SIGN>(k));   // W_2H^k Y_1[k]
   }
+  const T s = h ? T(-1) : T(1);
 #pragma unroll
-  for (int k = 0; k < H; ++k) a[k] = addsub(h, a[k], shfl_pair(a[k], mask));   // X[k] = Y0 + W Y1,  X[k + H] = Y0 - W Y1
+  for (int k = 0; k < H; ++k) {
+    const cplx<T> o = shfl_pair(a[k], mask);
+    a[k] = mk(fma_rn(s, a[k].x, o.x), fma_rn(s, a[k].y, o.y));   // X[k] = Y0 + W Y1,  X[k + H] = Y0 - W Y1
+  }
 }
 
 template <typename T, int H, int SIGN>
 __device__ __forceinline__ void fft_pair_dif(cplx<T> (&a)[H], int h, unsigned mask) {
+  const T s = h ? T(-1) : T(1);
 #pragma unroll
-  for (int j = 0; j < H; ++j) a[j] = addsub(h, a[j], shfl_pair(a[j], mask));   // x[j] + x[j + H], or x[j] - x[j + H]
+  for (int j = 0; j < H; ++j) {            // x[j] + x[j + H], or x[j] - x[j + H]
+    const cplx<T> o = shfl_pair(a[j], mask);
+    a[j] = mk(fma_rn(s, a[j].x, o.x), fma_rn(s, a[j].y, o.y));
+  }
   if (h) {
 #pragma unroll
     for (int j = 1; j < H; ++j) a[j] = cmul_rn(a[j], twiddle<T, 2 * H, SIGN>(j));

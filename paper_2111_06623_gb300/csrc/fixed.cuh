@@ -62,9 +62,6 @@ __host__ __device__ __forceinline__ void butterfly(cplx<fx64> a, cplx<fx64> b, F
 template <int SIGN> __host__ __device__ __forceinline__ FxTw turn_tw(FxTw w) {
   return SIGN > 0 ? FxTw{w.nh, w.nl, w.xh, w.xl, -w.xh, -w.xl} : FxTw{w.yh, w.yl, -w.xh, -w.xl, w.xh, w.xl};
 }
-__host__ __device__ __forceinline__ cplx<fx64> addsub(int h, cplx<fx64> a, cplx<fx64> o) {
-  return mk(fx64(h ? o.x.v - a.x.v : o.x.v + a.x.v), fx64(h ? o.y.v - a.y.v : o.y.v + a.y.v));
-}
 template <int SIGN> __host__ __device__ __forceinline__ void third(cplx<fx64> a, cplx<fx64> sum, cplx<fx64> dif, cplx<fx64>* v) {
   // sqrt(3)/2 in limbs
   constexpr int sh = 1859775393, sl = 815355111;

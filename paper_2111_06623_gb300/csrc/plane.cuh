@@ -14,6 +14,8 @@
 // buffers and back from it, and in the modes that read the orbital grids u(r) the plane of every
 // orbital, one batch ahead, while the rows of this batch and the next are transformed.
 //
+// FP64 chains run the same pass with fixed-point lines (plane64.cuh).
+//
 // What bounds it and why this shape (KB workload, FP32, W = 24, 2048 orbitals; the line FFTs are
 // 28 us of FMA issue, u(r) 34 us of HBM): the pass it replaces (128 threads, columns staged by
 // hand) took 94 / 135 / 87 us (pass 1 / density / pass 2): half its issue slots were index
