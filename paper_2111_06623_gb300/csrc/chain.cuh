@@ -644,6 +644,12 @@ class Chain : public ChainBase {
       // the chunked path also where the band groups are small: per-group CTAs would read the
       // projectors and U_{k+Q} once per group (32 times per k on the 16-atom cell)
       split_ = best == 0 || 4 * best < nbnd_ || (env && env[0] == '1' && env[1] == 0);
+      // fewer bands per CTA where the k-points alone leave SMs idle (the groups re-read U and B from
+      // L2, which costs less than the idle SMs): us per call, all bands -> this rule: two-atom cell
+      // (64 k-points, 4 bands, groups of 1) FP32 492 -> 471, FP64 3118 -> 3031; semimetal (6 bands, of
+      // 2) 668 -> 641; smallest cell (8 k-points, of 1) 2000 -> 1792
+      for (int b = bpc_ - 1; !split_ && b >= 1 && (long)nks_ * ngrp_ < nsm_; --b)
+        if (nbnd_ % b == 0) bpc_ = b, ngrp_ = nbnd_ / b;
       nchunk_ = split_ ? (pq + kChunk - 1) / kChunk : 1;
       npk_ = split_ ? nchunk_ : ngrp_;
       // FP32 path: the split path's dot blocks on the tensor cores (tcproj.cuh) where their
