@@ -1358,6 +1358,20 @@ __global__ void k_pad_rows(const double* __restrict__ src, const int* __restrict
     d[g] = g < n ? mk((T)(f * s[2 * g]), (T)(f * s[2 * g + 1])) : czero<T>();
 }
 
+// The padded rows of one batch vector back in the packed layout, in double.  grid (nks, nrow), block 256.
+template <typename T>
+__global__ void k_unpad_rows(const cplx<T>* __restrict__ src, const int* __restrict__ off, const int* __restrict__ npw,
+                             int nrow, int npw_pad, double* __restrict__ dst) {
+  const int k = blockIdx.x, r = blockIdx.y, n = npw[k];
+  const cplx<T>* s = src + ((long)k * nrow + r) * npw_pad;
+  double* d = dst + 2 * ((long)nrow * off[k] + (long)r * n);
+  for (int g = threadIdx.x; g < n; g += blockDim.x) {
+    const cplx<T> v = s[g];
+    d[2 * g] = (double)v.x;
+    d[2 * g + 1] = (double)v.y;
+  }
+}
+
 // A grid [j1][j2][j3] -> [j3][j2][j1] in T.
 template <typename T>
 __global__ void k_grid_in(int n, const double* __restrict__ src, T* __restrict__ dst) {

@@ -104,7 +104,7 @@ size_t footprint_bytes(const ll_system_desc* d, int side, int cols) {
   }
   const size_t ngroups = (4 * (size_t)nsm + w - 1) / w;
   // vectors: 3 nvec Lanczos vectors, nvec partial copies, y, U_{k+Q}, and the 2-vector scratch
-  // of the plane-pass tuner and ll_apply
+  // of ll_apply
   size_t b = elem * (vq * (3 * nvec + nvec + 2 + 2) + orb * pk + orb * w3 + cb + ngroups * w3 + 3 * w3 +
                      (size_t)d->nks * d->nproj * pq);
   // Lanczos partials: up to max(bands, plane-wave chunks) per k and step (band groups or the
