@@ -1547,9 +1547,12 @@ class Chain : public ChainBase {
     return LL_EUNSUPPORTED;
   }
 
-  template <typename F>
   // Opts the kernel in to `bytes` of dynamic shared memory (static shared memory counts
-  // against the same 48 KB default, so the opt-in is made whenever the sum passes it).
+  // against the same 48 KB default, so the opt-in is made whenever the sum passes it).  The limit
+  // belongs to the function on the device, not to the chain: it is raised to the largest size any
+  // chain of the process has asked for and never lowered, so that chains of other spheres (other
+  // Q, other threads) cannot take it away from one that launches later.
+  template <typename F>
   int set_smem(F* fn, size_t bytes, std::string& err) {
     const void* key = reinterpret_cast<const void*>(fn);
     for (auto& e : smem_set_)
@@ -1560,8 +1563,13 @@ class Chain : public ChainBase {
       err = "shared-memory tile exceeds 227 KB for this system";
       return LL_EUNSUPPORTED;
     }
-    if (bytes + at.sharedSizeBytes > 48 * 1024)
-      LL_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    if (bytes + at.sharedSizeBytes > 48 * 1024) {
+      static std::mutex mu;   // one per kernel type; the attribute itself is the maximum so far
+      std::lock_guard<std::mutex> lock(mu);
+      LL_CK(cudaFuncGetAttributes(&at, fn));
+      if ((size_t)at.maxDynamicSharedSizeBytes < bytes)
+        LL_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    }
     smem_set_.push_back({key, bytes});
     return LL_OK;
   }
