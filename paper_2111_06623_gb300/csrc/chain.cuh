@@ -1062,8 +1062,13 @@ class Chain : public ChainBase {
     }
     LL_CK(cudaMemcpyAsync(pk, x, packed * sizeof(double), cudaMemcpyHostToDevice, st_));
     k_pad_rows<T><<<dim3(nks_, nbnd_), 256, 0, st_>>>(pk, offq_, dq_.npw, nbnd_, hq_.npw_pad, nullptr, scratch_);
-    // a one-vector application reuses the cbuf/tbuf sized for nvec_ >= 1
-    if ((rc = op(1, scratch_, scratch_ + vq, (upper && approx_ != LL_APPROX_IPA) ? 0 : -1, err))) return rc;
+    // a one-vector application reuses the cbuf/tbuf sized for nvec_ >= 1; its norm partials go to a
+    // buffer of their own (part_ holds those of the recursion's last step, which the next one reads)
+    if (!apart_ && (rc = alloc(&apart_, (long)nks_ * npk_))) return rc;
+    std::swap(part_, apart_);
+    rc = op(1, scratch_, scratch_ + vq, (upper && approx_ != LL_APPROX_IPA) ? 0 : -1, err);
+    std::swap(part_, apart_);
+    if (rc) return rc;
     k_unpad_rows<T><<<dim3(nks_, nbnd_), 256, 0, st_>>>(scratch_ + vq, offq_, dq_.npw, nbnd_, hq_.npw_pad, pk);
     LL_CK(cudaGetLastError());
     if ((rc = oob_check(err))) return rc;
@@ -1706,6 +1711,7 @@ class Chain : public ChainBase {
   cplx<T>* scratch_ = nullptr;
   double* packed_ = nullptr;     // apply: the caller's packed vector where cbuf_ does not hold it
   int* offq_ = nullptr;          // apply: offsets of the packed k blocks
+  double* apart_ = nullptr;      // apply: norm partials
   T* rup_ = nullptr;             // W_ < N_: resampling table [N_][W_] (resample_table)
   cplx<T>* t1_ = nullptr;        // W_ < N_: n', then f_xc n', on W_ planes of the declared N_ x N_ grid
   cplx<double> *spart_ = nullptr, *gamma_ = nullptr, *z_ = nullptr, *zpart_ = nullptr, *spec_out_ = nullptr;

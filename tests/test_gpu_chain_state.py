@@ -28,3 +28,31 @@ def test_chains_of_other_spheres_take_turns(lib, precision, monkeypatch):  # noq
                 assert np.array_equal(p, q)
     for ch in chains:
         ch.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("flavour", ["ph", "nh"])
+@pytest.mark.parametrize("split", ["0", "1"])
+def test_applications_between_steps(lib, precision, flavour, split, monkeypatch):  # noqa: F811
+    """Chain.apply between Chain.lanczos calls: the coefficients are those of the recursion left
+    alone, bit for bit (graphs on, on a stream of its own, and eager), and the applications those of
+    a fresh chain."""
+    torch = pytest.importorskip("torch")
+    monkeypatch.setenv("LL_SPLIT_PERK", split)
+    d, x = _system(10.0, 18)
+    d["eps_k"] = d["eps_k"] - 30.0       # D is positive
+    kw = dict(approx="rpa", precision=precision, flavour=flavour, max_steps=12)
+    ref = lib.Chain(**kw, **d)
+    want, app = ref.lanczos(12), [ref.apply(x, up) for up in (True, False)]
+    ref.close()
+    for stream in (None, torch.cuda.Stream()):
+        ch = lib.Chain(stream=stream.cuda_stream if stream else None, **kw, **d)
+        got = []
+        for i in range(4):
+            for up, a in zip((True, False), app):
+                for p, q in zip(ch.apply(x, up), a):
+                    assert np.array_equal(p, q)
+            got = ch.lanczos(3)
+        ch.close()
+        for a, b in zip(got, want):
+            assert np.array_equal(a, b)
