@@ -41,6 +41,7 @@ def test_applications_between_steps(lib, precision, flavour, split, monkeypatch)
     monkeypatch.setenv("LL_SPLIT_PERK", split)
     d, x = _system(10.0, 18)
     d["eps_k"] = d["eps_k"] - 30.0       # D is positive
+    d["dij"] = abs(d["dij"])
     kw = dict(approx="rpa", precision=precision, flavour=flavour, max_steps=12)
     ref = lib.Chain(**kw, **d)
     want, app = ref.lanczos(12), [ref.apply(x, up) for up in (True, False)]
