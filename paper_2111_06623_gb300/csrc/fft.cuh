@@ -73,10 +73,6 @@ __device__ __forceinline__ typename TwTab<T>::type twiddle(int e) {
   const typename TwTab<T>::type w = TwTab<T>::get(TwOff<N>::v + e);
   return SIGN > 0 ? conj_tw(w) : w;
 }
-// SIGN i w
-template <int SIGN, typename T> __device__ __forceinline__ cplx<T> turn_tw(cplx<T> w) {
-  return (SIGN > 0) ? mk(-w.y, w.x) : mk(w.y, -w.x);
-}
 
 // Arithmetic with explicit rounding: what the compiler may contract is written out, so a
 // transform's result does not depend on what surrounds it (a pruned instantiation rounds as the
@@ -92,12 +88,6 @@ template <typename T> __device__ __forceinline__ cplx<T> csub(cplx<T> a, cplx<T>
 template <typename T> __device__ __forceinline__ cplx<T> cmul_rn(cplx<T> a, cplx<T> w) {
   return mk(fma_rn(a.x, w.x, mul_rn(-a.y, w.y)), fma_rn(a.x, w.y, mul_rn(a.y, w.x)));
 }
-// a + w b and a - w b in six FMAs (a complex product and two additions: eight operations)
-template <typename T> __device__ __forceinline__ void butterfly(cplx<T> a, cplx<T> b, cplx<T> w, cplx<T>& s, cplx<T>& d) {
-  s = mk(fma_rn(w.x, b.x, fma_rn(-w.y, b.y, a.x)), fma_rn(w.x, b.y, fma_rn(w.y, b.x, a.y)));
-  d = mk(fma_rn(T(2), a.x, -s.x), fma_rn(T(2), a.y, -s.y));
-}
-
 // the rest of a three-point DFT from a and sum, dif = b +- c
 template <int SIGN, typename T> __device__ __forceinline__ void third(cplx<T> a, cplx<T> sum, cplx<T> dif, cplx<T>* v) {
   // W_3 = -1/2 + SIGN i sqrt(3)/2
@@ -112,68 +102,53 @@ template <int SIGN, typename T> __device__ __forceinline__ void third(cplx<T> a,
 // R-point DFT in place with exponent sign SIGN.
 template <typename T, int R, int SIGN> struct Dft;
 
-// w1 multiplies input 1 and w1^2 input 2 (and w1^3 input 3) where TW (a twiddled pass).
 template <typename T, int SIGN> struct Dft<T, 2, SIGN> {
-  using Tw = typename TwTab<T>::type;
-  template <bool TW>
-  static __device__ __forceinline__ void run(cplx<T>* v, Tw w1, Tw) {
+  static __device__ __forceinline__ void run(cplx<T>* v) {
     const cplx<T> a = v[0], b = v[1];
-    if (TW) {
-      butterfly(a, b, w1, v[0], v[1]);
-    } else {
-      v[0] = cadd(a, b);
-      v[1] = csub(a, b);
-    }
+    v[0] = cadd(a, b);
+    v[1] = csub(a, b);
   }
 };
 
 template <typename T, int SIGN> struct Dft<T, 3, SIGN> {
-  using Tw = typename TwTab<T>::type;
-  template <bool TW>
-  static __device__ __forceinline__ void run(cplx<T>* v, Tw w1, Tw w2) {
-    const cplx<T> a = v[0];
-    cplx<T> sum, dif;
-    if (TW) butterfly(cmul_rn(v[1], w1), v[2], w2, sum, dif);
-    else sum = cadd(v[1], v[2]), dif = csub(v[1], v[2]);
+  static __device__ __forceinline__ void run(cplx<T>* v) {
+    const cplx<T> a = v[0], sum = cadd(v[1], v[2]), dif = csub(v[1], v[2]);
     v[0] = cadd(a, sum);
     third<SIGN>(a, sum, dif, v);
   }
 };
 
 template <typename T, int SIGN> struct Dft<T, 4, SIGN> {
-  using Tw = typename TwTab<T>::type;
-  template <bool TW>
-  static __device__ __forceinline__ void run(cplx<T>* v, Tw w1, Tw w2) {
-    cplx<T> a0, a1, b0, b1;
-    if (TW) {   // w1 v1 +- w3 v3 = w1 (v1 +- w2 v3): the factor w1 goes into the last butterflies
-      butterfly(v[0], v[2], w2, a0, a1);
-      butterfly(v[1], v[3], w2, b0, b1);
-      butterfly(a0, b0, w1, v[0], v[2]);
-      butterfly(a1, b1, turn_tw<SIGN>(w1), v[1], v[3]);
-    } else {
-      a0 = cadd(v[0], v[2]), a1 = csub(v[0], v[2]);
-      b0 = cadd(v[1], v[3]), b1 = csub(v[1], v[3]);
-      // SIGN i b1
-      const cplx<T> jb1 = (SIGN > 0) ? mk(-b1.y, b1.x) : mk(b1.y, -b1.x);
-      v[0] = cadd(a0, b0);
-      v[2] = csub(a0, b0);
-      v[1] = cadd(a1, jb1);
-      v[3] = csub(a1, jb1);
-    }
+  static __device__ __forceinline__ void run(cplx<T>* v) {
+    const cplx<T> a0 = cadd(v[0], v[2]), a1 = csub(v[0], v[2]);
+    const cplx<T> b0 = cadd(v[1], v[3]), b1 = csub(v[1], v[3]);
+    // SIGN i b1
+    const cplx<T> jb1 = (SIGN > 0) ? mk(-b1.y, b1.x) : mk(b1.y, -b1.x);
+    v[0] = cadd(a0, b0);
+    v[2] = csub(a0, b0);
+    v[1] = cadd(a1, jb1);
+    v[3] = csub(a1, jb1);
   }
 };
 
-// One Stockham pass of radix R after Ns points have been combined.
+// One Stockham pass of radix R after Ns points have been combined.  A twiddled input is a product
+// of its own: a butterfly that forms a + w b in FMAs and a - w b as 2 a - (a + w b) takes six
+// operations for eight, but the difference inherits the sum's rounding (FP32 transforms of 12 to
+// 48 points: errors 1.01 to 1.14 times these).
 template <typename T, int N, int R, int Ns, int SIGN>
 __device__ __forceinline__ void stockham_pass(const cplx<T>* in, cplx<T>* out) {
 #pragma unroll
   for (int j = 0; j < N / R; ++j) {
     cplx<T> v[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = in[j + r * (N / R)];
-    const int e = (j % Ns) * (N / (Ns * R));   // twiddle exponent of input 1
-    if (e != 0) Dft<T, R, SIGN>::template run<true>(v, twiddle<T, N, SIGN>(e), twiddle<T, N, SIGN>(2 * e));
-    else Dft<T, R, SIGN>::template run<false>(v, {}, {});
+    for (int r = 0; r < R; ++r) {
+      v[r] = in[j + r * (N / R)];
+      const int e = ((j % Ns) * r * (N / (Ns * R))) % N;
+      if (4 * e == N) v[r] = SIGN > 0 ? mk(-v[r].y, v[r].x) : mk(v[r].y, -v[r].x);   // SIGN i, exactly
+      else if (2 * e == N) v[r] = mk(-v[r].x, -v[r].y);
+      else if (e != 0) v[r] = cmul_rn(v[r], twiddle<T, N, SIGN>(e));
+    }
+    Dft<T, R, SIGN>::run(v);
     const int d = (j / Ns) * Ns * R + (j % Ns);
 #pragma unroll
     for (int r = 0; r < R; ++r) out[d + r * Ns] = v[r];
@@ -250,7 +225,7 @@ template <typename T, int SIGN> struct ZDft<T, 3, SIGN> {   // all zero, or the 
   static __device__ __forceinline__ void run(ZC<T>* v) {
     if (v[0].z && v[1].z && v[2].z) return;
     cplx<T> d[3] = {v[0].z ? czero<T>() : v[0].v, v[1].z ? czero<T>() : v[1].v, v[2].z ? czero<T>() : v[2].v};
-    Dft<T, 3, SIGN>::template run<false>(d, {}, {});
+    Dft<T, 3, SIGN>::run(d);
     for (int r = 0; r < 3; ++r) v[r] = {d[r], false};
   }
 };
