@@ -6,13 +6,15 @@
 // two integer instructions, a product with a twiddle three 32 x 32 -> 64 multiply-adds.
 //
 // Precision.  Every value keeps |v| <= 2^61; a transform over K inputs is entered at
-// |v| < 2^61 / (sqrt(2) K), so nothing overflows, and rounds at one unit: 2^-55 to 2^-53 of the
-// line's largest input, where FP64 rounds every operand at 2^-53 of itself.  Between transforms
-// the line is shifted back up to 2^61 and its exponent adjusted (fx_top, fx_up).
+// |v| < 2^61 / ((4/pi) K), so nothing overflows, and rounds to nearest at one unit: 2^-57 to 2^-55
+// of the line's largest input, where FP64 rounds every operand at 2^-53 of itself.  After EVERY
+// transform the line is shifted back up to 2^61 and its exponent adjusted (fx_top, fx_up): a
+// transform's outputs lie up to six bits below the headroom it was given, and a following one that
+// is entered at its own headroom would round them away.
 //
 // Inf and NaN: a line that holds one has exponent kFxBad and is NaN as a whole when it is
 // converted back, as the transform of such a line is.  Results beyond the range of a double are
-// Inf, subnormal ones 0 (inputs likewise).
+// Inf; subnormal inputs and results are kept.
 #pragma once
 #include "common.cuh"
 
@@ -28,7 +30,6 @@ __host__ __device__ __forceinline__ fx64 operator-(fx64 a) { return fx64(-a.v); 
 __host__ __device__ __forceinline__ fx64 operator+(fx64 a, fx64 b) { return fx64(a.v + b.v); }
 
 constexpr int kFxBad = 1 << 20;       // exponent of a line with an Inf or a NaN (sums stay above kFxBad / 2)
-constexpr int kFxNone = -(1 << 14);   // exponent of a line of zeros
 
 // A factor w, |w| <= 1, as w = (h + l 2^-31) 2^-31 with |l| <= 2^30 (h = 2^31 - 1, l = 2^31 - 1 for
 // w = 1).  A twiddle holds -y too: both occur in a complex product.
@@ -52,11 +53,6 @@ __host__ __device__ __forceinline__ cplx<fx64> cmul_rn(cplx<fx64> a, FxTw w) {
   const long long ti = (1LL << 30) + (long long)xh * w.yl + (long long)yh * w.xl + (long long)xl * w.yh + (long long)yl * w.xh;
   return mk(fx64((tr >> 31) + (long long)xh * w.xh + (long long)yh * w.nh),
             fx64((ti >> 31) + (long long)xh * w.yh + (long long)yh * w.xh));
-}
-__host__ __device__ __forceinline__ void butterfly(cplx<fx64> a, cplx<fx64> b, FxTw w, cplx<fx64>& s, cplx<fx64>& d) {
-  const cplx<fx64> p = cmul_rn(b, w);
-  s = mk(fx64(a.x.v + p.x.v), fx64(a.y.v + p.y.v));
-  d = mk(fx64(a.x.v - p.x.v), fx64(a.y.v - p.y.v));
 }
 // SIGN i w
 template <int SIGN> __host__ __device__ __forceinline__ FxTw turn_tw(FxTw w) {
@@ -110,23 +106,29 @@ static inline void fx_twiddle_limbs(int e, int n, int* out) {
 }
 
 // ---- doubles ------------------------------------------------------------------------------
-// A transform over k inputs is entered at |v| < 2^(61 - growth): ceil(log2(sqrt(2) k)).
+// A transform over k inputs is entered at |v| < 2^(61 - growth).  An output's real part is a sum of
+// k terms re cos - im sin: at most (4/pi) k times the largest input, the mean of |cos| + |sin| over
+// equally spaced angles with 0 among them being at most 4/pi (a trapezoid rule on a concave
+// function).  What lies between (a twiddled transform over a half or a third of the inputs, up to
+// two of its terms) stays below sqrt(2) (2/3) k.  ceil(log2 (4/pi) k), with 4% to spare for the
+// roundings at every side.
 __host__ __device__ constexpr int fx_growth(int k) {
   int g = 1;
-  while ((1L << (2 * g)) < 2L * k * k) ++g;
+  while ((1L << g) * 10000 < 12733L * k) ++g;
   return g;
 }
 __host__ __device__ __forceinline__ int fx_hiword(long long bits) { return (int)(bits >> 32); }
-// sign and fraction of the double `bits` as an integer below 2^(53 + s0) in a line whose largest
-// biased exponent is E (subnormals: 0); the line's exponent is fx_exp(E, s0)
+// sign and fraction of the double `bits` as an integer below 2^(53 + s0), rounded to nearest, in a
+// line whose largest biased exponent is E >= 1 (subnormals have exponent 1 and no leading bit);
+// the line's exponent is fx_exp(E, s0)
 __host__ __device__ __forceinline__ long long fx_from(long long bits, int E, int s0) {
   const int ex = (int)(bits >> 52) & 0x7ff;
-  long long m = ((bits & 0xfffffffffffffLL) | (1LL << 52)) << s0;
-  const int sh = E - ex;
-  m = (ex == 0 || sh > 63) ? 0 : m >> sh;
-  return bits < 0 ? -m : m;
+  const long long m = ((bits & 0xfffffffffffffLL) | ((long long)(ex > 0) << 52)) << s0;
+  const int sh = E - (ex > 1 ? ex : 1);
+  const long long r = sh > 62 ? 0 : (m + ((1LL << sh) >> 1)) >> sh;
+  return bits < 0 ? -r : r;
 }
-__host__ __device__ __forceinline__ int fx_exp(int E, int s0) { return E == 0x7ff ? kFxBad : (E == 0 ? kFxNone : E - 1075 - s0); }
+__host__ __device__ __forceinline__ int fx_exp(int E, int s0) { return E == 0x7ff ? kFxBad : E - 1075 - s0; }
 // v 2^e as a double, rounded to nearest (a tie away from zero)
 __host__ __device__ __forceinline__ long long fx_bits(long long v, int e) {
   if (e > kFxBad / 2) return 0x7ff8000000000000LL;
@@ -138,26 +140,27 @@ __host__ __device__ __forceinline__ long long fx_bits(long long v, int e) {
 #endif
   const int be = 63 + 1023 + e - lz;   // biased exponent of the leading bit
   const unsigned long long n = u << (lz & 63);
-  const unsigned long long m = (n >> 11) + ((n >> 10) & 1);
-  long long r = ((long long)(be - 1) << 52) + (long long)m;
+  const int sh = 11 + (be < 1 ? 1 - be : 0);   // a subnormal result keeps fewer bits
+  const unsigned long long m = (sh < 64 ? n >> sh : 0) + (sh < 65 ? (n >> (sh - 1)) & 1 : 0);
+  long long r = ((long long)(be < 1 ? 0 : be - 1) << 52) + (long long)m;
   if (be > 2046) r = 0x7ff0000000000000LL;
-  if (be < 1 || u == 0) r = 0;
+  if (u == 0) r = 0;
   return v < 0 ? (r | (long long)0x8000000000000000ull) : r;
 }
 // limbs of a factor: the double as a fraction below 1/2 of 2^e, e = fx_coef_exp(E) (E: the largest
 // biased exponent among the factors)
 __host__ __device__ __forceinline__ void fx_coef(long long bits, int E, int& h, int& l) { fx_limbs(fx_from(bits, E, 8), h, l); }
-__host__ __device__ __forceinline__ int fx_coef_exp(int E) { return fx_exp(E, 8) + (E == 0 ? 0 : 62); }
+__host__ __device__ __forceinline__ int fx_coef_exp(int E) { return fx_exp(E, 8) + 62; }
 
 // ---- a line in registers: H points of this lane, P lanes (mask: the pair) --------------------
-// The largest biased exponent of a line that holds doubles' bits.
+// The largest biased exponent of a line that holds doubles' bits (at least 1).
 template <int P, int H>
 __device__ __forceinline__ int fx_line_exp(const cplx<fx64> (&l)[H], unsigned mask) {
   int m = 0;
 #pragma unroll
   for (int i = 0; i < H; ++i) m = max(m, max(fx_hiword(l[i].x.v) & 0x7fffffff, fx_hiword(l[i].y.v) & 0x7fffffff));
   if (P == 2) m = max(m, __shfl_xor_sync(mask, m, 1));
-  return m >> 20;
+  return max(m >> 20, 1);
 }
 // doubles' bits -> fixed point at 2^(53 + S0)
 template <int S0, int H>

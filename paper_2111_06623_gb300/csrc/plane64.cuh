@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(PlaneCfg<double, W, MODE>::TH, PlaneCfg<double
     for (int i = t; i < n; i += TH) ev = max(ev, fx_hiword(fx_raw(src[i])) & 0x7fffffff);
     atomicMax(&s_ev, ev);
     __syncthreads();
-    ev = s_ev >> 20;
+    ev = max(s_ev >> 20, 1);
     for (int i = t; i < n; i += TH) {
       int2 w;
       fx_coef(fx_raw(src[i]), ev, w.x, w.y);
@@ -284,9 +284,14 @@ __global__ void __launch_bounds__(PlaneCfg<double, W, MODE>::TH, PlaneCfg<double
             fx_up<G>(l, c);
             e += G;
           }
-          if (h == 0) (ph == 0 ? s_er : s_el)[pr] = e;
+          if (ph == 0 && h == 0) s_er[pr] = e;
         }
         if (ph > 0) fx_line_fwd<W, P>(l, h, pmask);
+        if (ph == 1) {   // the rows' transform reads the line at its own headroom: up again first
+          const int c = fx_top<P>(l, pmask);
+          fx_up<0>(l, c);
+          if (h == 0) s_el[pr] = e - c;
+        }
         if (ph == 0) {
 #pragma unroll
           for (int i = 0; i < H; ++i) ysr[hb + pos(i)] = l[i];
