@@ -1491,16 +1491,52 @@ __device__ __forceinline__ double pow2_scale(double a, double b, double c, doubl
   return (e == 0 || e >= 0x7fe00000) ? 1.0 : __hiloint2double(0x7fe00000 - e, 0);
 }
 
+// Double-double values h + l, |l| <= ulp(h)/2 (Dekker 1971; Knuth's two-sum), and their complex
+// products, for the matrix power below.
+struct dd { double h, l; };
+__device__ __forceinline__ dd dd_norm(double h, double l) {   // |h| >= |l|
+  const double s = __dadd_rn(h, l);
+  return {s, __dadd_rn(l, -__dadd_rn(s, -h))};
+}
+__device__ __forceinline__ dd dd_prod(double a, double b) {
+  const double p = __dmul_rn(a, b);
+  return {p, __fma_rn(a, b, -p)};
+}
+__device__ __forceinline__ dd operator+(dd a, dd b) {
+  const double s = __dadd_rn(a.h, b.h), t = __dadd_rn(s, -a.h);
+  const double e = __dadd_rn(__dadd_rn(a.h, -__dadd_rn(s, -t)), __dadd_rn(b.h, -t));
+  return dd_norm(s, __dadd_rn(e, __dadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ dd operator-(dd a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ dd operator-(dd a, dd b) { return a + -b; }
+__device__ __forceinline__ dd operator*(dd a, dd b) {
+  const dd p = dd_prod(a.h, b.h);
+  return dd_norm(p.h, __fma_rn(a.h, b.l, __fma_rn(a.l, b.h, p.l)));
+}
+__device__ __forceinline__ cplx<dd> operator*(cplx<dd> a, cplx<dd> b) { return mk(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
+__device__ __forceinline__ cplx<dd> dd_sqr(cplx<dd> a) {
+  const dd t = a.x * a.y;
+  return mk(a.x * a.x - a.y * a.y, dd{2.0 * t.h, 2.0 * t.l});
+}
+__device__ __forceinline__ cplx<double> dd_hi(cplx<dd> a) { return mk(a.x.h, a.y.h); }
+__device__ __forceinline__ cplx<dd> dd_scale(cplx<dd> a, double s) {   // s a power of two
+  return mk(dd{a.x.h * s, a.x.l * s}, dd{a.y.h * s, a.y.l * s});
+}
+
 // The elimination without its divisions: with d_j = P_j / P_{j+1} and r_j = R_j / P_{j+1},
 //   P_j = w P_{j+1} - beta_{j+1} gamma_{j+1} P_{j+2},   R_j = z_j P_{j+1} + beta_{j+1} R_{j+1},
 // u_1 = R_1 / P_1; P, P_{j+1} and R are scaled together by an exact power of two every fourth
 // row.  m_total > m continues the chain with `tail` (T grows to m_total x m_total; z stays m
 // long): there R = 0 and the rows repeat with period two, so the whole tail is the
-// floor((m_total - m)/2)-th power of one 2 x 2 matrix, formed by repeated squaring.
+// floor((m_total - m)/2)-th power of one 2 x 2 matrix, formed by repeated squaring.  A squaring
+// doubles the relative error of its argument, so the k-th power would carry k roundings where
+// the rows carry about sqrt(k): the squarings run in double-double, the power is applied in double.
 // Bound by the FP64 pipe (one warp instruction per 16 cycles and SM): 14 FP64 instructions per row
 // against about 70 with two complex divisions; one warp per CTA puts 4001 frequencies on 126 SMs
-// where 128-thread CTAs used 32.  Errors as the division form's (both within 1e-14 on 1000
-// coefficients continued to 20000 at eta = 0.1 eV).  Block 32.
+// where 128-thread CTAs used 32.  1000 coefficients continued to 20000 at 4001 frequencies, us per
+// call: divisions 68900, this form 740 with every squaring in double, 850 with double-double.  Errors
+// against extended precision, divisions / double squarings / this form: 8.6e-15 / 2.1e-15 / 1e-15
+// there; 60 coefficients continued to 400 2.0e-14 / 3.0e-14 / 2.1e-15.  Block 32.
 static __global__ void __launch_bounds__(32) k_spectrum(int m, int m_total, const ExtrapTail* __restrict__ tail,
                                                         const double* __restrict__ beta,
                                                         const cplx<double>* __restrict__ gamma,
@@ -1523,23 +1559,24 @@ static __global__ void __launch_bounds__(32) k_spectrum(int m, int m_total, cons
       P = t;
     }
     // one period: [[w, -ca], [1, 0]] [[w, -cb], [1, 0]]
-    cplx<double> a = cmul(w, w) - ca, b = mk(-(cb.x * w.x - cb.y * w.y), -(cb.x * w.y + cb.y * w.x)), c = w,
-                 d = mk(-cb.x, -cb.y);
+    const cplx<dd> wd = mk(dd{w.x, 0.0}, dd{w.y, 0.0}), cad = mk(dd_prod(tail->g[pa].x, tail->b[pa]), dd_prod(tail->g[pa].y, tail->b[pa])),
+                   cbd = mk(dd_prod(-tail->g[pb].x, tail->b[pb]), dd_prod(-tail->g[pb].y, tail->b[pb]));
+    cplx<dd> a = dd_sqr(wd) - cad, b = cbd * wd, c = wd, d = cbd;
     for (int h = nt >> 1; h; h >>= 1) {
       if (h & 1) {
-        const cplx<double> t = cmul(a, P) + cmul(b, P1), u = cmul(c, P) + cmul(d, P1);
+        const cplx<double> t = cmul(dd_hi(a), P) + cmul(dd_hi(b), P1), u = cmul(dd_hi(c), P) + cmul(dd_hi(d), P1);
         const double s = pow2_scale(t.x, t.y, u.x, u.y);
         P = t * s;
         P1 = u * s;
       }
       if (h == 1) break;
-      const cplx<double> bc = cmul(b, c), tr = a + d;
-      const cplx<double> na = cmul(a, a) + bc, nd = cmul(d, d) + bc, nb = cmul(b, tr), nc = cmul(c, tr);
-      const double s = fmin(pow2_scale(na.x, na.y, nb.x, nb.y), pow2_scale(nc.x, nc.y, nd.x, nd.y));
-      a = na * s;
-      b = nb * s;
-      c = nc * s;
-      d = nd * s;
+      const cplx<dd> bc = b * c, tr = a + d;
+      const cplx<dd> na = dd_sqr(a) + bc, nd = dd_sqr(d) + bc, nb = b * tr, nc = c * tr;
+      const double s = fmin(pow2_scale(na.x.h, na.y.h, nb.x.h, nb.y.h), pow2_scale(nc.x.h, nc.y.h, nd.x.h, nd.y.h));
+      a = dd_scale(na, s);
+      b = dd_scale(nb, s);
+      c = dd_scale(nc, s);
+      d = dd_scale(nd, s);
     }
   }
   cplx<double> R = cmul(z[m - 1], P1);
