@@ -349,6 +349,30 @@ int ll_server_set_chunk(ll_server* s, int steps) {
   return LL_OK;
 }
 
+// ll_footprint's bound with the columns of the descriptor's spheres and the side of their grid
+static size_t spheres_footprint(const ll_system_desc* d) {
+  std::vector<ll::Extent> e[2];
+  int cols = 1;
+  for (int f = 0; f < 2; ++f) {
+    const int* m = f ? d->miller_kq : d->miller_k;
+    for (int k = 0; k < d->nks; ++k) {
+      const int np = (f ? d->npw_kq : d->npw_k)[k];
+      ll::Extent x{{m[0], m[1], m[2]}, {m[0], m[1], m[2]}};
+      int nc = 1;
+      for (int i = 0; i < np; ++i, m += 3) {
+        nc += i > 0 && (m[0] != m[-3] || m[1] != m[-2]);
+        for (int a = 0; a < 3; ++a) {
+          x.lo[a] = std::min(x.lo[a], m[a]);
+          x.hi[a] = std::max(x.hi[a], m[a]);
+        }
+      }
+      cols = std::max(cols, nc);
+      e[f].push_back(x);
+    }
+  }
+  return ll::footprint_bytes(d, ll::work_side(d, e[0].data(), e[1].data()), cols);
+}
+
 int ll_submit(ll_server* s, const ll_job_desc* jd, uint64_t* job_id) {
   if (!s || !jd || !job_id) return sfail(LL_EINVAL, "bad submit arguments");
   const ll_system_desc* d = &jd->sys;
@@ -362,6 +386,9 @@ int ll_submit(ll_server* s, const ll_job_desc* jd, uint64_t* job_id) {
     if (d->npw_k[k] < 1 || d->npw_kq[k] < 1) return sfail(LL_EINVAL, "malformed job: empty plane-wave sphere");
   size_t fp = 0;
   if (ll_footprint(d, &fp) != LL_OK) return sfail(LL_EINVAL, "footprint");
+  // refused and admitted by the bytes of the job's own spheres on the grid its chain will transform
+  // on (at most ll_footprint's, which reads no Miller index)
+  fp = std::min(fp, spheres_footprint(d));
   if (jd->n_omega > 0) fp += LL_SPECTRUM_BYTES(jd->n_omega);
   if (fp > s->budget) return sfail(LL_ENOMEM, "job footprint exceeds the whole HBM budget");
   Job* j = new Job();
@@ -426,29 +453,6 @@ int ll_submit(ll_server* s, const ll_job_desc* jd, uint64_t* job_id) {
   }
   j->n_steps = jd->n_steps;
   j->eta = jd->eta_ev;
-  {   // admitted by the bytes of the grid the chain will transform on (at most ll_footprint's)
-    std::vector<ll::Extent> e[2];
-    int cols = 1;
-    for (int f = 0; f < 2; ++f) {
-      const int* m = f ? j->desc.miller_kq : j->desc.miller_k;
-      for (int k = 0; k < j->desc.nks; ++k) {
-        const int np = (f ? j->desc.npw_kq : j->desc.npw_k)[k];
-        ll::Extent x{{m[0], m[1], m[2]}, {m[0], m[1], m[2]}};
-        int nc = 1;
-        for (int i = 0; i < np; ++i, m += 3) {
-          nc += i > 0 && (m[0] != m[-3] || m[1] != m[-2]);
-          for (int a = 0; a < 3; ++a) {
-            x.lo[a] = std::min(x.lo[a], m[a]);
-            x.hi[a] = std::max(x.hi[a], m[a]);
-          }
-        }
-        cols = std::max(cols, nc);
-        e[f].push_back(x);
-      }
-    }
-    fp = std::min(fp, ll::footprint_bytes(&j->desc, ll::work_side(&j->desc, e[0].data(), e[1].data()), cols) +
-                          LL_SPECTRUM_BYTES(jd->n_omega));
-  }
   j->footprint = fp;
   j->t_submit = now_s();
   std::lock_guard<std::mutex> lock(s->mu);
