@@ -898,7 +898,7 @@ class Chain : public ChainBase {
       LL_CK(cudaGetLastError());
     }
     if (n > 0) {
-      k_reduce_z<<<n, 128, 0, st_>>>(zpart_, nks_ * npk_, nks_, queued_, z_);
+      k_reduce_z<<<n, 128, 0, st_>>>(zpart_, nks_ * npk_, nks_, queued_, flavour_ == LL_FLAVOUR_PH ? beta_ : nullptr, z_);
       LL_CK(cudaGetLastError());
       prof_.count(LL_PROF_UPDATE);
     }

@@ -11,6 +11,7 @@
 // columns; the full N^3 grid of one orbital is never materialised.
 #pragma once
 #include "fft.cuh"
+#include "sums.cuh"
 
 namespace ll {
 
@@ -607,25 +608,6 @@ __device__ __forceinline__ T warp_sum_t(T v) {
   return v;
 }
 
-// A sum of T values held to at least twice T's precision without the FP64 pipe (2 lanes per SM
-// and cycle): FP32 adds with the rounding error of each kept (Knuth's two-sum, seven FP32
-// operations against a conversion and an add of 16 cycles each); plain for double.
-template <typename T> struct DSum;
-template <> struct DSum<double> {
-  double s = 0.0;
-  __device__ __forceinline__ void add(double v) { s += v; }
-  __device__ __forceinline__ double value() const { return s; }
-};
-template <> struct DSum<float> {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void add(float v) {
-    const float s = __fadd_rn(hi, v), b = __fadd_rn(s, -hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -b)), __fadd_rn(v, -b)));
-    hi = s;
-  }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
-
 // Warp sums of NV values per lane at once (NV a power of two <= 32): at every step a lane keeps
 // half of its values and gives its partner the other half, so 32 values take 31 exchanges
 // instead of 5 each.  Returns the total of value number lane / (32 / NV).
@@ -709,19 +691,16 @@ __device__ __forceinline__ void block_dots_nj(const cplx<T>* A0, const cplx<T>* 
                        nj - j0, red + q * 2 * TP);
     }
     __syncthreads();
-    for (int p = threadIdx.x; p < n * TP; p += blockDim.x) {
-      const int q = b0 + p / TP;
+    for (int e = threadIdx.x; e < 2 * n * TP; e += blockDim.x) {   // a component of a pair
+      const int p = e >> 1, q = b0 + p / TP;
       const bool first = q < t0n;
       const int t = first ? q : q - t0n, i = t / tj * 4 + (p % TP) / NJ, j = t % tj * NJ + p % NJ;
       if (i < (first ? n0 : n1) && j < nj) {
-        DSum<T> re, im;
+        DSum<T> sum;
 #pragma unroll 4
-        for (int w = 0; w < nw; ++w) {
-          re.add(red[w * 2 * kRedPairs + 2 * p]);
-          im.add(red[w * 2 * kRedPairs + 2 * p + 1]);
-        }
-        const double a = re.value(), b = im.value();
-        out[((first ? 0 : n0) + i) * nj + j] = first && mult ? mk(a * mult[i], b * mult[i]) : mk(a, b);
+        for (int w = 0; w < nw; ++w) sum.add(red[w * 2 * kRedPairs + e]);
+        const double a = sum.value();
+        reinterpret_cast<double*>(out + ((first ? 0 : n0) + i) * nj + j)[e & 1] = first && mult ? a * mult[i] : a;
       }
     }
     __syncthreads();
@@ -973,7 +952,7 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_ph_update(const
   const int np = s.npw[k];
   const long zi = (long)(j - 1) * nks * ngrp + (long)k * ngrp + grp;
   const T ib = (T)scal[1], bb = (T)scal[0];
-  T zr = T(0), zim = T(0);   // z_j partial = (y, r_j)/beta_j over the group's bands (r_j upper)
+  T zr = T(0), zim = T(0);   // z_j partial = (y, r_j) over the group's bands (r_j upper; beta_j: k_reduce_z)
 #pragma unroll 4
   for (int i = threadIdx.x; i < bpc * npw_pad; i += blockDim.x) {
     const cplx<T> r = R[base + i], x = X[base + i], v = Vp[base + i];
@@ -987,7 +966,7 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_ph_update(const
   }
   if (r_upper) block_sum2<T>(zr, zim, cf, red);
   else __syncthreads();
-  if (threadIdx.x == 0) co.zpart[zi] = r_upper ? mk(cf[0].x * scal[1], cf[0].y * scal[1]) : mk(0.0, 0.0);
+  if (threadIdx.x == 0) co.zpart[zi] = r_upper ? cf[0] : mk(0.0, 0.0);
   const cplx<T>* uk = ukq + (long)k * nbnd * npw_pad;
   block_dots<T>(uk, rs, npw_pad, np, nbnd, bpc, cf, red);
   if (keep) {  // a metal: only the states with c_mv = 0 are removed
@@ -1250,11 +1229,12 @@ __global__ void __launch_bounds__(256) k_nh_normalize(long n, cplx<T>* __restric
 // advances it).
 static __global__ void k_step_set(int* jdev, int j) { *jdev = j; }
 
-// z_j = (1/nks) sum zpart[j][0..nzp) for j in [j0, j0 + gridDim.x): nzp partials per step, one per
-// (k, band group) or (k, chunk) on the split path, one block per step, fixed order.  (One thread
-// per step took 68 us for the KB workload's 512 partials.)
+// z_j = (1/nks) sum zpart[j][0..nzp) for j in [j0, j0 + gridDim.x), divided by beta_j where given (the
+// pseudo-Hermitian partials are (y, r_j), v_j = r_j/beta_j): nzp partials per step, one per (k, band
+// group) or (k, chunk) on the split path, one block per step, fixed order.  (One thread per step
+// took 68 us for the KB workload's 512 partials.)
 static __global__ void __launch_bounds__(128) k_reduce_z(const cplx<double>* __restrict__ zpart, int nzp, int nks, int j0,
-                                                        cplx<double>* __restrict__ z) {
+                                                        const double* __restrict__ beta, cplx<double>* __restrict__ z) {
   __shared__ double wr[4], wi[4];
   const int j = j0 + blockIdx.x;
   double zr = 0, zi = 0;
@@ -1263,7 +1243,10 @@ static __global__ void __launch_bounds__(128) k_reduce_z(const cplx<double>* __r
   zi = warp_sum(zi);
   if ((threadIdx.x & 31) == 0) { wr[threadIdx.x >> 5] = zr; wi[threadIdx.x >> 5] = zi; }
   __syncthreads();
-  if (threadIdx.x == 0) z[j] = mk((wr[0] + wr[1] + wr[2] + wr[3]) / nks, (wi[0] + wi[1] + wi[2] + wi[3]) / nks);
+  if (threadIdx.x == 0) {
+    const double d = beta ? beta[j] * nks : (double)nks;
+    z[j] = mk((wr[0] + wr[1] + wr[2] + wr[3]) / d, (wi[0] + wi[1] + wi[2] + wi[3]) / d);
+  }
 }
 
 // ---------------------------------------------------------------------------------------

@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(256) k_sp_start(const int* __restrict__ jdev, 
   const long zi = (long)(j - 1) * nks * nchunk + k * nchunk + c;
   const T ib = (T)scal[1], bb = (T)scal[0];
   const int n = g1 - g0;
-  DSum<T> zr, zim;   // z_j partial = (y, r_j)/beta_j over the chunk (r_j upper)
+  DSum<T> zr, zim;   // z_j partial = (y, r_j) over the chunk (r_j upper; beta_j: k_reduce_z)
 #pragma unroll 4
   for (int e = threadIdx.x; e < nbnd * n; e += blockDim.x) {
     const int v = e / n, g = g0 + e - v * n;
@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(256) k_sp_start(const int* __restrict__ jdev, 
     if (threadIdx.x == 0) {
       double tr = 0.0, ti = 0.0;
       for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { tr += zred[0][w]; ti += zred[1][w]; }
-      co.zpart[zi] = mk(tr * scal[1], ti * scal[1]);
+      co.zpart[zi] = mk(tr, ti);
     }
   } else if (threadIdx.x == 0) {
     co.zpart[zi] = mk(0.0, 0.0);
