@@ -795,8 +795,11 @@ class Chain : public ChainBase {
       LL_CK(cudaMemcpyAsync(R(), y_, vq * sizeof(cplx<T>), cudaMemcpyDeviceToDevice, st_));
       if ((rc = op(1, R(), X(), -1, err))) return rc;               // X_1 = D y
       std::vector<double> hp(nzp);
+      int herr = DEV_OK;
       LL_CK(cudaMemcpyAsync(hp.data(), part_, nzp * sizeof(double), cudaMemcpyDeviceToHost, st_));
+      LL_CK(cudaMemcpyAsync(&herr, err_, sizeof(int), cudaMemcpyDeviceToHost, st_));
       LL_CK(cudaStreamSynchronize(st_));
+      if (herr != DEV_OK) { err = kGaveUp; return LL_ETIMEOUT; }
       double s = 0;
       for (double v : hp) s += v;
       s /= nks_;
@@ -993,7 +996,7 @@ class Chain : public ChainBase {
       queued_ = steps_;
       status = (herr[0] == DEV_NOTPD) ? LL_ENOTPD : (herr[0] == DEV_TIMEOUT ? LL_ETIMEOUT : LL_EBREAKDOWN);
       err = (status == LL_ENOTPD)     ? "pseudo-Hermitian metric not positive"
-            : (status == LL_ETIMEOUT) ? "a bounded tensor-core wait gave up"
+            : (status == LL_ETIMEOUT) ? kGaveUp
                                       : "Lanczos breakdown";
       stopped_ = true;
     }
@@ -1062,18 +1065,31 @@ class Chain : public ChainBase {
     }
     LL_CK(cudaMemcpyAsync(pk, x, packed * sizeof(double), cudaMemcpyHostToDevice, st_));
     k_pad_rows<T><<<dim3(nks_, nbnd_), 256, 0, st_>>>(pk, offq_, dq_.npw, nbnd_, hq_.npw_pad, nullptr, scratch_);
-    // a one-vector application reuses the cbuf/tbuf sized for nvec_ >= 1; its norm partials go to a
-    // buffer of their own (part_ holds those of the recursion's last step, which the next one reads)
-    if (!apart_ && (rc = alloc(&apart_, (long)nks_ * npk_))) return rc;
+    // a one-vector application reuses the cbuf/tbuf sized for nvec_ >= 1; its norm partials and its
+    // status word are its own (part_ holds the partials of the recursion's last step, which the
+    // next one reads, err_ what that recursion met)
+    if (!apart_) {
+      if ((rc = alloc(&aerr_, 2)) || (rc = alloc(&apart_, (long)nks_ * npk_))) return rc;
+      LL_CK(cudaMemsetAsync(aerr_, 0, 2 * sizeof(int), st_));
+    }
     std::swap(part_, apart_);
+    std::swap(err_, aerr_);
     rc = op(1, scratch_, scratch_ + vq, (upper && approx_ != LL_APPROX_IPA) ? 0 : -1, err);
     std::swap(part_, apart_);
+    std::swap(err_, aerr_);
     if (rc) return rc;
     k_unpad_rows<T><<<dim3(nks_, nbnd_), 256, 0, st_>>>(scratch_ + vq, offq_, dq_.npw, nbnd_, hq_.npw_pad, pk);
     LL_CK(cudaGetLastError());
     if ((rc = oob_check(err))) return rc;
+    int herr = DEV_OK;
+    LL_CK(cudaMemcpyAsync(&herr, aerr_, sizeof(int), cudaMemcpyDeviceToHost, st_));
     LL_CK(cudaMemcpyAsync(out, pk, packed * sizeof(double), cudaMemcpyDeviceToHost, st_));
     LL_CK(cudaStreamSynchronize(st_));
+    if (herr != DEV_OK) {
+      LL_CK(cudaMemsetAsync(aerr_, 0, 2 * sizeof(int), st_));
+      err = kGaveUp;
+      return LL_ETIMEOUT;
+    }
     return LL_OK;
   }
 
@@ -1118,6 +1134,8 @@ class Chain : public ChainBase {
   }
 
  private:
+  static constexpr const char* kGaveUp = "a bounded wait in a kernel gave up";
+
   // One axis of the band-limited resampling between N and W < N points, [N][W]:
   // f(j/N) = sum_s R[j][s] f(s/W) for f with |d| <= (W - 1)/2; its transpose times W/N limits a
   // function of the N points to those components and samples it on the W.
@@ -1433,6 +1451,8 @@ class Chain : public ChainBase {
     a.f_nbnd = FastDiv((unsigned)nbnd_);
     a.f_nks = FastDiv((unsigned)s.nks);
     a.f_pervec = FastDiv((unsigned)(s.nks * nbnd_));
+    const char* pe = getenv("LL_WAIT_POLLS");   // polls of a plane-pass wait before it gives up
+    a.polls = pe && pe[0] ? atoi(pe) : kWaitPolls;
     return a;
   }
   template <int N, int MODE>
@@ -1712,6 +1732,7 @@ class Chain : public ChainBase {
   double* packed_ = nullptr;     // apply: the caller's packed vector where cbuf_ does not hold it
   int* offq_ = nullptr;          // apply: offsets of the packed k blocks
   double* apart_ = nullptr;      // apply: norm partials
+  int* aerr_ = nullptr;          // apply: status word
   T* rup_ = nullptr;             // W_ < N_: resampling table [N_][W_] (resample_table)
   cplx<T>* t1_ = nullptr;        // W_ < N_: n', then f_xc n', on W_ planes of the declared N_ x N_ grid
   cplx<double> *spart_ = nullptr, *gamma_ = nullptr, *z_ = nullptr, *zpart_ = nullptr, *spec_out_ = nullptr;

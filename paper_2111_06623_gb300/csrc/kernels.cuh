@@ -120,6 +120,7 @@ struct XYArgs {
   FastDiv f_ncol, f_nrow;      // divisions by cb_ncol and by the sphere table's nrow_max
   FastDiv f_nbnd, f_nks;       // orbital -> k: (o / nbnd) mod nks
   FastDiv f_pervec;            // orbital -> vector: o / (nks nbnd)
+  int polls;                   // of a wait on a copy before it gives up (plane.cuh)
 };
 
 template <typename T, int N, int MODE>

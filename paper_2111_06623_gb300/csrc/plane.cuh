@@ -50,6 +50,17 @@ __device__ __forceinline__ void mbar_expect(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
 
+// Every wait on a copy is bounded (XYArgs::polls).  A thread whose wait has run out waits for no
+// other; once one of warp 0's has, no further copy is asked for (a barrier's next phase is armed only
+// when its last one is known to be complete), so the others' waits run out as well and the CTA
+// reaches its end.  There one thread records the error and waits, again with a limit, for the copies
+// still in flight: cols, us: batches whose columns and u(r) have been asked for.
+__device__ __forceinline__ void plane_gave_up(uint64_t* full, uint64_t* ufull, int cols, int us, int* err) {
+  flag_error(err, DEV_TIMEOUT, 1);
+  for (int b = cols > 2 ? cols - 2 : 0; b < cols; ++b) mbar_wait(&full[b & 1], (b >> 1) & 1);
+  if (us > 0) mbar_wait(ufull, (us - 1) & 1);
+}
+
 // ---- launch shape ------------------------------------------------------------------------
 // P lanes per line and SL line slots for a side, type and mode.  A lane holds W/P points; two
 // lanes where one would not keep a line in registers beside its temporaries (W >= 36 in FP32,
@@ -91,6 +102,7 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
   constexpr int LO = P == 1 ? PR : PR / 2, HI = P == 1 ? PR : (PR + 1) / 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t full[2], ufull;
+  __shared__ int s_asked[2];   // batches whose columns, u(r) have been asked for
   const SphereDev& s = a.s;
   const int iz = blockIdx.x, g = blockIdx.y, cb = a.cb_ncol;
   cplx<T>* Cs = reinterpret_cast<cplx<T>*>(smem_raw);
@@ -104,6 +116,7 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
     mbar_init(&full[0], 1);
     mbar_init(&full[1], 1);
     mbar_init(&ufull, 1);
+    s_asked[0] = s_asked[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
   }
@@ -123,7 +136,10 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
   // warp 0: the columns of batch `it` into its buffer; u(r) of batch `it`
   auto load_cols = [&](int it) {
     const int nb = min(SL, o_end - o_begin - it * SL);
-    if (t == 0) mbar_expect(&full[it & 1], nb * cbytes);
+    if (t == 0) {
+      s_asked[0] = it + 1;
+      mbar_expect(&full[it & 1], nb * cbytes);
+    }
     __syncwarp();
     if (t < nb) bulk_load(Cs + ((it & 1) * SL + t) * cb, row_of(o_begin + it * SL + t), cbytes, &full[it & 1]);
   };
@@ -131,7 +147,10 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
     const int o = o_begin + it * SL + t;
     const bool on = t < SL && o < o_end && dens_orb(o);
     const uint32_t n = __popc(__ballot_sync(0xffffffffu, on));
-    if (t == 0) mbar_expect(&ufull, n * (uint32_t)(WW * sizeof(cplx<T>)));
+    if (t == 0) {
+      s_asked[1] = it + 1;
+      mbar_expect(&ufull, n * (uint32_t)(WW * sizeof(cplx<T>)));
+    }
     __syncwarp();
     if (on)
       bulk_load(Us + t * WW, ur + ((long)a.f_pervec.mod(o) * W + iz) * WW, (uint32_t)(WW * sizeof(cplx<T>)), &ufull);
@@ -178,7 +197,7 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
     cplx<T>* cs = Cs + (it & 1) * SL * cb + (row_on ? rb * cb + rw.y - rw.z : 0);
     cplx<T>* ysr = Ys + (row_on ? pr * NP : 0);
     if (MODE != XY_PASS2) {
-      if (!bad) bad = !mbar_wait(&full[it & 1], (it >> 1) & 1);
+      if (!bad) bad = !mbar_wait(&full[it & 1], (it >> 1) & 1, a.polls);
       if (row_on) {
         cplx<T> l[H];
 #pragma unroll
@@ -200,7 +219,7 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
     const int4 rwc = rw;
     const bool rowc = row_on;
     if (it + 1 < nbat) tables(ob + SL);
-    if (HAS_U && !bad) bad = !mbar_wait(&ufull, it & 1);
+    if (HAS_U && !bad) bad = !mbar_wait(&ufull, it & 1, a.polls);
     if (line_on) {
       cplx<T> l[H];
       cplx<T>* ysl = Ys + (ls * s.nrow_max - lm2) * NP + j1;
@@ -238,8 +257,8 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
         }
     }
     __syncthreads();
-    if (HAS_U && t < 32 && it + 1 < nbat) load_u(it + 1);
-    if (MODE == XY_PASS2 && !bad) bad = !mbar_wait(&full[it & 1], (it >> 1) & 1);
+    if (HAS_U && t < 32 && it + 1 < nbat && !__any_sync(0xffffffffu, bad)) load_u(it + 1);
+    if (MODE == XY_PASS2 && !bad) bad = !mbar_wait(&full[it & 1], (it >> 1) & 1, a.polls);
     if (rowc) {
       cplx<T> l[H];
 #pragma unroll
@@ -263,14 +282,14 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
         bulk_store(row_of(ob + t), Cs + ((it & 1) * SL + t) * cb, cbytes);
         bulk_commit();
       }
-      if (it + 2 < nbat) {   // the same buffer's next batch, once the store has read it
+      if (it + 2 < nbat && !__any_sync(0xffffffffu, bad)) {   // the same buffer's next batch, once the store has read it
         if (t < nb) bulk_wait_read();
         __syncwarp();
         load_cols(it + 2);
       }
     }
   }
-  if (bad && t == 0 && err) flag_error(err, DEV_TIMEOUT, 1);
+  if (__syncthreads_or(bad) && t == 0) plane_gave_up(full, &ufull, s_asked[0], s_asked[1], err);
   if (MODE == XY_PASS1_DENS) {   // the slots summed in order
     __syncthreads();
     for (int q = 0; q < SL; ++q) {

@@ -91,6 +91,7 @@ __global__ void __launch_bounds__(PlaneCfg<double, W, MODE>::TH, PlaneCfg<double
   constexpr int G = fx_growth(W);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t full[2], ufull;
+  __shared__ int s_asked[2];   // batches whose columns, u(r) have been asked for
   __shared__ int s_er[SL * W], s_el[SL * W], s_ev;   // exponents of the rows and lines; largest of V or v'
   const SphereDev& s = a.s;
   const int iz = blockIdx.x, g = blockIdx.y, cb = a.cb_ncol;
@@ -104,6 +105,7 @@ __global__ void __launch_bounds__(PlaneCfg<double, W, MODE>::TH, PlaneCfg<double
     mbar_init(&full[0], 1);
     mbar_init(&full[1], 1);
     mbar_init(&ufull, 1);
+    s_asked[0] = s_asked[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
     s_ev = 0;
@@ -137,7 +139,10 @@ __global__ void __launch_bounds__(PlaneCfg<double, W, MODE>::TH, PlaneCfg<double
   // warp 0: the columns of batch `it` into its buffer; u(r) of batch `it`
   auto load_cols = [&](int it) {
     const int nb = min(SL, o_end - o_begin - it * SL);
-    if (t == 0) mbar_expect(&full[it & 1], nb * cbytes);
+    if (t == 0) {
+      s_asked[0] = it + 1;
+      mbar_expect(&full[it & 1], nb * cbytes);
+    }
     __syncwarp();
     if (t < nb) bulk_load(Cs + ((it & 1) * SL + t) * cb, row_of(o_begin + it * SL + t), cbytes, &full[it & 1]);
   };
@@ -145,7 +150,10 @@ __global__ void __launch_bounds__(PlaneCfg<double, W, MODE>::TH, PlaneCfg<double
     const int o = o_begin + it * SL + t;
     const bool on = t < SL && o < o_end && dens_orb(o);
     const uint32_t n = __popc(__ballot_sync(0xffffffffu, on));
-    if (t == 0) mbar_expect(&ufull, n * (uint32_t)(WW * sizeof(cplx<T>)));
+    if (t == 0) {
+      s_asked[1] = it + 1;
+      mbar_expect(&ufull, n * (uint32_t)(WW * sizeof(cplx<T>)));
+    }
     __syncwarp();
     if (on)
       bulk_load(Us + t * WW, ur + ((long)a.f_pervec.mod(o) * W + iz) * WW, (uint32_t)(WW * sizeof(cplx<T>)), &ufull);
@@ -200,8 +208,8 @@ __global__ void __launch_bounds__(PlaneCfg<double, W, MODE>::TH, PlaneCfg<double
     // phase 0: rows inverse; 1: lines; 2: rows forward (pass 2 has no inverse transforms)
 #pragma unroll 1
     for (int ph = MODE == XY_PASS2 ? 1 : 0; ph < 3; ++ph) {
-      if (HAS_U && ph == 1 && !bad) bad = !mbar_wait(&ufull, it & 1);
-      if (ph == (MODE == XY_PASS2 ? 2 : 0) && !bad) bad = !mbar_wait(&full[it & 1], (it >> 1) & 1);
+      if (HAS_U && ph == 1 && !bad) bad = !mbar_wait(&ufull, it & 1, a.polls);
+      if (ph == (MODE == XY_PASS2 ? 2 : 0) && !bad) bad = !mbar_wait(&full[it & 1], (it >> 1) & 1, a.polls);
       cplx<fx64> l[H];
       int e = 0;
       if (ph == 1 ? line_on : row_on) {
@@ -317,7 +325,7 @@ __global__ void __launch_bounds__(PlaneCfg<double, W, MODE>::TH, PlaneCfg<double
       }
       if (ph == 2) fence_async_smem();
       __syncthreads();
-      if (HAS_U && ph == 1 && t < 32 && it + 1 < nbat) load_u(it + 1);
+      if (HAS_U && ph == 1 && t < 32 && it + 1 < nbat && !__any_sync(0xffffffffu, bad)) load_u(it + 1);
     }
     if (t < 32) {
       const int nb = min(SL, o_end - ob);
@@ -325,14 +333,14 @@ __global__ void __launch_bounds__(PlaneCfg<double, W, MODE>::TH, PlaneCfg<double
         bulk_store(row_of(ob + t), Cs + ((it & 1) * SL + t) * cb, cbytes);
         bulk_commit();
       }
-      if (it + 2 < nbat) {   // the same buffer's next batch, once the store has read it
+      if (it + 2 < nbat && !__any_sync(0xffffffffu, bad)) {   // the same buffer's next batch, once the store has read it
         if (t < nb) bulk_wait_read();
         __syncwarp();
         load_cols(it + 2);
       }
     }
   }
-  if (bad && t == 0 && err) flag_error(err, DEV_TIMEOUT, 1);
+  if (__syncthreads_or(bad) && t == 0) plane_gave_up(full, &ufull, s_asked[0], s_asked[1], err);
   if (MODE == XY_PASS1_DENS) {   // the slots summed in order
     __syncthreads();
     for (int i = t; i < WW; i += TH) {

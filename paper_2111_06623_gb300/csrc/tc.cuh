@@ -100,8 +100,9 @@ __device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
 }
 
 // Wait for the phase with the given parity to complete; false when the bounded wait ran out.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  for (long it = 0; it < (1L << 24); ++it)
+constexpr int kWaitPolls = 1 << 24;
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int polls = kWaitPolls) {
+  for (int it = 0; it < polls; ++it)
     if (mbar_try(bar, parity)) return true;
   return false;
 }
