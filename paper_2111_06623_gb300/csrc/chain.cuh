@@ -274,7 +274,8 @@ static inline void recip(const double a[3][3], double b[3][3]) {
 // (k_hxcw_*).  The smallest built side that holds the differences is taken: cells whose grid is
 // a size or more above the smallest product grid gain (25 Ry on 32^3: 24^3; 10 Ry on 18^3:
 // 16^3), the others keep W = N.  LL_PRUNE=0 or 1 in the environment: W = N.
-static inline int work_side(const ll_system_desc* d, const Extent* ek, const Extent* eq) {
+// eq: extents of the spheres at k+Q as indexed from c (fold_index; null: from zero).
+static inline int work_side(const ll_system_desc* d, const Extent* ek, const Extent* eq, const int* c = nullptr) {
   const int n = d->nfft, nsym = d->sym ? d->nsym : 1;
   const char* pe = getenv("LL_PRUNE");
   if (pe && (pe[0] == '0' || pe[0] == '1') && pe[1] == 0) return n;
@@ -288,8 +289,8 @@ static inline int work_side(const ll_system_desc* d, const Extent* ek, const Ext
   }
   if (nsym > 1) {
     // the density averaged over the small group has the rotated differences too: all of
-    // |G| <= max|k+G| + max|k+Q+G| + |Q|, a ball the group's operations keep; they must be
-    // isometries of the lattice (M^T g M = g with g_ij = a_i . a_j)
+    // |G| <= max|k+G| + max|k+Q+G| + |Q| (indices from c: |Q + c|), a ball the group's operations
+    // keep; they must be isometries of the lattice (M^T g M = g with g_ij = a_i . a_j)
     double g[3][3], gmax = 0, r[2] = {0, 0}, q2 = 0;
     for (int i = 0; i < 3; ++i)
       for (int j = 0; j < 3; ++j) {
@@ -322,7 +323,10 @@ static inline int work_side(const ll_system_desc* d, const Extent* ek, const Ext
           r[f] = std::max(r[f], t);
         }
     }
-    for (int a = 0; a < 3; ++a) q2 += d->q_cart[a] * d->q_cart[a];
+    for (int a = 0; a < 3; ++a) {
+      const double x = d->q_cart[a] + (c ? c[0] * b[0][a] + c[1] * b[1][a] + c[2] * b[2][a] : 0.0);
+      q2 += x * x;
+    }
     const double rad = std::sqrt(r[0]) + std::sqrt(r[1]) + std::sqrt(q2);
     for (int a = 0; a < 3; ++a)
       dmax = std::max(dmax, (int)std::min(1e6, rad * std::sqrt(g[a][a]) / (2.0 * 3.14159265358979323846) + 1e-9));
@@ -330,6 +334,63 @@ static inline int work_side(const ll_system_desc* d, const Extent* ek, const Ext
   for (int s : kGridSides)
     if (s < n && 2 * dmax + 1 <= s && mmax <= s) return s;
   return n;
+}
+
+// The Miller index c that the spheres at k+Q are indexed from on the grid.  A Q far outside the
+// first zone moves them beyond half the grid, where signed indices are not unique and only the
+// general plane kernel (k_xy) applies.  Seen from c, x'(r) = exp(-i c r) x(r): V x, v' u and f_xc n'
+// are products in r and keep the factor, the density conj(u) x carries it into v', so that only
+// the Hartree kernel has to be taken at G + c; the spheres' data and every other table stay as
+// they are.  c = 0 unless the spheres need it and then fit the pruned kernels' range -W/2 .. W/2
+// (one sphere never holds both ends); with a symmetry group, only a c that its operations keep
+// (they act on n').  us per step, k_xy in FP32 | FP64 -> so: 32^3, 64 k-points, 4 bands 133 | 2033
+// -> 112 | 981; 48^3, 64 k-points, 8 bands 1146 | 19767 -> 575 | 8939.
+static inline bool in_signed_range(const ll_system_desc* d, const Extent* eq, const int* c, int w) {
+  for (int k = 0; k < d->nks; ++k)
+    for (int a = 0; a < 3; ++a)
+      if (eq[k].lo[a] - c[a] < -(w / 2) || eq[k].hi[a] - c[a] > w / 2) return false;
+  return true;
+}
+static inline void fold_index(const ll_system_desc* d, const Extent* ek, const Extent* eq, int* c) {
+  const int zero[3] = {0, 0, 0};
+  c[0] = c[1] = c[2] = 0;
+  if (in_signed_range(d, eq, zero, work_side(d, ek, eq))) return;
+  int f[3];
+  for (int a = 0; a < 3; ++a) {
+    int lo = eq[0].lo[a], hi = eq[0].hi[a];
+    for (int k = 1; k < d->nks; ++k) lo = std::min(lo, eq[k].lo[a]), hi = std::max(hi, eq[k].hi[a]);
+    f[a] = lo + (hi - lo + 1) / 2;
+  }
+  for (int s = 0; d->sym && s < d->nsym; ++s)   // c (M j) = c j at every grid point j
+    for (int b = 0; b < 3; ++b) {
+      const int* m = d->sym + 9 * s;
+      if (f[0] * m[b] + f[1] * m[3 + b] + f[2] * m[6 + b] != f[b]) return;
+    }
+  std::vector<Extent> e(eq, eq + d->nks);
+  for (Extent& x : e)
+    for (int a = 0; a < 3; ++a) x.lo[a] -= f[a], x.hi[a] -= f[a];
+  if (in_signed_range(d, eq, f, work_side(d, ek, e.data(), f)))
+    for (int a = 0; a < 3; ++a) c[a] = f[a];
+}
+// Moves a family's tables to indices from c; with w > 0 then to bases modulo w (what the kernels
+// for any index need where a sphere lies beyond w).
+static inline void index_from(HostSphere& h, const int* c, int w = 0) {
+  auto mod = [&](int m) { return w > 0 ? ((m % w) + w) % w : m; };
+  for (int k = 0; k < h.nks; ++k) {
+    const int y0 = h.row[(size_t)k * h.nrow_max].x - c[1], y = y0 - mod(y0) + c[1];   // rows of a sphere stay consecutive
+    for (int i = 0; i < h.ncol[k]; ++i) {
+      int4& e = h.col[(size_t)k * h.ncol_max + i];
+      e.x = mod(e.x - c[0]);
+      e.y -= y;
+      e.z = mod(e.z - c[2]);
+    }
+    for (int i = 0; i < h.nrow[k]; ++i) {
+      int4& e = h.row[(size_t)k * h.nrow_max + i];
+      e.x -= y;
+      e.z = mod(e.z - c[0]);
+    }
+    for (int a = 0; a < 3; ++a) h.ext[k].lo[a] -= c[a], h.ext[k].hi[a] -= c[a];
+  }
 }
 
 // Orbitals per batch of the per-plane kernel: enough axis-1 lines for the 128 threads when
@@ -498,16 +559,23 @@ class Chain : public ChainBase {
                   d->lattice[0][1] * (d->lattice[1][0] * d->lattice[2][2] - d->lattice[1][2] * d->lattice[2][0]) +
                   d->lattice[0][2] * (d->lattice[1][0] * d->lattice[2][1] - d->lattice[1][1] * d->lattice[2][0]));
     for (int a = 0; a < 3; ++a) q_[a] = d->q_cart[a];
-    W_ = work_side(d, hk_.ext.data(), hq_.ext.data());
+    int c[3];
+    fold_index(d, hk_.ext.data(), hq_.ext.data(), c);
+    index_from(hq_, c);
+    W_ = work_side(d, hk_.ext.data(), hq_.ext.data(), c);
     {   // the largest |m| of the k+Q spheres on any axis picks the bound the lines are built with:
-        // the smallest of plane_level's that holds every sphere, 0 (k_xy) where none does
+        // the smallest of plane_level's that holds every sphere (the largest holds -W/2 and W/2
+        // too), 0 (k_xy) where none does
       int pmax = 0;
       for (const Extent& e : hq_.ext)
-        for (int a = 0; a < 3; ++a) pmax = std::max({pmax, std::abs(e.lo[a]), std::abs(e.hi[a])});
+        for (int a = 0; a < 3; ++a) pmax = std::max({pmax, -e.lo[a] - (e.lo[a] == -(W_ / 2)), e.hi[a] - (e.hi[a] == W_ / 2)});
       const char* pe = getenv("LL_PRUNE");   // 0: lines not pruned (the largest bound); 1: W = N
       prune_ = 0;
       for (int l = (pe && pe[0] == '0' && pe[1] == 0) ? 2 : 0; l < 3 && !prune_; ++l)
         if (pmax <= plane_level(W_, l)) prune_ = plane_level(W_, l);
+      const int zero[3] = {0, 0, 0};
+      index_from(hk_, zero, W_);
+      if (!prune_) index_from(hq_, zero, W_);
     }
     const int w = W_;
     const long w3 = (long)w * w * w;
@@ -516,25 +584,30 @@ class Chain : public ChainBase {
     const long vq = (long)nks_ * nbnd_ * pq;  // one batch vector
     nvec_ = (flavour_ == LL_FLAVOUR_NH) ? 2 : 1;
 
-    // Hartree kernel 4 pi / |Q + G|^2 / W^3 over the work grid's box, [m3][m2][m1]; Q + G = 0 is
-    // looked for over the whole declared box
+    // Hartree kernel 4 pi / |Q + G|^2 / W^3 over the work grid's box, [m3][m2][m1], at the box index
+    // of m + c on the declared grid; Q + G = 0 is looked for over the whole declared box
     std::vector<T> wh(w3);
-    for (int i3 = 0; i3 < n; ++i3)
-      for (int i2 = 0; i2 < n; ++i2)
-        for (int i1 = 0; i1 < n; ++i1) {
-          const int m[3] = {i1 < n / 2 ? i1 : i1 - n, i2 < n / 2 ? i2 : i2 - n, i3 < n / 2 ? i3 : i3 - n};
-          double g[3];
-          for (int a = 0; a < 3; ++a) g[a] = q_[a] + m[0] * b[0][a] + m[1] * b[1][a] + m[2] * b[2][a];
-          const double g2 = g[0] * g[0] + g[1] * g[1] + g[2] * g[2];
-          if (!(g2 > 1e-20)) { err = "Q + G = 0 on the grid (Q is a reciprocal lattice vector)"; return LL_EINVAL; }
-          bool in = true;
-          int i[3];
-          for (int a = 0; a < 3; ++a) {
-            in = in && m[a] >= -(w / 2) && m[a] < (w + 1) / 2;
-            i[a] = m[a] < 0 ? m[a] + w : m[a];
-          }
-          if (in) wh[((long)i[2] * w + i[1]) * w + i[0]] = (T)(4.0 * 3.14159265358979323846 / g2 / (double)w3);
-        }
+    auto qg2 = [&](int m1, int m2, int m3) {
+      double t = 0;
+      for (int a = 0; a < 3; ++a) {
+        const double g = q_[a] + m1 * b[0][a] + m2 * b[1][a] + m3 * b[2][a];
+        t += g * g;
+      }
+      return t;
+    };
+    for (int m3 = -(n / 2); m3 < n - n / 2; ++m3)
+      for (int m2 = -(n / 2); m2 < n - n / 2; ++m2)
+        for (int m1 = -(n / 2); m1 < n - n / 2; ++m1)
+          if (!(qg2(m1, m2, m3) > 1e-20)) { err = "Q + G = 0 on the grid (Q is a reciprocal lattice vector)"; return LL_EINVAL; }
+    auto box = [&](int i, int a) {   // work-grid point i of axis a -> its index on the declared box
+      const int m = (i < (w + 1) / 2 ? i : i - w) + c[a] + n / 2;
+      return ((m % n) + n) % n - n / 2;
+    };
+    for (int i3 = 0; i3 < w; ++i3)
+      for (int i2 = 0; i2 < w; ++i2)
+        for (int i1 = 0; i1 < w; ++i1)
+          wh[((long)i3 * w + i2) * w + i1] =
+              (T)(4.0 * 3.14159265358979323846 / qg2(box(i1, 0), box(i2, 1), box(i3, 2)) / (double)w3);
     // kinetic 1/2 |k + Q + G|^2 on sphere(k+Q)
     std::vector<T> kin((size_t)nks_ * pq, T(0));
     for (int k = 0; k < nks_; ++k) {

@@ -34,10 +34,18 @@ __device__ __forceinline__ int wrapn(int m) { return (int)((unsigned)(m + N) % (
 
 // Pruned lines: with PR > 0 every sphere of the system has |m| <= PR on all three axes, so only the
 // points p <= PR and p >= N - PR of a line are kept; with the stores of the other points gone at
-// compile time, the compiler drops the butterflies that only feed them.  PR = 0: every point.
+// compile time, the compiler drops the butterflies that only feed them.  PR = N/2 - 1 keeps the whole
+// line (line_hi): m = -N/2 or N/2 too, whichever lies in a sphere's run of indices that starts at
+// lo (line_m).  PR = 0: every point, of any indices.
+__host__ __device__ constexpr int line_hi(int n, int pr) { return pr == n / 2 - 1 ? n / 2 : pr; }
+template <int N, int PR>
+__device__ __forceinline__ int line_m(int p, int lo) {
+  if (PR == N / 2 - 1 && p == N / 2) return lo > -N / 2 ? N / 2 : -N / 2;
+  return p <= PR ? p : p - N;
+}
 template <int N, int PR>
 __device__ __forceinline__ constexpr bool line_kept(int p) {
-  return PR == 0 || p <= PR || p >= N - PR;
+  return PR == 0 || p <= PR || p >= N - line_hi(N, PR);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -62,11 +70,11 @@ __global__ void __launch_bounds__(128) k_zinv(SphereDev s, const cplx<T>* __rest
     for (int p = 0; p < N; ++p) {
       a[p] = czero<T>();
       if (line_kept<N, PR>(p)) {
-        const int i = PR > 0 ? (p <= PR ? p : p - N) - cl.z : wrapn<N>(p - cl.z);
+        const int i = PR > 0 ? line_m<N, PR>(p, cl.z) - cl.z : wrapn<N>(p - cl.z);
         if ((unsigned)i < (unsigned)cl.w && LL_INB(st >= 0 && st + i < s.npw_pad)) a[p] = src[i];
       }
     }
-    if constexpr (PR > 0) line_transform<T, N, +1, PR, PR>(a);
+    if constexpr (PR > 0) line_transform<T, N, +1, PR, line_hi(N, PR)>(a);
     else line_transform<T, N, +1>(a);
     if (!LL_INB(c < cb_ncol)) continue;
     cplx<T>* dst = cbuf + o * (long)N * cb_ncol + c;
@@ -84,8 +92,8 @@ __device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
 
 // ---------------------------------------------------------------------------------------
 // Per-plane pass of one operator application, for any Miller indices that fit the grid (the
-// orbital grids at set-up, and spheres beyond |m| < N/2, a Q far outside the first zone; every
-// other application takes k_plane, plane.cuh, with the same modes).  grid (N planes, groups),
+// orbital grids at set-up, and spheres that no index shift brings within -N/2 .. N/2, fold_index;
+// every other application takes k_plane, plane.cuh, with the same modes).  grid (N planes, groups),
 // block 128.
 // The sphere's columns are ordered by (m2, m1) and grouped in rows of equal m2 (consecutive
 // m1).  For every orbital of the group (BO at a time), at plane j3 = blockIdx.x:
@@ -1032,7 +1040,7 @@ __global__ void __launch_bounds__(kLines) k_zfwd(SphereDev s, int nbnd, const cp
 #pragma unroll
   for (int p = 0; p < N; ++p)
     if (line_kept<N, PR>(p)) {
-      const int i = PR > 0 ? (p <= PR ? p : p - N) - cl.z : wrapn<N>(p - cl.z);
+      const int i = PR > 0 ? line_m<N, PR>(p, cl.z) - cl.z : wrapn<N>(p - cl.z);
       if ((unsigned)i < (unsigned)cl.w && LL_INB(st >= 0 && st + i < npw_pad)) t[i] = x[i] * (kn[i] - ev) + a[p] * scale;
     }
 }

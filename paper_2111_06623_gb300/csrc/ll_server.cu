@@ -370,7 +370,11 @@ static size_t spheres_footprint(const ll_system_desc* d) {
       e[f].push_back(x);
     }
   }
-  return ll::footprint_bytes(d, ll::work_side(d, e[0].data(), e[1].data()), cols);
+  int c[3];
+  ll::fold_index(d, e[0].data(), e[1].data(), c);
+  for (ll::Extent& x : e[1])
+    for (int a = 0; a < 3; ++a) x.lo[a] -= c[a], x.hi[a] -= c[a];
+  return ll::footprint_bytes(d, ll::work_side(d, e[0].data(), e[1].data(), c), cols);
 }
 
 int ll_submit(ll_server* s, const ll_job_desc* jd, uint64_t* job_id) {

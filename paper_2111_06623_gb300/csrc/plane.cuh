@@ -1,5 +1,6 @@
 // The per-plane pass of k_xy (kernels.cuh) for spheres whose Miller indices lie within
-// |m| <= PR < W/2 on every axis (signed indices are then unique on the grid), pipelined with
+// |m| <= PR < W/2 on every axis (PR = W/2 - 1: -W/2 too; signed indices are then unique on the grid),
+// pipelined with
 // bulk copies.  grid (W planes, groups); a CTA takes SL orbitals per batch, one per line slot,
 // so every thread (P = 1) or lane pair (P = 2) has exactly one axis-1 row and one axis-2 line of
 // the batch:
@@ -99,7 +100,7 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
   constexpr int NP = W + 1, WW = W * W;
   constexpr bool HAS_U = MODE != XY_PASS1;
   // kept points of a lane's half line (P = 2: p = 2 i + h), i <= LO or i >= H - HI
-  constexpr int LO = P == 1 ? PR : PR / 2, HI = P == 1 ? PR : (PR + 1) / 2;
+  constexpr int LO = P == 1 ? PR : PR / 2, HI = P == 1 ? line_hi(W, PR) : (PR + 1) / 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t full[2], ufull;
   __shared__ int s_asked[2];   // batches whose columns, u(r) have been asked for
@@ -187,8 +188,12 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
   cplx<T> acc[MODE == XY_PASS1_DENS ? H : 1];
 #pragma unroll
   for (int i = 0; i < (MODE == XY_PASS1_DENS ? H : 1); ++i) acc[i] = czero<T>();
-  // signed index of point i of this lane: m(i) = (p <= PR ? p : p - W) at h = 0, + h
-  auto m_of = [](int i) constexpr { return P == 1 ? (i <= LO ? i : i - W) : (i <= LO ? 2 * i : 2 * i - W); };
+  // signed index of point i of this lane, in a run of indices that starts at lo: m(i) = (p <= PR ? p : p - W)
+  // at h = 0, + h; the middle point of a whole line is -W/2 or W/2 (line_m)
+  auto m_of = [&](int i, int lo) {
+    if (PR == W / 2 - 1 && i == H / 2 && (P == 1 || h == 0)) return lo > -W / 2 ? W / 2 : -W / 2;
+    return P == 1 ? (i <= LO ? i : i - W) : (i <= LO ? 2 * i : 2 * i - W);
+  };
   auto kept = [](int i) constexpr { return i <= LO || i >= H - HI; };
   bool bad = false;
 
@@ -204,7 +209,7 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
         for (int i = 0; i < H; ++i) {
           l[i] = czero<T>();
           if (kept(i)) {
-            const int m = m_of(i) + h, j = m - rw.z;
+            const int m = m_of(i, rw.z) + h, j = m - rw.z;
             if ((unsigned)j < (unsigned)rw.w && LL_INB(rw.y >= 0 && rw.y + j < cb)) l[i] = cs[m];
           }
         }
@@ -232,7 +237,7 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
         for (int i = 0; i < H; ++i) {
           l[i] = czero<T>();
           if (kept(i)) {
-            const int m = m_of(i) + h;
+            const int m = m_of(i, lm2) + h;
             if ((unsigned)(m - lm2) < (unsigned)lnr && LL_INB(m - lm2 < s.nrow_max)) l[i] = ysl[m * NP];
           }
         }
@@ -252,7 +257,7 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
 #pragma unroll
       for (int i = 0; i < H; ++i)
         if (kept(i)) {
-          const int m = m_of(i) + h;
+          const int m = m_of(i, lm2) + h;
           if ((unsigned)(m - lm2) < (unsigned)lnr && LL_INB(m - lm2 < s.nrow_max)) ysl[m * NP] = l[i];
         }
     }
@@ -267,7 +272,7 @@ __global__ void __launch_bounds__(PlaneCfg<T, W, MODE>::TH, PlaneCfg<T, W, MODE>
 #pragma unroll
       for (int i = 0; i < H; ++i)
         if (kept(i)) {
-          const int m = m_of(i) + h, j = m - rwc.z;
+          const int m = m_of(i, rwc.z) + h, j = m - rwc.z;
           if ((unsigned)j < (unsigned)rwc.w && LL_INB(rwc.y >= 0 && rwc.y + j < cb)) {
             if (MODE == XY_PASS2) cs[m] = cs[m] + l[i];
             else cs[m] = l[i];

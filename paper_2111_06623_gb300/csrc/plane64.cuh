@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(PlaneCfg<double, W, MODE>::TH, PlaneCfg<double
   constexpr int NP = W + 1, WW = W * W;
   constexpr bool HAS_U = MODE != XY_PASS1;
   // kept points of a lane's half line (P = 2: p = 2 i + h), i <= LO or i >= H - HI
-  constexpr int LO = P == 1 ? PR : PR / 2, HI = P == 1 ? PR : (PR + 1) / 2;
+  constexpr int LO = P == 1 ? PR : PR / 2, HI = P == 1 ? line_hi(W, PR) : (PR + 1) / 2;
   // headroom of a transform's inputs (of the whole line, so that results do not depend on PR)
   constexpr int G = fx_growth(W);
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -168,8 +168,12 @@ __global__ void __launch_bounds__(PlaneCfg<double, W, MODE>::TH, PlaneCfg<double
   const unsigned pmask = 3u << (t & 30);
   const int rb = a.f_nrow.div(pr), rr = pr - rb * s.nrow_max;
   const int ls = pr / W, j1 = pr - ls * W;
-  // signed index of point i of this lane: m(i) = (p <= PR ? p : p - W) at h = 0, + h
-  auto m_of = [](int i) constexpr { return P == 1 ? (i <= LO ? i : i - W) : (i <= LO ? 2 * i : 2 * i - W); };
+  // signed index of point i of this lane, in a run of indices that starts at lo: m(i) = (p <= PR ? p : p - W)
+  // at h = 0, + h; the middle point of a whole line is -W/2 or W/2 (line_m)
+  auto m_of = [&](int i, int lo) {
+    if (PR == W / 2 - 1 && i == H / 2 && (P == 1 || h == 0)) return lo > -W / 2 ? W / 2 : -W / 2;
+    return P == 1 ? (i <= LO ? i : i - W) : (i <= LO ? 2 * i : 2 * i - W);
+  };
   auto kept = [](int i) constexpr { return i <= LO || i >= H - HI; };
   // the next batch's row: (m2, first column, m1 of it, columns); line: the orbital's rows and first m2
   int4 rw_n = make_int4(0, 0, 0, 0);
@@ -218,7 +222,7 @@ __global__ void __launch_bounds__(PlaneCfg<double, W, MODE>::TH, PlaneCfg<double
           for (int i = 0; i < H; ++i) {
             l[i] = czero<fx64>();
             if (kept(i)) {
-              const int m = m_of(i) + h, j = m - rw.z;
+              const int m = m_of(i, rw.z) + h, j = m - rw.z;
               if ((unsigned)j < (unsigned)rw.w && LL_INB(rw.y >= 0 && rw.y + j < cb)) l[i] = fx_raw(cs[m]);
             }
           }
@@ -232,7 +236,7 @@ __global__ void __launch_bounds__(PlaneCfg<double, W, MODE>::TH, PlaneCfg<double
           for (int i = 0; i < H; ++i) {
             l[i] = czero<fx64>();
             if (kept(i)) {
-              const int m = m_of(i) + h;
+              const int m = m_of(i, lm2) + h;
               if ((unsigned)(m - lm2) < (unsigned)lnr && LL_INB(m - lm2 < s.nrow_max))
                 l[i] = fx_down(ysl[m * NP], min(e - er[m - lm2] + G, 63));
             }
@@ -307,14 +311,14 @@ __global__ void __launch_bounds__(PlaneCfg<double, W, MODE>::TH, PlaneCfg<double
 #pragma unroll
           for (int i = 0; i < H; ++i)
             if (kept(i)) {
-              const int m = m_of(i) + h;
+              const int m = m_of(i, lm2) + h;
               if ((unsigned)(m - lm2) < (unsigned)lnr && LL_INB(m - lm2 < s.nrow_max)) ysl[m * NP] = l[i];
             }
         } else {
 #pragma unroll
           for (int i = 0; i < H; ++i)
             if (kept(i)) {
-              const int m = m_of(i) + h, j = m - rw.z;
+              const int m = m_of(i, rw.z) + h, j = m - rw.z;
               if ((unsigned)j < (unsigned)rw.w && LL_INB(rw.y >= 0 && rw.y + j < cb)) {
                 const cplx<T> r = fx_value(l[i], e);
                 if (MODE == XY_PASS2) cs[m] = cs[m] + r;
