@@ -1122,7 +1122,11 @@ class Chain : public ChainBase {
   int apply(int upper, const double* x, double* out, std::string& err) override {
     int rc;
     const long vq = (long)nks_ * nbnd_ * hq_.npw_pad;
-    if (!scratch_ && (rc = alloc(&scratch_, 2 * vq))) return rc;
+    if (!scratch_) {
+      if ((rc = alloc(&scratch_, 2 * vq))) return rc;
+      // the spheres' padding of the output stays zero: no kernel writes it before k_op_proj reads it
+      LL_CK(cudaMemsetAsync(scratch_, 0, 2 * vq * sizeof(cplx<T>), st_));
+    }
     if (!offq_) {
       if ((rc = alloc(&offq_, nks_ + 1))) return rc;
       LL_CK(cudaMemcpyAsync(offq_, hq_.off.data(), (nks_ + 1) * sizeof(int), cudaMemcpyHostToDevice, st_));
@@ -1698,6 +1702,9 @@ class Chain : public ChainBase {
     const size_t nbytes = sizeof(cplx<T>) * (size_t)std::max(1L, count);
     if (cudaMalloc(&q, nbytes) != cudaSuccess) { cudaGetLastError(); return LL_ENOMEM; }
     ur_share_ = std::shared_ptr<void>(q, [](void* a) { cudaFree(a); });
+#ifdef LL_CHECK
+    if (cudaMemsetAsync(q, 0xff, nbytes, st_) != cudaSuccess) return LL_ECUDA;
+#endif
     ur_ = static_cast<cplx<T>*>(q);
     bytes_ += nbytes;
     return LL_OK;
@@ -1708,6 +1715,10 @@ class Chain : public ChainBase {
     void* q = nullptr;
     const size_t nbytes = sizeof(U) * (size_t)std::max(1L, count);
     if (cudaMalloc(&q, nbytes) != cudaSuccess) { cudaGetLastError(); return LL_ENOMEM; }
+#ifdef LL_CHECK   // a value that is read before it is written is NaN and shows
+    if (std::is_floating_point<U>::value || std::is_same<U, cplx<T>>::value || std::is_same<U, cplx<double>>::value)
+      if (cudaMemsetAsync(q, 0xff, nbytes, st_) != cudaSuccess) { cudaFree(q); return LL_ECUDA; }
+#endif
     ptrs_.push_back({q, nbytes});
     bytes_ += nbytes;
     *p = static_cast<U*>(q);

@@ -1114,6 +1114,7 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_op_proj(SphereD
       if (v < n) {
         const long o = base + (long)(b0 + v) * npw_pad + gi;
         const cplx<T> x = xin[o];
+        (void)LL_INB(gi < np || (acc[v].x == T(0) && acc[v].y == T(0)));   // the padding is zero
         nr += x.x * acc[v].x + x.y * acc[v].y;
         xout[o] = acc[v];
       }
