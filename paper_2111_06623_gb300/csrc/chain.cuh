@@ -441,10 +441,14 @@ static inline uint64_t ground_state_hash(const ll_system_desc* d) {
   return h;
 }
 
-// The bounds |m| <= PR the plane pass is built for at side W: W/4 (spheres whose products just
-// fit the grid), two ninths more at W = 48 (the sixteen-atom cell's |m| <= 13), and W/2 - 1, the
-// largest with unique signed indices.
-constexpr int plane_level(int w, int l) { return l == 0 ? w / 4 : l == 1 && w == 48 ? 14 : w / 2 - 1; }
+// The bounds |m| <= PR the lines are built for at side W: W/4, spheres whose products just fit the
+// grid; W/4 + 2, those of the same cut-off at k and Q inside the zone, each up to one index further;
+// W/2 - 1, the largest with unique signed indices.  Below W = 24 the second is within two of the
+// third, which serves for both.  us with the lines built for the tighter bound | for W/2 - 1: KB
+// workload on 32^3 (W/4) FP32 3517 | 3814, FP64 38578 | 44824; spheres that reach W/4 + 2, 64
+// k-points, 4 bands, per step, FP32, FP64: W = 24 71.0 | 71.6, 540 | 552; 32 126 | 129, 1112 | 1158;
+// 36 174 | 179, 2047 | 2204; 48 340 | 353, 4937 | 5364.
+constexpr int plane_level(int w, int l) { return l == 0 ? w / 4 : l == 1 && w >= 24 ? w / 4 + 2 : w / 2 - 1; }
 
 template <typename T>
 class Chain : public ChainBase {
@@ -1299,8 +1303,10 @@ class Chain : public ChainBase {
     const dim3 grid(nks_, nvec, (nbnd_ * hq_.ncol_max + kLines - 1) / kLines);
     if (prune_ == plane_level(N, 0))
       k_zfwd<T, N, plane_level(N, 0)><<<grid, kLines, 0, st_>>>(dq_, nbnd_, cbuf_, cb_ncol_, in, kin_, eps_, out);
-    else if (prune_ > 0 && prune_ == plane_level(N, 1))
+    else if (prune_ == plane_level(N, 1))
       k_zfwd<T, N, plane_level(N, 1)><<<grid, kLines, 0, st_>>>(dq_, nbnd_, cbuf_, cb_ncol_, in, kin_, eps_, out);
+    else if (prune_ == plane_level(N, 2))
+      k_zfwd<T, N, plane_level(N, 2)><<<grid, kLines, 0, st_>>>(dq_, nbnd_, cbuf_, cb_ncol_, in, kin_, eps_, out);
     else
       k_zfwd<T, N><<<grid, kLines, 0, st_>>>(dq_, nbnd_, cbuf_, cb_ncol_, in, kin_, eps_, out);
     return cudaGetLastError() == cudaSuccess ? LL_OK : LL_ECUDA;
@@ -1475,10 +1481,13 @@ class Chain : public ChainBase {
   int zinv_n(const SphereDev& s, const cplx<T>* in, int nvec) {
     // pruned where the spheres are the k+Q ones the bound holds for (not sphere(k) at set-up)
     const dim3 grid(nks_, nvec, zsplit());
-    if (s.col == dq_.col && prune_ == plane_level(N, 0))
+    const int pr = s.col == dq_.col ? prune_ : 0;
+    if (pr == plane_level(N, 0))
       k_zinv<T, N, plane_level(N, 0)><<<grid, 128, 0, st_>>>(s, in, nbnd_, cbuf_, cb_ncol_);
-    else if (s.col == dq_.col && prune_ > 0 && prune_ == plane_level(N, 1))
+    else if (pr == plane_level(N, 1))
       k_zinv<T, N, plane_level(N, 1)><<<grid, 128, 0, st_>>>(s, in, nbnd_, cbuf_, cb_ncol_);
+    else if (pr == plane_level(N, 2))
+      k_zinv<T, N, plane_level(N, 2)><<<grid, 128, 0, st_>>>(s, in, nbnd_, cbuf_, cb_ncol_);
     else
       k_zinv<T, N><<<grid, 128, 0, st_>>>(s, in, nbnd_, cbuf_, cb_ncol_);
     return cudaGetLastError() == cudaSuccess ? LL_OK : LL_ECUDA;

@@ -45,3 +45,20 @@ def test_fp32_application_with_tensor_core_projections(lib, nfft, ecut, monkeypa
     for upper in (False, True):
         _check(ch.apply(x, upper), _with_projectors(d, x, upper))
     ch.close()
+
+
+# side, cut-off, largest |m|: one beyond side/4, at side/4 + 2 and one beyond (the bounds of the lines)
+BOUNDS = [(24, 37.0, 7), (24, 48.0, 8), (24, 61.0, 9), (32, 61.0, 9), (32, 75.0, 10), (32, 91.0, 11), (36, 75.0, 10), (36, 90.0, 11),
+          (36, 108.0, 12), (48, 127.0, 13), (48, 147.0, 14), (48, 170.0, 15)]
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-12), ("fp32", 2e-5)])
+@pytest.mark.parametrize("nfft,ecut,mmax", BOUNDS)
+def test_line_bounds(lib, nfft, ecut, mmax, precision, tol, monkeypatch):  # noqa: F811
+    monkeypatch.setenv("LL_PRUNE", "1")
+    d, x = _system(ecut, nfft, nbnd=2)
+    assert max(abs(m).max() for m in d["miller_kq"]) == mmax
+    ch = lib.Chain(approx="rpa", precision=precision, max_steps=1, flavour="nh", **d)
+    for upper in (False, True):
+        _check(ch.apply(x, upper), _with_projectors(d, x, upper), tol)
+    ch.close()
