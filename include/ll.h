@@ -211,7 +211,8 @@ int ll_spectrum_static(const double* beta, const double* gamma, const double* z,
 /* One application of the SBR operator to a batch (Eqs. 24-28): out = (D + K) x when
  * upper != 0 (K omitted for IPA), out = D x otherwise, with D = P_c (H_{k+Q} - eps_{vk})
  * and the P_c of Eq. 16 on the output.  x and out are complex batches laid out per k as
- * [nbnd][npw_kq[k]] concatenated over k (host). */
+ * [nbnd][npw_kq[k]] concatenated over k (host).  Calls between ll_lanczos calls leave the recursion
+ * as it is.  LL_ETIMEOUT: a bounded wait in a kernel gave up, out is not valid. */
 int ll_apply(ll_handle* h, int upper, const double* x, double* out);
 
 /* Bit-exact index map: for each k, each Miller of sphere(k+Q) -> its position in sphere(k)

@@ -53,7 +53,7 @@ __device__ __forceinline__ constexpr bool line_kept(int p) {
 // grid (nks, nvec, split), block 128; item = (v, column), the k block's items spread over
 // the split CTAs.  PR > 0: every point of the spheres has |m| <= PR (PR < N/2), so a point's
 // offset is a compile-time constant and the zeros outside are known (PR = 0: any indices).
-// FP64 through fixed point (line_transform): KB workload 107 -> 54 us per launch, k_zfwd 146 -> 68.
+// FP64 through fixed point (line_transform): KB workload 107 -> 58 us per launch, k_zfwd 146 -> 71.
 template <typename T, int N, int PR = 0>
 __global__ void __launch_bounds__(128) k_zinv(SphereDev s, const cplx<T>* __restrict__ x, int nbnd,
                                               cplx<T>* __restrict__ cbuf, int cb_ncol) {
@@ -610,13 +610,6 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-template <typename T>
-__device__ __forceinline__ T warp_sum_t(T v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // Warp sums of NV values per lane at once (NV a power of two <= 32): at every step a lane keeps
 // half of its values and gives its partner the other half, so 32 values take 31 exchanges
 // instead of 5 each.  Returns the total of value number lane / (32 / NV).
@@ -894,21 +887,6 @@ __device__ __forceinline__ void flag_error(int* err, int code, int step) {
   if (atomicCAS(err, 0, code) == 0) err[1] = step;
 }
 
-// (1/n) sum_i p[i*stride + offset], i < n, by the whole block in a fixed order; every thread
-// gets the result.
-__device__ __forceinline__ double block_mean(const double* p, int n, int stride = 1, int offset = 0) {
-  __shared__ double wsum[32];
-  double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s += p[(long)i * stride + offset];
-  s = warp_sum(s);
-  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = s;
-  __syncthreads();
-  double t = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += wsum[w];
-  __syncthreads();
-  return t / n;
-}
-
 // Start of pseudo-Hermitian step j: the device step counter is advanced to j (so that a captured
 // step can be replayed), and beta_j from the n partials of Re(r_j^H X_j) in a fixed order;
 // scal = {beta_j, 1/beta_j} for the update kernels.  One block.  (Every CTA of the update
@@ -1045,10 +1023,10 @@ __global__ void __launch_bounds__(kLines) k_zfwd(SphereDev s, int nbnd, const cp
     }
 }
 
-// Threads of the per-k projection kernels: 512 where a band has more plane waves than two rounds
-// of 256 hold three times over (their loops then have few, long rounds of loads in flight: the
-// eight-atom cell has 1.7 CTAs per SM), else 256 (four CTAs per SM: the KB workload's 512
-// k-points are one wave).
+// Threads of the per-k projection kernels: 512 beyond three rounds of 256 (a band's 1632 plane waves
+// of the eight-atom cell are then four long rounds of loads in flight; it has 1.7 CTAs per SM), else
+// 256 (four CTAs per SM: the KB workload's 512 k-points of 570 plane waves are one wave).  In FP64
+// on the KB workload, us per launch at 128 | 256: k_op_proj 411 | 429, k_ph_update 176 | 170.
 static inline int proj_threads(int npw_pad) { return npw_pad > 768 ? 512 : 256; }
 
 // Last stage of the operator, for one group of bpc bands of one k-point (the KB and P_c terms act
@@ -1063,8 +1041,8 @@ static inline int proj_threads(int npw_pad) { return npw_pad > 768 ? 512 : 256; 
 // A kernel of its own: with the column transforms in front it needed 123 registers, two CTAs per
 // SM and 1.7 waves on the KB workload's 512 k-points, and shared memory for x and t.  Measured
 // (GB300, FP32, us per launch; the one kernel -> k_zfwd + this one): eight-atom cell (16 bands,
-// 1632 plane waves) 128 -> 27 + 79, KB workload (4 bands, 570) 61 -> 18 + 41, two-atom 10 Ry cell
-// (147) 15 -> 6 + 11.
+// 1632 plane waves) 128 -> 27 + 82, KB workload (4 bands, 570) 61 -> 19 + 42, two-atom 10 Ry cell
+// (147) 15 -> 6 + 9.
 template <typename T>
 __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_op_proj(SphereDev s, int nbnd, int bpc,
                                                    const cplx<T>* __restrict__ xin, const cplx<T>* __restrict__ ukq,

@@ -23,9 +23,9 @@
 // arithmetic (m mod W per point), 24-point lines left its warps partly filled, and its u(r) loads
 // waited on HBM inside the line loop.  With signed indices every point's offset is a compile-time
 // constant and its test one compare, W SL P threads fill their warps for W = 16, 24, 32, 48, and
-// the bulk copies are in flight two phases ahead: 62 / 90 / 53 us.  Eight-atom cell (W = 32):
-// 115 / 176 / 108 -> 63 / 127 / 61 us; sixteen-atom cell (W = 48): 1654 / 1969 / 1080 -> 843 /
-// 1009 / 650 us.
+// the bulk copies are in flight two phases ahead: 63 / 91 / 55 us.  Eight-atom cell (W = 32):
+// 115 / 176 / 108 -> 68 / 129 / 62 us; sixteen-atom cell (W = 48): 1654 / 1969 / 1080 -> 868 /
+// 1024 / 664 us.
 #pragma once
 #include "kernels.cuh"
 #include "tc.cuh"

@@ -15,7 +15,8 @@
 // one lane per line 2206 / 2478 / 1423, bound by the FP64 pipe; fixed point written out phase by
 // phase on one lane per line 867 / 2196 / 1142 (half the issue slots lost to instruction
 // fetch, six warps per SM in the modes with u(r)); shared transforms, two lanes per line 956 / 1166 /
-// 640; the pair's butterflies halved between the lanes (below) 757 / 936 / 565.  Two CTAs per SM:
+// 640; the pair's butterflies halved between the lanes (below) 757 / 936 / 565; one product per twiddled
+// input, every line shifted up again after its transform 748 / 944 / 592.  Two CTAs per SM:
 // the 96 registers that a third would leave spill 580 bytes per thread.
 #pragma once
 #include "plane.cuh"

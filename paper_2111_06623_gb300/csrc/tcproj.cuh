@@ -359,7 +359,7 @@ static inline int tc_apply_tiles(int nkv, int npw_pad, int nsm) {
 // next stage is split into the other.  One CTA per SM (coefficients 72 KB, tiles 48 KB, ring
 // 85 KB on the sixteen-atom cell), so it has 16 warps; the split, not HBM or the tensor pipe, is
 // what it spends its issue slots on.  Sixteen-atom cell, per launch (operator / update):
-// 269 / 111 us.
+// 274 / 115 us.
 static __global__ void __launch_bounds__(kTaThreads, 1) k_tc_apply(TcApplyArgs a) {
   extern __shared__ __align__(1024) unsigned char tsm[];
   __shared__ __align__(8) uint64_t bar[2];

@@ -21,13 +21,18 @@ import numpy as np
 sys.path.insert(0, {root!r})
 os.environ["LL_PRUNE"] = "1"
 from tests.test_gpu_fixed_lines import GRIDS
+from tests.test_gpu_far_q import FAR, WIDE, zones
 from tests.test_gpu_work_grid import _system
 from paper_2111_06623_gb300 import ll
+systems = [_system(e, n) for n, e in GRIDS] + [_system(e, n, q=(q, 0.2, 0.1)) for n, e, q in FAR]
+systems += [_system(e, n, q=q, nbnd=2) for n, e, q in WIDE[:3]]
+for n, e in ((12, 4.4), (18, 10.0), (24, 17.8), (48, 50.0)):
+    systems.append(_system(e, n))
+    zones(systems[-1][0])
 out = []
 for split in ("0", "1"):
     os.environ["LL_SPLIT_PERK"] = split
-    for nfft, ecut in GRIDS:
-        d, x = _system(ecut, nfft)
+    for d, x in systems:
         for prec in ("fp32", "fp64"):
             ch = ll.Chain(approx="rpa", precision=prec, flavour="nh", max_steps=2, **d)
             for up in (False, True):

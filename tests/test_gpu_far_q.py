@@ -47,18 +47,23 @@ def test_spheres_that_fill_the_grid(lib, nfft, ecut, q, precision):  # noqa: F81
         _check(got, _with_projectors(d, x, up), TOL[precision])
 
 
-@pytest.mark.parametrize("precision", ["fp64", "fp32"])
-@pytest.mark.parametrize("nfft,ecut", [(12, 4.4), (18, 10.0), (24, 17.8), (32, 20.0), (36, 40.0), (48, 50.0)])
-def test_k_points_in_different_zones(lib, nfft, ecut, precision):  # noqa: F811
-    """k-points given in different zones: no one shift fits, the general plane kernel (k_xy)."""
-    d, x = _system(ecut, nfft, nbnd=2)
-    b = 2 * np.pi * np.linalg.inv(d["lattice"]).T
+def zones(d):
+    """Some of the k-points given in other zones: no one index shift fits the spheres."""
+    n, b = d["nfft"], 2 * np.pi * np.linalg.inv(d["lattice"]).T
     d["kcart"] = d["kcart"].copy()
     for k in (1, 4, 6):
-        g = np.array([nfft, -nfft // 2, 3])
+        g = np.array([n, -n // 2, 3])
         d["kcart"][k] += g @ b
         for name in ("miller_k", "miller_kq"):
             d[name][k] = d[name][k] - g
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("nfft,ecut", [(12, 4.4), (18, 10.0), (24, 17.8), (32, 20.0), (36, 40.0), (48, 50.0)])
+def test_k_points_in_different_zones(lib, nfft, ecut, precision):  # noqa: F811
+    """The general plane kernel (k_xy)."""
+    d, x = _system(ecut, nfft, nbnd=2)
+    zones(d)
     for up, got in enumerate(_apply(lib, d, x, precision)):
         _check(got, _with_projectors(d, x, up), TOL[precision])
 
