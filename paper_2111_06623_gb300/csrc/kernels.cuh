@@ -661,11 +661,12 @@ __device__ __forceinline__ void dots_tile(const cplx<T>* __restrict__ A, long ld
     for (int j = 0; j < NJ; ++j) y[j] = pb[j][g];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
+      if (sizeof(T) == 4 || i < ni)   // (FP64: the pipe is what bounds the block)
 #pragma unroll
-      for (int j = 0; j < NJ; ++j) {
-        acc[(i * NJ + j) * 2] += x[i].x * y[j].x + x[i].y * y[j].y;
-        acc[(i * NJ + j) * 2 + 1] += x[i].x * y[j].y - x[i].y * y[j].x;
-      }
+        for (int j = 0; j < NJ; ++j) {
+          acc[(i * NJ + j) * 2] += x[i].x * y[j].x + x[i].y * y[j].y;
+          acc[(i * NJ + j) * 2 + 1] += x[i].x * y[j].y - x[i].y * y[j].x;
+        }
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (warp * 32 >= npw) return;   // a warp without plane waves
@@ -714,6 +715,7 @@ __device__ __forceinline__ void block_dots2(const cplx<T>* A0, const cplx<T>* B0
                                             const cplx<T>* A1, const cplx<T>* B1, int n1, long ld, int npw, int nj,
                                             cplx<double>* out, T* red) {
   if (nj == 1) block_dots_nj<T, 1>(A0, B0, n0, mult, A1, B1, n1, ld, npw, nj, out, red);
+  else if (nj == 2) block_dots_nj<T, 2>(A0, B0, n0, mult, A1, B1, n1, ld, npw, nj, out, red);
   else block_dots_nj<T, 4>(A0, B0, n0, mult, A1, B1, n1, ld, npw, nj, out, red);
 }
 template <typename T>
@@ -739,16 +741,16 @@ __device__ __forceinline__ void block_sum2(T re, T im, cplx<double>* out, T* red
   __syncthreads();
 }
 
-// acc[v] += sign sum_r M[r][g] C[r*ldc + v], v < 4, over nr rows of M (row stride ldm; C in shared
-// memory): every value of M is loaded once for four bands.
-template <typename T, int SIGN>
-__device__ __forceinline__ void rows_times(cplx<T> (&acc)[4], const cplx<T>* __restrict__ M, long ldm, int nr,
+// acc[v] += sign sum_r M[r][g] C[r*ldc + v], v < nv <= NV, over nr rows of M (row stride ldm; C in
+// shared memory): every value of M is loaded once for NV bands.
+template <typename T, int SIGN, int NV>
+__device__ __forceinline__ void rows_times(cplx<T> (&acc)[NV], const cplx<T>* __restrict__ M, long ldm, int nr,
                                            const cplx<T>* C, int ldc, int nv) {
 #pragma unroll 4
   for (int r = 0; r < nr; ++r) {
     const cplx<T> m = M[r * ldm];
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
+    for (int v = 0; v < NV; ++v) {
       const cplx<T> c = C[r * ldc + min(v, nv - 1)];
       if (SIGN > 0) {
         acc[v].x += m.x * c.x - m.y * c.y;
@@ -761,6 +763,18 @@ __device__ __forceinline__ void rows_times(cplx<T> (&acc)[4], const cplx<T>* __r
   }
 }
 
+// f(NV) with the block of bands that a thread takes per plane wave: four, and one or two for groups
+// of as many bands (a block of four would do four or two times their arithmetic: FP64, 8 k-points of
+// 4800 plane waves, groups of one band, us per step 481 with blocks of four, 291 so; 420 with the
+// pair-by-pair form before).
+template <int N> struct IntC { static constexpr int v = N; };
+template <typename F>
+__device__ __forceinline__ void band_blocks(int nv, F&& f) {
+  if (nv == 1) f(IntC<1>{});
+  else if (nv == 2) f(IntC<2>{});
+  else f(IntC<4>{});
+}
+
 // x[v][g] -= sum_w U[w][g] S[w][v] for nv orbitals x of one k against its nbnd occupied
 // states U (S = U^H x, nbnd x nv).  The coefficients are rounded to T once: conversions from
 // double run on the slow FP64 pipe.
@@ -771,17 +785,20 @@ __device__ __forceinline__ void subtract_projection(cplx<T>* x, const cplx<T>* _
   __shared__ cplx<T> St[NB * 32 * 32];
   for (int i = threadIdx.x; i < nbnd * nv; i += blockDim.x) St[i] = mk((T)S[i].x, (T)S[i].y);
   __syncthreads();
-  const int nb4 = (nv + 3) / 4;
-  for (int i = threadIdx.x; i < nb4 * npw_pad; i += blockDim.x) {
-    const int v0 = i / npw_pad * 4, gi = i % npw_pad, n = min(4, nv - v0);
-    cplx<T> acc[4];
+  band_blocks(nv, [&](auto nc) {
+    constexpr int NV = decltype(nc)::v;
+    const int nb = (nv + NV - 1) / NV;
+    for (int i = threadIdx.x; i < nb * npw_pad; i += blockDim.x) {
+      const int v0 = i / npw_pad * NV, gi = i % npw_pad, n = min(NV, nv - v0);
+      cplx<T> acc[NV];
 #pragma unroll
-    for (int v = 0; v < 4; ++v) acc[v] = v < n ? x[(long)(v0 + v) * npw_pad + gi] : czero<T>();
-    rows_times<T, -1>(acc, uk + gi, npw_pad, nbnd, St + v0, nv, n);
+      for (int v = 0; v < NV; ++v) acc[v] = v < n ? x[(long)(v0 + v) * npw_pad + gi] : czero<T>();
+      rows_times<T, -1>(acc, uk + gi, npw_pad, nbnd, St + v0, nv, n);
 #pragma unroll
-    for (int v = 0; v < 4; ++v)
-      if (v < n) x[(long)(v0 + v) * npw_pad + gi] = acc[v];
-  }
+      for (int v = 0; v < NV; ++v)
+        if (v < n) x[(long)(v0 + v) * npw_pad + gi] = acc[v];
+    }
+  });
   __syncthreads();
 }
 
@@ -1036,7 +1053,7 @@ static inline int proj_threads(int npw_pad) { return npw_pad > 768 ? 512 : 256; 
 // partial Re(z^H X)).
 // P_c of the KB term goes through the overlaps ub = U^H B of the set-up, S = U^H t + ub c, so
 // both dot blocks are formed on the same data and KB, P_c, the output and the norm partial
-// are one pass over the plane waves, four bands of a plane wave per thread (rows_times).
+// are one pass over the plane waves, a block of bands of a plane wave per thread (band_blocks).
 // grid (nks, nvec, ngrp), block proj_threads.  smem: coefficients, scratch.
 // A kernel of its own: with the column transforms in front it needed 123 registers, two CTAs per
 // SM and 1.7 waves on the KB workload's 512 k-points, and shared memory for x and t.  Measured
@@ -1078,25 +1095,28 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_op_proj(SphereD
       md.sp ? metal_operator_coefs(md, k, v0, nbnd, bpc, zp + (long)vec * nks * nbnd * nbnd, sf) : 0.0;
   for (int i = threadIdx.x; i < (nproj + nbnd) * bpc; i += blockDim.x) ct[i] = mk((T)cf[i].x, (T)cf[i].y);
   __syncthreads();
-  const int nb4 = (bpc + 3) / 4;
   T nr = T(0);
-  for (int i = threadIdx.x; i < nb4 * npw_pad; i += blockDim.x) {
-    const int b0 = i / npw_pad * 4, gi = i % npw_pad, n = min(4, bpc - b0);
-    cplx<T> acc[4];
+  band_blocks(bpc, [&](auto nc) {
+    constexpr int NV = decltype(nc)::v;
+    const int nb = (bpc + NV - 1) / NV;
+    for (int i = threadIdx.x; i < nb * npw_pad; i += blockDim.x) {
+      const int b0 = i / npw_pad * NV, gi = i % npw_pad, n = min(NV, bpc - b0);
+      cplx<T> acc[NV];
 #pragma unroll
-    for (int v = 0; v < 4; ++v) acc[v] = v < n ? ts[(b0 + v) * npw_pad + gi] : czero<T>();
-    rows_times<T, +1>(acc, bk + gi, npw_pad, nproj, ct + b0, bpc, n);
-    rows_times<T, -1>(acc, uk + gi, npw_pad, nbnd, ct + nproj * bpc + b0, bpc, n);
+      for (int v = 0; v < NV; ++v) acc[v] = v < n ? ts[(b0 + v) * npw_pad + gi] : czero<T>();
+      rows_times<T, +1>(acc, bk + gi, npw_pad, nproj, ct + b0, bpc, n);
+      rows_times<T, -1>(acc, uk + gi, npw_pad, nbnd, ct + nproj * bpc + b0, bpc, n);
 #pragma unroll
-    for (int v = 0; v < 4; ++v)
-      if (v < n) {
-        const long o = base + (long)(b0 + v) * npw_pad + gi;
-        const cplx<T> x = xin[o];
-        (void)LL_INB(gi < np || (acc[v].x == T(0) && acc[v].y == T(0)));   // the padding is zero
-        nr += x.x * acc[v].x + x.y * acc[v].y;
-        xout[o] = acc[v];
-      }
-  }
+      for (int v = 0; v < NV; ++v)
+        if (v < n) {
+          const long o = base + (long)(b0 + v) * npw_pad + gi;
+          const cplx<T> x = xin[o];
+          (void)LL_INB(gi < np || (acc[v].x == T(0) && acc[v].y == T(0)));   // the padding is zero
+          nr += x.x * acc[v].x + x.y * acc[v].y;
+          xout[o] = acc[v];
+        }
+    }
+  });
   block_sum2<T>(nr, T(0), cf, red);
   if (threadIdx.x == 0) part[((long)vec * nks + k) * ngrp + grp] = cf[0].x + corr;
 }

@@ -62,3 +62,21 @@ def test_line_bounds(lib, nfft, ecut, mmax, precision, tol, monkeypatch):  # noq
     for upper in (False, True):
         _check(ch.apply(x, upper), _with_projectors(d, x, upper), tol)
     ch.close()
+
+
+# bands, copies of the eight k-points: groups of 1, 2 (and 4 bands of the non-Hermitian update), 3 and 4
+# bands per CTA, and the bands that blocks of two and four leave over
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-12), ("fp32", 2e-5)])
+@pytest.mark.parametrize("nbnd,copies", [(1, 1), (2, 1), (3, 1), (5, 24), (6, 8), (9, 8), (12, 8), (13, 24)])
+def test_band_groups(lib, nbnd, copies, precision, tol):  # noqa: F811
+    for nproj in (1, 2, 6):
+        d, x = _system(5.5, 12, nbnd=nbnd, nproj=nproj)
+        for name in ("miller_k", "miller_kq", "u_k", "u_kq", "beta_kq"):
+            d[name] = d[name] * copies
+        d["kcart"], d["eps_k"] = (np.tile(d[name], (copies, 1)) for name in ("kcart", "eps_k"))
+        rng = np.random.default_rng(nbnd)
+        x = [v * rng.normal() for v in x * copies]
+        ch = lib.Chain(approx="rpa", precision=precision, max_steps=1, flavour="nh", **d)
+        for upper in (False, True):
+            _check(ch.apply(x, upper), _with_projectors(d, x, upper), tol)
+        ch.close()
