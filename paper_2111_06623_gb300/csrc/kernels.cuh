@@ -632,6 +632,18 @@ __device__ __forceinline__ T warp_sums(T (&v)[NV]) {
   return t;
 }
 
+// f(NV) with the block of bands (or of rows of a dot tile) that a thread takes per plane wave: four,
+// and one or two for groups of as many, which a block of four would make four or two times the
+// arithmetic.  FP64, 8 k-points of 4820 plane waves, groups of one band, us per step: blocks of four 481,
+// so 291, the pair-by-pair form before 420.
+template <int N> struct IntC { static constexpr int v = N; };
+template <typename F>
+__device__ __forceinline__ void band_blocks(int nv, F&& f) {
+  if (nv == 1) f(IntC<1>{});
+  else if (nv == 2) f(IntC<2>{});
+  else f(IntC<4>{});
+}
+
 // Dot blocks of the per-k kernels, in tiles of 4 x NJ pairs whose sums a thread keeps in registers
 // (4 + NJ loads per 4 NJ complex products); warp sums in T by halving exchange (warp_sums), warps
 // summed with DSum.  `red`: kRedPairs complex T per warp; the tiles fill it before the block
@@ -642,35 +654,34 @@ __device__ __forceinline__ T warp_sums(T (&v)[NV]) {
 constexpr int kRedPairs = 128;
 __host__ __device__ constexpr size_t red_elems(int threads) { return (size_t)(threads / 32) * 2 * kRedPairs; }
 
-template <typename T, int NJ>
+template <typename T, int NI, int NJ>
 __device__ __forceinline__ void dots_tile(const cplx<T>* __restrict__ A, long lda, const cplx<T>* B, long ldb, int npw,
                                           int ni, int nj, T* red) {
-  T acc[8 * NJ];   // [i][j][re, im]
+  T acc[2 * NI * NJ];   // [i][j][re, im]
 #pragma unroll
-  for (int q = 0; q < 8 * NJ; ++q) acc[q] = T(0);
-  const cplx<T>*pa[4], *pb[NJ];   // rows past the block's edge repeat its last one
+  for (int q = 0; q < 2 * NI * NJ; ++q) acc[q] = T(0);
+  const cplx<T>*pa[NI], *pb[NJ];   // rows past the block's edge repeat its last one
 #pragma unroll
-  for (int i = 0; i < 4; ++i) pa[i] = A + (long)min(i, ni - 1) * lda;
+  for (int i = 0; i < NI; ++i) pa[i] = A + (long)min(i, ni - 1) * lda;
 #pragma unroll
   for (int j = 0; j < NJ; ++j) pb[j] = B + (long)min(j, nj - 1) * ldb;
   for (int g = threadIdx.x; g < npw; g += blockDim.x) {
-    cplx<T> x[4], y[NJ];
+    cplx<T> x[NI], y[NJ];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) x[i] = pa[i][g];
+    for (int i = 0; i < NI; ++i) x[i] = pa[i][g];
 #pragma unroll
     for (int j = 0; j < NJ; ++j) y[j] = pb[j][g];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (sizeof(T) == 4 || i < ni)   // (FP64: the pipe is what bounds the block)
+    for (int i = 0; i < NI; ++i)
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-          acc[(i * NJ + j) * 2] += x[i].x * y[j].x + x[i].y * y[j].y;
-          acc[(i * NJ + j) * 2 + 1] += x[i].x * y[j].y - x[i].y * y[j].x;
-        }
+      for (int j = 0; j < NJ; ++j) {
+        acc[(i * NJ + j) * 2] += x[i].x * y[j].x + x[i].y * y[j].y;
+        acc[(i * NJ + j) * 2 + 1] += x[i].x * y[j].y - x[i].y * y[j].x;
+      }
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (warp * 32 >= npw) return;   // a warp without plane waves
-  constexpr int NV = 8 * NJ;
+  constexpr int NV = 2 * NI * NJ;
   const T t = warp_sums<T, NV>(acc);
   if (lane % (32 / NV) == 0) red[(long)warp * 2 * kRedPairs + lane / (32 / NV)] = t;
 }
@@ -690,8 +701,13 @@ __device__ __forceinline__ void block_dots_nj(const cplx<T>* A0, const cplx<T>* 
     for (int q = 0; q < n; ++q) {
       const bool first = b0 + q < t0n;
       const int t = first ? b0 + q : b0 + q - t0n, i0 = t / tj * 4, j0 = t % tj * NJ;
-      dots_tile<T, NJ>((first ? A0 : A1) + i0 * ld, ld, (first ? B0 : B1) + j0 * ld, ld, npw, (first ? n0 : n1) - i0,
-                       nj - j0, red + q * 2 * TP);
+      auto tile = [&](auto nc) {
+        dots_tile<T, decltype(nc)::v, NJ>((first ? A0 : A1) + i0 * ld, ld, (first ? B0 : B1) + j0 * ld, ld, npw,
+                                          (first ? n0 : n1) - i0, nj - j0, red + q * 2 * TP);
+      };
+      // (FP64: the pipe bounds the block, so that no row is done for nothing)
+      if constexpr (sizeof(T) == 8) band_blocks((first ? n0 : n1) - i0, tile);
+      else tile(IntC<4>{});
     }
     __syncthreads();
     for (int e = threadIdx.x; e < 2 * n * TP; e += blockDim.x) {   // a component of a pair
@@ -761,18 +777,6 @@ __device__ __forceinline__ void rows_times(cplx<T> (&acc)[NV], const cplx<T>* __
       }
     }
   }
-}
-
-// f(NV) with the block of bands that a thread takes per plane wave: four, and one or two for groups
-// of as many bands (a block of four would do four or two times their arithmetic: FP64, 8 k-points of
-// 4800 plane waves, groups of one band, us per step 481 with blocks of four, 291 so; 420 with the
-// pair-by-pair form before).
-template <int N> struct IntC { static constexpr int v = N; };
-template <typename F>
-__device__ __forceinline__ void band_blocks(int nv, F&& f) {
-  if (nv == 1) f(IntC<1>{});
-  else if (nv == 2) f(IntC<2>{});
-  else f(IntC<4>{});
 }
 
 // x[v][g] -= sum_w U[w][g] S[w][v] for nv orbitals x of one k against its nbnd occupied
