@@ -724,8 +724,8 @@ class Chain : public ChainBase {
       // fewer bands per CTA where the k-points alone leave SMs idle (the groups re-read U and B from
       // L2, which costs less than the idle SMs): us per call, all bands -> this rule -> with blocks of as
       // many bands (band_blocks): two-atom cell (64 k-points, 4 bands, groups of 1) FP32 492 -> 471,
-      // FP64 3118 -> 3031 -> 2693; semimetal (6 bands, of 2) 668 -> 641 -> 609; smallest cell (8
-      // k-points, of 1) 2000 -> 1792 -> 1780
+      // FP64 3118 -> 3031 -> 2672; semimetal (6 bands, of 2) 668 -> 641 -> 602; smallest cell (8
+      // k-points, of 1) 2000 -> 1792 -> 1732
       for (int b = bpc_ - 1; !split_ && b >= 1 && (long)nks_ * ngrp_ < nsm_; --b)
         if (nbnd_ % b == 0) bpc_ = b, ngrp_ = nbnd_ / b;
       nchunk_ = split_ ? (pq + kChunk - 1) / kChunk : 1;

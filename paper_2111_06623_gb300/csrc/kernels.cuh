@@ -1062,7 +1062,7 @@ static inline int proj_threads(int npw_pad) { return npw_pad > 768 ? 512 : 256; 
 // A kernel of its own: with the column transforms in front it needed 123 registers, two CTAs per
 // SM and 1.7 waves on the KB workload's 512 k-points, and shared memory for x and t.  Measured
 // (GB300, FP32, us per launch; the one kernel -> k_zfwd + this one): eight-atom cell (16 bands,
-// 1632 plane waves) 128 -> 27 + 82, KB workload (4 bands, 570) 61 -> 19 + 42, two-atom 10 Ry cell
+// 1632 plane waves) 128 -> 27 + 77, KB workload (4 bands, 570) 61 -> 19 + 40, two-atom 10 Ry cell
 // (147) 15 -> 6 + 9.
 template <typename T>
 __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_op_proj(SphereDev s, int nbnd, int bpc,
